@@ -95,8 +95,9 @@ typedef struct {
                           * in 32-byte pieces (SPMV_SPMM_*): AUTO = tuned when autotune is on,
                           * else the measured default (UNROLLED).  Every form gives the same
                           * bits. */
-    int pq_ctas;         /* CG product grid: CTAs per SM (0 = tuned when autotune is on, else
-                          * 4; 2..4 explicit).  The grid fixes the reduction order of p.q. */
+    int pq_ctas;         /* CG product grid: at most this many times 256 threads per SM (0 =
+                          * tuned when autotune is on, else 4; 2..4 explicit).  The grid fixes
+                          * the reduction order of p.q. */
     int pq_unroll;       /* CG product entries in flight per lane: 0 = tuned / automatic, 2, 5 */
     int gather_bytes;    /* cg_solve_multi: bytes of a row of P each product lane gathers
                           * (0 = tuned when autotune is on, else 32; 16 or 32) */
@@ -182,7 +183,7 @@ typedef struct {
     int32_t spmm_form[2][4]; /* SPMV_SPMM_* used by the multi-vector product, per precision
                               * (0 FP64, 1 FP32) and lanes per row (1, 2, 4, 8: k = 4, 8, 16,
                               * 32 FP64 or 8, 16, 32, 64 FP32) */
-    int32_t pq_ctas;         /* CG product grid: CTAs per SM                        */
+    int32_t pq_ctas;         /* CG product grid: 256-thread units per SM            */
     int32_t pq_unroll;       /* CG product entries in flight per lane (FP64 handle)  */
     int32_t gather_bytes;    /* cg_solve_multi product: bytes gathered per lane      */
     int32_t chain_form[2];   /* SPMV_CHAIN_* of spmv_apply_chain(_f32) with this B      */

@@ -4,14 +4,18 @@
 //
 // One CG iteration is three kernels, each a grid-stride sweep over a fixed grid (the product
 // over a grid of its own, see cg_pq_grid):
-//   cg_spmv_pq   q = A p and p.q                      -> alpha = rho / (p.q)
-//   cg_update_xr x += alpha p, r -= alpha q, r.(D^-1 r), r.r -> beta, rho, convergence
-//   cg_update_p  p = D^-1 r + beta p
-// Every kernel ends with a deterministic reduction: each CTA writes its partial sums, the
-// last CTA to arrive (atomic ticket) reduces all partials in a fixed order and computes the
-// scalars the next kernel reads.  Results therefore do not depend on CTA scheduling.  A
-// "done" flag set by that last CTA turns the remaining kernels of a CUDA-graph batch into
-// no-ops, so the host only checks convergence once per batch of iterations.
+//   cg_spmv_pq   q = A p, partial p.q
+//   cg_update_xr alpha = rho / (p.q); x += alpha p, r -= alpha q, partial r.(D^-1 r), r.r
+//   cg_update_p  beta, rho, convergence; p = D^-1 r + beta p
+// The reductions are deterministic: each CTA writes its partial sums, and every CTA of the next
+// kernel adds all of them in one fixed order (reduce_parts), so results do not depend on CTA
+// scheduling.  Measured against a last-CTA reduction at the end of every kernel (atomic ticket,
+// four 256-thread CTAs per SM, plain launches), per FP64 iteration of a CUDA-graph batch: 10K
+// rows 16.9 -> 7.7 us, 48K 17.3 -> 8.5, 304K 24.1 -> 15.5, 1M 44.6 -> 36.6, 6M 175.0 -> 167.0;
+// FP32 6M 76.2 -> 71.8, 1M 28.9 -> 18.7.  Each kernel is a programmatic dependent of the one before: its CTAs start as
+// the previous kernel's leave, request what no kernel of the solve writes (matrix, D^-1) and
+// then wait.  A "done" flag turns the remaining kernels of a CUDA-graph batch into no-ops, so
+// the host only checks convergence once per batch of iterations.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -97,96 +101,162 @@ cg_residual(int32_t n, int32_t n_slices, const int64_t *sp, ColT col, const T *v
     }
 }
 
-// q = A p; partial p.q; last CTA: alpha = rho / (p.q).  Grid cg_pq_grid (see cgkern.cuh).
-// UU: entries in flight per lane (pq_unroll, or 2 for matrices whose widest slice needs fewer
-// load rounds that way; the per-row order, hence the result, is the same).
+// q = A p and the CTA's partial p.q.  Grid cg_pq_grid (see cgkern.cuh).  UU: entries in flight
+// per lane (pq_unroll, or 2 for matrices whose widest slice needs fewer load rounds that way;
+// the per-row order, hence the result, is the same).  The first round of matrix entries is
+// requested before the previous kernel (which finishes p) has ended.
 template <typename T, int R, int L, typename ColT, int UU>
-__global__ void __launch_bounds__(kCgBlock, pq_min_ctas((int)sizeof(T) * R))
-cg_spmv_pq(int32_t n, int32_t n_slices, const int64_t *sp, ColT col, const T *val,
+__global__ void __launch_bounds__(kCgBlock * pq_min_ctas((int)sizeof(T) * R))
+cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, const int64_t *sp, ColT col, const T *val,
            const T *p, T *q, double *part, CgScalars *sc) {
-    // start the first slice's pointer loads while the stop flag is read, so that memory
-    // traffic begins at once (a CTA would otherwise wait a full round trip for the flag)
-    const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g0 < (int64_t)n_slices * L) {
-        prefetch_l1(sp + g0 / L);
-        prefetch_l1(sp + g0 / L + 1);
-        prefetch_col_base(col, g0 / L);
-    }
-    if (sc->done) return;
-    constexpr int S = L * R;
     const uint64_t pol = policy_evict_first();
-    const int64_t lanes = (int64_t)gridDim.x * blockDim.x;
+    const int64_t g0 = iter_begin(chunk), end = iter_end(chunk, (int64_t)n_slices * L);
+    // lanes of 64 bytes per entry have no registers for a round held across the wait
+    constexpr bool kEarly = sizeof(T) * R <= 32;
+    SliceLane s{};
+    SliceRound<T, R, UU> rd;
+    if constexpr (kEarly) {
+        if (g0 < end) {
+            s = slice_open<R, L>(g0, sp, col);
+            if (s.w >= UU) rd.template load<L>(s, 0, col, val, pol);
+        }
+    }
+    dep_wait();
+    dep_allow();
+    const int done = sc->done;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->cur_rho = sc->rho;
+        sc->cur_iters = sc->iters;
+        sc->cur_done = done;
+    }
+    if (done) return;
     T vt = T(0);
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < (int64_t)n_slices * L;
-         g += lanes) {
-        const int64_t slice = g / L;
-        const int lane = (int)(g % L);
+    for (int64_t g = g0; g < end; g += blockDim.x) {
         T acc[R];
-        slice_rows<T, R, L, false, UU>(slice, lane, sp, col, val, p, pol, acc);
-        const int64_t row0 = slice * S + (int64_t)lane * R;
+        if constexpr (kEarly) {
+            if (g != g0) {
+                s = slice_open<R, L>(g, sp, col);
+                if (s.w >= UU) rd.template load<L>(s, 0, col, val, pol);
+            }
+            slice_multiply<T, R, L, false, UU>(s, rd, col, val, p, pol, acc);
+        } else {
+            slice_rows<T, R, L, false, UU>(g / L, (int)(g % L), sp, col, val, p, pol, acc);
+        }
+        const int64_t row0 = g * R;
         store_rows<T, R>(q, row0, n, acc);
 #pragma unroll
         for (int i = 0; i < R; ++i)
             if (row0 + i < n) vt = fma_t(p[row0 + i], acc[i], vt);
     }
     double v[1] = {(double)vt};
-    double tot[1];
-    if (grid_sum_last<1>(v, part, &sc->tickets[1], tot) && threadIdx.x == 0) {
-        if (tot[0] == 0.0 || !isfinite(tot[0])) {
-            sc->done = 3;
+    store_parts<1>(v, part);
+}
+
+// alpha = rho / (p.q) from the product's partials; x += alpha p; r -= alpha q; the CTA's partial
+// r.(D^-1 r) and r.r.  ONE: the grid has a thread for every vector, whose loads then travel with
+// those of the partials (one round trip); otherwise the sweep's own loads overlap each other.
+template <typename T, bool ONE>
+__global__ void __launch_bounds__(kIterThreads)
+cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const T *dinv,
+             const double *pq_part, int pq_count, double *part, CgScalars *sc) {
+    constexpr int V = Vec16<T>::n;
+    const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
+    const bool mine = k0 < end && k0 < n / V;
+    XrVec<T> v;
+    if (mine) {
+        if (ONE) v.load_d(dinv, k0 * V);
+        else prefetch_l1(dinv + k0 * V);
+    }
+    dep_wait();
+    dep_allow();
+    const uint64_t pol = policy_evict_first();
+    if (mine) {
+        if (ONE) {
+            v.load(x, r, p, q, k0 * V, pol);
         } else {
-            sc->alpha = sc->rho / tot[0];
+            prefetch_l1(x + k0 * V);
+            prefetch_l1(r + k0 * V);
+            prefetch_l1(p + k0 * V);
+            prefetch_l1(q + k0 * V);
         }
     }
-}
-
-// x += alpha p; r -= alpha q; partials r.(D^-1 r), r.r; last CTA: beta, rho, convergence
-template <typename T>
-__global__ void __launch_bounds__(kCgBlock)
-cg_update_xr(int32_t n, T *x, T *r, const T *p, const T *q, const T *dinv, double *part,
-             CgScalars *sc) {
-    // the first vectors of the sweep and the scalars are requested together (one round trip)
-    const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * Vec16<T>::n;
-    if (i0 < n) {
-        prefetch_l1(x + i0);
-        prefetch_l1(r + i0);
-        prefetch_l1(p + i0);
-        prefetch_l1(q + i0);
-        prefetch_l1(dinv + i0);
+    if (sc->cur_done) return;
+    __shared__ StepScalars<T> step;
+    if (threadIdx.x < 32) {
+        const double pq = reduce_parts(pq_part, pq_count);
+        if (threadIdx.x == 0) step_alpha(sc->cur_rho, pq, step);
     }
-    const int done = sc->done;
-    const T alpha = (T)sc->alpha;
-    if (done) return;
+    __syncthreads();
+    if (step.done) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) sc->broke = 1;
+        return;
+    }
+    const T alpha = step.coef;
     T vz = T(0), vr = T(0);
-    sweep_update_xr<T>(n, alpha, x, r, p, q, dinv, vz, vr);
-    double v[2] = {(double)vz, (double)vr};
-    double tot[2];
-    if (grid_sum_last<2>(v, part, &sc->tickets[2], tot) && threadIdx.x == 0) {
-        const double rho_new = tot[0];
-        sc->beta = rho_new / sc->rho;
-        sc->rho = rho_new;
-        sc->rr = tot[1];
-        sc->iters += 1;
-        if (tot[1] <= sc->tol2 * sc->bb) sc->done = 1;
-        else if (!isfinite(tot[1])) sc->done = 3;
-        else if (sc->iters >= sc->max_iter) sc->done = 2;
-    }
+    if (ONE && mine) v.update(alpha, x, r, k0 * V, pol, vz, vr);
+    else sweep_update_xr<T>(n, k0, end, blockDim.x, alpha, x, r, p, q, dinv, vz, vr);
+    double t[2] = {(double)vz, (double)vr};
+    store_parts<2>(t, part);
 }
 
-// p = D^-1 r + beta p
-template <typename T>
-__global__ void __launch_bounds__(kCgBlock)
-cg_update_p(int32_t n, const T *r, const T *dinv, T *p, const CgScalars *sc) {
-    const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * Vec16<T>::n;
-    if (i0 < n) {
-        prefetch_l1(r + i0);
-        prefetch_l1(dinv + i0);
-        prefetch_l1(p + i0);
+// beta, rho and the convergence test from the x/r update's partials; p = D^-1 r + beta p.  ONE as
+// in cg_update_xr.
+template <typename T, bool ONE>
+__global__ void __launch_bounds__(kIterThreads)
+cg_update_p(int32_t n, int64_t chunk, const T *r, const T *dinv, T *p, const double *part,
+            int count, CgScalars *sc) {
+    constexpr int V = Vec16<T>::n;
+    const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
+    const bool mine = k0 < end && k0 < n / V;
+    const uint64_t pol = policy_evict_first();
+    PVec<T> v;
+    if (mine) {
+        if (ONE) v.load_d(dinv, k0 * V, pol);
+        else prefetch_l1(dinv + k0 * V);
     }
-    const int done = sc->done;
-    const T beta = (T)sc->beta;
-    if (done) return;
-    sweep_update_p<T>(n, beta, r, dinv, p);
+    dep_wait();
+    dep_allow();
+    if (mine) {
+        if (ONE) {
+            v.load(r, p, k0 * V, pol);
+        } else {
+            prefetch_l1(r + k0 * V);
+            prefetch_l1(p + k0 * V);
+        }
+    }
+    const bool first_cta = blockIdx.x == 0;
+    if (sc->cur_done) return;
+    if (sc->broke) {
+        if (first_cta && threadIdx.x == 0) sc->done = 3;
+        return;
+    }
+    __shared__ StepScalars<T> step;
+    if (threadIdx.x < 32) {  // warp 0: r.z, beta
+        const double rz = reduce_parts(part, count);
+        if (threadIdx.x == 0) {
+            step_beta(sc->cur_rho, rz, step);
+            if (first_cta) {
+                sc->beta = (double)step.coef;
+                sc->rho = rz;
+            }
+        }
+    } else if (threadIdx.x < 64) {  // warp 1: r.r, convergence
+        const double rr = reduce_parts(part + count, count);
+        if (threadIdx.x == 32) {
+            const int iters = sc->cur_iters + 1;
+            step.done = step_done(rr, sc->tol2 * sc->bb, iters, sc->max_iter);
+            if (first_cta) {
+                sc->rr = rr;
+                sc->iters = iters;
+                sc->done = step.done;
+            }
+        }
+    }
+    __syncthreads();
+    if (step.done) return;
+    const T beta = step.coef;
+    if (ONE && mine) v.update(beta, p, k0 * V);
+    else sweep_update_p<T>(n, k0, end, blockDim.x, beta, r, dinv, p);
 }
 
 // refinement: right-hand side of the inner solve r32 = fp32(r64 / ||r64||), start of the
@@ -231,8 +301,8 @@ __global__ void set_scalars(CgScalars *sc, double tol2, int max_iter) {
     sc->max_iter = max_iter;
     sc->iters = 0;
     sc->done = 0;
+    sc->broke = 0;
     for (int k = 0; k < 4; ++k) sc->tickets[k] = 0u;
-    sc->bar_count = 0u;
     sc->budget_ns = 0;
 }
 
@@ -240,15 +310,26 @@ __global__ void add_iters(CgScalars *inner, int *total) { *total += inner->iters
 
 }  // namespace
 
-// Grid of the CG product q = A p: one thread per slice-lane, at most the handle's pq_ctas CTAs
-// per SM (tuned, or set by option; default pq_min_ctas).  The grid fixes the order of the p.q
-// reduction, so it is a property of the handle, shared by the graph path and the persistent
-// kernel (which runs it as virtual CTAs): both give identical results.
-int cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes) {
-    const int per_sm = A->pq_ctas > 0 ? A->pq_ctas : pq_min_ctas(value_bytes);
-    const int64_t cap = (int64_t)device_facts().sm_count * per_sm;
-    const int64_t want = ((int64_t)A->n_slices * L + kCgBlock - 1) / kCgBlock;
-    return (int)(want < 1 ? 1 : (want > cap ? cap : want));
+IterGrid cg_iter_grid(int64_t items, int max_threads) {
+    const int sms = std::min(device_facts().sm_count, 32 * kPartLoads);
+    IterGrid g;
+    g.chunk = std::max<int64_t>(64, ((items + sms - 1) / sms + 31) / 32 * 32);
+    g.threads = (int)std::min<int64_t>(max_threads, g.chunk);
+    g.ctas = (int)std::max<int64_t>(1, (items + g.chunk - 1) / g.chunk);
+    return g;
+}
+
+// Grid of the CG product q = A p: at most 256 threads per unit of the handle's pq_ctas (tuned, or
+// set by option; default pq_min_ctas).
+IterGrid cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes) {
+    const int units = std::min(A->pq_ctas > 0 ? A->pq_ctas : 4, pq_min_ctas(value_bytes));
+    return cg_iter_grid((int64_t)A->n_slices * L, kCgBlock * units);
+}
+
+// Grid of the CG sweeps over 16-byte vectors of `vec` rows (counted to the end of the last slice,
+// so that it is the product's grid where a slice-lane is such a vector).
+IterGrid cg_sweep_grid(const spmv_matrix_t A, int vec) {
+    return cg_iter_grid((int64_t)A->n_slices * (A->S / vec), kIterThreads);
 }
 
 // Entries the product keeps in flight per lane: the handle's pq_unroll (tuned, or set by
@@ -259,20 +340,9 @@ bool cg_pq_deep(const spmv_matrix_t A, int uu) {
     return load_rounds(A->max_width, uu) < load_rounds(A->max_width, 2);
 }
 
-// (lanes per slice, value bytes per lane entry) of the FP64 and FP32 product kernels for a
-// slice height, as with_shape picks them
-static int pq_grid64(const spmv_matrix_t A) {
-    return cg_pq_grid(A, 32, 8 * (A->S / 32));
-}
-static int pq_grid32(const spmv_matrix_t A) {
-    const int L = A->S / 4 < 32 ? A->S / 4 : 32;
-    return cg_pq_grid(A, L, 4 * (A->S / L));
-}
-
-// Grid of the CG sweeps of a matrix with n rows: about 1,024 rows (4 per thread) per CTA, at
-// most kCgCtasPerSm CTAs per SM (the persistent kernel uses the same grid).  It depends only
-// on n and the device, so the reduction order is fixed per handle and both paths give
-// identical results; small systems use fewer CTAs and leave room for concurrent solves.
+// Grid of the kernels around the iteration: about 1,024 rows (4 per thread) per CTA, at most
+// kCgCtasPerSm CTAs per SM.  It depends only on n and the device, so the reduction order is fixed
+// per handle.
 int cg_grid(int32_t n) {
     const int cap = device_facts().sm_count * kCgCtasPerSm;
     const int64_t want = ((int64_t)n + 1023) / 1024;
@@ -284,11 +354,11 @@ spmv_status_t ensure_cg_work(spmv_matrix_t A, bool mixed, cudaStream_t st) {
     size_t *t = &A->bytes;
     const size_t n = (size_t)A->n;
     if (!w.ready) {
-        const int G = cg_grid(A->n);
+        // the product's p.q partials, then the sweeps' (kMaxParts per CTA of the largest grid,
+        // that of the kernels around the iteration)
+        const int G = std::max(cg_grid(A->n), 32 * kPartLoads);
         w.part_len = G;
-        // the product's p.q partials (room for the largest grid any pq_ctas gives), then
-        // kMaxParts partials per CTA of the sweeps
-        w.pq_len = device_facts().sm_count * 4;
+        w.pq_len = 32 * kPartLoads;
         GB_TRY(w.part.alloc((size_t)w.pq_len + (size_t)G * kMaxParts * 2, t));
         GB_TRY(w.scal.alloc(2 * ((sizeof(CgScalars) + 7) / 8), t));
         GB_CUDA(cudaMemsetAsync(w.scal.p, 0, w.scal.n * sizeof(double), st));
@@ -332,35 +402,64 @@ static spmv_status_t with_cols(spmv_matrix_t A, F &&f) {
     return f(Cols32{A->sell_col.p});
 }
 
-// enqueue `iters` FP64 iterations (3 kernels each)
-static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st) {
-    CgWork &w = A->cg;
-    const int G = cg_grid(A->n);
-    CgScalars *sc = outer_scalars(A);
+// the product, the x/r sweep and the p sweep of an iteration (pq_count: CTAs of the product)
+template <typename T>
+static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q, CgScalars *sc,
+                                cudaStream_t st, int *pq_count) {
     return with_cols(A, [&](auto cols) -> spmv_status_t {
         using ColT = decltype(cols);
-        return with_shape(A->S, false, [&](auto rt, auto lt) -> spmv_status_t {
+        return with_shape<T>(A->S, [&](auto rt, auto lt) -> spmv_status_t {
             constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
-            const int Gpq = pq_grid64(A);
-            constexpr int UU = pq_unroll(8 * R);
-            const bool deep = cg_pq_deep(A, UU);
-            for (int it = 0; it < iters; ++it) {
-                if (deep)
-                    cg_spmv_pq<double, R, L, ColT, UU><<<Gpq, kCgBlock, 0, st>>>(
-                        A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.p.p, w.q.p,
-                        w.part.p, sc);
-                else
-                    cg_spmv_pq<double, R, L, ColT, 2><<<Gpq, kCgBlock, 0, st>>>(
-                        A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.p.p, w.q.p,
-                        w.part.p, sc);
-                cg_update_xr<double><<<G, kCgBlock, 0, st>>>(A->n, w.x.p, w.r.p, w.p.p, w.q.p,
-                                                             w.dinv.p, w.part.p + w.pq_len, sc);
-                cg_update_p<double><<<G, kCgBlock, 0, st>>>(A->n, w.r.p, w.dinv.p, w.p.p, sc);
-            }
-            GB_LAUNCHED();
-            return SPMV_OK;
+            constexpr int UU = pq_unroll((int)sizeof(T) * R);
+            const IterGrid g = cg_pq_grid(A, L, (int)sizeof(T) * R);
+            *pq_count = g.ctas;
+            return launch_dependent(cg_pq_deep(A, UU) ? cg_spmv_pq<T, R, L, ColT, UU>
+                                                      : cg_spmv_pq<T, R, L, ColT, 2>,
+                                    g.ctas, g.threads, st, A->n, A->n_slices, g.chunk,
+                                    A->slice_ptr.p, cols, val, p, q, A->cg.part.p, sc);
         });
     });
+}
+template <typename T>
+static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const T *p, const T *q,
+                                const T *dinv, CgScalars *sc, cudaStream_t st) {
+    constexpr int V = Vec16<T>::n;
+    const IterGrid g = cg_sweep_grid(A, V);
+    return launch_dependent(g.single() ? cg_update_xr<T, true> : cg_update_xr<T, false>, g.ctas,
+                            g.threads, st, A->n, g.chunk, x, r, p, q, dinv, A->cg.part.p,
+                            pq_count, A->cg.part.p + A->cg.pq_len, sc);
+}
+template <typename T>
+static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p, CgScalars *sc,
+                               cudaStream_t st) {
+    constexpr int V = Vec16<T>::n;
+    const IterGrid g = cg_sweep_grid(A, V);
+    return launch_dependent(g.single() ? cg_update_p<T, true> : cg_update_p<T, false>, g.ctas,
+                            g.threads, st, A->n, g.chunk, r, dinv, p,
+                            A->cg.part.p + A->cg.pq_len, g.ctas, sc);
+}
+template <typename T>
+static spmv_status_t enqueue_iterations(spmv_matrix_t A, int iters, const T *val, T *x, T *r, T *p,
+                                        T *q, const T *dinv, CgScalars *sc, cudaStream_t st) {
+    for (int it = 0; it < iters; ++it) {
+        int pq_count = 0;
+        GB_TRY(enqueue_pq<T>(A, val, p, q, sc, st, &pq_count));
+        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, st));
+        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, st));
+    }
+    return SPMV_OK;
+}
+
+// enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each)
+static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st) {
+    CgWork &w = A->cg;
+    return enqueue_iterations<double>(A, iters, A->sell_val.p, w.x.p, w.r.p, w.p.p, w.q.p,
+                                      w.dinv.p, outer_scalars(A), st);
+}
+static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st) {
+    CgWork &w = A->cg;
+    return enqueue_iterations<float>(A, iters, A->sell_val32.p, w.d32.p, w.r32.p, w.p32.p, w.q32.p,
+                                     w.dinv32.p, inner_scalars(A), st);
 }
 
 __global__ void fill_value(int32_t n, double *v, double value) {
@@ -369,29 +468,7 @@ __global__ void fill_value(int32_t n, double *v, double value) {
         v[i] = value;
 }
 
-// one FP64 product q = A p with p.q (the first kernel of an iteration), on scalar block sc
-static spmv_status_t enqueue_pq64(spmv_matrix_t A, CgScalars *sc, cudaStream_t st) {
-    CgWork &w = A->cg;
-    return with_cols(A, [&](auto cols) -> spmv_status_t {
-        using ColT = decltype(cols);
-        return with_shape(A->S, false, [&](auto rt, auto lt) -> spmv_status_t {
-            constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
-            constexpr int UU = pq_unroll(8 * R);
-            if (cg_pq_deep(A, UU))
-                cg_spmv_pq<double, R, L, ColT, UU><<<pq_grid64(A), kCgBlock, 0, st>>>(
-                    A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.p.p, w.q.p,
-                    w.part.p, sc);
-            else
-                cg_spmv_pq<double, R, L, ColT, 2><<<pq_grid64(A), kCgBlock, 0, st>>>(
-                    A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.p.p, w.q.p,
-                    w.part.p, sc);
-            GB_LAUNCHED();
-            return SPMV_OK;
-        });
-    });
-}
-
-// Tuner of the CG product: its grid (2, 3 or 4 CTAs per SM) and the entries each lane keeps in
+// Tuner of the CG product: its grid (2, 3 or 4 times 256 threads per SM) and the entries each lane keeps in
 // flight (2 or 5).  Each candidate computes q = A p with p = 1 (the gathers and multiply-adds
 // of a solve; the scalars go to the inner block, which every solve resets before use), timed
 // as the median of three launches each after writing a buffer of twice the L2 size, as in
@@ -424,7 +501,9 @@ static spmv_status_t tune_cg_product(spmv_matrix_t A, cudaStream_t st) {
                 s = cuda_status(cudaGetLastError());
                 if (s == SPMV_OK) s = cuda_status(cudaMemsetAsync(flush, i + 2, fb, st));
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e0, st));
-                if (s == SPMV_OK) s = enqueue_pq64(A, sc, st);
+                int count = 0;
+                if (s == SPMV_OK)
+                    s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, st, &count);
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e1, st));
                 if (s == SPMV_OK) s = cuda_status(cudaEventSynchronize(e1));
                 if (s == SPMV_OK && i >= 0) s = cuda_status(cudaEventElapsedTime(&t[i], e0, e1));
@@ -446,37 +525,6 @@ static spmv_status_t tune_cg_product(spmv_matrix_t A, cudaStream_t st) {
     return s;
 }
 
-static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st) {
-    CgWork &w = A->cg;
-    const int G = cg_grid(A->n);
-    CgScalars *sc = inner_scalars(A);
-    return with_cols(A, [&](auto cols) -> spmv_status_t {
-        using ColT = decltype(cols);
-        return with_shape(A->S, true, [&](auto rt, auto lt) -> spmv_status_t {
-            constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
-            const int Gpq = pq_grid32(A);
-            constexpr int UU = pq_unroll(4 * R);
-            const bool deep = cg_pq_deep(A, UU);
-            for (int it = 0; it < iters; ++it) {
-                if (deep)
-                    cg_spmv_pq<float, R, L, ColT, UU><<<Gpq, kCgBlock, 0, st>>>(
-                        A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val32.p, w.p32.p,
-                        w.q32.p, w.part.p, sc);
-                else
-                    cg_spmv_pq<float, R, L, ColT, 2><<<Gpq, kCgBlock, 0, st>>>(
-                        A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val32.p, w.p32.p,
-                        w.q32.p, w.part.p, sc);
-                cg_update_xr<float><<<G, kCgBlock, 0, st>>>(A->n, w.d32.p, w.r32.p, w.p32.p,
-                                                            w.q32.p, w.dinv32.p,
-                                                            w.part.p + w.pq_len, sc);
-                cg_update_p<float><<<G, kCgBlock, 0, st>>>(A->n, w.r32.p, w.dinv32.p, w.p32.p, sc);
-            }
-            GB_LAUNCHED();
-            return SPMV_OK;
-        });
-    });
-}
-
 // r = b - A x on the FP64 values, p = D^-1 r when want_p
 static spmv_status_t enqueue_residual64(spmv_matrix_t A, const double *b, bool x_zero,
                                         bool want_p, cudaStream_t st) {
@@ -484,7 +532,7 @@ static spmv_status_t enqueue_residual64(spmv_matrix_t A, const double *b, bool x
     const int G = cg_grid(A->n);
     return with_cols(A, [&](auto cols) -> spmv_status_t {
         using ColT = decltype(cols);
-        return with_shape(A->S, false, [&](auto rt, auto lt) -> spmv_status_t {
+        return with_shape<double>(A->S, [&](auto rt, auto lt) -> spmv_status_t {
             constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
             cg_residual<double, R, L, ColT><<<G, kCgBlock, 0, st>>>(
                 A->n, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.x.p, x_zero ? 1 : 0, b,
@@ -753,7 +801,8 @@ void release_cg(spmv_matrix_t A) {
     CgWork &w = A->cg;
     w.x.release(t); w.r.release(t); w.p.release(t); w.q.release(t); w.dinv.release(t);
     w.r32.release(t); w.p32.release(t); w.q32.release(t); w.d32.release(t); w.dinv32.release(t);
-    w.part.release(t); w.scal.release(t); w.flags.release(t);
+    w.part.release(t); w.scal.release(t); w.slots.release(t); w.zp.release(t);
+    w.zp32.release(t); w.flags.release(t);
     if (w.graph64) cudaGraphExecDestroy(w.graph64);
     if (w.graph32) cudaGraphExecDestroy(w.graph32);
     w = CgWork{};
@@ -786,7 +835,6 @@ spmv_status_t cg_timing(spmv_matrix_t A, int iters, double *out, cudaStream_t st
         GB_CUDA(cudaEventElapsedTime(ms, e[0], e[1]));
         return SPMV_OK;
     };
-    const int G = cg_grid(A->n);
     float ms = 0.f;
     cudaGraphExec_t g = nullptr;
     if (s == SPMV_OK) s = get_graph(A, false, iters, &g);
@@ -803,17 +851,17 @@ spmv_status_t cg_timing(spmv_matrix_t A, int iters, double *out, cudaStream_t st
     if (s == SPMV_OK) s = elapsed(&ms);
     out[1] = ms / iters;
     double sum[3] = {0.0, 0.0, 0.0};
+    int pq_count = 0;
     for (int it = 0; it < iters && s == SPMV_OK; ++it) {
         for (int k = 0; k < 3 && s == SPMV_OK; ++k) {
             s = cuda_status(cudaEventRecord(e[0], st));
             if (s != SPMV_OK) break;
-            if (k == 0) s = enqueue_pq64(A, sc, st);
+            if (k == 0)
+                s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, st, &pq_count);
             else if (k == 1)
-                cg_update_xr<double><<<G, kCgBlock, 0, st>>>(A->n, w.x.p, w.r.p, w.p.p, w.q.p,
-                                                             w.dinv.p, w.part.p + w.pq_len, sc);
-            else
-                cg_update_p<double><<<G, kCgBlock, 0, st>>>(A->n, w.r.p, w.dinv.p, w.p.p, sc);
-            if (s == SPMV_OK) s = cuda_status(cudaGetLastError());
+                s = enqueue_xr<double>(A, pq_count, w.x.p, w.r.p, w.p.p, w.q.p, w.dinv.p, sc,
+                                       st);
+            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, st);
             if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e[1], st));
             if (s == SPMV_OK) s = elapsed(&ms);
             sum[k] += ms;

@@ -9,34 +9,58 @@
 
 namespace gb {
 
-constexpr int kCgBlock = 256;
-constexpr int kCgCtasPerSm = 4;  // at most this many CTAs per SM in a CG sweep
+constexpr int kCgBlock = 256;    // CTAs of the kernels around the iteration (residual, start)
+constexpr int kCgCtasPerSm = 4;  // at most this many of them per SM
 
 int cg_grid(int32_t n);
 
-// The product phase q = A p, p.q runs on a grid of its own: the sweeps' grid (at most
-// kCgCtasPerSm CTAs per SM) leaves the latency-bound gathers without enough warps in flight.
-// A lane holding at most 16 bytes of values per entry keeps pq_unroll = 5 entries in flight
-// (a whole row of the tetrahedral meshes) at four CTAs per SM and 64 registers -- measured on
-// the 6M-row mesh against two entries at six CTAs per SM (40 registers): FP64 CG 185 -> 176 us
-// per iteration, the FP32 refinement solve 4.7 % faster; wider lanes keep two entries at
-// pq_min_ctas CTAs per SM, and so do matrices whose widest slice needs fewer load rounds
-// that way (load_rounds).  The persistent kernel runs the same grid as virtual CTAs, so
-// both paths stay bit-identical.
+// The kernels of an iteration run one CTA per SM, as many threads as the work needs (64 to
+// kIterThreads).  GB300 executes 2 FP64 operations per SM and clock, so a warp-wide FP64 add
+// costs 16 clocks of the SM: with four 256-thread CTAs per SM the shuffle trees of their
+// reductions alone took 2.5 us per summed quantity and kernel.  One CTA per SM leaves 152
+// partial sums, few enough for every CTA of the next kernel to add them itself, and small
+// systems still spread over every SM's FP64 pipe.
+//
+// A lane of the product holding at most 16 bytes of values per entry keeps pq_unroll = 5
+// entries in flight (a whole row of the tetrahedral meshes) at 1,024 threads per SM and 64
+// registers -- measured on the 6M-row mesh against two entries at 1,536 threads (40
+// registers): FP64 CG 185 -> 176 us per iteration, the FP32 refinement solve 4.7 % faster;
+// wider lanes keep two entries, and so do matrices whose widest slice needs fewer load
+// rounds that way (load_rounds).
+constexpr int kIterThreads = 1024;
 constexpr int pq_min_ctas(int value_bytes) { return value_bytes >= 64 ? 3 : 4; }
 constexpr int pq_unroll(int value_bytes) { return value_bytes <= 16 ? 5 : 2; }
-int cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes);
 bool cg_pq_deep(const spmv_matrix_t A, int uu);
+
+// Grid of an iteration kernel over `items` slice-lanes or 16-byte vectors: CTA c takes the `chunk`
+// items from c * chunk, its thread t those t, t + threads, ... into the chunk.  Equal contiguous
+// chunks, since a grid stride leaves the last, partly filled round of items to some of the SMs:
+// the 6M-row product takes 19.3 rounds of 152 x 1,024 items, 20 on a third of the SMs.  The grid
+// fixes the order of the reductions, so it depends on the handle and the device only; the
+// persistent kernel uses the same grid and gives identical results.
+struct IterGrid {
+    int ctas, threads;
+    int64_t chunk;
+    bool operator==(const IterGrid &o) const {
+        return ctas == o.ctas && threads == o.threads && chunk == o.chunk;
+    }
+    bool single() const { return chunk <= threads; }  // a thread for every item
+};
+// first item and end of the calling thread's items
+__device__ __forceinline__ int64_t iter_begin(int64_t chunk) {
+    return (int64_t)blockIdx.x * chunk + threadIdx.x;
+}
+__device__ __forceinline__ int64_t iter_end(int64_t chunk, int64_t items) {
+    const int64_t e = ((int64_t)blockIdx.x + 1) * chunk;
+    return e < items ? e : items;
+}
+IterGrid cg_iter_grid(int64_t items, int max_threads);
+IterGrid cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes);
+IterGrid cg_sweep_grid(const spmv_matrix_t A, int vec);
 
 // Hint: bring the line holding p into L1 without waiting for it (a later load of it hits).
 __device__ __forceinline__ void prefetch_l1(const void *p) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-// prefetch of a slice's column base (16-bit relative columns only)
-__device__ __forceinline__ void prefetch_col_base(const Cols32 &, int64_t) {}
-__device__ __forceinline__ void prefetch_col_base(const Cols16 &c, int64_t slice) {
-    prefetch_l1(c.col_start + slice);
 }
 
 // Sum over the CTA in a fixed tree; the total is left in every lane of warp 0.
@@ -66,19 +90,131 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
     }
 }
 
-// Same sum, broadcast to every thread of the CTA.
+// ---- reductions of the iteration kernels ----------------------------------------------------
+// Sum of v[k] over the first T threads of the CTA (T >= 32 NV, a multiple of 32), in one fixed
+// order: quantity k's total is returned in every lane of warp k, k < NV.  The values are folded
+// in shared memory to 128 per quantity before the one shuffle tree, 36 warp-wide adds per
+// quantity at 1,024 threads where a tree in each warp takes 165 (see kIterThreads).
 template <int NV>
-__device__ __forceinline__ void block_sum_all(double (&v)[NV]) {
-    __shared__ double bc[NV];
-    block_sum<NV>(v);
-    if (threadIdx.x == 0) {
+struct FoldSmem {
+    double all[NV][kIterThreads];
+    double part[NV][128];
+};
+template <int NV, int NS>
+__device__ __forceinline__ double fold_block(const double (&v)[NV], int T, FoldSmem<NS> &sm) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int F = T < 128 ? T : 128;
+    __syncthreads();  // the arrays may still be read from a previous call
+    if (t < T) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) bc[k] = v[k];
+        for (int k = 0; k < NV; ++k) sm.all[k][t] = v[k];
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = bc[k];
+    for (int k = 0; k < NV; ++k) {
+        // quantity k on threads k F .. k F + F - 1, or on the first F when the CTA is smaller
+        const int j = T >= NV * F ? t - k * F : t;
+        if (j >= 0 && j < F) {
+            double s = sm.all[k][j];
+            for (int m = j + F; m < T; m += F) s += sm.all[k][m];
+            sm.part[k][j] = s;
+        }
+    }
     __syncthreads();
+    double s = 0.0;
+    if (warp < NV) {
+        s = sm.part[warp][lane];
+        for (int m = lane + 32; m < F; m += 32) s += sm.part[warp][m];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    return s;
+}
+
+// Sum of one value per CTA (at most 32 kPartLoads CTAs) by one warp: lane l holds the values
+// of CTAs l, l + 32, ...
+constexpr int kPartLoads = 5;
+__device__ __forceinline__ double sum_parts(const double (&a)[kPartLoads]) {
+    double s = a[0];
+#pragma unroll
+    for (int j = 1; j < kPartLoads; ++j) s += a[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// The CTA's sums of v to part[k * ctas + cta].
+template <int NV>
+__device__ __forceinline__ void store_parts(const double (&v)[NV], double *part) {
+    __shared__ FoldSmem<NV> sm;
+    const double s = fold_block<NV>(v, blockDim.x, sm);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < NV && lane == 0) part[warp * gridDim.x + blockIdx.x] = s;
+}
+
+// The scalars of an iteration from its sums, computed by one thread of each CTA and shared: an
+// FP64 division is some twenty operations, which all 32 warps of a CTA would put through the
+// SM's 2-per-clock pipe in 3 us.
+template <typename T>
+struct StepScalars {
+    double rho, rr;
+    T coef;    // alpha, or beta
+    int done;  // 0, or the reason to stop after this step (CgScalars::done)
+};
+
+// alpha = rho / (p.q); done = 3 when it does not exist
+template <typename T>
+__device__ __forceinline__ void step_alpha(double rho, double pq, StepScalars<T> &s) {
+    s.done = (pq == 0.0 || !isfinite(pq)) ? 3 : 0;
+    s.coef = (T)(rho / pq);
+}
+// beta = r.z / rho, from the sums r.z and r.r
+template <typename T>
+__device__ __forceinline__ void step_beta(double rho, double rz, StepScalars<T> &s) {
+    s.rho = rz;
+    s.coef = (T)(rz / rho);
+}
+__device__ __forceinline__ int step_done(double rr, double limit, int iters, int max_iter) {
+    return rr <= limit ? 1 : (!isfinite(rr) ? 3 : (iters >= max_iter ? 2 : 0));
+}
+
+// Sum over i < count of part[i], by the calling warp (in every lane).  The kernels of a CG
+// iteration leave their CTAs' sums in part and each CTA of the next kernel adds them up: one
+// read of a few KB from L2, where a last-CTA reduction costs a fence, an atomic ticket and a
+// second pass at the end of every kernel.
+__device__ __forceinline__ double reduce_parts(const double *part, int count) {
+    const int lane = threadIdx.x & 31;
+    double a[kPartLoads];
+#pragma unroll
+    for (int j = 0; j < kPartLoads; ++j)
+        a[j] = lane + 32 * j < count ? __ldcg(part + lane + 32 * j) : 0.0;
+    return sum_parts(a);
+}
+
+// Programmatic dependent launch (a kernel launched by launch_dependent).  dep_wait: returns once
+// the kernels this one depends on have finished and their writes are visible; before it, only
+// data that no kernel of the solve writes may be read (the matrix, D^-1).  dep_allow: lets the
+// next kernel's CTAs start as SM slots become free; they stop at their own dep_wait.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_allow() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches a kernel that begins with dep_wait so that it may start while the kernel before it on
+// the stream still runs (also as an edge of a captured graph).
+template <typename... K, typename... A>
+spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t st,
+                               A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_status(cudaLaunchKernelEx(&cfg, kern, K(args)...));
 }
 
 // Each CTA stores its partial sums in part[k * gridDim.x + cta]; the CTA that arrives last
@@ -113,30 +249,53 @@ __device__ bool grid_sum_last(double (&v)[NV], double *part, unsigned *ticket, d
     return true;
 }
 
-// y-rows (R of them) of lane `lane` in slice `slice`: sum over the slice's columns in order,
-// fused multiply-add from +0.0, padding skipped (the same order as spmv_sell).  COHERENT
-// selects coherent gathers of x, for kernels in which other CTAs rewrite x between barriers.
-template <typename T, int R, int L, bool COHERENT = false, int UU = 2, typename ColT>
-__device__ __forceinline__ void slice_rows(int64_t slice, int lane, const int64_t *sp,
-                                           const ColT &cols, const T *val, const T *x,
-                                           uint64_t pol, T (&acc)[R]) {
-    constexpr int S = L * R;
+// A slice-lane: R rows of one slice, held by one thread.
+struct SliceLane {
+    int64_t at;     // first stored entry of the lane's first row
+    int w;          // stored entries per row of the slice
+    int32_t cbase;  // column base of 16-bit relative columns
+};
+
+template <int R, int L, typename ColT>
+__device__ __forceinline__ SliceLane slice_open(int64_t g, const int64_t *sp, const ColT &cols) {
+    const int64_t slice = g / L;
+    const int lane = (int)(g % L);
     const int64_t base = sp[slice];
-    const int w = (int)((sp[slice + 1] - base) / S);
-    const int32_t cbase = cols.base(slice);
-    const T *vp = val + base + lane * R;
-    const int64_t cat = base + lane * R;
-#pragma unroll
-    for (int i = 0; i < R; ++i) acc[i] = T(0);
-    int t = 0;
-    for (; t + UU <= w; t += UU) {
-        T v[UU][R];
-        int32_t c[UU][R];
+    SliceLane s;
+    s.w = (int)((sp[slice + 1] - base) / (L * R));
+    s.cbase = cols.base(slice);
+    s.at = base + lane * R;
+    return s;
+}
+
+// UU stored entries of each of a lane's R rows, in flight together.  MASKED: entries past the
+// slice's width are not loaded (column -1).
+template <typename T, int R, int UU>
+struct SliceRound {
+    T v[UU][R];
+    int32_t c[UU][R];
+
+    template <int L, bool MASKED = false, typename ColT>
+    __device__ __forceinline__ void load(const SliceLane &s, int t, const ColT &cols,
+                                         const T *val, uint64_t pol) {
+        constexpr int S = L * R;
 #pragma unroll
         for (int u = 0; u < UU; ++u) {
-            ld_stream(vp + (int64_t)(t + u) * S, pol, v[u]);
-            cols.template load<R>(cat + (int64_t)(t + u) * S, slice, pol, cbase, c[u]);
+            if (!MASKED || t + u < s.w) {
+                ld_stream(val + s.at + (int64_t)(t + u) * S, pol, v[u]);
+                cols.template load<R>(s.at + (int64_t)(t + u) * S, 0, pol, s.cbase, c[u]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    v[u][i] = T(0);
+                    c[u][i] = -1;
+                }
+            }
         }
+    }
+
+    template <bool COHERENT>
+    __device__ __forceinline__ void multiply(const T *x, T (&acc)[R]) const {
         T xv[UU][R];
 #pragma unroll
         for (int u = 0; u < UU; ++u)
@@ -150,15 +309,50 @@ __device__ __forceinline__ void slice_rows(int64_t slice, int lane, const int64_
             for (int i = 0; i < R; ++i)
                 if (c[u][i] >= 0) acc[i] = fma_t(v[u][i], xv[u][i], acc[i]);
     }
-    for (; t < w; ++t) {
-        T v[R];
-        int32_t c[R];
-        ld_stream(vp + (int64_t)t * S, pol, v);
-        cols.template load<R>(cat + (int64_t)t * S, slice, pol, cbase, c);
+};
+
+// The R row sums of a slice-lane: its entries in column order, fused multiply-add from +0.0,
+// padding skipped (the order of spmv_sell).  rd holds the first round when the slice has at
+// least UU entries (the caller loads it, as early as it can); the remainder of a row shorter
+// than a round is one more round with the missing entries masked.  COHERENT selects coherent
+// gathers of x, for kernels in which other CTAs rewrite x between barriers.
+template <typename T, int R, int L, bool COHERENT, int UU, typename ColT>
+__device__ __forceinline__ void slice_multiply(const SliceLane &s, SliceRound<T, R, UU> &rd,
+                                               const ColT &cols, const T *val, const T *x,
+                                               uint64_t pol, T (&acc)[R]) {
 #pragma unroll
-        for (int i = 0; i < R; ++i)
-            if (c[i] >= 0)
-                acc[i] = fma_t(v[i], COHERENT ? ld_x_coherent(x + c[i]) : ld_x(x + c[i]), acc[i]);
+    for (int i = 0; i < R; ++i) acc[i] = T(0);
+    int t = 0;
+    if (s.w >= UU) {
+        rd.template multiply<COHERENT>(x, acc);
+        for (t = UU; t + UU <= s.w; t += UU) {
+            rd.template load<L>(s, t, cols, val, pol);
+            rd.template multiply<COHERENT>(x, acc);
+        }
+    }
+    if (t < s.w) {
+        rd.template load<L, true>(s, t, cols, val, pol);
+        rd.template multiply<COHERENT>(x, acc);
+    }
+}
+
+template <typename T, int R, int L, bool COHERENT = false, int UU = 2, typename ColT>
+__device__ __forceinline__ void slice_rows(int64_t slice, int lane, const int64_t *sp,
+                                           const ColT &cols, const T *val, const T *x,
+                                           uint64_t pol, T (&acc)[R]) {
+    const SliceLane s = slice_open<R, L>(slice * L + lane, sp, cols);
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = T(0);
+    int t = 0;
+    for (; t + UU <= s.w; t += UU) {
+        SliceRound<T, R, UU> rd;
+        rd.template load<L>(s, t, cols, val, pol);
+        rd.template multiply<COHERENT>(x, acc);
+    }
+    if (t < s.w) {
+        SliceRound<T, R, UU> rd;
+        rd.template load<L, true>(s, t, cols, val, pol);
+        rd.template multiply<COHERENT>(x, acc);
     }
 }
 
@@ -235,73 +429,113 @@ __device__ __forceinline__ void vstore_h(T *p, const T (&v)[Vec16<T>::n], uint64
     else vstore(p, v);
 }
 
-// x += alpha p; r -= alpha q; accumulates r.(D^-1 r) into vz and r.r into vr.  x and q are
-// not needed again in this iteration (evict-first in FP32); r, p and D^-1 are read by the p
-// update.
+// One thread's vector of the x/r update.  D^-1 does not change during a solve, so a kernel may
+// load it before the kernel it depends on has finished (load_d); the rest comes after.
 template <typename T>
-__device__ __forceinline__ void sweep_update_xr(int32_t n, T alpha, T *x, T *r, const T *p,
-                                                const T *q, const T *dinv, T &vz, T &vr) {
-    constexpr int V = Vec16<T>::n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nv = n / V;
-    const uint64_t pol = policy_evict_first();
-    for (int64_t v = tid; v < nv; v += stride) {
-        const int64_t i = v * V;
-        T xv[V], rv[V], pv[V], qv[V], dv[V];
-        vload_h(x + i, xv, pol);
-        vload(r + i, rv);
-        vload(p + i, pv);
-        vload_h(q + i, qv, pol);
-        vload(dinv + i, dv);
+struct XrVec {
+    static constexpr int V = Vec16<T>::n;
+    T x[V], r[V], p[V], q[V], d[V];
+    __device__ __forceinline__ void load_d(const T *dinv, int64_t i) { vload(dinv + i, d); }
+    __device__ __forceinline__ void load(const T *xg, const T *rg, const T *pg, const T *qg,
+                                         int64_t i, uint64_t pol) {
+        vload_h(xg + i, x, pol);
+        vload(rg + i, r);
+        vload(pg + i, p);
+        vload_h(qg + i, q, pol);
+    }
+    // x += alpha p; r -= alpha q; r.(D^-1 r) into vz, r.r into vr
+    __device__ __forceinline__ void update(T alpha, T *xg, T *rg, int64_t i, uint64_t pol, T &vz,
+                                           T &vr) {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-            xv[e] = fma_t(alpha, pv[e], xv[e]);
-            rv[e] = fma_t(-alpha, qv[e], rv[e]);
-            vz = fma_t(rv[e], dv[e] * rv[e], vz);
-            vr = fma_t(rv[e], rv[e], vr);
+            x[e] = fma_t(alpha, p[e], x[e]);
+            r[e] = fma_t(-alpha, q[e], r[e]);
+            vz = fma_t(r[e], d[e] * r[e], vz);
+            vr = fma_t(r[e], r[e], vr);
         }
-        vstore_h(x + i, xv, pol);
-        vstore(r + i, rv);
+        vstore_h(xg + i, x, pol);
+        vstore(rg + i, r);
     }
-    for (int64_t i = nv * V + tid; i < n; i += stride) {
-        const T xi = fma_t(alpha, p[i], x[i]);
-        const T ri = fma_t(-alpha, q[i], r[i]);
-        x[i] = xi;
-        r[i] = ri;
-        vz = fma_t(ri, dinv[i] * ri, vz);
-        vr = fma_t(ri, ri, vr);
+};
+
+// x += alpha p; r -= alpha q over the vectors k = from, from + stride, ... below end (n may cut the
+// last one short); accumulates r.(D^-1 r) into vz and r.r into vr.  x and q are not needed again
+// in this iteration (evict-first in FP32); r, p and D^-1 are read by the p update.
+template <typename T, int UNROLL = 4>
+__device__ __forceinline__ void sweep_update_xr(int32_t n, int64_t from, int64_t end,
+                                                int64_t stride, T alpha, T *x, T *r,
+                                                const T *p, const T *q, const T *dinv, T &vz,
+                                                T &vr) {
+    constexpr int V = Vec16<T>::n;
+    const int64_t nv = n / V, full = nv < end ? nv : end;
+    const uint64_t pol = policy_evict_first();
+    int64_t k = from;
+#pragma unroll UNROLL
+    for (; k < full; k += stride) {
+        XrVec<T> v;
+        v.load(x, r, p, q, k * V, pol);
+        v.load_d(dinv, k * V);
+        v.update(alpha, x, r, k * V, pol, vz, vr);
+    }
+    if (k == nv && k < end) {
+        for (int64_t i = k * V; i < n; ++i) {
+            const T xi = fma_t(alpha, p[i], x[i]);
+            const T ri = fma_t(-alpha, q[i], r[i]);
+            x[i] = xi;
+            r[i] = ri;
+            vz = fma_t(ri, dinv[i] * ri, vz);
+            vr = fma_t(ri, ri, vr);
+        }
     }
 }
 
-// p = D^-1 r + beta p.  r and D^-1 are next read by the next iteration's x/r update
-// (evict-first in FP32); the new p stays in L2 for the product's gathers.
+// One thread's vector of the p update (D^-1 apart, as in XrVec).
 template <typename T>
-__device__ __forceinline__ void sweep_update_p(int32_t n, T beta, const T *r, const T *dinv,
+struct PVec {
+    static constexpr int V = Vec16<T>::n;
+    T r[V], d[V], p[V];
+    __device__ __forceinline__ void load_d(const T *dinv, int64_t i, uint64_t pol) {
+        vload_h(dinv + i, d, pol);
+    }
+    __device__ __forceinline__ void load(const T *rg, const T *pg, int64_t i, uint64_t pol) {
+        vload_h(rg + i, r, pol);
+        vload(pg + i, p);
+    }
+    __device__ __forceinline__ void update(T beta, T *pg, int64_t i) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) p[e] = fma_t(beta, p[e], d[e] * r[e]);
+        vstore(pg + i, p);
+    }
+};
+
+// p = D^-1 r + beta p over the vectors k = from, from + stride, ... below end.  r and D^-1 are next read by
+// the next iteration's x/r update (evict-first in FP32); the new p stays in L2 for the
+// product's gathers.
+template <typename T, int UNROLL = 4>
+__device__ __forceinline__ void sweep_update_p(int32_t n, int64_t from, int64_t end,
+                                               int64_t stride, T beta, const T *r, const T *dinv,
                                                T *p) {
     constexpr int V = Vec16<T>::n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nv = n / V;
+    const int64_t nv = n / V, full = nv < end ? nv : end;
     const uint64_t pol = policy_evict_first();
-    for (int64_t v = tid; v < nv; v += stride) {
-        const int64_t i = v * V;
-        T rv[V], dv[V], pv[V];
-        vload_h(r + i, rv, pol);
-        vload_h(dinv + i, dv, pol);
-        vload(p + i, pv);
-#pragma unroll
-        for (int e = 0; e < V; ++e) pv[e] = fma_t(beta, pv[e], dv[e] * rv[e]);
-        vstore(p + i, pv);
+    int64_t k = from;
+#pragma unroll UNROLL
+    for (; k < full; k += stride) {
+        PVec<T> v;
+        v.load(r, p, k * V, pol);
+        v.load_d(dinv, k * V, pol);
+        v.update(beta, p, k * V);
     }
-    for (int64_t i = nv * V + tid; i < n; i += stride) p[i] = fma_t(beta, p[i], dinv[i] * r[i]);
+    if (k == nv && k < end) {
+        for (int64_t i = k * V; i < n; ++i) p[i] = fma_t(beta, p[i], dinv[i] * r[i]);
+    }
 }
 
 // (R, L) of the sliced kernels for a slice height and value type.
-template <typename F>
-spmv_status_t with_shape(int S, bool f32, F &&f) {
+template <typename T, typename F>
+spmv_status_t with_shape(int S, F &&f) {
     using std::integral_constant;
-    if (!f32) {
+    if constexpr (sizeof(T) == 8) {
         switch (S) {
             case 32: return f(integral_constant<int, 1>{}, integral_constant<int, 32>{});
             case 64: return f(integral_constant<int, 2>{}, integral_constant<int, 32>{});

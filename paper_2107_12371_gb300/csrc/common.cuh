@@ -106,15 +106,20 @@ struct DevBuf {
     }
 };
 
-// Device scalars of one CG recurrence (written by the last CTA of a reduction).
+// Device scalars of one CG recurrence.  The kernel that ends an iteration writes rho, beta, rr,
+// iters and done while its CTAs still need the iteration's own values, so these are kept in
+// the cur_ fields, which the first kernel of the iteration copies.
 struct CgScalars {
-    double alpha, beta, rho, rr, bb, tol2, s, inv_s;
+    double alpha, beta, rho, rr, bb, tol2, s, inv_s;  // alpha: allocation-free solve only
+    double cur_rho;
+    int cur_done, cur_iters;
+    int broke;  // the iteration's p.q was zero or not finite: its updates are left out
+    int pad0;
     int done;   // 0 running, 1 converged, 2 iteration cap, 3 breakdown, 4 timeout
     int iters;
     int max_iter;
     int pad;
     unsigned tickets[4];
-    unsigned bar_count, bar_gen;    // grid barrier of the persistent kernel
     long long budget_ns;            // persistent kernel: wall-clock budget (0 = none)
 };
 
@@ -124,16 +129,18 @@ struct CgWork {
     DevBuf<float> r32, p32, q32, d32, dinv32;
     DevBuf<double> part;        // per-CTA partial sums
     DevBuf<double> scal;        // two CgScalars blocks (outer / inner)
+    DevBuf<double> zp;          // persistent kernel, resident form: (D^-1 r, p) of every row
+    DevBuf<float> zp32;
+    DevBuf<ulonglong2> slots;   // persistent kernel: what each CTA posts to the others
     DevBuf<int> flags;          // status flags
     int h_flags[16] = {};       // host mirrors (read back synchronously; no pinned buffers)
     CgScalars h_scal[2] = {};
     int part_len = 0;
-    int pq_len = 0;  // leading p.q partials: one per CTA of the product grid (cg_pq_grid)
+    int pq_len = 0;  // leading p.q partials (room for one per CTA of the product)
     bool ready = false;
     bool mixed_ready = false;
     cudaGraphExec_t graph64 = nullptr, graph32 = nullptr, graph_pers = nullptr;
     int graph64_iters = 0, graph32_iters = 0;
-    int pers_grid = 0;
 };
 
 struct McgWork;  // multi-right-hand-side CG work (mcg.cu)

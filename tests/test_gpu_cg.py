@@ -116,6 +116,72 @@ def test_persistent_equals_graph_path_shapes(oracle, case, bits, S):
         assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b)
 
 
+def banded(n, width, seed=0):
+    """SPD matrix with `width` entries per row (a symmetric band of ones' negatives, diagonally
+    dominant)."""
+    k = (width - 1) // 2
+    i = np.repeat(np.arange(n, dtype=np.int64), 2 * k + 1)
+    j = i + np.tile(np.arange(-k, k + 1), n)
+    keep = (j >= 0) & (j < n)
+    i, j = i[keep], j[keep]
+    v = np.where(i == j, 2.0 * k + 0.05 * (1 + i % 5), -1.0)
+    rp = np.zeros(n + 1, np.int64)
+    np.add.at(rp, i + 1, 1)
+    return np.cumsum(rp).astype(np.int32), j.astype(np.int32), v
+
+
+@pytest.mark.parametrize("rows_per_sm,extra,width,mixed", [
+    (0, 1, 1, 0), (0, 63, 3, 1), (64, 0, 3, 0), (64, 1, 3, 1),
+    (1024, 0, 5, 0), (1024, 1, 5, 0), (2048, 0, 3, 0), (2048, 1, 3, 0), (2048, 0, 3, 1),
+    (2048, 3, 3, 1), (4096, 0, 3, 1), (4096, 5, 3, 1), (1024, -1, 25, 0), (2048, -7, 11, 0)])
+def test_iteration_grids_at_their_edges(oracle, rows_per_sm, extra, width, mixed):
+    """The grids change form where a chunk of rows per SM fills 64, 512 and 1,024 threads (1,024
+    and 2,048 rows per SM in FP64, twice that in FP32), and the persistent kernel where the rows
+    no longer fit a thread each or the matrix no longer fits shared memory (wide rows): on both
+    sides of each, the persistent kernel equals the graph path bit for bit and the oracle's
+    product confirms the residual."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = rows_per_sm * sms + extra
+    rp, ci, v = banded(n, width)
+    b = np.random.default_rng(n).uniform(-1, 1, n)
+    A = capi.Matrix(n, rp, ci, v, precision=capi.SPMV_PREC_DUAL)
+    x1, r1 = solve(A, b, rtol=1e-10, mixed=mixed)
+    x2, r2 = solve(A, b, rtol=1e-10, mixed=mixed, persistent=1)
+    assert r1["status"] == r2["status"] == capi.SPMV_OK, (r1, r2)
+    assert r1["iterations"] == r2["iterations"]
+    assert np.array_equal(x1, x2)
+    r = b - oracle.spmv(rp, ci, v, x1)
+    assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b)
+
+
+def test_concurrent_persistent_solves_of_different_sizes(oracle):
+    """Host threads that launch the persistent kernel for handles of different sizes (so with
+    different amounts of shared memory) on streams of their own do not disturb each other."""
+    import threading
+    cases = []
+    for n in (3, 8, 14, 20):
+        m, b = workloads.kuhn(n, seed=n, dirichlet=True)
+        A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values)
+        cases.append((A, dev(b), solve(A, b, rtol=1e-10)[0], torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(A, bd, ref, stream):
+        xd = torch.zeros_like(bd)
+        torch.cuda.current_stream().synchronize()
+        for _ in range(6):
+            res = A.solve(bd, xd, stream=stream, raise_on_error=False, rtol=1e-10, persistent=1)
+            if res["status"] != capi.SPMV_OK or not np.array_equal(xd.cpu().numpy(), ref):
+                bad.append(res)
+
+    threads = [threading.Thread(target=work, args=c) for c in cases]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+
+
 def mixed_solve(oracle, m, b, reorder, **opts):
     """GPU refinement through the C ABI in the handle's numbering; x returned in the original one."""
     A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values, reorder=reorder,
