@@ -148,7 +148,7 @@ cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, const int64_t *sp, ColT c
         for (int i = 0; i < R; ++i)
             if (row0 + i < n) vt = fma_t(p[row0 + i], acc[i], vt);
     }
-    double v[1] = {(double)vt};
+    const T v[1] = {vt};
     store_parts<1>(v, part);
 }
 
@@ -195,7 +195,7 @@ cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const
     T vz = T(0), vr = T(0);
     if (ONE && mine) v.update(alpha, x, r, k0 * V, pol, vz, vr);
     else sweep_update_xr<T>(n, k0, end, blockDim.x, alpha, x, r, p, q, dinv, vz, vr);
-    double t[2] = {(double)vz, (double)vr};
+    const T t[2] = {vz, vr};
     store_parts<2>(t, part);
 }
 

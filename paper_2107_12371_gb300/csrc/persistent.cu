@@ -95,7 +95,7 @@ struct PersSmem {
 // the grid waits.  PUBLISH: the CTAs' earlier writes are visible to all after the exchange.
 // Returns false on a wait that ran out or CTA 0's vote to stop.
 template <int NV, bool PUBLISH, typename T, typename F>
-__device__ __forceinline__ bool exchange(const double (&v)[NV], int TT, int ctas,
+__device__ __forceinline__ bool exchange(const T (&v)[NV], int TT, int ctas,
                                          ulonglong2 *slots, unsigned long long iter, int my_vote,
                                          PersSmem<T> &sm, F &&use) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -303,7 +303,7 @@ cg_persistent(PersArgs<T> a, ColT col) {
                     if (g * R + i < n) vt = fma_t(a.p[g * R + i], acc[i], vt);
             }
         }
-        const double v1[1] = {(double)vt};
+        const T v1[1] = {vt};
         // CTA 0's vote to stop on the wall-clock budget
         const int my_vote =
             blockIdx.x == 0 && budget > 0 && global_timer_ns() - t_start > budget ? 1 : 0;
@@ -340,7 +340,7 @@ cg_persistent(PersArgs<T> a, ColT col) {
         } else {
             sweep_update_xr<T, 1>(n, k0, k1, a.sw.threads, alpha, a.x, a.r, a.p, a.q, a.dinv, vz, vr);
         }
-        const double v2[2] = {(double)vz, (double)vr};
+        const T v2[2] = {vz, vr};
         ++iters;
         if (!exchange<2, PAIRS>(v2, a.sw.threads, a.sw.ctas, a.slots + kSlotsR, it, 0, sm,
                                 [&](int k, double sum) {
