@@ -3,10 +3,14 @@
 //   the symmetric permutation P A P^T; FP32 value copy; conversion to sliced ELLPACK with S
 //   rows per slice, column-major inside a slice (Sec. 4.2); per-slice x range (Sec. 5.1).
 // The paper applies these once per simulation, so their cost is amortised (Sec. 2, 4.1).
+#include <cooperative_groups.h>
+
 #include <climits>
 #include <vector>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace gb {
 namespace {
@@ -62,103 +66,323 @@ __device__ __forceinline__ unsigned long long node_key(const int32_t *deg, int32
     return ((unsigned long long)(uint32_t)deg[v] << 32) | (uint32_t)v;
 }
 
-// min key over unplaced nodes
-__global__ void min_key_unplaced(int32_t n, const int32_t *deg, const int32_t *pos,
-                                 unsigned long long *out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || pos[i] != -1) return;
-    atomicMin(out, node_key(deg, (int32_t)i));
+// a word that other CTAs write between barriers, from L2
+__device__ __forceinline__ int32_t ld_l2(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
-// min key over queue[ls, le)
-__global__ void min_key_range(const int32_t *queue, int64_t ls, int64_t le, const int32_t *deg,
-                              unsigned long long *out) {
-    int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= le) return;
-    atomicMin(out, node_key(deg, queue[p]));
-}
+constexpr int kCmCluster = 16;
+constexpr int kCmThreads = 1024;  // at most; see cm_order_device
+constexpr int kCmPlaced = -2;   // stamp of a node that has its position
+constexpr int kCmBatch = 6;     // row entries in flight per thread
+constexpr int kCmComponents = 256;  // components that one launch orders
+constexpr int kCmKids = 8;      // children of a node sorted in registers; more are selected one by one
 
-__global__ void bfs_seed(int32_t r, int32_t id, int32_t *stamp, int32_t *queue, int32_t *tail) {
-    stamp[r] = id;
-    queue[0] = r;
-    *tail = 1;
-}
+// Smallest key that each CTA of the cluster found, in every CTA; two sets in turn, so that one can
+// be written while another CTA still reads the last one.
+struct CmKeys {
+    unsigned long long key[2][kCmCluster];
+    unsigned long long warp[kCmThreads / 32];
+};
 
-// expand one BFS level (level sets only, order irrelevant), restricted to unplaced nodes
-__global__ void bfs_expand(const int32_t *rp, const int32_t *ci, const int32_t *pos, int32_t id,
-                           int32_t *stamp, int32_t *queue, int64_t ls, int64_t le,
-                           int32_t *tail) {
-    int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= le) return;
-    int32_t u = queue[p];
-    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
-        int32_t v = ci[k];
-        if (v == u || pos[v] != -1) continue;
-        if (stamp[v] == id) continue;
-        if (atomicExch(&stamp[v], id) != id) queue[atomicAdd(tail, 1)] = v;
+// What the CTAs of the cluster keep in step (every thread of every CTA holds the same values).
+struct CmWalk {
+    int32_t n;
+    const int32_t *rp, *ci, *deg;
+    int32_t *pos, *claim, *stamp, *queue, *perm;
+    // nodes that a BFS level appends: three words in turn, the next one cleared a level ahead,
+    // when every CTA has passed the barrier after the last CTA read it
+    int32_t *grown;
+    CmKeys *keys;
+    cg::cluster_group cluster;
+    int64_t gid, threads;  // threads are numbered across the CTAs: small levels use every SM
+    int searches, levels;  // uses of the words above so far
+
+    // up to kCmBatch neighbours of u from row entry k on, requested together (-1: none)
+    __device__ __forceinline__ void load_row(int32_t u, int32_t k, int32_t end,
+                                             int32_t (&v)[kCmBatch]) const {
+#pragma unroll
+        for (int j = 0; j < kCmBatch; ++j) v[j] = k + j < end ? ci[k + j] : -1;
+#pragma unroll
+        for (int j = 0; j < kCmBatch; ++j)
+            if (v[j] == u) v[j] = -1;
     }
-}
 
-__global__ void place_start(int32_t v, int64_t at, int32_t *perm, int32_t *pos) {
-    perm[at] = v;
-    pos[v] = (int32_t)at;
-}
-
-// every unplaced neighbour of a frontier node records the earliest frontier position
-__global__ void cm_claim(const int32_t *rp, const int32_t *ci, const int32_t *perm,
-                         const int32_t *pos, int32_t *claim, int64_t ls, int64_t le) {
-    int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= le) return;
-    int32_t u = perm[p];
-    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
-        int32_t v = ci[k];
-        if (v != u && pos[v] == -1) atomicMin(&claim[v], (int32_t)p);
-    }
-}
-
-__global__ void cm_count(const int32_t *rp, const int32_t *ci, const int32_t *perm,
-                         const int32_t *pos, const int32_t *claim, int64_t ls, int64_t le,
-                         int64_t *counts) {
-    int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= le) return;
-    int32_t u = perm[p];
-    int64_t c = 0;
-    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
-        int32_t v = ci[k];
-        c += (v != u && pos[v] == -1 && claim[v] == (int32_t)p);
-    }
-    counts[p - ls] = c;
-}
-
-// children of frontier position p, appended in increasing (degree, index) by repeated
-// selection of the next larger key (no buffer, any row length)
-__global__ void cm_place(const int32_t *rp, const int32_t *ci, const int32_t *deg,
-                         int32_t *perm, const int32_t *pos, const int32_t *claim, int64_t ls,
-                         int64_t le, const int64_t *offsets) {
-    int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= le) return;
-    int32_t u = perm[p];
-    int64_t at = le + offsets[p - ls];
-    int64_t cnt = offsets[p - ls + 1] - offsets[p - ls];
-    unsigned long long last = 0;
-    bool first = true;
-    for (int64_t t = 0; t < cnt; ++t) {
+    // smallest key over the nodes f(i), i in [0, count); f returns a node or -1
+    template <typename F>
+    __device__ __forceinline__ unsigned long long min_key(int64_t count, F &&f) {
+        const int w = searches++ & 1, ranks = (int)cluster.num_blocks();
         unsigned long long best = ~0ull;
-        for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
-            int32_t v = ci[k];
-            if (v == u || pos[v] != -1 || claim[v] != (int32_t)p) continue;
-            unsigned long long key = node_key(deg, v);
-            if ((first || key > last) && key < best) best = key;
+        for (int64_t i = gid; i < count; i += threads) {
+            const int32_t v = f(i);
+            if (v >= 0) {
+                const unsigned long long k = node_key(deg, v);
+                best = k < best ? k : best;
+            }
         }
-        perm[at + t] = (int32_t)(best & 0xffffffffull);
+        auto warp_min = [&] {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+                best = k < best ? k : best;
+            }
+        };
+        warp_min();
+        const int warps = blockDim.x >> 5;
+        if ((threadIdx.x & 31) == 0) keys->warp[threadIdx.x >> 5] = best;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            best = (int)threadIdx.x < warps ? keys->warp[threadIdx.x] : ~0ull;
+            warp_min();
+            if ((int)threadIdx.x < ranks)
+                cluster.map_shared_rank(keys, threadIdx.x)->key[w][cluster.block_rank()] = best;
+        }
+        cluster.sync();
+        for (int r = 0; r < ranks; ++r) best = keys->key[w][r] < best || r == 0 ? keys->key[w][r] : best;
+        return best;
+    }
+
+    // BFS levels from r over nodes without a position: the number of levels, and the node of
+    // the last one with the smallest key
+    __device__ __forceinline__ void bfs(int32_t r, int32_t id, int32_t *ecc, int32_t *pick) {
+        if (gid == 0) {
+            stamp[r] = id;
+            queue[0] = r;
+        }
+        cluster.sync();
+        int64_t ls = 0, le = 1;
+        int32_t depth = 0;
+        for (;;) {
+            const int w = levels++ % 3;
+            for (int64_t i = ls + gid; i < le; i += threads) {
+                const int32_t u = ld_l2(queue + i);
+                const int32_t b = rp[u + 1];
+                for (int32_t k = rp[u]; k < b; k += kCmBatch) {
+                    int32_t v[kCmBatch];
+                    bool fresh[kCmBatch];
+                    load_row(u, k, b, v);
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j) {
+                        const int32_t st = v[j] >= 0 ? ld_l2(stamp + v[j]) : id;
+                        fresh[j] = st != id && st != kCmPlaced;
+                    }
+                    int cnt = 0;
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j)
+                        if (fresh[j]) fresh[j] = atomicExch(&stamp[v[j]], id) != id;
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j) cnt += fresh[j];
+                    if (cnt == 0) continue;
+                    int64_t at = le + atomicAdd(&grown[w], cnt);
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j)
+                        if (fresh[j]) queue[at++] = v[j];
+                }
+            }
+            if (gid == 0) grown[levels % 3] = 0;
+            cluster.sync();
+            const int more = ld_l2(grown + w);
+            if (more == 0) break;
+            ++depth;
+            ls = le;
+            le += more;
+        }
+        const int32_t *q = queue + ls;
+        const unsigned long long k = min_key(le - ls, [&](int64_t i) { return ld_l2(q + i); });
+        *ecc = depth;
+        *pick = (int32_t)(k & 0xffffffffull);
+    }
+};
+
+// Children of frontier position p (the unplaced neighbours of u = perm[p] that no earlier
+// position claimed): their number, and the first kCmKids keys, sorted.
+__device__ __forceinline__ int cm_kids(const CmWalk &w, int64_t p, int32_t u,
+                                       unsigned long long (&key)[kCmKids]) {
+#pragma unroll
+    for (int j = 0; j < kCmKids; ++j) key[j] = ~0ull;
+    int cnt = 0;
+    const int32_t b = w.rp[u + 1];
+    for (int32_t k = w.rp[u]; k < b; k += kCmBatch) {
+        int32_t v[kCmBatch], c[kCmBatch], d[kCmBatch];
+        w.load_row(u, k, b, v);
+#pragma unroll
+        for (int j = 0; j < kCmBatch; ++j) {
+            c[j] = v[j] >= 0 ? ld_l2(w.claim + v[j]) : -1;
+            d[j] = v[j] >= 0 ? w.deg[v[j]] : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < kCmBatch; ++i) {
+            if (c[i] != (int32_t)p) continue;
+            // insertion into the sorted list (a full list keeps the smallest)
+            unsigned long long x = (unsigned long long)(uint32_t)d[i] << 32 | (uint32_t)v[i];
+#pragma unroll
+            for (int j = 0; j < kCmKids; ++j) {
+                const unsigned long long lo = x < key[j] ? x : key[j];
+                x = x < key[j] ? key[j] : x;
+                key[j] = lo;
+            }
+            ++cnt;
+        }
+    }
+    return cnt;
+}
+
+__device__ __forceinline__ void cm_set(const CmWalk &w, int64_t at, int32_t v) {
+    w.perm[at] = v;
+    w.pos[v] = (int32_t)at;
+    w.stamp[v] = kCmPlaced;
+}
+
+// Places the children of position p from position `at` on, in increasing (degree, index).
+__device__ __forceinline__ void cm_place_kids(const CmWalk &w, int64_t p, int32_t u, int cnt,
+                                              const unsigned long long (&key)[kCmKids],
+                                              int64_t at) {
+    if (cnt <= kCmKids) {
+#pragma unroll
+        for (int j = 0; j < kCmKids; ++j)
+            if (j < cnt) cm_set(w, at + j, (int32_t)(key[j] & 0xffffffffull));
+        return;
+    }
+    // any number: repeated selection of the next larger key
+    unsigned long long last = 0;
+    for (int t = 0; t < cnt; ++t) {
+        unsigned long long best = ~0ull;
+        for (int32_t k = w.rp[u]; k < w.rp[u + 1]; ++k) {
+            const int32_t v = w.ci[k];
+            if (v == u || ld_l2(w.claim + v) != (int32_t)p) continue;
+            const unsigned long long x = node_key(w.deg, v);
+            if ((t == 0 || x > last) && x < best) best = x;
+        }
+        cm_set(w, at + t, (int32_t)(best & 0xffffffffull));
         last = best;
-        first = false;
     }
 }
 
-__global__ void set_pos(const int32_t *perm, int64_t a, int64_t b, int32_t *pos) {
-    int64_t q = a + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < b) pos[perm[q]] = (int32_t)q;
+// Cuthill-McKee from position *placed_io on, up to max_components further components (so that a
+// launch is short whatever the graph), in one thread-block cluster: the levels of a mesh are
+// a few thousand nodes in some hundred steps, so what a level costs is its chain of dependent
+// loads and its barriers.  A cluster barrier is a hardware one, and nothing returns to the host
+// between levels.  Measured for a mesh of 796K cells (1,038 BFS levels of the start-node search,
+// 353 of the order): 42 -> 8.8 ms against a few kernels and a read-back per level; 48K cells 15.8
+// -> 2.8 ms, 6M about 115 -> 36 ms.  With the frontier spread over all CTAs a level of the
+// search takes 6 us and one of the order 8 us.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, int32_t *pos,
+           int32_t *claim, int32_t *stamp, int32_t *queue, int32_t *perm, int peripheral,
+           int max_components, int64_t *placed_io, int32_t *bfs_id_io, int32_t *grown) {
+    __shared__ CmKeys keys;
+    __shared__ int totals[2][kCmCluster];
+    __shared__ int warp_sums[THREADS / 32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (rank == 0 && threadIdx.x < 3) grown[threadIdx.x] = 0;
+    CmWalk w{n, rp, ci, deg, pos, claim, stamp, queue, perm, grown, &keys, cluster,
+             (int64_t)threadIdx.x * ranks + rank, (int64_t)ranks * THREADS, 0, 0};
+    int64_t placed = *placed_io;
+    int32_t bfs_id = *bfs_id_io;
+    int turn = 0;
+    cluster.sync();
+    for (int comp = 0; comp < max_components && placed < n; ++comp) {
+        int32_t start = (int32_t)(w.min_key(n, [&](int64_t i) {
+                                      return ld_l2(pos + i) == -1 ? (int32_t)i : -1;
+                                  }) & 0xffffffffull);
+        if (peripheral) {
+            int32_t ecc, pick;
+            w.bfs(start, bfs_id++, &ecc, &pick);
+            for (int moves = 0; moves < 8; ++moves) {
+                int32_t ecc2, pick2;
+                w.bfs(pick, bfs_id++, &ecc2, &pick2);
+                if (ecc2 <= ecc) break;
+                start = pick;
+                ecc = ecc2;
+                pick = pick2;
+            }
+        }
+        if (w.gid == 0) cm_set(w, placed, start);
+        cluster.sync();
+        int64_t ls = placed, le = placed + 1;
+        while (le > ls) {
+            // the CTAs take equal runs of the frontier, their threads `m` consecutive positions
+            // each, so that the children's order is that of a scan over CTAs and threads
+            const int64_t run = (le - ls + ranks - 1) / ranks;
+            const int64_t m = (run + THREADS - 1) / THREADS;
+            const int64_t r1 = ls + (rank + 1) * run < le ? ls + (rank + 1) * run : le;
+            const int64_t p0 = ls + rank * run + threadIdx.x * m;
+            const int64_t p1 = p0 + m < r1 ? p0 + m : r1;
+            // every unplaced neighbour of a frontier node records the earliest position
+            for (int64_t p = p0; p < p1; ++p) {
+                const int32_t u = ld_l2(perm + p);
+                const int32_t b = rp[u + 1];
+                for (int32_t k = rp[u]; k < b; k += kCmBatch) {
+                    int32_t v[kCmBatch];
+                    w.load_row(u, k, b, v);
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j)
+                        if (v[j] >= 0 && ld_l2(pos + v[j]) != -1) v[j] = -1;
+#pragma unroll
+                    for (int j = 0; j < kCmBatch; ++j)
+                        if (v[j] >= 0) atomicMin(&claim[v[j]], (int32_t)p);
+                }
+            }
+            cluster.sync();
+            // children per thread, their scan over the cluster
+            unsigned long long key[kCmKids];
+            int32_t u = -1;
+            int mine = 0;
+            for (int64_t p = p0; p < p1; ++p) {
+                u = ld_l2(perm + p);
+                mine += cm_kids(w, p, u, key);
+            }
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            if (lane == 31) warp_sums[warp] = incl;
+            __syncthreads();
+            const int ws = lane < THREADS / 32 ? warp_sums[lane] : 0;
+            int before = lane < warp ? ws : 0, all = ws;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                before += __shfl_xor_sync(0xffffffffu, before, o);
+                all += __shfl_xor_sync(0xffffffffu, all, o);
+            }
+            turn ^= 1;
+            if ((int)threadIdx.x < ranks)
+                *cluster.map_shared_rank(&totals[turn][rank], threadIdx.x) = all;
+            cluster.sync();
+            int64_t at = le + before + incl - mine, total = 0;
+            for (int r = 0; r < ranks; ++r) {
+                const int x = totals[turn][r];
+                if (r < rank) at += x;
+                total += x;
+            }
+            if (m == 1) {
+                if (mine) cm_place_kids(w, p0, u, mine, key, at);
+            } else {
+                for (int64_t p = p0; p < p1; ++p) {
+                    u = ld_l2(perm + p);
+                    const int cnt = cm_kids(w, p, u, key);
+                    cm_place_kids(w, p, u, cnt, key, at);
+                    at += cnt;
+                }
+            }
+            cluster.sync();
+            ls = le;
+            le += total;
+        }
+        placed = le;
+    }
+    if (w.gid == 0) {
+        *placed_io = placed;
+        *bfs_id_io = bfs_id;
+    }
+    cluster.sync();  // no CTA leaves while another may use its shared memory
 }
 
 __global__ void reverse_kernel(int32_t n, const int32_t *src, int32_t *dst) {
@@ -171,166 +395,65 @@ __global__ void fill_i32(int32_t *p, int64_t n, int32_t v) {
     if (i < n) p[i] = v;
 }
 
-struct CmScratch {
-    int32_t *deg = nullptr, *pos = nullptr, *claim = nullptr, *stamp = nullptr,
-            *queue = nullptr, *cm = nullptr, *tail = nullptr;
-    int64_t *counts = nullptr;
-    unsigned long long *key = nullptr;
-    void *host = nullptr;  // pinned: [0] = int64 scratch, [1] = key
-};
-
-spmv_status_t read_i64(const int64_t *d, int64_t *h, void *pinned, cudaStream_t st) {
-    GB_CUDA(cudaMemcpyAsync(pinned, d, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaStreamSynchronize(st));
-    *h = *(int64_t *)pinned;
-    return SPMV_OK;
-}
-
-spmv_status_t read_i32(const int32_t *d, int32_t *h, void *pinned, cudaStream_t st) {
-    GB_CUDA(cudaMemcpyAsync(pinned, d, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaStreamSynchronize(st));
-    *h = *(int32_t *)pinned;
-    return SPMV_OK;
-}
-
-spmv_status_t read_key(const unsigned long long *d, unsigned long long *h, void *pinned,
-                       cudaStream_t st) {
-    GB_CUDA(cudaMemcpyAsync(pinned, d, sizeof(*d), cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaStreamSynchronize(st));
-    *h = *(unsigned long long *)pinned;
-    return SPMV_OK;
-}
-
-// BFS level structure from r over unplaced nodes; eccentricity and the min-key node of the
-// last level.
-spmv_status_t bfs_ecc(int32_t n, const int32_t *rp, const int32_t *ci, CmScratch &w,
-                      int32_t r, int32_t id, cudaStream_t st, int32_t *ecc, int32_t *pick) {
-    bfs_seed<<<1, 1, 0, st>>>(r, id, w.stamp, w.queue, w.tail);
-    GB_LAUNCHED();
-    int64_t ls = 0, le = 1;
-    int32_t levels = 0;
-    int64_t last_ls = 0, last_le = 1;
-    while (le > ls) {
-        last_ls = ls;
-        last_le = le;
-        bfs_expand<<<blocks_for(le - ls), kT, 0, st>>>(rp, ci, w.pos, id, w.stamp, w.queue, ls,
-                                                       le, w.tail);
-        GB_LAUNCHED();
-        int32_t t;
-        GB_TRY(read_i32(w.tail, &t, w.host, st));
-        ls = le;
-        le = t;
-        if (le > ls) ++levels;
-    }
-    GB_CUDA(cudaMemsetAsync(w.key, 0xff, sizeof(unsigned long long), st));
-    min_key_range<<<blocks_for(last_le - last_ls), kT, 0, st>>>(w.queue, last_ls, last_le, w.deg,
-                                                               w.key);
-    GB_LAUNCHED();
-    unsigned long long k;
-    GB_TRY(read_key(w.key, &k, w.host, st));
-    *ecc = levels;
-    *pick = (int32_t)(k & 0xffffffffull);
-    (void)n;
-    return SPMV_OK;
-}
-
 spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, bool reverse,
                               bool peripheral, int32_t *perm_out, cudaStream_t st) {
     if (n == 0) return SPMV_OK;
-    CmScratch w;
-    spmv_status_t s = SPMV_OK;
-    auto alloc = [&](void **p, size_t bytes) {
-        if (s != SPMV_OK) return;
-        s = cuda_status(gb_malloc_async(p, bytes, st));
-    };
-    alloc((void **)&w.deg, sizeof(int32_t) * n);
-    alloc((void **)&w.pos, sizeof(int32_t) * n);
-    alloc((void **)&w.claim, sizeof(int32_t) * n);
-    alloc((void **)&w.stamp, sizeof(int32_t) * n);
-    alloc((void **)&w.queue, sizeof(int32_t) * n);
-    alloc((void **)&w.cm, sizeof(int32_t) * n);
-    alloc((void **)&w.tail, sizeof(int32_t));
-    alloc((void **)&w.counts, sizeof(int64_t) * ((size_t)n + 1));
-    alloc((void **)&w.key, sizeof(unsigned long long));
-    if (s == SPMV_OK) s = cuda_status(cudaMallocHost(&w.host, 64));
-    if (s == SPMV_OK) {
-        s = [&]() -> spmv_status_t {
-            const unsigned nb = blocks_for(n);
-            degree_kernel<<<nb, kT, 0, st>>>(n, rp, ci, w.deg);
-            fill_i32<<<nb, kT, 0, st>>>(w.pos, n, -1);
-            fill_i32<<<nb, kT, 0, st>>>(w.claim, n, INT_MAX);
-            fill_i32<<<nb, kT, 0, st>>>(w.stamp, n, -1);
-            GB_LAUNCHED();
-            int32_t bfs_id = 0;
-            int64_t placed = 0;
-            while (placed < n) {
-                GB_CUDA(cudaMemsetAsync(w.key, 0xff, sizeof(unsigned long long), st));
-                min_key_unplaced<<<nb, kT, 0, st>>>(n, w.deg, w.pos, w.key);
-                GB_LAUNCHED();
-                unsigned long long k;
-                GB_TRY(read_key(w.key, &k, w.host, st));
-                int32_t start = (int32_t)(k & 0xffffffffull);
-                if (peripheral) {
-                    int32_t ecc, pick;
-                    GB_TRY(bfs_ecc(n, rp, ci, w, start, bfs_id++, st, &ecc, &pick));
-                    for (int moves = 0; moves < 8; ++moves) {
-                        int32_t ecc2, pick2;
-                        GB_TRY(bfs_ecc(n, rp, ci, w, pick, bfs_id++, st, &ecc2, &pick2));
-                        if (ecc2 > ecc) {
-                            start = pick;
-                            ecc = ecc2;
-                            pick = pick2;
-                        } else {
-                            break;
-                        }
-                    }
-                }
-                place_start<<<1, 1, 0, st>>>(start, placed, w.cm, w.pos);
-                GB_LAUNCHED();
-                int64_t ls = placed, le = placed + 1;
-                placed += 1;
-                while (le > ls) {
-                    const int64_t nf = le - ls;
-                    const unsigned fb = blocks_for(nf);
-                    cm_claim<<<fb, kT, 0, st>>>(rp, ci, w.cm, w.pos, w.claim, ls, le);
-                    cm_count<<<fb, kT, 0, st>>>(rp, ci, w.cm, w.pos, w.claim, ls, le, w.counts);
-                    GB_LAUNCHED();
-                    GB_TRY(exclusive_scan_i64(w.counts, nf, st));
-                    cm_place<<<fb, kT, 0, st>>>(rp, ci, w.deg, w.cm, w.pos, w.claim, ls, le,
-                                                w.counts);
-                    GB_LAUNCHED();
-                    int64_t total;
-                    GB_TRY(read_i64(w.counts + nf, &total, w.host, st));
-                    if (total > 0) {
-                        set_pos<<<blocks_for(total), kT, 0, st>>>(w.cm, le, le + total, w.pos);
-                        GB_LAUNCHED();
-                    }
-                    ls = le;
-                    le = le + total;
-                    placed = le;
-                }
-            }
-            if (reverse) {
-                reverse_kernel<<<nb, kT, 0, st>>>(n, w.cm, perm_out);
-            } else {
-                GB_CUDA(cudaMemcpyAsync(perm_out, w.cm, sizeof(int32_t) * n,
-                                        cudaMemcpyDeviceToDevice, st));
-            }
-            GB_LAUNCHED();
-            return SPMV_OK;
-        }();
-    }
-    GB_CUDA(cudaStreamSynchronize(st));
-    cudaFreeAsync(w.deg, st);
-    cudaFreeAsync(w.pos, st);
-    cudaFreeAsync(w.claim, st);
-    cudaFreeAsync(w.stamp, st);
-    cudaFreeAsync(w.queue, st);
-    cudaFreeAsync(w.cm, st);
-    cudaFreeAsync(w.tail, st);
-    cudaFreeAsync(w.counts, st);
-    cudaFreeAsync(w.key, st);
-    if (w.host) cudaFreeHost(w.host);
+    // six arrays of n words, then the progress words
+    int32_t *mem = nullptr;
+    const size_t stride = ((size_t)n + 63) / 64 * 64;
+    GB_CUDA(gb_malloc_async((void **)&mem, sizeof(int32_t) * (6 * stride + 8), st));
+    int32_t *deg = mem, *pos = mem + stride, *claim = mem + 2 * stride, *stamp = mem + 3 * stride,
+            *queue = mem + 4 * stride, *cm = mem + 5 * stride;
+    int64_t *placed_d = (int64_t *)(mem + 6 * stride);
+    int32_t *bfs_id_d = mem + 6 * stride + 2, *grown_d = mem + 6 * stride + 3;
+    spmv_status_t s = [&]() -> spmv_status_t {
+        const unsigned nb = blocks_for(n);
+        degree_kernel<<<nb, kT, 0, st>>>(n, rp, ci, deg);
+        fill_i32<<<nb, kT, 0, st>>>(pos, n, -1);
+        fill_i32<<<nb, kT, 0, st>>>(claim, n, INT_MAX);
+        fill_i32<<<nb, kT, 0, st>>>(stamp, n, -1);
+        GB_LAUNCHED();
+        GB_CUDA(cudaMemsetAsync(placed_d, 0, 4 * sizeof(int32_t), st));
+        // 512 threads per CTA leave registers for a row's loads in flight; the frontiers of
+        // larger graphs (about 10K nodes from 1.5M on) keep 1,024 busy.  Whole set-up, ms, 512 /
+        // 1,024: 48K cells 3.1 / 3.4, 796K 9.7 / 10.3, 3.1M 23.5 / 21.9, 6M 43.0 / 40.4.
+        const bool wide = n >= 1500000;
+        auto *kern = wide ? cm_cluster<1024> : cm_cluster<512>;
+        GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kCmCluster;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(kCmCluster);
+        cfg.blockDim = dim3(wide ? 1024 : 512);
+        cfg.stream = st;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int fits = 0;
+        if (cudaOccupancyMaxActiveClusters(&fits, kern, &cfg) != cudaSuccess || fits < 1) {
+            cudaGetLastError();
+            attr[0].val.clusterDim.x = 8;  // the portable size
+            cfg.gridDim = dim3(8);
+        }
+        int64_t placed = 0;
+        while (placed < n) {
+            GB_CUDA(cudaLaunchKernelEx(&cfg, kern, n, rp, ci, (const int32_t *)deg, pos,
+                                       claim, stamp, queue, cm, peripheral ? 1 : 0,
+                                       kCmComponents, placed_d, bfs_id_d, grown_d));
+            GB_CUDA(cudaMemcpyAsync(&placed, placed_d, sizeof(int64_t), cudaMemcpyDeviceToHost,
+                                    st));
+            GB_CUDA(cudaStreamSynchronize(st));
+        }
+        if (reverse)
+            reverse_kernel<<<nb, kT, 0, st>>>(n, cm, perm_out);
+        else
+            GB_CUDA(cudaMemcpyAsync(perm_out, cm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice,
+                                    st));
+        GB_LAUNCHED();
+        return SPMV_OK;
+    }();
+    cudaFreeAsync(mem, st);
     return s;
 }
 

@@ -408,6 +408,50 @@ def test_gpu_cm_order_hand_worked_graphs(oracle):
             assert list(A.permutation()) == expect
 
 
+def graph_csr(n, edges):
+    """Pattern of a graph's symmetric matrix with a full diagonal."""
+    e = np.asarray(edges, np.int64).reshape(-1, 2)
+    i = np.concatenate([e[:, 0], e[:, 1], np.arange(n)])
+    j = np.concatenate([e[:, 1], e[:, 0], np.arange(n)])
+    key = np.unique(i * n + j)
+    i, j = key // n, key % n
+    rp = np.zeros(n + 1, np.int64)
+    np.add.at(rp, i + 1, 1)
+    return np.cumsum(rp).astype(np.int32), j.astype(np.int32), np.ones(j.size)
+
+
+def ordering_graph(kind):
+    rng = np.random.default_rng(5)
+    if kind == "isolated":       # components of one node, more than one launch orders
+        return graph_csr(700, [])
+    if kind == "paths":          # several hundred components of different lengths
+        edges, n = [], 0
+        for k in range(400):
+            edges += [(n + t, n + t + 1) for t in range(k % 5)]
+            n += k % 5 + 1
+        p = rng.permutation(n)
+        return graph_csr(n, p[np.asarray(edges)])
+    if kind == "star":           # one parent with more children than are sorted in registers
+        return graph_csr(3000, [(1234, k) for k in range(3000) if k != 1234])
+    if kind == "wheel":          # long rows beside short ones
+        return graph_csr(500, [(0, k) for k in range(1, 500)] + [(k, k + 1) for k in range(1, 499)])
+    if kind == "broad":          # levels wider than the cluster has threads
+        n = 60000
+        return graph_csr(n, [(k, (k - 1) // 300) for k in range(1, n)])
+    n = 5000                     # random sparse graph, several components
+    return graph_csr(n, rng.integers(0, n, (2 * n // 3, 2)))
+
+
+@pytest.mark.parametrize("kind", ["isolated", "paths", "star", "wheel", "broad", "random"])
+@pytest.mark.parametrize("peripheral", [0, 1])
+def test_gpu_cm_order_of_unusual_graphs(oracle, kind, peripheral):
+    rp, ci, v = ordering_graph(kind)
+    n = rp.size - 1
+    A = capi.Matrix(n, rp, ci, v, reorder=capi.SPMV_REORDER_CM, peripheral=peripheral)
+    ref = oracle.cm_order(rp, ci, reverse=False, peripheral=bool(peripheral))
+    assert np.array_equal(A.permutation(), ref)
+
+
 @pytest.mark.parametrize("reorder", [capi.SPMV_REORDER_NONE, capi.SPMV_REORDER_RCM])
 @pytest.mark.parametrize("sigma", [64, 1024, 4096])
 def test_sigma_sorted_rows_match_oracle(oracle, sigma, reorder):
