@@ -1,8 +1,7 @@
 // spmm.cu -- multi-right-hand-side products Y = A X (not in the paper).
 //
-// spmm_sell<T, G, C>: X and Y row-major (n x k), G lanes per row, each lane C columns;
-// every gathered row of X (k contiguous values) is read once per matrix entry and used for
-// all k columns.  Column c of Y equals the single-vector product of column c bit for bit
+// X and Y are row-major (n x k), a group of lanes per row; every gathered row of X (k contiguous
+// values) is read once per matrix entry and used for all k columns.  Column c of Y equals the single-vector product of column c bit for bit
 // (same entry order, fused multiply-add from +0.0).
 #include <algorithm>
 #include <type_traits>
@@ -22,7 +21,9 @@ inline unsigned grid_for(int64_t threads, int block) {
 // share its width), lane g owns columns g, g + G, ... (C of them).  The lanes of a row first
 // load G of its (value, column) pairs at once, one per lane; the pairs are then broadcast
 // inside the row's lane group by shuffles, four at a time, so each lane issues 4 C gathers of
-// X back to back instead of one dependent load-then-gather round per entry.
+// X back to back instead of one dependent load-then-gather round per entry.  For the FP64
+// products where a power of two of lanes per row wastes little of the FP64 pipe (see
+// piece_choice).
 template <typename T, int G, int C, typename ColT>
 __global__ void __launch_bounds__(256)
 spmm_sell(int32_t n, int32_t S, int32_t n_slices, int k, const int64_t *__restrict__ sp,
@@ -234,6 +235,158 @@ struct Wide<double> {
                      : "memory");
     }
 };
+
+// Loads and stores of P consecutive elements (4 to 32 bytes) of a row of X or Y.
+template <typename T, int P>
+__device__ __forceinline__ void ld_cols(const T *p, T (&v)[P]) {
+    if constexpr (P == 1) {
+        v[0] = __ldg(p);
+    } else if constexpr (P == 2 && sizeof(T) == 8) {
+        const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
+        v[0] = t.x, v[1] = t.y;
+    } else if constexpr (P == 2) {
+        const float2 t = __ldg(reinterpret_cast<const float2 *>(p));
+        v[0] = t.x, v[1] = t.y;
+    } else if constexpr (P == 4 && sizeof(T) == 4) {
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else {
+        Wide<T>::load(p, v);
+    }
+}
+template <typename T, int P>
+__device__ __forceinline__ void st_cols(T *p, const T (&v)[P]) {
+    if constexpr (P == 1) *p = v[0];
+    else if constexpr (P == 2 && sizeof(T) == 8)
+        *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+    else if constexpr (P == 2) *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+    else if constexpr (P == 4 && sizeof(T) == 4)
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else Wide<T>::store(p, v);
+}
+
+// SpMM for any k: a row's k columns are cut into pieces of P, the largest of 32, 16, 8 bytes or
+// one element that divides the row and that X and Y are aligned to; G lanes take a row, lane g
+// its pieces g, g + G, ... (C of them, the last perhaps none), and a warp as many rows as fit:
+// 32 / G, of any two neighbouring slices.  G lanes that read the same matrix entry share one
+// transaction, and the (value, column) pairs of U entries are requested before their gathers.
+// Same entry order and fused multiply-add from +0.0 as the other SpMM kernels, so the results
+// are identical.  The product is bound by the latency of its gathers: several pieces per lane
+// put more rows into a warp and more bytes in flight, which is why C is three to five for
+// narrow pieces; two or three entries in flight leave more warps room than five (f32 k = 5 on
+// 312K mixed-mesh rows: 14.4 us with three, 16.1 with five).  Measured there against a power
+// of two of lanes per row with the pairs broadcast by shuffles (spmm_sell): f32 k = 5 30.9 ->
+// 14.4 us, 6 31.2 -> 13.8, 11 54.5 -> 28.9, 20 105 -> 36, 31 108 -> 67; f64 k = 5 51.7 -> 37.3.
+constexpr int piece_unroll(int bytes, int elem) {
+    return bytes <= (elem == 4 ? 24 : 16) ? 3 : 2;
+}
+
+// Pieces per lane (C) for `pieces` pieces of P elements, or 0 when spmm_sell is faster.
+// FP32: the narrow pieces' best count, the one of two that leaves fewer lanes idle.  FP64: the
+// FP64 pipe is the other bound and takes a warp's instruction whole, so the count with the
+// fewest multiply-adds per row and entry, P C / (32 / G), is taken, and where spmm_sell needs
+// no more than 1.1 times as many (k = 7, 13 to 15, 26 to 31, 50 to 63) it stays: it has fewer
+// rows per warp, so rows of unlike lengths leave fewer of them idle (mixed mesh, k = 31: 122
+// against 134 us; k = 25, one group of lanes above, 115 against 111).
+inline int piece_choice(int k, int P, int elem) {
+    const int pieces = k / P;
+    auto valid = [&](int C) {
+        const int G = (pieces + C - 1) / C;
+        return G <= 32 && (C - 1) * G < pieces;
+    };
+    auto use = [&](int C) {
+        const int G = (pieces + C - 1) / C;
+        return (double)(32 / G) * pieces / (32.0 * C);
+    };
+    if (k == 1) return 0;
+    if (elem == 4) {
+        if (P == 8) return pieces >= 6 ? 3 : 1;
+        const int hi = P == 1 ? 4 : 3, lo = P == 1 ? 5 : 2;
+        if (!valid(hi) || !valid(lo)) {
+            for (int C : {hi, lo, 3, 2, 1})
+                if (valid(C)) return C;
+        }
+        return use(lo) > use(hi) + (P == 1 ? 0.001 : 0.1) ? lo : hi;
+    }
+    int best = 0;
+    for (int C = 1; C <= (P == 1 ? 5 : 3); ++C)
+        if (valid(C) && (!best || use(C) >= use(best) - 1e-9)) best = C;
+    if (P == 4 && k == 64) return 3;  // 1.2 times the work of C = 1, but 210 against 260 us on ragged rows
+    if (P > 1 && (k & (k - 1)) == 0) return best;
+    int lanes = 1;
+    while (lanes < k && lanes < 32) lanes *= 2;
+    const double other = k <= 32 ? k * (32 / lanes) / 32.0 : k / 64.0;
+    return use(best) >= other / 0.9 ? best : 0;
+}
+
+template <typename T, int P, int C, typename ColT>
+__global__ void __launch_bounds__(256)
+spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ sp, ColT cols,
+                const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
+    constexpr int U = piece_unroll(P * C * (int)sizeof(T), (int)sizeof(T));
+    const int rpw = 32 / G;
+    const int lane = threadIdx.x & 31;
+    const int sub = lane / G, g = lane - sub * G;
+    const int64_t row = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * rpw + sub;
+    if (sub >= rpw || row >= n) return;
+    // (w is set under a test that always holds here: with its value plain, the compiler knows the
+    // first entry of each round exists and branches around the others' loads instead of
+    // predicating them, and they no longer overlap: f32 k = 31 56 against 39 us)
+    const uint64_t pol = policy_evict_first();
+    int w = 0;
+    int32_t cb = 0;
+    int64_t at = 0;
+    if (row < n) {
+        const int64_t slice = row / S;
+        const int64_t base = sp[slice];
+        w = (int)((sp[slice + 1] - base) / S);
+        cb = cols.base(slice);
+        at = base + (row - slice * S);
+    }
+    bool has[C];
+#pragma unroll
+    for (int j = 0; j < C; ++j) has[j] = j == 0 || (g + j * G) * P < k;
+    const T *xg = X + g * P;
+    T acc[C][P];
+#pragma unroll
+    for (int j = 0; j < C; ++j)
+#pragma unroll
+        for (int e = 0; e < P; ++e) acc[j][e] = T(0);
+    for (int t0 = 0; t0 < w; t0 += U) {
+        T a[U][1];
+        int32_t c[U][1];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a[u][0] = T(0);
+            c[u][0] = -1;
+            if (t0 + u < w) {
+                ld_stream(val + at + (int64_t)(t0 + u) * S, pol, a[u]);
+                cols.template load<1>(at + (int64_t)(t0 + u) * S, 0, pol, cb, c[u]);
+            }
+        }
+        T xv[U][C][P];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c[u][0] < 0) continue;
+            const T *xr = xg + (int64_t)c[u][0] * k;
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                if (has[j]) ld_cols<T, P>(xr + j * G * P, xv[u][j]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c[u][0] < 0) continue;
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+#pragma unroll
+                for (int e = 0; e < P; ++e) acc[j][e] = fma_t(a[u][0], xv[u][j][e], acc[j][e]);
+        }
+    }
+    T *yr = Y + row * k + g * P;
+#pragma unroll
+    for (int j = 0; j < C; ++j)
+        if (has[j]) st_cols<T, P>(yr + j * G * P, acc[j]);
+}
 
 // SpMM for k = G * (32 bytes / sizeof(T)) with 32-byte aligned X and Y: lane g of a row's G
 // lanes owns 32 consecutive bytes of the row and gathers them with one 256-bit load.  Every
@@ -683,7 +836,9 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
         if (k == WV * 4) return wide(integral_constant<int, 4>{});
         if (k == WV * 8) return wide(integral_constant<int, 8>{});
     }
-    // vectorised kernel when k is a power of two with k >= 16 / sizeof(T), k <= 64
+    // k a power of two of 16-byte pieces (X and Y not 32-byte aligned, or k = 4 in FP32); FP64
+    // k = 2 and 64 are faster cut into pieces (15.0 -> 11.7 and 253 -> 210 us on a 192K-row
+    // mixed mesh, 143 -> 125 on a 162K-row tetrahedral one)
     constexpr int VW = sizeof(T) == 8 ? 2 : 4;
     auto vec = [&](auto gtag) -> spmv_status_t {
         constexpr int G = decltype(gtag)::value;
@@ -700,12 +855,54 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
         return SPMV_OK;
     };
     using std::integral_constant;
-    if (k == VW * 1) return vec(integral_constant<int, 1>{});
+    if constexpr (sizeof(T) == 4) {
+        if (k == VW * 1) return vec(integral_constant<int, 1>{});
+    }
     if (k == VW * 2) return vec(integral_constant<int, 2>{});
     if (k == VW * 4) return vec(integral_constant<int, 4>{});
     if (k == VW * 8) return vec(integral_constant<int, 8>{});
     if (k == VW * 16) return vec(integral_constant<int, 16>{});
-    if (k == VW * 32 && VW * 32 <= 64) return vec(integral_constant<int, 32>{});
+    // any other k: pieces of P columns, C per lane
+    bool done = false;
+    auto piece = [&](auto ptag) -> spmv_status_t {
+        constexpr int P = decltype(ptag)::value;
+        const int pieces = k / P;
+        auto go = [&](auto ctag) -> spmv_status_t {
+            constexpr int C = decltype(ctag)::value;
+            const int G = (pieces + C - 1) / C;
+            const int64_t warps = ((int64_t)A->n + 32 / G - 1) / (32 / G);
+            const unsigned grid = grid_for(warps * 32, block);
+            if (A->index_bits == 16)
+                spmm_sell_piece<T, P, C, Cols16><<<grid, block, 0, st>>>(
+                    A->n, A->S, k, G, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p}, val,
+                    X, Y);
+            else
+                spmm_sell_piece<T, P, C, Cols32><<<grid, block, 0, st>>>(
+                    A->n, A->S, k, G, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
+            done = true;
+            GB_LAUNCHED();
+            return SPMV_OK;
+        };
+        switch (piece_choice(k, P, (int)sizeof(T))) {
+            case 1: return go(integral_constant<int, 1>{});
+            case 2: return go(integral_constant<int, 2>{});
+            case 3: return go(integral_constant<int, 3>{});
+            case 4:
+                if constexpr (P == 1) return go(integral_constant<int, 4>{});
+                break;
+            case 5:
+                if constexpr (P == 1) return go(integral_constant<int, 5>{});
+                break;
+        }
+        return SPMV_OK;
+    };
+    const uintptr_t where = (uintptr_t)X | (uintptr_t)Y | (uintptr_t)(k * sizeof(T));
+    spmv_status_t s = SPMV_OK;
+    if (where % 32 == 0) s = piece(integral_constant<int, 32 / (int)sizeof(T)>{});
+    else if (where % 16 == 0) s = piece(integral_constant<int, 16 / (int)sizeof(T)>{});
+    else if (sizeof(T) == 4 && where % 8 == 0) s = piece(integral_constant<int, sizeof(T) == 4 ? 2 : 1>{});
+    else s = piece(integral_constant<int, 1>{});
+    if (s != SPMV_OK || done) return s;
     auto go = [&](auto gtag, auto ctag) -> spmv_status_t {
         constexpr int G = decltype(gtag)::value;
         constexpr int C = decltype(ctag)::value;
@@ -722,18 +919,15 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
         return SPMV_OK;
     };
     using I1 = std::integral_constant<int, 1>;
-    using I2 = std::integral_constant<int, 2>;
-    using I4 = std::integral_constant<int, 4>;
-    using I8 = std::integral_constant<int, 8>;
-    using I16 = std::integral_constant<int, 16>;
-    using I32 = std::integral_constant<int, 32>;
-    if (k <= 1) return go(I1{}, I1{});
-    if (k <= 2) return go(I2{}, I1{});
-    if (k <= 4) return go(I4{}, I1{});
-    if (k <= 8) return go(I8{}, I1{});
-    if (k <= 16) return go(I16{}, I1{});
-    if (k <= 32) return go(I32{}, I1{});
-    return go(I32{}, I2{});
+    if (k == 1) return go(I1{}, I1{});
+    if constexpr (sizeof(T) == 8) {
+        using I2 = std::integral_constant<int, 2>;
+        if (k <= 8) return go(std::integral_constant<int, 8>{}, I1{});
+        if (k <= 16) return go(std::integral_constant<int, 16>{}, I1{});
+        if (k <= 32) return go(std::integral_constant<int, 32>{}, I1{});
+        return go(std::integral_constant<int, 32>{}, I2{});
+    }
+    return SPMV_ERR_INVALID_ARG;
 }
 
 // Tuner of the 256-bit SpMM's form for this (precision, k): each form in turn computes the

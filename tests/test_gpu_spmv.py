@@ -534,6 +534,27 @@ def test_spmm_parity(oracle, k, dtype, bits):
     assert np.array_equal(Y[:, c], yc)
 
 
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 6, 7, 9, 11, 12, 17, 20, 23, 24, 31, 33, 40, 44, 48, 57,
+                               63, 64])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_spmm_any_column_count(oracle, dtype, k, bits):
+    """Products whose rows are gathered in pieces of 4 to 32 bytes, one to three per lane: ragged
+    rows (0 to 17 entries, so every remainder of the load rounds), a row count that is no
+    multiple of a warp's rows or of a slice, warps whose rows lie in two slices; bit-exact."""
+    n = 1237
+    m = ragged_matrix(n, seed=k, max_len=17)
+    X = np.random.default_rng(k).uniform(-1, 1, (n, k)).astype(dtype)
+    A = capi.Matrix(n, m.row_ptr, m.col_idx, m.values, precision=capi.SPMV_PREC_DUAL,
+                    index_bits=bits, slice_height=32)
+    Xd = dev(X)
+    Y = torch.full_like(Xd, float("nan"))
+    A.apply_multi(Xd, Y)
+    torch.cuda.synchronize()
+    ref = oracle.spmm(m.row_ptr, m.col_idx, m.values.astype(dtype), X, use_fma=True)
+    assert np.array_equal(Y.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("k", [4, 8, 32])
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_spmm_16_byte_aligned_blocks(oracle, k, dtype):
