@@ -162,6 +162,7 @@ struct spmv_matrix_s {
     int32_t max_span = 0;
     int32_t n_slices = 0;
     int32_t max_width = 0;  // widest slice: its stored entries per row
+    float mean_width = 0.f;  // stored entries per row, padding included, over all slices
     int64_t sell_entries = 0;
     size_t bytes = 0;  // device bytes owned
 

@@ -666,6 +666,7 @@ spmv_status_t build_sell(spmv_matrix_t A, int S, cudaStream_t st) {
                             cudaMemcpyDeviceToHost, st));
     GB_CUDA(cudaStreamSynchronize(st));
     A->sell_entries = total;
+    A->mean_width = n_slices > 0 ? (float)((double)total / ((double)n_slices * S)) : 0.f;
     GB_TRY(A->sell_col.alloc((size_t)total, tally));
     if (A->has64()) GB_TRY(A->sell_val.alloc((size_t)total, tally));
     else A->sell_val.release(tally);

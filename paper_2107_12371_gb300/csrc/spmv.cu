@@ -15,6 +15,8 @@
 //   with five entries of each row in flight; the one whose widest slice needs fewer dependent
 //   load rounds is launched.
 // spmv_csr: the naive baseline of Sec. 4.3, thread per CSR row.
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -125,6 +127,75 @@ spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT c
         spmv_sell_body<T, R, L, U, ColT, AXPBY>(gt, n, n_slices, sp, cols, val, x, y, alpha, beta);
 }
 
+// The product of small and of ragged matrices (see use_thin): one or two rows per lane, S / R
+// lanes per slice (a slice may span several warps), U entries in flight, and the remainder of
+// a row as one more round with the missing entries masked instead of one dependent round per
+// entry.  At these sizes the chip is not full: a row is a chain of three or four dependent
+// loads of 0.6 us, and what helps is more threads (four rows per lane leave 400K rows a third
+// of the thread slots) and fewer rounds (a 13-entry row took five with U = 5 and a plain loop
+// behind it).  Measured (us, before -> now): FP32 398K mixed-mesh rows 10.9 -> 6.6 (int32
+// columns), 24K 5.9 -> 2.7, 48K tetrahedra 3.8 -> 2.9, 1.3M 10.8 -> 8.8; FP64 24K mixed 6.4 ->
+// 3.7, 192K 9.6 -> 7.1, 48K tetrahedra 3.4 -> 3.0.  Same order and bits as spmv_sell.
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
+__global__ void __launch_bounds__(1024, 1)
+spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
+               const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
+               T beta) {
+    constexpr int S = L * R;
+    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t slice = gt / L;
+    if (slice >= n_slices) return;
+    const int lane = (int)(gt % L);
+    const int64_t base = sp[slice];
+    const int w = (int)((sp[slice + 1] - base) / S);
+    const int32_t cbase = cols.base(slice);
+    const int64_t at = base + lane * R;
+    const uint64_t pol = policy_evict_first();
+    T acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = T(0);
+    auto round = [&](int t, auto masked) {
+        constexpr bool kMasked = decltype(masked)::value;
+        T v[U][R];
+        int32_t c[U][R];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (!kMasked || t + u < w) {
+                ld_stream(val + at + (int64_t)(t + u) * S, pol, v[u]);
+                cols.template load<R>(at + (int64_t)(t + u) * S, slice, pol, cbase, c[u]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    v[u][i] = T(0);
+                    c[u][i] = -1;
+                }
+            }
+        }
+        T xv[U][R];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < R; ++i) xv[u][i] = c[u][i] >= 0 ? ld_x(x + c[u][i]) : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                if (c[u][i] >= 0) acc[i] = fma_t(v[u][i], xv[u][i], acc[i]);
+    };
+    int t = 0;
+    for (; t + U <= w; t += U) round(t, std::false_type{});
+    if (t < w) round(t, std::true_type{});
+    const int64_t row0 = gt * R;
+    if constexpr (AXPBY) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            if (row0 + i < n)
+                acc[i] = beta != T(0) ? fma_t(alpha, acc[i], beta * y[row0 + i]) : alpha * acc[i];
+        }
+    }
+    store_rows<T, R>(y, row0, n, acc);
+}
+
 // naive CSR baseline (Sec. 4.3): the column index is read first, then x[col] from global
 // memory, thread per row
 template <typename T>
@@ -183,10 +254,75 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
     return SPMV_OK;
 }
 
+// Where spmv_sell_thin is the faster kernel (old / thin, measured on tetrahedral and mixed meshes
+// in random, RCM and sorted order).  FP32, whose other kernels take four or eight rows per lane:
+// 1.1 to 2.6 up to 1.5M rows (2.0M: 0.93); with alpha and beta and at S = 256 up to 512K (750K:
+// 0.93 to 0.97).  FP64: up to 64K rows (1.0 to 1.7), at S >= 128, whose other kernels take four
+// and eight rows per lane (1.1 to 4 up to 2M), and at S = 64 for slices wider than the five
+// entries that the other kernels take in one round, up to 512K rows (1.0 to 1.75; 1M: 0.89 to
+// 1.09).  Not for FP64 rows of up to five entries above 64K (304K tetrahedra: 0.94 to 1.04, the
+// gradient's two-entry rows of a chain 0.79).
+bool use_thin(const spmv_matrix_t A, bool f32, bool axpby) {
+    if (f32) return A->n <= (axpby || A->S == 256 ? 512 * 1024 : 1500000);
+    if (A->n <= 64 * 1024) return true;
+    if (A->S >= 128) return A->n <= 2000000;
+    return A->S == 64 && A->max_width > 5 && A->n <= 512 * 1024;
+}
+// FP32 lanes take one row up to here and two above (24K mixed-mesh rows 2.4 against 2.8 us, 192K
+// 3.6 and 3.8; 398K 5.7 and 5.5, 1.3M tetrahedra 9.0 and 8.2).
+constexpr int32_t kThinRows32 = 256 * 1024;
+
+template <typename T, bool AXPBY>
+spmv_status_t go_thin(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, T beta,
+                      cudaStream_t st) {
+    auto shape = [&](auto rt, auto ut, auto st_) -> spmv_status_t {
+        constexpr int R = decltype(rt)::value, U = decltype(ut)::value;
+        constexpr int L = decltype(st_)::value / R;
+        const int64_t lanes = (int64_t)A->n_slices * L;
+        // smaller CTAs while they do not fill the chip: they spread over more SMs (48K rows 2.8
+        // against 3.1 us)
+        const int block = A->block > 128 && lanes < (int64_t)device_facts().sm_count * 2048 ? 128
+                                                                                           : A->block;
+        const unsigned grid = grid_for(lanes, block);
+        if (A->index_bits == 16)
+            spmv_sell_thin<T, R, L, U, Cols16, AXPBY><<<grid, block, 0, st>>>(
+                A->n, A->n_slices, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p}, val, x,
+                y, alpha, beta);
+        else
+            spmv_sell_thin<T, R, L, U, Cols32, AXPBY><<<grid, block, 0, st>>>(
+                A->n, A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, x, y, alpha, beta);
+        GB_LAUNCHED();
+        return SPMV_OK;
+    };
+    auto go = [&](auto rt, auto ut) -> spmv_status_t {
+        switch (A->S) {
+            case 32: return shape(rt, ut, std::integral_constant<int, 32>{});
+            case 64: return shape(rt, ut, std::integral_constant<int, 64>{});
+            case 128: return shape(rt, ut, std::integral_constant<int, 128>{});
+            case 256: return shape(rt, ut, std::integral_constant<int, 256>{});
+        }
+        return SPMV_ERR_INVALID_ARG;
+    };
+    using std::integral_constant;
+    // entries in flight: a whole row of the tetrahedral meshes; for longer rows four in FP64
+    // (whose gathers then still leave the SM enough warps), six in FP32
+    const bool longer = A->mean_width > 6.f;
+    if constexpr (sizeof(T) == 8) {
+        if (longer) return go(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+        return go(integral_constant<int, 1>{}, integral_constant<int, 5>{});
+    } else {
+        if (A->n > kThinRows32) return go(integral_constant<int, 2>{}, integral_constant<int, 5>{});
+        if (longer) return go(integral_constant<int, 1>{}, integral_constant<int, 6>{});
+        return go(integral_constant<int, 1>{}, integral_constant<int, 5>{});
+    }
+}
+
 template <typename T, bool AXPBY = false>
 spmv_status_t launch_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha = T(1),
                           T beta = T(0), cudaStream_t st = nullptr) {
     if (A->n == 0) return SPMV_OK;
+    if (use_thin(A, sizeof(T) == 4, AXPBY))
+        return go_thin<T, AXPBY>(A, val, x, y, alpha, beta, st);
     if constexpr (sizeof(T) == 8) {
         switch (A->S) {
             case 32: return go_sell<T, 1, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);

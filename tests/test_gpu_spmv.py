@@ -534,6 +534,63 @@ def test_spmm_parity(oracle, k, dtype, bits):
     assert np.array_equal(Y[:, c], yc)
 
 
+@pytest.mark.parametrize("S", [32, 64, 128, 256])
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("n,max_len", [(1, 3), (31, 5), (1237, 4), (1237, 5), (1238, 6), (5003, 13),
+                                       (5001, 23)])
+def test_small_products_every_row_remainder(oracle, n, max_len, bits, S):
+    """The kernel of small and ragged matrices: rows of every remainder of its four to six
+    entries in flight, row counts at the ends of lanes, slices and CTAs, with and without alpha and
+    beta, both precisions; bit-exact."""
+    m = ragged_matrix(n, seed=n + max_len, max_len=max_len)
+    x = np.random.default_rng(n).uniform(-1, 1, n)
+    A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values, precision=capi.SPMV_PREC_DUAL,
+                    index_bits=bits, slice_height=S)
+    ref = oracle.spmv(m.row_ptr, m.col_idx, m.values, x, use_fma=True)
+    assert np.array_equal(gpu_spmv(A, x), ref)
+    v32, x32 = m.values.astype(np.float32), x.astype(np.float32)
+    assert np.array_equal(gpu_spmv(A, x32, f32=True),
+                          oracle.spmv_f32(m.row_ptr, m.col_idx, v32, x32))
+    y0 = np.random.default_rng(n + 1).uniform(-1, 1, n)
+    y = dev(y0)
+    A.apply_axpby(1.5, dev(x), -0.25, y)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), oracle.spmv_axpby(m.row_ptr, m.col_idx, m.values, 1.5, x,
+                                                             -0.25, y0))
+
+
+@pytest.mark.parametrize("rows", [64 * 1024, 64 * 1024 + 1, 256 * 1024, 256 * 1024 + 1, 512 * 1024,
+                                  512 * 1024 + 1, 1500000, 1500001, 2000000, 2000001])
+def test_product_kernels_agree_at_the_edges_of_their_ranges(rows):
+    """Products on both sides of each row count where another kernel is chosen, equal bit for bit
+    to the thread-per-row CSR kernel's (FP64) and to a mirrored matrix of another slice height."""
+    i = np.arange(rows, dtype=np.int64)
+    offs = np.array([-777, -1, 0, 1, 777, 1201])
+    j = i[:, None] + offs[None, :]
+    keep = (j >= 0) & (j < rows) & ((np.arange(6)[None, :] < 5) | (i[:, None] % 3 == 0))
+    rp = np.zeros(rows + 1, np.int64)
+    np.cumsum(keep.sum(1), out=rp[1:])
+    ci = j[keep].astype(np.int32)
+    v = np.random.default_rng(1).uniform(-1, 1, ci.size)
+    x = dev(np.random.default_rng(2).uniform(-1, 1, rows))
+    ys, y32 = [], []
+    for S in (64, 128, 32):
+        A = capi.Matrix(rows, rp.astype(np.int32), ci, v, precision=capi.SPMV_PREC_DUAL,
+                        slice_height=S)
+        y = torch.empty_like(x)
+        A.apply(x, y)
+        ys.append(y)
+        z = torch.empty(rows, dtype=torch.float32, device="cuda")
+        A.apply_f32(x.float(), z)
+        y32.append(z)
+        w = torch.empty_like(x)
+        A.apply_csr(x, w)
+        torch.cuda.synchronize()
+        assert torch.equal(y, w)
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
+    assert torch.equal(y32[0], y32[1]) and torch.equal(y32[0], y32[2])
+
+
 @pytest.mark.parametrize("bits", [16, 32])
 @pytest.mark.parametrize("k", [1, 2, 3, 5, 6, 7, 9, 11, 12, 17, 20, 23, 24, 31, 33, 40, 44, 48, 57,
                                63, 64])
