@@ -14,8 +14,8 @@
 //   r sweep  r_c -= alpha_c q_c, r_c.(D^-1 r_c), r_c.r_c -> beta_c, rho_c, convergence
 //   p sweep  x_c += alpha_c p_c (the x update of the same iteration, applied here where p_c is
 //            read anyway: one pass over P fewer), p_c = D^-1 r_c + beta_c p_c
-// Every per-column sum is reduced deterministically: per CTA in a fixed tree, then over the
-// CTAs in a fixed order (by the last CTA to arrive, or by every CTA after a grid barrier).
+// Every per-column sum is reduced deterministically: per CTA, then over the CTAs in a fixed order
+// (by every CTA of the next kernel, or by every CTA after a grid barrier).
 //
 // With opt->mixed the same kernels run in FP32 as the inner solves of FP64 iterative
 // refinement (per column: FP64 residual, FP32 inner Jacobi-PCG on r_c / ||r_c|| to the inner
@@ -49,7 +49,12 @@ struct McgCol {
 struct McgScalars {
     McgCol col[kMcgMaxCols];
     int active;      // columns with done == 0
-    int pending;     // an r sweep ran since the last product: the p sweep applies
+    // The kernel that ends an iteration writes col and active while its CTAs still need the
+    // iteration's own values: the iteration's first kernel copies those here, and its second
+    // adds the step (see mcg_product).
+    int cur_active;
+    int cur_done[kMcgMaxCols], cur_iters[kMcgMaxCols], cur_run[kMcgMaxCols];
+    double cur_rho[kMcgMaxCols], cur_alpha[kMcgMaxCols];
     int max_iter;
     int timed_out;   // persistent kernel: a grid-barrier wait or the wall-clock budget ran out
     unsigned tickets[4];
@@ -141,6 +146,8 @@ __device__ __forceinline__ void st_piece(T *p, const T (&v)[Piece<T, BYTES>::n])
 }
 
 // ---- deterministic per-column reductions ------------------------------------------------------
+// The kernels around the iteration (residual, start of an inner solve): 256-thread CTAs, fixed
+// shuffle trees, the totals by the last CTA to arrive.
 // v[q][j]: this thread's partial of quantity q for column (lane % CG) * V + j; lanes of a warp
 // with the same lane % CG hold the same columns.  The CTA's sums (fixed shuffle tree, then the
 // warps in order) go to part[(q * KP + c) * vgrid + vb].
@@ -175,18 +182,55 @@ __device__ __forceinline__ void cta_cols(double (&v)[NQ][V], double *part, int v
     }
 }
 
-// tot[q][c] = the sum over i < count of part[(q * KP + c) * count + i], in a fixed order
-// (warp w takes (q, c) pairs w, w + 8, ...; its lanes stride over i; a fixed shuffle tree).
-// Valid in every thread after return.
+// The same per-CTA sums for the kernels of an iteration (T threads, at most kIterThreads): the
+// threads' values go to shared memory ordered by column, and each (quantity, column) is added by
+// one warp in fixed point (fx_warp), so the FP64 pipe, which the iteration needs for its own
+// arithmetic, takes no part: in FP64 shuffles a CTA of 1,024 threads cost it 8,000 clocks.
+template <typename E, int CG, int V, int NQ>
+struct ColsSmem {
+    // the pitch between lane classes keeps the strided writes off each other's banks
+    static constexpr int kPitch = kIterThreads / CG + (CG < 16 ? 16 / CG : 1);
+    E v[NQ * V][CG * kPitch];
+};
+template <int CG, int V, int NQ, typename E>
+__device__ __forceinline__ void cta_cols_fx(const E (&v)[NQ][V], ColsSmem<E, CG, V, NQ> &sm, int T,
+                                            double *part, int vb, int vgrid) {
+    constexpr int KP = CG * V;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    __syncthreads();  // sm may still be read by a previous call
+    if (t < T) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                sm.v[q * V + j][(t % CG) * ColsSmem<E, CG, V, NQ>::kPitch + t / CG] = v[q][j];
+    }
+    __syncthreads();
+    const int per = T / CG;  // threads holding a column
+    for (int qc = warp; qc < NQ * KP; qc += (int)blockDim.x >> 5) {
+        const int q = qc / KP, c = qc % KP;
+        const E *src = sm.v[q * V + c % V] + (c / V) * ColsSmem<E, CG, V, NQ>::kPitch;
+        // at most 512 / 32 values per lane, eight at a time
+        constexpr int M = 8;
+        double s = 0.0;
+        for (int i0 = 0; i0 < per; i0 += 32 * M) {
+            E a[M];
+#pragma unroll
+            for (int m = 0; m < M; ++m)
+                a[m] = i0 + 32 * m + lane < per ? src[i0 + 32 * m + lane] : E(0);
+            s += fx_value(fx_warp<M>(a));
+        }
+        if (lane == 0) part[(int64_t)qc * vgrid + vb] = s;
+    }
+}
+
+// tot[q][c] = the sum over i < count of part[(q * KP + c) * count + i] (count <= 32 kPartLoads),
+// one warp per sum.  Valid in every thread after return.
 template <int KP, int NQ>
 __device__ __forceinline__ void grid_cols(const double *part, int count, double (&tot)[NQ][KP]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int qc = warp; qc < NQ * KP; qc += kMcgWarps) {
-        const double *pp = part + (int64_t)qc * count;
-        double s = 0.0;
-        for (int i = lane; i < count; i += 32) s += __ldcg(pp + i);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int qc = warp; qc < NQ * KP; qc += (int)blockDim.x >> 5) {
+        const double s = reduce_parts(part + (int64_t)qc * count, count);
         if (lane == 0) tot[qc / KP][qc % KP] = s;
     }
     __syncthreads();
@@ -204,6 +248,21 @@ __device__ __forceinline__ bool last_cta(unsigned *ticket) {
     __syncthreads();
     if (last) __threadfence();
     return last;
+}
+
+// tot[q][c] as grid_cols, over any number of CTAs' sums, in a fixed order
+template <int KP, int NQ>
+__device__ __forceinline__ void last_cols(const double *part, int count, double (&tot)[NQ][KP]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int qc = warp; qc < NQ * KP; qc += kMcgWarps) {
+        const double *pp = part + (int64_t)qc * count;
+        double s = 0.0;
+        for (int i = lane; i < count; i += 32) s += __ldcg(pp + i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) tot[qc / KP][qc % KP] = s;
+    }
+    __syncthreads();
 }
 
 // ---- per-column scalar updates (shared by the graph kernels and the persistent kernel) ------
@@ -225,15 +284,19 @@ __device__ __forceinline__ void col_after_r(McgCol &c, double rz, double rr, int
     else if (c.iters >= max_iter) c.done = 2;
 }
 
-// ---- phase bodies (virtual CTA vb of a grid of vgrid CTAs) -----------------------------------
+// ---- phase bodies -------------------------------------------------------------------------------
+// Each runs on the first g.threads threads of CTAs [0, g.ctas); CTA b takes the g.chunk items
+// (groups of rows, 16-byte pieces) from b * g.chunk (see IterGrid).
+//
 // Q = A P and per-column p.q.  G lanes per row, each owning a BYTES-wide piece (VW columns) of
 // the row; entries two at a time so two gathers are in flight, in stored order with fused
 // multiply-add from +0.0 (column c of Q equals spmv_apply on column c of P bit for bit).
 template <typename T, int G, int BYTES, bool COH, typename ColT>
-__device__ __forceinline__ void product_phase(int vb, int vgrid, int32_t n, int32_t S,
+__device__ __forceinline__ void product_phase(IterGrid g_, int32_t n, int32_t S,
                                               int32_t n_slices, const int64_t *__restrict__ sp,
                                               ColT cols, const T *__restrict__ val, const T *P,
-                                              T *Q, double *part) {
+                                              T *Q, double *part,
+                                              ColsSmem<T, G, Piece<T, BYTES>::n, 1> &sm) {
     constexpr int VW = Piece<T, BYTES>::n;
     constexpr int KP = VW * G;
     constexpr int RPW = 32 / G;
@@ -241,12 +304,13 @@ __device__ __forceinline__ void product_phase(int vb, int vgrid, int32_t n, int3
     const int sub = lane / G, g = lane % G;
     const int64_t groups = (int64_t)n_slices * S / RPW;
     const uint64_t pol = policy_evict_first();
-    double pq[1][VW];
-    T pqt[VW];
+    T pq[1][VW];
 #pragma unroll
-    for (int j = 0; j < VW; ++j) pqt[j] = T(0);
-    for (int64_t wg = (int64_t)vb * kMcgWarps + warp; wg < groups;
-         wg += (int64_t)vgrid * kMcgWarps) {
+    for (int j = 0; j < VW; ++j) pq[0][j] = T(0);
+    const int64_t end = iter_end(g_.chunk, groups);
+    const bool in = (int)threadIdx.x < g_.threads && (int)blockIdx.x < g_.ctas;
+    for (int64_t wg = in ? (int64_t)blockIdx.x * g_.chunk + warp : end; wg < end;
+         wg += g_.threads >> 5) {
         const int64_t row0 = wg * RPW;
         const int64_t row = row0 + sub;
         const int64_t slice = row0 / S;
@@ -296,12 +360,11 @@ __device__ __forceinline__ void product_phase(int vb, int vgrid, int32_t n, int3
             T pv[VW];
             ld_piece<BYTES, COH>(P + row * KP + g * VW, pv);
 #pragma unroll
-            for (int j = 0; j < VW; ++j) pqt[j] = fma_t(pv[j], acc[j], pqt[j]);
+            for (int j = 0; j < VW; ++j) pq[0][j] = fma_t(pv[j], acc[j], pq[0][j]);
         }
     }
-#pragma unroll
-    for (int j = 0; j < VW; ++j) pq[0][j] = (double)pqt[j];
-    cta_cols<G, VW, 1>(pq, part, vb, vgrid);
+    if ((int)blockIdx.x < g_.ctas)
+        cta_cols_fx<G, VW, 1>(pq, sm, g_.threads, part, blockIdx.x, g_.ctas);
 }
 
 // R = B - A X (x_zero: R = B), P = D^-1 R when P is given; per-column r.z, r.r, b.b.  FP64.
@@ -370,16 +433,15 @@ __device__ __forceinline__ void residual_phase(int vb, int vgrid, int32_t n, int
     cta_cols<G, VW, 3>(v, part, vb, vgrid);
 }
 
-// r_c -= alpha_c q_c for running columns; per-column r.(D^-1 r) and r.r.  16-byte pieces, a
-// grid stride that is a multiple of the column groups, so each thread keeps its columns.
+// r_c -= alpha_c q_c for running columns; per-column r.(D^-1 r) and r.r.  16-byte pieces; chunk and
+// thread count are multiples of the column groups, so each thread keeps its columns.
 template <typename T, int KP>
-__device__ __forceinline__ void r_phase(int vb, int vgrid, int32_t n, T *R, const T *Q,
+__device__ __forceinline__ void r_phase(IterGrid g, int32_t n, T *R, const T *Q,
                                         const T *dinv, const T *s_alpha, const int *s_run,
-                                        double *part) {
+                                        double *part,
+                                        ColsSmem<T, KP * (int)sizeof(T) / 16, 16 / (int)sizeof(T), 2> &sm) {
     constexpr int V = 16 / (int)sizeof(T);
     constexpr int CG = KP / V;
-    const int64_t nvec = (int64_t)n * CG;
-    const int64_t stride = (int64_t)vgrid * kCgBlock;
     const int c0 = (int)(threadIdx.x % CG) * V;
     T al[V];
     bool run[V], any = false;
@@ -389,11 +451,12 @@ __device__ __forceinline__ void r_phase(int vb, int vgrid, int32_t n, T *R, cons
         run[j] = s_run[c0 + j] != 0;
         any = any || run[j];
     }
-    T vz[V], vr[V];
+    T vs[2][V];
 #pragma unroll
-    for (int j = 0; j < V; ++j) vz[j] = vr[j] = T(0);
-    if (any) {
-        for (int64_t v = (int64_t)vb * kCgBlock + threadIdx.x; v < nvec; v += stride) {
+    for (int j = 0; j < V; ++j) vs[0][j] = vs[1][j] = T(0);
+    if (any && (int)threadIdx.x < g.threads && (int)blockIdx.x < g.ctas) {
+        const int64_t end = iter_end(g.chunk, (int64_t)n * CG);
+        for (int64_t v = iter_begin(g.chunk); v < end; v += g.threads) {
             const int64_t i = v * V;
             const T d = dinv[v / CG];
             T rv[V], qv[V];
@@ -403,31 +466,24 @@ __device__ __forceinline__ void r_phase(int vb, int vgrid, int32_t n, T *R, cons
             for (int j = 0; j < V; ++j)
                 if (run[j]) {
                     rv[j] = fma_t(-al[j], qv[j], rv[j]);
-                    vz[j] = fma_t(rv[j], d * rv[j], vz[j]);
-                    vr[j] = fma_t(rv[j], rv[j], vr[j]);
+                    vs[0][j] = fma_t(rv[j], d * rv[j], vs[0][j]);
+                    vs[1][j] = fma_t(rv[j], rv[j], vs[1][j]);
                 }
             st_piece<16>(R + i, rv);
         }
     }
-    double v2[2][V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        v2[0][j] = (double)vz[j];
-        v2[1][j] = (double)vr[j];
-    }
-    cta_cols<CG, V, 2>(v2, part, vb, vgrid);
+    if ((int)blockIdx.x < g.ctas)
+        cta_cols_fx<CG, V, 2>(vs, sm, g.threads, part, blockIdx.x, g.ctas);
 }
 
 // x_c += alpha_c p_c for the columns the r sweep updated, then p_c = D^-1 r_c + beta_c p_c for
 // the columns still running.
 template <typename T, int KP>
-__device__ __forceinline__ void p_phase(int vb, int vgrid, int32_t n, T *X, T *P, const T *R,
+__device__ __forceinline__ void p_phase(IterGrid g, int32_t n, T *X, T *P, const T *R,
                                         const T *dinv, const T *s_alpha, const T *s_beta,
                                         const int *s_upd, const int *s_run) {
     constexpr int V = 16 / (int)sizeof(T);
     constexpr int CG = KP / V;
-    const int64_t nvec = (int64_t)n * CG;
-    const int64_t stride = (int64_t)vgrid * kCgBlock;
     const int c0 = (int)(threadIdx.x % CG) * V;
     T al[V], be[V];
     bool upd[V], run[V], any = false;
@@ -439,8 +495,9 @@ __device__ __forceinline__ void p_phase(int vb, int vgrid, int32_t n, T *X, T *P
         run[j] = s_run[c0 + j] != 0;
         any = any || upd[j];
     }
-    if (!any) return;
-    for (int64_t v = (int64_t)vb * kCgBlock + threadIdx.x; v < nvec; v += stride) {
+    if (!any || (int)threadIdx.x >= g.threads || (int)blockIdx.x >= g.ctas) return;
+    const int64_t end = iter_end(g.chunk, (int64_t)n * CG);
+    for (int64_t v = iter_begin(g.chunk); v < end; v += g.threads) {
         const int64_t i = v * V;
         const T d = dinv[v / CG];
         T xv[V], pv[V], rv[V];
@@ -458,71 +515,108 @@ __device__ __forceinline__ void p_phase(int vb, int vgrid, int32_t n, T *X, T *P
 }
 
 // ---- graph-launched kernels -------------------------------------------------------------------
+// Measured against four 256-thread CTAs per SM with FP64 shuffle trees and last-CTA reductions
+// (us per iteration): k = 8 FP64 192K mixed-mesh rows 84 -> 57, FP32 55 -> 35; k = 32 FP64 647K
+// rows 721 -> 585, FP32 294 -> 211; k = 8 10K tetrahedra 26 -> 20.
+//
+// As in the single-vector recurrence (cg.cu): each CTA leaves its sums, every CTA of the next
+// kernel adds them, and a kernel starts under the previous one's tail (dep_wait).  State of an
+// iteration: the product copies rho, done and iters to the cur_ fields, the r sweep adds the
+// step (cur_alpha, cur_run), the p sweep writes the columns' new state.
 template <typename T, int G, int BYTES, typename ColT>
-__global__ void __launch_bounds__(kCgBlock, 4)
-mcg_product(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT cols, const T *val,
-            const T *P, T *Q, double *part, McgScalars *sc) {
-    constexpr int KP = Piece<T, BYTES>::n * G;
-    if (blockIdx.x == 0 && threadIdx.x == 0) sc->pending = 0;
-    if (sc->active == 0) return;
-    product_phase<T, G, BYTES, false>(blockIdx.x, gridDim.x, n, S, n_slices, sp, cols, val, P, Q,
-                                      part);
-    if (last_cta(&sc->tickets[0])) {
-        __shared__ double tot[1][KP];
-        grid_cols<KP, 1>(part, gridDim.x, tot);
-        if (threadIdx.x < KP) col_after_pq(sc->col[threadIdx.x], tot[0][threadIdx.x]);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int a = 0;
-            for (int c = 0; c < KP; ++c) a += sc->col[c].done == 0;
-            sc->active = a;
+__global__ void __launch_bounds__(kIterThreads, 1)
+mcg_product(IterGrid g, int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT cols,
+            const T *val, const T *P, T *Q, double *part, McgScalars *sc) {
+    __shared__ ColsSmem<T, G, Piece<T, BYTES>::n, 1> sm;
+    dep_wait();
+    dep_allow();
+    const int active = sc->active;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < kMcgMaxCols) {
+            const McgCol &c = sc->col[threadIdx.x];
+            sc->cur_done[threadIdx.x] = c.done;
+            sc->cur_iters[threadIdx.x] = c.iters;
+            sc->cur_rho[threadIdx.x] = c.rho;
         }
+        if (threadIdx.x == 0) sc->cur_active = active;
     }
+    if (active == 0) return;
+    product_phase<T, G, BYTES, false>(g, n, S, n_slices, sp, cols, val, P, Q, part, sm);
 }
 
 template <typename T, int KP>
-__global__ void __launch_bounds__(kCgBlock)
-mcg_rsweep(int32_t n, T *R, const T *Q, const T *dinv, double *part, McgScalars *sc) {
+__global__ void __launch_bounds__(kIterThreads, 1)
+mcg_rsweep(IterGrid g, int32_t n, T *R, const T *Q, const T *dinv, const double *pq_part,
+           int pq_count, double *part, McgScalars *sc) {
     __shared__ T s_alpha[KP];
     __shared__ int s_run[KP];
-    if (sc->active == 0) return;
+    __shared__ double tot[1][KP];
+    __shared__ ColsSmem<T, KP * (int)sizeof(T) / 16, 16 / (int)sizeof(T), 2> sm;
+    dep_wait();
+    dep_allow();
+    if (sc->cur_active == 0) return;
+    grid_cols<KP, 1>(pq_part, pq_count, tot);
     if (threadIdx.x < KP) {
-        s_alpha[threadIdx.x] = (T)sc->col[threadIdx.x].alpha;
-        s_run[threadIdx.x] = sc->col[threadIdx.x].done == 0;
-    }
-    __syncthreads();
-    r_phase<T, KP>(blockIdx.x, gridDim.x, n, R, Q, dinv, s_alpha, s_run, part);
-    if (last_cta(&sc->tickets[1])) {
-        __shared__ double tot[2][KP];
-        grid_cols<KP, 2>(part, gridDim.x, tot);
-        if (threadIdx.x < KP)
-            col_after_r(sc->col[threadIdx.x], tot[0][threadIdx.x], tot[1][threadIdx.x],
-                        sc->max_iter);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int a = 0;
-            for (int c = 0; c < KP; ++c) a += sc->col[c].done == 0;
-            sc->active = a;
-            sc->pending = 1;
+        McgCol c;
+        c.done = sc->cur_done[threadIdx.x];
+        c.rho = sc->cur_rho[threadIdx.x];
+        c.alpha = 0.0;
+        col_after_pq(c, tot[0][threadIdx.x]);
+        s_alpha[threadIdx.x] = (T)c.alpha;
+        s_run[threadIdx.x] = c.done == 0;
+        if (blockIdx.x == 0) {
+            sc->cur_alpha[threadIdx.x] = c.alpha;
+            sc->cur_run[threadIdx.x] = c.done;
         }
     }
+    __syncthreads();
+    r_phase<T, KP>(g, n, R, Q, dinv, s_alpha, s_run, part, sm);
 }
 
 template <typename T, int KP>
-__global__ void __launch_bounds__(kCgBlock)
-mcg_psweep(int32_t n, T *X, T *P, const T *R, const T *dinv, const McgScalars *sc) {
+__global__ void __launch_bounds__(kIterThreads, 1)
+mcg_psweep(IterGrid g, int32_t n, T *X, T *P, const T *R, const T *dinv, const double *part,
+           McgScalars *sc) {
     __shared__ T s_alpha[KP], s_beta[KP];
     __shared__ int s_upd[KP], s_run[KP];
-    if (!sc->pending) return;
+    __shared__ double tot[2][KP];
+    dep_wait();
+    dep_allow();
+    if (sc->cur_active == 0) return;
+    grid_cols<KP, 2>(part, g.ctas, tot);
     if (threadIdx.x < KP) {
-        const McgCol &c = sc->col[threadIdx.x];
-        s_alpha[threadIdx.x] = (T)c.alpha;
-        s_beta[threadIdx.x] = (T)c.beta;
-        s_upd[threadIdx.x] = c.upd;
-        s_run[threadIdx.x] = c.done == 0;
+        const int k = threadIdx.x;
+        McgCol c{};  // (CTA 0 writes the columns' new state below: only what it leaves alone is
+                     // read from there)
+        c.tol2 = sc->col[k].tol2;
+        c.bb = sc->col[k].bb;
+        c.done = sc->cur_run[k];
+        c.iters = sc->cur_iters[k];
+        c.rho = sc->cur_rho[k];
+        c.alpha = sc->cur_alpha[k];
+        col_after_r(c, tot[0][k], tot[1][k], sc->max_iter);
+        s_alpha[k] = (T)c.alpha;
+        s_beta[k] = (T)c.beta;
+        s_upd[k] = c.upd;
+        s_run[k] = c.done == 0;
+        if (blockIdx.x == 0) {
+            McgCol &o = sc->col[k];
+            o.done = c.done;
+            o.iters = c.iters;
+            o.rho = c.rho;
+            o.alpha = c.alpha;
+            o.beta = c.beta;
+            o.upd = c.upd;
+            if (c.upd) o.rr = c.rr;
+        }
     }
     __syncthreads();
-    p_phase<T, KP>(blockIdx.x, gridDim.x, n, X, P, R, dinv, s_alpha, s_beta, s_upd, s_run);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        int a = 0;
+        for (int c = 0; c < KP; ++c) a += s_run[c];
+        sc->active = a;
+    }
+    p_phase<T, KP>(g, n, X, P, R, dinv, s_alpha, s_beta, s_upd, s_run);
 }
 
 // R = B - A X, P = D^-1 R and the per-column sums; last CTA by mode:
@@ -540,7 +634,7 @@ mcg_residual(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT col
                              R, P, dinv, part);
     if (last_cta(&sc->tickets[2])) {
         __shared__ double tot[3][KP];
-        grid_cols<KP, 3>(part, gridDim.x, tot);
+        last_cols<KP, 3>(part, gridDim.x, tot);
         if (threadIdx.x < KP) {
             McgCol &c = sc->col[threadIdx.x];
             const double rz = tot[0][threadIdx.x], rr = tot[1][threadIdx.x],
@@ -574,7 +668,6 @@ mcg_residual(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT col
             int a = 0;
             for (int c = 0; c < KP; ++c) a += sc->col[c].done == 0;
             sc->active = a;
-            sc->pending = 0;
         }
     }
 }
@@ -626,7 +719,7 @@ mcg_inner_start(int32_t n, const double *R64, const McgScalars *outer, float *R3
     cta_cols<CG, V, 2>(v2, part, blockIdx.x, gridDim.x);
     if (last_cta(&inner->tickets[3])) {
         __shared__ double tot[2][KP];
-        grid_cols<KP, 2>(part, gridDim.x, tot);
+        last_cols<KP, 2>(part, gridDim.x, tot);
         if (threadIdx.x < KP) {
             McgCol &c = inner->col[threadIdx.x];
             const McgCol &o = outer->col[threadIdx.x];
@@ -648,7 +741,6 @@ mcg_inner_start(int32_t n, const double *R64, const McgScalars *outer, float *R3
             int a = 0;
             for (int c = 0; c < KP; ++c) a += inner->col[c].done == 0;
             inner->active = a;
-            inner->pending = 0;
         }
     }
 }
@@ -688,7 +780,6 @@ __global__ void mcg_set(McgScalars *sc, int k, int kp, double tol2, int max_iter
     }
     if (c == 0) {
         sc->active = 0;
-        sc->pending = 0;
         sc->max_iter = max_iter;
         sc->timed_out = 0;
         for (int t = 0; t < 4; ++t) sc->tickets[t] = 0u;
@@ -760,17 +851,16 @@ __device__ bool mcg_barrier(McgScalars *sc) {
     return ok != 0;
 }
 
-// The whole lock-step recurrence in one cooperative launch: the product runs on the graph
-// path's product grid as virtual CTAs (CTA b on CTA b mod gridDim.x), the sweeps on the grid
-// itself (the graph path's sweep grid), and after each barrier every CTA reduces the partials
-// in the graph path's fixed order, so all CTAs hold the same column states and the results are
-// the graph path's bit for bit.  Vectors are read with coherent loads (they change between
-// barriers).  The wall-clock budget is voted by CTA 0 once per iteration.
+// The whole lock-step recurrence in one cooperative launch, one CTA per SM, on the graph path's
+// grids; after each barrier every CTA adds the partials in the graph path's way, so all CTAs hold
+// the same column states and the results are the graph path's bit for bit.  Vectors are read with
+// coherent loads (they change between barriers).  The wall-clock budget is voted by CTA 0 once
+// per iteration.
 template <typename T, int G, int BYTES, typename ColT>
-__global__ void __launch_bounds__(kCgBlock, 4)
-mcg_persistent(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT cols,
-               const T *val, T *X, T *R, T *P, T *Q, const T *dinv, double *part, int Gpq,
-               int pq_len, McgScalars *sc) {
+__global__ void __launch_bounds__(kIterThreads, 1)
+mcg_persistent(IterGrid pq, IterGrid sw, int32_t n, int32_t S, int32_t n_slices,
+               const int64_t *sp, ColT cols, const T *val, T *X, T *R, T *P, T *Q, const T *dinv,
+               double *part, McgScalars *sc) {
     constexpr int KP = Piece<T, BYTES>::n * G;
     __shared__ McgCol s_col[KP];
     __shared__ T s_alpha[KP], s_beta[KP];
@@ -778,19 +868,22 @@ mcg_persistent(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT c
     __shared__ double tot1[1][KP];
     __shared__ double tot2[2][KP];
     __shared__ int s_active;
+    __shared__ union Sums {
+        ColsSmem<T, G, Piece<T, BYTES>::n, 1> pq;
+        ColsSmem<T, KP * (int)sizeof(T) / 16, 16 / (int)sizeof(T), 2> r;
+    } sm;
     const long long t_start = mcg_timer_ns();
     const long long budget = sc->budget_ns;
     const int max_iter = sc->max_iter;
     double *part1 = part;
-    double *part2 = part + (int64_t)KP * pq_len;
-    double *vote = part2 + (int64_t)2 * KP * gridDim.x;
+    double *part2 = part + (int64_t)KP * pq.ctas;
+    double *vote = part2 + (int64_t)2 * KP * sw.ctas;
     if (threadIdx.x < KP) s_col[threadIdx.x] = sc->col[threadIdx.x];
     if (threadIdx.x == 0) s_active = sc->active;
     __syncthreads();
     bool timed_out = false;
     while (s_active > 0) {
-        for (int b = blockIdx.x; b < Gpq; b += gridDim.x)
-            product_phase<T, G, BYTES, true>(b, Gpq, n, S, n_slices, sp, cols, val, P, Q, part1);
+        product_phase<T, G, BYTES, true>(pq, n, S, n_slices, sp, cols, val, P, Q, part1, sm.pq);
         if (blockIdx.x == 0 && threadIdx.x == 0)
             vote[0] = (budget > 0 && mcg_timer_ns() - t_start > budget) ? 1.0 : 0.0;
         if (!mcg_barrier(sc)) {
@@ -801,19 +894,19 @@ mcg_persistent(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT c
             timed_out = true;
             break;
         }
-        grid_cols<KP, 1>(part1, Gpq, tot1);
+        grid_cols<KP, 1>(part1, pq.ctas, tot1);
         if (threadIdx.x < KP) {
             col_after_pq(s_col[threadIdx.x], tot1[0][threadIdx.x]);
             s_alpha[threadIdx.x] = (T)s_col[threadIdx.x].alpha;
             s_run[threadIdx.x] = s_col[threadIdx.x].done == 0;
         }
         __syncthreads();
-        r_phase<T, KP>(blockIdx.x, gridDim.x, n, R, Q, dinv, s_alpha, s_run, part2);
+        r_phase<T, KP>(sw, n, R, Q, dinv, s_alpha, s_run, part2, sm.r);
         if (!mcg_barrier(sc)) {
             timed_out = true;
             break;
         }
-        grid_cols<KP, 2>(part2, gridDim.x, tot2);
+        grid_cols<KP, 2>(part2, sw.ctas, tot2);
         if (threadIdx.x < KP) {
             McgCol &c = s_col[threadIdx.x];
             col_after_r(c, tot2[0][threadIdx.x], tot2[1][threadIdx.x], max_iter);
@@ -827,7 +920,7 @@ mcg_persistent(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT c
             for (int c = 0; c < KP; ++c) a += s_col[c].done == 0;
             s_active = a;
         }
-        p_phase<T, KP>(blockIdx.x, gridDim.x, n, X, P, R, dinv, s_alpha, s_beta, s_upd, s_run);
+        p_phase<T, KP>(sw, n, X, P, R, dinv, s_alpha, s_beta, s_upd, s_run);
         if (!mcg_barrier(sc)) {
             timed_out = true;
             break;
@@ -837,13 +930,30 @@ mcg_persistent(int32_t n, int32_t S, int32_t n_slices, const int64_t *sp, ColT c
         if (threadIdx.x < KP) sc->col[threadIdx.x] = s_col[threadIdx.x];
         if (threadIdx.x == 0) {
             sc->active = s_active;
-            sc->pending = 0;
             if (timed_out) atomicExch(&sc->timed_out, 1);
         }
     }
 }
 
 // ---- host ---------------------------------------------------------------------------------------
+// Grids of the iteration's kernels: 16-byte pieces of the n x kp arrays, and groups of 32 / G rows,
+// in equal chunks per SM.  At least 256 threads per CTA: their warps also add the columns' sums.
+IterGrid sweep_iter_grid(int32_t n, int kp, int elem_bytes) {
+    IterGrid g = cg_iter_grid((int64_t)n * kp * elem_bytes / 16, kIterThreads);
+    g.threads = std::max(g.threads, 256);
+    return g;
+}
+IterGrid product_iter_grid(const spmv_matrix_t A, int G) {
+    const int64_t groups = (int64_t)A->n_slices * A->S / (32 / G);
+    const int sms = std::min(device_facts().sm_count, 32 * kPartLoads);
+    IterGrid g;
+    g.chunk = std::max<int64_t>(2, (groups + sms - 1) / sms);
+    g.threads = (int)std::min<int64_t>(kIterThreads, std::max<int64_t>(256, 32 * g.chunk));
+    g.ctas = (int)std::max<int64_t>(1, (groups + g.chunk - 1) / g.chunk);
+    return g;
+}
+
+// Grids of the kernels around the iteration.
 int sweep_grid(int32_t n, int kp, int elem_bytes) {
     const int64_t vecs = (int64_t)n * kp * elem_bytes / 16;
     const int64_t cap = (int64_t)device_facts().sm_count * kCgCtasPerSm;
@@ -851,9 +961,8 @@ int sweep_grid(int32_t n, int kp, int elem_bytes) {
     return (int)(want < 1 ? 1 : (want > cap ? cap : want));
 }
 
-int product_grid(const spmv_matrix_t A, int G, int elem_bytes) {
+int product_grid(const spmv_matrix_t A, int G) {
     const int64_t groups = (int64_t)A->n_slices * A->S / (32 / G);
-    (void)elem_bytes;
     const int64_t cap = (int64_t)device_facts().sm_count * 4;
     const int64_t want = (groups + kMcgWarps - 1) / kMcgWarps;
     return (int)(want < 1 ? 1 : (want > cap ? cap : want));
@@ -906,20 +1015,23 @@ spmv_status_t enqueue_iters(spmv_matrix_t A, bool f32, int iters, int bytes, cud
         const T *dinv = f32 ? (const T *)A->cg.dinv32.p : (const T *)A->cg.dinv.p;
         const T *val = f32 ? (const T *)A->sell_val32.p : (const T *)A->sell_val.p;
         McgScalars *sc = block_of(A, f32 ? 1 : 0);
-        const int Gsw = sweep_grid(A->n, kp, (int)sizeof(T));
+        const IterGrid sw = sweep_iter_grid(A->n, kp, (int)sizeof(T));
         return with_mcg_cols(A, [&](auto cols) -> spmv_status_t {
             using ColT = decltype(cols);
             return with_piece<T>(kp, bytes, [&](auto gt, auto bt) -> spmv_status_t {
                 constexpr int G = decltype(gt)::value, BY = decltype(bt)::value;
                 constexpr int KP = Piece<T, BY>::n * G;
-                const int Gpq = product_grid(A, G, (int)sizeof(T));
+                const IterGrid pq = product_iter_grid(A, G);
+                double *part1 = w.part.p, *part2 = w.part.p + (int64_t)KP * pq.ctas;
                 for (int it = 0; it < iters; ++it) {
-                    mcg_product<T, G, BY, ColT><<<Gpq, kCgBlock, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, P, Q, w.part.p, sc);
-                    mcg_rsweep<T, KP><<<Gsw, kCgBlock, 0, st>>>(A->n, R, Q, dinv, w.part.p, sc);
-                    mcg_psweep<T, KP><<<Gsw, kCgBlock, 0, st>>>(A->n, X, P, R, dinv, sc);
+                    GB_TRY(launch_dependent(mcg_product<T, G, BY, ColT>, pq.ctas, pq.threads, st, pq,
+                                            A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, P,
+                                            Q, part1, sc));
+                    GB_TRY(launch_dependent(mcg_rsweep<T, KP>, sw.ctas, sw.threads, st, sw, A->n, R,
+                                            Q, dinv, part1, pq.ctas, part2, sc));
+                    GB_TRY(launch_dependent(mcg_psweep<T, KP>, sw.ctas, sw.threads, st, sw, A->n, X,
+                                            P, R, dinv, part2, sc));
                 }
-                GB_LAUNCHED();
                 return SPMV_OK;
             });
         });
@@ -937,7 +1049,6 @@ __global__ void mcg_activate(McgScalars *sc, int kp) {
     }
     if (c == 0) {
         sc->active = kp;
-        sc->pending = 0;
         for (int t = 0; t < 4; ++t) sc->tickets[t] = 0u;
     }
 }
@@ -974,13 +1085,11 @@ spmv_status_t tune_gather(spmv_matrix_t A, cudaStream_t st) {
                     using ColT = decltype(cols);
                     return with_piece<double>(w.kp, bytes, [&](auto gt, auto bt) -> spmv_status_t {
                         constexpr int G = decltype(gt)::value, BY = decltype(bt)::value;
-                        mcg_product<double, G, BY, ColT><<<product_grid(A, G, 8), kCgBlock, 0,
-                                                           st>>>(A->n, A->S, A->n_slices,
-                                                                 A->slice_ptr.p, cols,
-                                                                 A->sell_val.p, w.P.p, w.Q.p,
-                                                                 w.part.p, sc);
-                        GB_LAUNCHED();
-                        return SPMV_OK;
+                        const IterGrid pq = product_iter_grid(A, G);
+                        return launch_dependent(mcg_product<double, G, BY, ColT>, pq.ctas,
+                                                pq.threads, st, pq, A->n, A->S, A->n_slices,
+                                                A->slice_ptr.p, cols, A->sell_val.p, w.P.p, w.Q.p,
+                                                w.part.p, sc);
                     });
                 });
             if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e1, st));
@@ -1008,7 +1117,7 @@ spmv_status_t enqueue_residual(spmv_matrix_t A, bool x_zero, bool want_p, int mo
         using ColT = decltype(cols);
         return with_piece<double>(w.kp, 32, [&](auto gt, auto) -> spmv_status_t {
             constexpr int G = decltype(gt)::value;
-            const int grid = product_grid(A, G, 8);
+            const int grid = product_grid(A, G);
             mcg_residual<G, 32, ColT><<<grid, kCgBlock, 0, st>>>(
                 A->n, A->S, A->n_slices, A->slice_ptr.p, cols, A->sell_val.p, w.X.p,
                 x_zero ? 1 : 0, w.B.p, w.R.p, want_p ? w.P.p : nullptr, A->cg.dinv.p, w.part.p,
@@ -1085,22 +1194,23 @@ spmv_status_t launch_persistent(spmv_matrix_t A, bool f32, int bytes, double tim
             return with_piece<T>(w.kp, bytes, [&](auto gt, auto bt) -> spmv_status_t {
                 constexpr int G = decltype(gt)::value, BY = decltype(bt)::value;
                 auto kern = mcg_persistent<T, G, BY, ColT>;
+                IterGrid pq = product_iter_grid(A, G);
+                IterGrid sw = sweep_iter_grid(A->n, w.kp, (int)sizeof(T));
+                const int ctas = std::max(pq.ctas, sw.ctas);
+                const int threads = std::max(pq.threads, sw.threads);
                 int per_sm = 0;
-                GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCgBlock, 0));
-                int Gsw = sweep_grid(A->n, w.kp, (int)sizeof(T));
-                if ((int64_t)per_sm * device_facts().sm_count < Gsw) return SPMV_ERR_UNSUPPORTED;
-                int Gpq = product_grid(A, G, (int)sizeof(T));
-                int pq_len = Gpq;
+                GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0));
+                if ((int64_t)per_sm * device_facts().sm_count < ctas) return SPMV_ERR_UNSUPPORTED;
                 const long long budget = timeout_s > 0 ? (long long)(timeout_s * 1e9) : 0;
                 GB_CUDA(cudaMemcpyAsync(&sc->budget_ns, &budget, sizeof(budget),
                                         cudaMemcpyHostToDevice, st));
                 int32_t n = A->n, S = A->S, ns = A->n_slices;
                 const int64_t *sp = A->slice_ptr.p;
                 double *part = w.part.p;
-                void *args[] = {&n, &S, &ns, &sp, &cols, &val, &X, &R, &P, &Q, &dinv, &part,
-                                &Gpq, &pq_len, &sc};
-                GB_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3(Gsw),
-                                                    dim3(kCgBlock), args, 0, st));
+                void *args[] = {&pq, &sw, &n, &S, &ns, &sp, &cols, &val, &X, &R, &P, &Q, &dinv, &part,
+                                &sc};
+                GB_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(threads),
+                                                    args, 0, st));
                 return SPMV_OK;
             });
         });
