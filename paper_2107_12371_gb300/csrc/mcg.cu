@@ -324,35 +324,73 @@ __device__ __forceinline__ void product_phase(IterGrid g_, int32_t n, int32_t S,
         T acc[VW];
 #pragma unroll
         for (int j = 0; j < VW; ++j) acc[j] = T(0);
-        int t = 0;
-        for (; t + 2 <= w; t += 2) {
-            T a[2][1];
-            int32_t c[2][1];
-            ld_stream(vp + (int64_t)t * S, pol, a[0]);
-            cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c[0]);
-            ld_stream(vp + (int64_t)(t + 1) * S, pol, a[1]);
-            cols.template load<1>(cat + (int64_t)(t + 1) * S, slice, pol, cbase, c[1]);
-            T xv[2][VW];
+        // One FP32 lane per row (k <= 8) has few loads in flight per warp: the next two entries'
+        // values and columns travel with the current two's gathers (647K mixed-mesh rows 87 -> 65
+        // us per iteration).  With more lanes per row or FP64 it is slower (57 -> 62 us), and with
+        // coherent gathers, whose order the compiler keeps (33 -> 36 us).
+        if constexpr (sizeof(T) == 4 && G == 1 && !COH) {
+            T a[2][1], an[2][1];
+            int32_t c[2][1], cn[2][1];
+            auto load_pair = [&](int t, T (&av)[2][1], int32_t (&cv)[2][1]) {
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (c[u][0] >= 0) ld_piece<BYTES, COH>(pg + (int64_t)c[u][0] * KP, xv[u]);
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (c[u][0] >= 0) {
-#pragma unroll
-                    for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[u][0], xv[u][j], acc[j]);
+                for (int u = 0; u < 2; ++u) {
+                    av[u][0] = T(0);
+                    cv[u][0] = -1;
+                    if (t + u < w) {
+                        ld_stream(vp + (int64_t)(t + u) * S, pol, av[u]);
+                        cols.template load<1>(cat + (int64_t)(t + u) * S, slice, pol, cbase, cv[u]);
+                    }
                 }
-        }
-        if (t < w) {
-            T a[1];
-            int32_t c[1];
-            ld_stream(vp + (int64_t)t * S, pol, a);
-            cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c);
-            if (c[0] >= 0) {
-                T xv[VW];
-                ld_piece<BYTES, COH>(pg + (int64_t)c[0] * KP, xv);
+            };
+            load_pair(0, a, c);
+#pragma unroll 1
+            for (int t = 0; t < w; t += 2) {
+                T xv[2][VW];
 #pragma unroll
-                for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[0], xv[j], acc[j]);
+                for (int u = 0; u < 2; ++u)
+                    if (c[u][0] >= 0) ld_piece<BYTES, COH>(pg + (int64_t)c[u][0] * KP, xv[u]);
+                load_pair(t + 2, an, cn);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (c[u][0] >= 0) {
+#pragma unroll
+                        for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[u][0], xv[u][j], acc[j]);
+                    }
+                    a[u][0] = an[u][0];
+                    c[u][0] = cn[u][0];
+                }
+            }
+        } else {
+            int t = 0;
+            for (; t + 2 <= w; t += 2) {
+                T a[2][1];
+                int32_t c[2][1];
+                ld_stream(vp + (int64_t)t * S, pol, a[0]);
+                cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c[0]);
+                ld_stream(vp + (int64_t)(t + 1) * S, pol, a[1]);
+                cols.template load<1>(cat + (int64_t)(t + 1) * S, slice, pol, cbase, c[1]);
+                T xv[2][VW];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (c[u][0] >= 0) ld_piece<BYTES, COH>(pg + (int64_t)c[u][0] * KP, xv[u]);
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (c[u][0] >= 0) {
+#pragma unroll
+                        for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[u][0], xv[u][j], acc[j]);
+                    }
+            }
+            if (t < w) {
+                T a[1];
+                int32_t c[1];
+                ld_stream(vp + (int64_t)t * S, pol, a);
+                cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c);
+                if (c[0] >= 0) {
+                    T xv[VW];
+                    ld_piece<BYTES, COH>(pg + (int64_t)c[0] * KP, xv);
+#pragma unroll
+                    for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[0], xv[j], acc[j]);
+                }
             }
         }
         if (row < n) {
