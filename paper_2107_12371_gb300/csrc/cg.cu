@@ -107,9 +107,9 @@ cg_residual(int32_t n, int32_t n_slices, const int64_t *sp, ColT col, const T *v
 // requested before the previous kernel (which finishes p) has ended.
 template <typename T, int R, int L, typename ColT, int UU>
 __global__ void __launch_bounds__(kCgBlock * pq_min_ctas((int)sizeof(T) * R))
-cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, const int64_t *sp, ColT col, const T *val,
-           const T *p, T *q, double *part, CgScalars *sc) {
-    const uint64_t pol = policy_evict_first();
+cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, bool keep, const int64_t *sp, ColT col,
+           const T *val, const T *p, T *q, double *part, CgScalars *sc) {
+    const uint64_t pol = policy_stream(keep);
     const int64_t g0 = iter_begin(chunk), end = iter_end(chunk, (int64_t)n_slices * L);
     // lanes of 64 bytes per entry have no registers for a round held across the wait
     constexpr bool kEarly = sizeof(T) * R <= 32;
@@ -157,8 +157,8 @@ cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, const int64_t *sp, ColT c
 // those of the partials (one round trip); otherwise the sweep's own loads overlap each other.
 template <typename T, bool ONE>
 __global__ void __launch_bounds__(kIterThreads)
-cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const T *dinv,
-             const double *pq_part, int pq_count, double *part, CgScalars *sc) {
+cg_update_xr(int32_t n, int64_t chunk, bool keep, T *x, T *r, const T *p, const T *q,
+             const T *dinv, const double *pq_part, int pq_count, double *part, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
     const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
     const bool mine = k0 < end && k0 < n / V;
@@ -169,7 +169,7 @@ cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const
     }
     dep_wait();
     dep_allow();
-    const uint64_t pol = policy_evict_first();
+    const uint64_t pol = policy_stream(keep);
     if (mine) {
         if (ONE) {
             v.load(x, r, p, q, k0 * V, pol);
@@ -194,7 +194,7 @@ cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const
     const T alpha = step.coef;
     T vz = T(0), vr = T(0);
     if (ONE && mine) v.update(alpha, x, r, k0 * V, pol, vz, vr);
-    else sweep_update_xr<T>(n, k0, end, blockDim.x, alpha, x, r, p, q, dinv, vz, vr);
+    else sweep_update_xr<T>(n, k0, end, blockDim.x, pol, alpha, x, r, p, q, dinv, vz, vr);
     const T t[2] = {vz, vr};
     store_parts<2>(t, part);
 }
@@ -203,12 +203,12 @@ cg_update_xr(int32_t n, int64_t chunk, T *x, T *r, const T *p, const T *q, const
 // in cg_update_xr.
 template <typename T, bool ONE>
 __global__ void __launch_bounds__(kIterThreads)
-cg_update_p(int32_t n, int64_t chunk, const T *r, const T *dinv, T *p, const double *part,
-            int count, CgScalars *sc) {
+cg_update_p(int32_t n, int64_t chunk, bool keep, const T *r, const T *dinv, T *p,
+            const double *part, int count, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
     const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
     const bool mine = k0 < end && k0 < n / V;
-    const uint64_t pol = policy_evict_first();
+    const uint64_t pol = policy_stream(keep);
     PVec<T> v;
     if (mine) {
         if (ONE) v.load_d(dinv, k0 * V, pol);
@@ -256,7 +256,7 @@ cg_update_p(int32_t n, int64_t chunk, const T *r, const T *dinv, T *p, const dou
     if (step.done) return;
     const T beta = step.coef;
     if (ONE && mine) v.update(beta, p, k0 * V);
-    else sweep_update_p<T>(n, k0, end, blockDim.x, beta, r, dinv, p);
+    else sweep_update_p<T>(n, k0, end, blockDim.x, pol, beta, r, dinv, p);
 }
 
 // refinement: right-hand side of the inner solve r32 = fp32(r64 / ||r64||), start of the
@@ -317,6 +317,13 @@ IterGrid cg_iter_grid(int64_t items, int max_threads) {
     g.threads = (int)std::min<int64_t>(max_threads, g.chunk);
     g.ctas = (int)std::max<int64_t>(1, (items + g.chunk - 1) / g.chunk);
     return g;
+}
+
+IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes) {
+    const double l2 = device_facts().l2_bytes;
+    const double vectors = 5.0 * elem_bytes * A->n;
+    const double matrix = (double)A->sell_entries * (elem_bytes + A->index_bits / 8);
+    return {matrix + vectors <= 0.75 * l2, vectors <= 0.5 * l2};
 }
 
 // Grid of the CG product q = A p: at most 256 threads per unit of the handle's pq_ctas (tuned, or
@@ -416,7 +423,7 @@ static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q,
             return launch_dependent(cg_pq_deep(A, UU) ? cg_spmv_pq<T, R, L, ColT, UU>
                                                       : cg_spmv_pq<T, R, L, ColT, 2>,
                                     g.ctas, g.threads, st, A->n, A->n_slices, g.chunk,
-                                    A->slice_ptr.p, cols, val, p, q, A->cg.part.p, sc);
+                                    cg_keep(A, sizeof(T)).matrix, A->slice_ptr.p, cols, val, p, q, A->cg.part.p, sc);
         });
     });
 }
@@ -426,8 +433,8 @@ static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const
     constexpr int V = Vec16<T>::n;
     const IterGrid g = cg_sweep_grid(A, V);
     return launch_dependent(g.single() ? cg_update_xr<T, true> : cg_update_xr<T, false>, g.ctas,
-                            g.threads, st, A->n, g.chunk, x, r, p, q, dinv, A->cg.part.p,
-                            pq_count, A->cg.part.p + A->cg.pq_len, sc);
+                            g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, x, r, p, q,
+                            dinv, A->cg.part.p, pq_count, A->cg.part.p + A->cg.pq_len, sc);
 }
 template <typename T>
 static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p, CgScalars *sc,
@@ -435,7 +442,7 @@ static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p,
     constexpr int V = Vec16<T>::n;
     const IterGrid g = cg_sweep_grid(A, V);
     return launch_dependent(g.single() ? cg_update_p<T, true> : cg_update_p<T, false>, g.ctas,
-                            g.threads, st, A->n, g.chunk, r, dinv, p,
+                            g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, r, dinv, p,
                             A->cg.part.p + A->cg.pq_len, g.ctas, sc);
 }
 template <typename T>

@@ -52,6 +52,16 @@ __device__ __forceinline__ int64_t iter_end(int64_t chunk, int64_t items) {
     const int64_t e = ((int64_t)blockIdx.x + 1) * chunk;
     return e < items ? e : items;
 }
+// What an iteration leaves in L2 for the next one.  The matrix is streamed evict-first unless it
+// and the vectors fit (three quarters of) the L2 together; the vectors that a FP32 sweep is the
+// last to touch are, unless the five vectors take no more than half of it.  Per FP32 iteration,
+// evict-first / kept: matrix 1.5M rows 23.1 / 21.3 us (75 MB in all; 2.1M rows, 103 MB: 27.8 /
+// 30.8), vectors 2.1M rows 29.1 / 27.8, 3.1M (61 MB) 35.6 / 34.5 (4.4M: 50.2 / 51.5).
+struct IterKeep {
+    bool matrix, vectors;
+};
+IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes);
+
 IterGrid cg_iter_grid(int64_t items, int max_threads);
 IterGrid cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes);
 IterGrid cg_sweep_grid(const spmv_matrix_t A, int vec);
@@ -567,15 +577,14 @@ struct XrVec {
 
 // x += alpha p; r -= alpha q over the vectors k = from, from + stride, ... below end (n may cut the
 // last one short); accumulates r.(D^-1 r) into vz and r.r into vr.  x and q are not needed again
-// in this iteration (evict-first in FP32); r, p and D^-1 are read by the p update.
+// in this iteration (pol, in FP32); r, p and D^-1 are read by the p update.
 template <typename T, int UNROLL = 4>
 __device__ __forceinline__ void sweep_update_xr(int32_t n, int64_t from, int64_t end,
-                                                int64_t stride, T alpha, T *x, T *r,
-                                                const T *p, const T *q, const T *dinv, T &vz,
-                                                T &vr) {
+                                                int64_t stride, uint64_t pol, T alpha, T *x,
+                                                T *r, const T *p, const T *q, const T *dinv,
+                                                T &vz, T &vr) {
     constexpr int V = Vec16<T>::n;
     const int64_t nv = n / V, full = nv < end ? nv : end;
-    const uint64_t pol = policy_evict_first();
     int64_t k = from;
 #pragma unroll UNROLL
     for (; k < full; k += stride) {
@@ -616,15 +625,14 @@ struct PVec {
 };
 
 // p = D^-1 r + beta p over the vectors k = from, from + stride, ... below end.  r and D^-1 are next read by
-// the next iteration's x/r update (evict-first in FP32); the new p stays in L2 for the
-// product's gathers.
+// the next iteration's x/r update (pol, in FP32); the new p stays in L2 for the product's
+// gathers.
 template <typename T, int UNROLL = 4>
 __device__ __forceinline__ void sweep_update_p(int32_t n, int64_t from, int64_t end,
-                                               int64_t stride, T beta, const T *r, const T *dinv,
-                                               T *p) {
+                                               int64_t stride, uint64_t pol, T beta, const T *r,
+                                               const T *dinv, T *p) {
     constexpr int V = Vec16<T>::n;
     const int64_t nv = n / V, full = nv < end ? nv : end;
-    const uint64_t pol = policy_evict_first();
     int64_t k = from;
 #pragma unroll UNROLL
     for (; k < full; k += stride) {

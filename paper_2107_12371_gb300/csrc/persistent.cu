@@ -157,6 +157,7 @@ struct PersArgs {
     T *zp;  // resident form with PAIRS: (D^-1 r, p) of every row
     IterGrid pq, sw;
     bool same;  // pq == sw
+    IterKeep keep;
     ulonglong2 *slots;
     CgScalars *sc;
 };
@@ -185,7 +186,7 @@ cg_persistent(PersArgs<T> a, ColT col) {
     const int t = threadIdx.x;
     const int32_t n = a.n;
     CgScalars *sc = a.sc;
-    const uint64_t pol = policy_evict_first();
+    const uint64_t pol = policy_stream(a.keep.matrix), pol_v = policy_stream(a.keep.vectors);
     const long long t_start = global_timer_ns();
     const long long budget = sc->budget_ns;
     double rho = sc->rho;  // thread 0's is the current one
@@ -338,7 +339,7 @@ cg_persistent(PersArgs<T> a, ColT col) {
                 }
             }
         } else {
-            sweep_update_xr<T, 1>(n, k0, k1, a.sw.threads, alpha, a.x, a.r, a.p, a.q, a.dinv, vz, vr);
+            sweep_update_xr<T, 1>(n, k0, k1, a.sw.threads, pol_v, alpha, a.x, a.r, a.p, a.q, a.dinv, vz, vr);
         }
         const T v2[2] = {vz, vr};
         ++iters;
@@ -368,7 +369,7 @@ cg_persistent(PersArgs<T> a, ColT col) {
             for (int i = 0; i < R; ++i) p[i] = fma_t(beta, p[i], z[i]);
             if (g0 < g1) store_rows<T, R>(a.p, row0, n, p);
         } else {
-            sweep_update_p<T, 1>(n, k0, k1, a.sw.threads, beta, a.r, a.dinv, a.p);
+            sweep_update_p<T, 1>(n, k0, k1, a.sw.threads, pol_v, beta, a.r, a.dinv, a.p);
         }
         if (!grid_barrier(a.slots + kSlotsP, (int)gridDim.x, it, &sm.late)) {
             done = 4;
@@ -442,6 +443,7 @@ static spmv_status_t run_persistent(spmv_matrix_t A, PersArgs<T> a, const cg_opt
     a.sp = A->slice_ptr.p;
     a.sc = (CgScalars *)w.scal.p + (f32 ? 1 : 0);
     a.sw = cg_sweep_grid(A, Vec16<T>::n);
+    a.keep = cg_keep(A, (int)sizeof(T));
     if (!w.slots.p) GB_TRY(w.slots.alloc(kSlotsTotal, &A->bytes));
     a.slots = w.slots.p;
     GB_CUDA(cudaMemsetAsync(w.slots.p, 0, sizeof(ulonglong2) * kSlotsTotal, st));

@@ -17,10 +17,12 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
     return p;
 }
 
-__device__ __forceinline__ uint64_t policy_evict_last() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
+// evict-first, or the ordinary priority for data that stays in L2 until its next use
+__device__ __forceinline__ uint64_t policy_stream(bool keep) {
+    uint64_t first, normal;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
+    return keep ? normal : first;
 }
 
 // ---- streamed matrix loads -------------------------------------------------------------
