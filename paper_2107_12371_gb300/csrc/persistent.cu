@@ -93,19 +93,20 @@ struct PersSmem {
 // Sums over CTAs [0, ctas) of their first TT threads' v[k]: use(k, sum) runs in one thread of
 // each CTA per quantity, and the other threads see what it wrote after the call.  Every CTA of
 // the grid waits.  PUBLISH: the CTAs' earlier writes are visible to all after the exchange.
-// Returns false on a wait that ran out or CTA 0's vote to stop.
-template <int NV, bool PUBLISH, typename T, typename F>
+// meanwhile runs in every thread while the sums travel.  Returns false on a wait that ran out or CTA 0's vote to stop.
+template <int NV, bool PUBLISH, typename T, typename F, typename M>
 __device__ __forceinline__ bool exchange(const T (&v)[NV], int TT, int ctas,
                                          ulonglong2 *slots, unsigned long long iter, int my_vote,
-                                         PersSmem<T> &sm, F &&use) {
+                                         PersSmem<T> &sm, F &&use, M &&meanwhile) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double s = fold_block<NV>(v, TT, sm.fold);
+    ulonglong2 *mine = slots + (int64_t)warp * ctas;
+    if (warp < NV && lane == 0 && (int)blockIdx.x < ctas) {
+        if (PUBLISH) __threadfence();
+        st_slot(mine + blockIdx.x, s, 2 * iter + my_vote);
+    }
+    meanwhile();
     if (warp < NV) {
-        ulonglong2 *mine = slots + (int64_t)warp * ctas;
-        if (lane == 0 && (int)blockIdx.x < ctas) {
-            if (PUBLISH) __threadfence();
-            st_slot(mine + blockIdx.x, s, 2 * iter + my_vote);
-        }
         double a[kPartLoads];
         int vt = 0;
         const bool ok = wait_slots(mine, ctas, iter, a, &vt);
@@ -311,10 +312,10 @@ cg_persistent(PersArgs<T> a, ColT col) {
         auto take_pq = [&](int, double pq) { step_alpha(rho, pq, sm.step); };
         const bool go = (RES || own) ? exchange<1, false>(v1, a.pq.threads, a.pq.ctas,
                                                           a.slots + kSlotsPq, it, my_vote, sm,
-                                                          take_pq)
+                                                          take_pq, [] {})
                                      : exchange<1, true>(v1, a.pq.threads, a.pq.ctas,
                                                          a.slots + kSlotsPq, it, my_vote, sm,
-                                                         take_pq);
+                                                         take_pq, [] {});
         if (!go) {
             done = 4;
             break;
@@ -330,7 +331,6 @@ cg_persistent(PersArgs<T> a, ColT col) {
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 if (g0 < g1 && row0 + i < n) {
-                    x[i] = fma_t(alpha, p[i], x[i]);
                     r[i] = fma_t(-alpha, acc[i], r[i]);
                     z[i] = d[i] * r[i];
                     vz = fma_t(r[i], z[i], vz);
@@ -351,6 +351,13 @@ cg_persistent(PersArgs<T> a, ColT col) {
                                     } else {
                                         sm.step.rr = sum;
                                         sm.step.done = step_done(sum, limit, iters, max_iter);
+                                    }
+                                },
+                                [&] {  // nothing waits for x
+                                    if constexpr (RES) {
+#pragma unroll
+                                        for (int i = 0; i < R; ++i)
+                                            x[i] = fma_t(alpha, p[i], x[i]);
                                     }
                                 })) {
             done = 4;
