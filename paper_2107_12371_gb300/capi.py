@@ -198,17 +198,47 @@ def _check(status, where):
 
 def _ptr(t):
     """Device/host pointer of a torch tensor or numpy array (None -> NULL)."""
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        return t.ctypes.data if isinstance(t, np.ndarray) else _no_pointer(t)
+
+
+def _no_pointer(t):
     if t is None:
         return None
-    if isinstance(t, np.ndarray):
-        return t.ctypes.data
-    return t.data_ptr()
+    raise AttributeError("%r has no data pointer" % type(t).__name__)
+
+
+def _find_stream_reader():
+    """A function returning the current stream's handle.  Small products take a few microseconds,
+    of which building torch's Stream object for its handle alone would be one: torch's raw
+    accessors give the same handle once CUDA is initialised (before, the ordinary call does it)."""
+    import torch
+
+    def ordinary():
+        return torch.cuda.current_stream().cuda_stream
+
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is None or raw is None:
+        return ordinary
+    initialised = torch.cuda.is_initialized
+
+    def current():
+        return raw(device()) if initialised() else ordinary()
+    return current
+
+
+_current_stream = None
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _current_stream
+        if _current_stream is None:
+            _current_stream = _find_stream_reader()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
