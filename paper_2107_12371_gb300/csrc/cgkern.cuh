@@ -308,32 +308,6 @@ __device__ __forceinline__ double reduce_parts(const double *part, int count) {
     return sum_parts(a);
 }
 
-// Programmatic dependent launch (a kernel launched by launch_dependent).  dep_wait: returns once
-// the kernels this one depends on have finished and their writes are visible; before it, only
-// data that no kernel of the solve writes may be read (the matrix, D^-1).  dep_allow: lets the
-// next kernel's CTAs start as SM slots become free; they stop at their own dep_wait.
-__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void dep_allow() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// Launches a kernel that begins with dep_wait so that it may start while the kernel before it on
-// the stream still runs (also as an edge of a captured graph).
-template <typename... K, typename... A>
-spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t st,
-                               A... args) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cuda_status(cudaLaunchKernelEx(&cfg, kern, K(args)...));
-}
-
 // Each CTA stores its partial sums in part[k * gridDim.x + cta]; the CTA that arrives last
 // (atomic ticket) sums all partials in a fixed order.  Returns true in that CTA, with the
 // grid totals in tot[] (valid in thread 0); the ticket is reset for the next launch.

@@ -53,6 +53,23 @@ inline spmv_status_t cuda_status(cudaError_t e) {
 
 #define GB_LAUNCHED() GB_CUDA(cudaGetLastError())
 
+// Launches a kernel that begins with dep_wait so that it may start while the kernel before it on
+// the stream still runs (also as an edge of a captured graph).
+template <typename... K, typename... A>
+spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t st,
+                               A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_status(cudaLaunchKernelEx(&cfg, kern, K(args)...));
+}
+
 // Stream on which handle buffers are allocated and freed (stream-ordered allocator), set for
 // the duration of an entry point by AllocStream.  Stream-ordered frees never synchronize the
 // whole device, so solves running concurrently on other streams are not stalled.

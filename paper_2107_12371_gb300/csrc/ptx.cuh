@@ -160,6 +160,11 @@ struct Cols16 {
     __device__ __forceinline__ int32_t base(int64_t slice) const { return col_start[slice]; }
 };
 
+// Hint: bring the line holding p into L2 without waiting for it.
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // ---- gathers of the multiplying vector (read-only path, L1 allocating) ----------------
 // Only for vectors that no thread writes while the kernel runs.
 __device__ __forceinline__ double ld_x(const double *p) { return __ldg(p); }
@@ -208,5 +213,15 @@ __device__ __forceinline__ void store_rows(T *y, int64_t row0, int32_t n, const 
 
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// Programmatic dependent launch (a kernel launched by launch_dependent).  dep_wait: returns once
+// the kernels this one depends on have finished and their writes are visible; before it, only
+// data that no kernel still running may write is read (a handle's matrix, a solve's D^-1).
+// dep_allow: lets the next kernel's CTAs start as SM slots become free; they stop at their own
+// dep_wait.  Called after dep_wait, so that no more than two kernels of a stream are in flight.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_allow() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 }  // namespace gb

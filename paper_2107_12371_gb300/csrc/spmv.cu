@@ -28,17 +28,21 @@ namespace {
 // gt: the slice-lane this thread computes (slice gt / L, lane gt % L).  The entries of a row
 // go in blocks of U (all loads of a block issued before its gathers, and those before its
 // FMAs), the rest one at a time.
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
+// DEP: a dependent launch (dep_wait), done by the thread's first slice-lane.
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP = false>
 __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_slices,
                                                const int64_t *__restrict__ sp, ColT cols,
                                                const T *__restrict__ val,
                                                const T *__restrict__ x, T *__restrict__ y,
-                                               T alpha, T beta) {
+                                               T alpha, T beta, bool first = false) {
     // L lanes per slice, R rows per lane: S = L R rows per slice
     constexpr int S = L * R;
     const int64_t slice = gt / L;
     const int lane = (int)(gt % L);
-    if (slice >= n_slices) return;
+    if (slice >= n_slices) {
+        if (DEP && first) dep_wait();
+        return;
+    }
     const int64_t base = sp[slice];
     const int w = (int)((sp[slice + 1] - base) / S);
     const int32_t cbase = cols.base(slice);
@@ -48,6 +52,19 @@ __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_
     T acc[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) acc[i] = T(0);
+    // the matrix does not depend on the kernel before: while that one ends, the first entries are
+    // brought into L2 (held in registers they spill)
+    if (DEP && first) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (u < w) {
+                prefetch_l2(vp + (int64_t)u * S);
+                prefetch_l2(cols.col + cat + (int64_t)u * S);
+            }
+        }
+        dep_wait();
+        dep_allow();
+    }
     int t = 0;
     for (; t + U <= w; t += U) {
         T v[U][R];
@@ -100,13 +117,13 @@ spmv_sell(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols
 // FP64 with one or two rows per lane, capped at 32 registers (2 x 1024 threads per SM), four
 // entries in flight: for matrices whose widest slice needs fewer load rounds in blocks of four
 // than of five (see go_sell).
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP>
 __global__ void __launch_bounds__(1024, 2)
 spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
               const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
               T beta) {
-    spmv_sell_body<T, R, L, U, ColT, AXPBY>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
-                                            n_slices, sp, cols, val, x, y, alpha, beta);
+    spmv_sell_body<T, R, L, U, ColT, AXPBY, DEP>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
+                                                 n_slices, sp, cols, val, x, y, alpha, beta, true);
 }
 
 // FP64 with one or two rows per lane: a grid of at most kGsCtasPerSm 256-thread CTAs per SM
@@ -116,15 +133,18 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
 // SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.
 constexpr int kGsBlock = 256;
 constexpr int kGsCtasPerSm = 4;
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP>
 __global__ void __launch_bounds__(kGsBlock, kGsCtasPerSm)
 spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
              const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
              T beta) {
     const int64_t items = (int64_t)n_slices * L;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gt < items; gt += stride)
-        spmv_sell_body<T, R, L, U, ColT, AXPBY>(gt, n, n_slices, sp, cols, val, x, y, alpha, beta);
+    const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (DEP && g0 >= items) dep_wait();
+    for (int64_t gt = g0; gt < items; gt += stride)
+        spmv_sell_body<T, R, L, U, ColT, AXPBY, DEP>(gt, n, n_slices, sp, cols, val, x, y, alpha,
+                                                     beta, gt == g0);
 }
 
 // The product of small and of ragged matrices (see use_thin): one or two rows per lane, S / R
@@ -144,7 +164,10 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
     constexpr int S = L * R;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t slice = gt / L;
-    if (slice >= n_slices) return;
+    if (slice >= n_slices) {
+        dep_wait();
+        return;
+    }
     const int lane = (int)(gt % L);
     const int64_t base = sp[slice];
     const int w = (int)((sp[slice + 1] - base) / S);
@@ -154,10 +177,10 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
     T acc[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) acc[i] = T(0);
-    auto round = [&](int t, auto masked) {
+    T v[U][R];
+    int32_t c[U][R];
+    auto load = [&](int t, auto masked) {
         constexpr bool kMasked = decltype(masked)::value;
-        T v[U][R];
-        int32_t c[U][R];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (!kMasked || t + u < w) {
@@ -171,6 +194,8 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
                 }
             }
         }
+    };
+    auto multiply = [&] {
         T xv[U][R];
 #pragma unroll
         for (int u = 0; u < U; ++u)
@@ -182,9 +207,22 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
             for (int i = 0; i < R; ++i)
                 if (c[u][i] >= 0) acc[i] = fma_t(v[u][i], xv[u][i], acc[i]);
     };
-    int t = 0;
-    for (; t + U <= w; t += U) round(t, std::false_type{});
-    if (t < w) round(t, std::true_type{});
+    // the matrix does not depend on the kernel before: its first entries are requested while that
+    // one ends
+    if (U <= w) load(0, std::false_type{});
+    else load(0, std::true_type{});
+    dep_wait();
+    dep_allow();
+    multiply();
+    int t = U;
+    for (; t + U <= w; t += U) {
+        load(t, std::false_type{});
+        multiply();
+    }
+    if (t < w) {
+        load(t, std::true_type{});
+        multiply();
+    }
     const int64_t row0 = gt * R;
     if constexpr (AXPBY) {
 #pragma unroll
@@ -230,28 +268,41 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
                       cudaStream_t st) {
     const int block = A->block;
     const unsigned grid = grid_for((int64_t)A->n_slices * L, block);
-    auto go = [&](auto c) {
+    // Dependent launches, so that a product starts under the tail of the kernel before it: the
+    // chain of 304K tetrahedra and their 600K faces 16.5 -> 13.4 us, a 1.3M-row product 18.6 ->
+    // 16.9 in a stream of products; the long kernels above gain nothing and run 2 % slower with
+    // the wait in them (6M rows 68.0 -> 69.6).
+    const bool dep = A->n <= 2000000;
+    auto go = [&](auto c) -> spmv_status_t {
         using ColT = decltype(c);
         if constexpr (sizeof(T) == 8 && R <= 2) {
             if (load_rounds(A->max_width, 5) < load_rounds(A->max_width, 4)) {
                 const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
                 const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
                 const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
-                spmv_sell_gs<T, R, L, 5, ColT, AXPBY><<<g, kGsBlock, 0, st>>>(
+                if (dep)
+                    return launch_dependent(spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>, g, kGsBlock,
+                                            st, A->n, A->n_slices, A->slice_ptr.p, c, val, x, y,
+                                            alpha, beta);
+                spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false><<<g, kGsBlock, 0, st>>>(
                     A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
             } else {
-                spmv_sell_occ<T, R, L, U, ColT, AXPBY><<<grid, block, 0, st>>>(
+                if (dep)
+                    return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY, true>, grid,
+                                            block, st, A->n, A->n_slices, A->slice_ptr.p, c, val, x,
+                                            y, alpha, beta);
+                spmv_sell_occ<T, R, L, U, ColT, AXPBY, false><<<grid, block, 0, st>>>(
                     A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
             }
         } else {
             spmv_sell<T, R, L, U, ColT, AXPBY><<<grid, block, 0, st>>>(
                 A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
         }
+        GB_LAUNCHED();
+        return SPMV_OK;
     };
-    if (A->index_bits == 16) go(Cols16{A->sell_col16.p, A->col_start.p});
-    else go(Cols32{A->sell_col.p});
-    GB_LAUNCHED();
-    return SPMV_OK;
+    if (A->index_bits == 16) return go(Cols16{A->sell_col16.p, A->col_start.p});
+    return go(Cols32{A->sell_col.p});
 }
 
 // Where spmv_sell_thin is the faster kernel (old / thin, measured on tetrahedral and mixed meshes
@@ -285,14 +336,13 @@ spmv_status_t go_thin(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
                                                                                            : A->block;
         const unsigned grid = grid_for(lanes, block);
         if (A->index_bits == 16)
-            spmv_sell_thin<T, R, L, U, Cols16, AXPBY><<<grid, block, 0, st>>>(
-                A->n, A->n_slices, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p}, val, x,
-                y, alpha, beta);
-        else
-            spmv_sell_thin<T, R, L, U, Cols32, AXPBY><<<grid, block, 0, st>>>(
-                A->n, A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, x, y, alpha, beta);
-        GB_LAUNCHED();
-        return SPMV_OK;
+            return launch_dependent(spmv_sell_thin<T, R, L, U, Cols16, AXPBY>, grid, block, st,
+                                    A->n, A->n_slices, A->slice_ptr.p,
+                                    Cols16{A->sell_col16.p, A->col_start.p}, val, x, y, alpha,
+                                    beta);
+        return launch_dependent(spmv_sell_thin<T, R, L, U, Cols32, AXPBY>, grid, block, st, A->n,
+                                A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, x, y,
+                                alpha, beta);
     };
     auto go = [&](auto rt, auto ut) -> spmv_status_t {
         switch (A->S) {

@@ -591,6 +591,50 @@ def test_product_kernels_agree_at_the_edges_of_their_ranges(rows):
     assert torch.equal(y32[0], y32[1]) and torch.equal(y32[0], y32[2])
 
 
+@pytest.mark.parametrize("rows,per_row", [(33, 3), (5003, 4), (300000, 5), (1000003, 6),
+                                          (2000000, 5), (2000001, 5)])
+def test_products_that_wait_for_one_another(rows, per_row):
+    """Products in a row on one stream, each the next one's input (dependent launches up to 2M
+    rows), with a copy, another stream's product and other kernels between them; then the same
+    captured in a graph.  Equal bit for bit to the CSR kernel with a synchronisation after each."""
+    i = np.arange(rows, dtype=np.int64)
+    j = (i[:, None] + np.array([0, 1, -1, 29, -29, 777])[None, :per_row]) % rows
+    rp = np.arange(rows + 1, dtype=np.int64) * per_row
+    v = np.random.default_rng(1).uniform(-0.3, 0.3, rows * per_row)
+    A = capi.Matrix(rows, rp.astype(np.int32), np.sort(j, 1).astype(np.int32).ravel(), v)
+    x = dev(np.random.default_rng(2).uniform(-1, 1, rows))
+    side = torch.cuda.Stream()
+    b = [torch.empty_like(x) for _ in range(4)]
+
+    def row(apply, sync):
+        here = torch.cuda.current_stream()
+        b[0].copy_(x)
+        for step in range(12):
+            src, dst = b[step % 3], b[(step + 1) % 3]
+            apply(src, dst)
+            sync()
+            if step % 4 == 1:
+                dst.mul_(1.25)
+            if step % 4 == 2:
+                side.wait_stream(here)
+                with torch.cuda.stream(side):
+                    apply(dst, b[3])
+                here.wait_stream(side)
+                dst.copy_(b[3])
+            sync()
+        return b[0]
+
+    ref = row(A.apply_csr, torch.cuda.synchronize).clone()
+    assert torch.equal(row(A.apply, lambda: None), ref)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = row(A.apply, lambda: None)
+    out.fill_(float("nan"))
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+
+
 @pytest.mark.parametrize("bits", [16, 32])
 @pytest.mark.parametrize("k", [1, 2, 3, 5, 6, 7, 9, 11, 12, 17, 20, 23, 24, 31, 33, 40, 44, 48, 57,
                                63, 64])
