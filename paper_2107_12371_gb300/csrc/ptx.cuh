@@ -160,11 +160,6 @@ struct Cols16 {
     __device__ __forceinline__ int32_t base(int64_t slice) const { return col_start[slice]; }
 };
 
-// Hint: bring the line holding p into L2 without waiting for it.
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 // ---- gathers of the multiplying vector (read-only path, L1 allocating) ----------------
 // Only for vectors that no thread writes while the kernel runs.
 __device__ __forceinline__ double ld_x(const double *p) { return __ldg(p); }

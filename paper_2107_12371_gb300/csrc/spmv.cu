@@ -1,19 +1,19 @@
 // spmv.cu -- SpMV kernels (the multi-vector products are in spmm.cu).
 //
-// spmv_sell<T, R, L>: L lanes per slice of S = L R rows, lane l owns rows l R .. l R + R - 1
-//   of the slice.  Because a slice is stored column-major (Sec. 4.2), step t of the lanes
-//   reads S consecutive values and column indices: one R-wide vector load per lane, fully
+// spmv_sell_thin<T, R, L>: L lanes per slice of S = L R rows, lane l owns rows l R .. l R + R - 1
+//   of the slice (one or two).  Because a slice is stored column-major (Sec. 4.2), step t of the
+//   lanes reads S consecutive values and column indices: one R-wide vector load per lane, fully
 //   coalesced, streamed evict-first so the matrix never displaces x from L2.  x is gathered
 //   through the read-only L1 path; with a banded (Cuthill-McKee) order the gathers of
 //   neighbouring rows hit the same lines (Sec. 4.3, 5.1).  Each row accumulates its entries
 //   in ascending column order with fused multiply-add from +0.0; padding entries (column -1)
 //   are skipped.  Column indices come as int32 or (when every slice spans fewer than 65,535
 //   columns) as 16-bit offsets from the slice's col_start (Sec. 5.1), 10 instead of 12 bytes
-//   per FP64 non-zero.
-// spmv_sell_occ / spmv_sell_gs: the FP64 forms with one or two rows per lane, one slice-lane
-//   per thread at 32 registers, or a grid of four CTAs per SM striding over the slice-lanes
-//   with five entries of each row in flight; the one whose widest slice needs fewer dependent
-//   load rounds is launched.
+//   per FP64 non-zero.  All FP32 products, and the FP64 ones up to a few million rows (use_thin).
+// spmv_sell_occ / spmv_sell_gs: FP64 products of larger matrices at one or two rows per lane, one
+//   slice-lane per thread at 32 registers, or a grid of four CTAs per SM striding over the
+//   slice-lanes with five entries of each row in flight; the one whose widest slice needs fewer
+//   dependent load rounds is launched.  spmv_sell: the same at four or eight rows per lane.
 // spmv_csr: the naive baseline of Sec. 4.3, thread per CSR row.
 #include <type_traits>
 
@@ -28,21 +28,17 @@ namespace {
 // gt: the slice-lane this thread computes (slice gt / L, lane gt % L).  The entries of a row
 // go in blocks of U (all loads of a block issued before its gathers, and those before its
 // FMAs), the rest one at a time.
-// DEP: a dependent launch (dep_wait), done by the thread's first slice-lane.
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP = false>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_slices,
                                                const int64_t *__restrict__ sp, ColT cols,
                                                const T *__restrict__ val,
                                                const T *__restrict__ x, T *__restrict__ y,
-                                               T alpha, T beta, bool first = false) {
+                                               T alpha, T beta) {
     // L lanes per slice, R rows per lane: S = L R rows per slice
     constexpr int S = L * R;
     const int64_t slice = gt / L;
     const int lane = (int)(gt % L);
-    if (slice >= n_slices) {
-        if (DEP && first) dep_wait();
-        return;
-    }
+    if (slice >= n_slices) return;
     const int64_t base = sp[slice];
     const int w = (int)((sp[slice + 1] - base) / S);
     const int32_t cbase = cols.base(slice);
@@ -52,19 +48,6 @@ __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_
     T acc[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) acc[i] = T(0);
-    // the matrix does not depend on the kernel before: while that one ends, the first entries are
-    // brought into L2 (held in registers they spill)
-    if (DEP && first) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (u < w) {
-                prefetch_l2(vp + (int64_t)u * S);
-                prefetch_l2(cols.col + cat + (int64_t)u * S);
-            }
-        }
-        dep_wait();
-        dep_allow();
-    }
     int t = 0;
     for (; t + U <= w; t += U) {
         T v[U][R];
@@ -117,13 +100,13 @@ spmv_sell(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols
 // FP64 with one or two rows per lane, capped at 32 registers (2 x 1024 threads per SM), four
 // entries in flight: for matrices whose widest slice needs fewer load rounds in blocks of four
 // than of five (see go_sell).
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __global__ void __launch_bounds__(1024, 2)
 spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
               const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
               T beta) {
-    spmv_sell_body<T, R, L, U, ColT, AXPBY, DEP>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
-                                                 n_slices, sp, cols, val, x, y, alpha, beta, true);
+    spmv_sell_body<T, R, L, U, ColT, AXPBY>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
+                                            n_slices, sp, cols, val, x, y, alpha, beta);
 }
 
 // FP64 with one or two rows per lane: a grid of at most kGsCtasPerSm 256-thread CTAs per SM
@@ -133,34 +116,33 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
 // SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.
 constexpr int kGsBlock = 256;
 constexpr int kGsCtasPerSm = 4;
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool DEP>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __global__ void __launch_bounds__(kGsBlock, kGsCtasPerSm)
 spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
              const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
              T beta) {
     const int64_t items = (int64_t)n_slices * L;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (DEP && g0 >= items) dep_wait();
-    for (int64_t gt = g0; gt < items; gt += stride)
-        spmv_sell_body<T, R, L, U, ColT, AXPBY, DEP>(gt, n, n_slices, sp, cols, val, x, y, alpha,
-                                                     beta, gt == g0);
+    for (int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gt < items; gt += stride)
+        spmv_sell_body<T, R, L, U, ColT, AXPBY>(gt, n, n_slices, sp, cols, val, x, y, alpha, beta);
 }
 
-// The product of small and of ragged matrices (see use_thin): one or two rows per lane, S / R
-// lanes per slice (a slice may span several warps), U entries in flight, and the remainder of
-// a row as one more round with the missing entries masked instead of one dependent round per
-// entry.  At these sizes the chip is not full: a row is a chain of three or four dependent
-// loads of 0.6 us, and what helps is more threads (four rows per lane leave 400K rows a third
-// of the thread slots) and fewer rounds (a 13-entry row took five with U = 5 and a plain loop
-// behind it).  Measured (us, before -> now): FP32 398K mixed-mesh rows 10.9 -> 6.6 (int32
-// columns), 24K 5.9 -> 2.7, 48K tetrahedra 3.8 -> 2.9, 1.3M 10.8 -> 8.8; FP64 24K mixed 6.4 ->
-// 3.7, 192K 9.6 -> 7.1, 48K tetrahedra 3.4 -> 3.0.  Same order and bits as spmv_sell.
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
-__global__ void __launch_bounds__(1024, 1)
+// One or two rows per lane, S / R lanes per slice (a slice may span several warps), U entries in
+// flight, and the remainder of a row as one more round with the missing entries masked instead of
+// one dependent round per entry.  A row is a chain of three or four dependent loads of 0.6 us, so
+// below a few million rows time goes by how many waves of threads an SM takes and how many rounds
+// a row takes: CTAS (CTAs of kThinBlock per SM) sets the registers, 64, 40 or 32, and with them
+// the 1,024, 1,536 or 2,048 threads that an SM holds (see go_thin).  A dependent launch: slices
+// and the first round of entries are requested while the kernel before still runs.  Measured (us,
+// against four rows per lane, plain launches and registers as they fell): FP64 48K tetrahedra 3.4
+// -> 2.0, 304K 5.9 -> 4.2, 1.3M 18.7 -> 13.7, 398K mixed-mesh rows 16 -> 11.7; FP32 304K 8 -> 2.4,
+// 1.3M 10.8 -> 7.1, 6M 36 -> 32, 398K mixed 16.6 -> 5.9.  Same order and bits as spmv_sell.
+constexpr int kThinBlock = 128;
+template <typename T, int R, int L, int U, int CTAS, typename ColT, bool AXPBY>
+__global__ void __launch_bounds__(kThinBlock, CTAS)
 spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
                const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
-               T beta) {
+               T beta, bool add) {
     constexpr int S = L * R;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t slice = gt / L;
@@ -213,6 +195,16 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
     else load(0, std::true_type{});
     dep_wait();
     dep_allow();
+    const int64_t row0 = gt * R;
+    // y of the rows: in FP32 with the first gathers (0.2 us of a small product); in FP64, where the
+    // registers are short, at the end (1.3M rows 20.8 against 26.0 us).  `add` is beta != 0: the
+    // comparison in FP64 costs as much of the FP64 pipe as a multiply-add
+    T y0[AXPBY ? R : 1];
+    auto load_y = [&] {
+#pragma unroll
+        for (int i = 0; i < R; ++i) y0[i] = add && row0 + i < n ? y[row0 + i] : T(0);
+    };
+    if constexpr (AXPBY && sizeof(T) == 4) load_y();
     multiply();
     int t = U;
     for (; t + U <= w; t += U) {
@@ -223,13 +215,11 @@ spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT
         load(t, std::true_type{});
         multiply();
     }
-    const int64_t row0 = gt * R;
     if constexpr (AXPBY) {
+        if constexpr (sizeof(T) == 8) load_y();
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-            if (row0 + i < n)
-                acc[i] = beta != T(0) ? fma_t(alpha, acc[i], beta * y[row0 + i]) : alpha * acc[i];
-        }
+        for (int i = 0; i < R; ++i)
+            acc[i] = add ? fma_t(alpha, acc[i], beta * y0[i]) : alpha * acc[i];
     }
     store_rows<T, R>(y, row0, n, acc);
 }
@@ -261,37 +251,24 @@ inline unsigned grid_for(int64_t threads, int block) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// (R, L) per slice height: FP64 lanes read 8R bytes of values (16 B at S = 64, 32 B at
-// S >= 128); FP32 lanes read 16 B (R = 4) or 32 B (R = 8).
+// The FP64 products of larger matrices; (R, L) per slice height: lanes read 8 R bytes of values per
+// entry (16 B at S = 64, 32 B at S = 128).
 template <typename T, int R, int L, int U, bool AXPBY>
 spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, T beta,
                       cudaStream_t st) {
     const int block = A->block;
     const unsigned grid = grid_for((int64_t)A->n_slices * L, block);
-    // Dependent launches, so that a product starts under the tail of the kernel before it: the
-    // chain of 304K tetrahedra and their 600K faces 16.5 -> 13.4 us, a 1.3M-row product 18.6 ->
-    // 16.9 in a stream of products; the long kernels above gain nothing and run 2 % slower with
-    // the wait in them (6M rows 68.0 -> 69.6).
-    const bool dep = A->n <= 2000000;
     auto go = [&](auto c) -> spmv_status_t {
         using ColT = decltype(c);
-        if constexpr (sizeof(T) == 8 && R <= 2) {
+        if constexpr (R <= 2) {
             if (load_rounds(A->max_width, 5) < load_rounds(A->max_width, 4)) {
                 const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
                 const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
                 const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
-                if (dep)
-                    return launch_dependent(spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>, g, kGsBlock,
-                                            st, A->n, A->n_slices, A->slice_ptr.p, c, val, x, y,
-                                            alpha, beta);
-                spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false><<<g, kGsBlock, 0, st>>>(
+                spmv_sell_gs<T, R, L, 5, ColT, AXPBY><<<g, kGsBlock, 0, st>>>(
                     A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
             } else {
-                if (dep)
-                    return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY, true>, grid,
-                                            block, st, A->n, A->n_slices, A->slice_ptr.p, c, val, x,
-                                            y, alpha, beta);
-                spmv_sell_occ<T, R, L, U, ColT, AXPBY, false><<<grid, block, 0, st>>>(
+                spmv_sell_occ<T, R, L, U, ColT, AXPBY><<<grid, block, 0, st>>>(
                     A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
             }
         } else {
@@ -305,65 +282,93 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
     return go(Cols32{A->sell_col.p});
 }
 
-// Where spmv_sell_thin is the faster kernel (old / thin, measured on tetrahedral and mixed meshes
-// in random, RCM and sorted order).  FP32, whose other kernels take four or eight rows per lane:
-// 1.1 to 2.6 up to 1.5M rows (2.0M: 0.93); with alpha and beta and at S = 256 up to 512K (750K:
-// 0.93 to 0.97).  FP64: up to 64K rows (1.0 to 1.7), at S >= 128, whose other kernels take four
-// and eight rows per lane (1.1 to 4 up to 2M), and at S = 64 for slices wider than the five
-// entries that the other kernels take in one round, up to 512K rows (1.0 to 1.75; 1M: 0.89 to
-// 1.09).  Not for FP64 rows of up to five entries above 64K (304K tetrahedra: 0.94 to 1.04, the
-// gradient's two-entry rows of a chain 0.79).
-bool use_thin(const spmv_matrix_t A, bool f32, bool axpby) {
-    if (f32) return A->n <= (axpby || A->S == 256 ? 512 * 1024 : 1500000);
-    if (A->n <= 64 * 1024) return true;
-    if (A->S >= 128) return A->n <= 2000000;
-    return A->S == 64 && A->max_width > 5 && A->n <= 512 * 1024;
+// FP64 products that spmv_sell_thin takes (us, spmv_sell_gs or _occ / thin).  Rows of up to six
+// entries in Cuthill-McKee order: 304K 4.5 / 4.2, 796K 10.5 / 8.7, 3.1M 35.1 / 29.9, 6M 68.1 /
+// 71.1; of two entries (a gradient's faces): 600K 5.3 / 4.5, 2.6M 22.6 / 17.2.  Longer rows: 647K
+// 20.8 / 17.1, 1.8M 44.6 / 43.5, 3M 70.8 / 69.9 but with alpha and beta 82.6 / 84.5.
+bool use_thin(const spmv_matrix_t A) {
+    return A->n <= (A->max_width > 2 && A->mean_width > 6.f ? 2000000 : 3500000);
 }
-// FP32 lanes take one row up to here and two above (24K mixed-mesh rows 2.4 against 2.8 us, 192K
-// 3.6 and 3.8; 398K 5.7 and 5.5, 1.3M tetrahedra 9.0 and 8.2).
-constexpr int32_t kThinRows32 = 256 * 1024;
 
+// Rows per lane, entries in flight and registers of spmv_sell_thin, by the threads that an SM
+// then has to run.
 template <typename T, bool AXPBY>
 spmv_status_t go_thin(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, T beta,
                       cudaStream_t st) {
-    auto shape = [&](auto rt, auto ut, auto st_) -> spmv_status_t {
+    using std::integral_constant;
+    auto launch = [&](auto rt, auto ut, auto ct, auto heightt) -> spmv_status_t {
         constexpr int R = decltype(rt)::value, U = decltype(ut)::value;
-        constexpr int L = decltype(st_)::value / R;
-        const int64_t lanes = (int64_t)A->n_slices * L;
-        // smaller CTAs while they do not fill the chip: they spread over more SMs (48K rows 2.8
-        // against 3.1 us)
-        const int block = A->block > 128 && lanes < (int64_t)device_facts().sm_count * 2048 ? 128
-                                                                                           : A->block;
-        const unsigned grid = grid_for(lanes, block);
+        constexpr int CTAS = decltype(ct)::value, L = decltype(heightt)::value / R;
+        const int block = A->block < kThinBlock ? A->block : kThinBlock;
+        const unsigned grid = grid_for((int64_t)A->n_slices * L, block);
         if (A->index_bits == 16)
-            return launch_dependent(spmv_sell_thin<T, R, L, U, Cols16, AXPBY>, grid, block, st,
-                                    A->n, A->n_slices, A->slice_ptr.p,
+            return launch_dependent(spmv_sell_thin<T, R, L, U, CTAS, Cols16, AXPBY>, grid, block,
+                                    st, A->n, A->n_slices, A->slice_ptr.p,
                                     Cols16{A->sell_col16.p, A->col_start.p}, val, x, y, alpha,
-                                    beta);
-        return launch_dependent(spmv_sell_thin<T, R, L, U, Cols32, AXPBY>, grid, block, st, A->n,
-                                A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, x, y,
-                                alpha, beta);
+                                    beta, beta != T(0));
+        return launch_dependent(spmv_sell_thin<T, R, L, U, CTAS, Cols32, AXPBY>, grid, block, st,
+                                A->n, A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, x,
+                                y, alpha, beta, beta != T(0));
     };
-    auto go = [&](auto rt, auto ut) -> spmv_status_t {
+    auto go = [&](auto rt, auto ut, auto ct) -> spmv_status_t {
         switch (A->S) {
-            case 32: return shape(rt, ut, std::integral_constant<int, 32>{});
-            case 64: return shape(rt, ut, std::integral_constant<int, 64>{});
-            case 128: return shape(rt, ut, std::integral_constant<int, 128>{});
-            case 256: return shape(rt, ut, std::integral_constant<int, 256>{});
+            case 32: return launch(rt, ut, ct, integral_constant<int, 32>{});
+            case 64: return launch(rt, ut, ct, integral_constant<int, 64>{});
+            case 128: return launch(rt, ut, ct, integral_constant<int, 128>{});
+            case 256: return launch(rt, ut, ct, integral_constant<int, 256>{});
         }
         return SPMV_ERR_INVALID_ARG;
     };
-    using std::integral_constant;
-    // entries in flight: a whole row of the tetrahedral meshes; for longer rows four in FP64
-    // (whose gathers then still leave the SM enough warps), six in FP32
-    const bool longer = A->mean_width > 6.f;
-    if constexpr (sizeof(T) == 8) {
-        if (longer) return go(integral_constant<int, 1>{}, integral_constant<int, 4>{});
-        return go(integral_constant<int, 1>{}, integral_constant<int, 5>{});
+    constexpr bool f32 = sizeof(T) == 4;
+    constexpr integral_constant<int, 1> one{};
+    constexpr integral_constant<int, 2> two{};
+    constexpr integral_constant<int, 5> u5{};
+    constexpr integral_constant<int, 6> u6{};
+    constexpr integral_constant<int, 7> u7{};
+    constexpr integral_constant<int, 8> regs64{};
+    constexpr integral_constant<int, 12> regs40{};
+    constexpr integral_constant<int, 16> regs32{};
+    // The entries in flight are a whole row of the tetrahedral meshes (5), two for two-entry rows
+    // (five, four masked: 600K rows 6.8 against 4.5 us), and for longer rows what the registers
+    // hold: FP64 6 (4: 192K mixed-mesh rows 8.0 against 6.5 us, 7: 7.2), FP32 7 (5: 292K rows 5.2
+    // against 4.2).
+    const bool narrow = A->max_width <= 2;
+    const bool longer = !narrow && A->mean_width > 6.f;
+    auto threads_per_sm = [&](int R) {
+        return (int64_t)A->n_slices * (A->S / R) / device_facts().sm_count;
+    };
+    // Two rows per lane halve the threads where one would need more than the SM holds in a single
+    // wave: FP32 (304K rows 3.9 against 2.4 us; 192K mixed 3.2 against 4.1, 222K even), and
+    // two-entry rows.  Other FP64 rows have no registers for two (304K rows 7.0 against 4.9).
+    const bool two_rows = narrow || (f32 && (longer ? threads_per_sm(1) > 1280
+                                                    : A->n > 256 * 1024));
+    const int64_t threads = threads_per_sm(two_rows ? 2 : 1);
+    // 64 registers for up to 1,024 threads; else those that let one wave of 1,536 or 2,048 threads
+    // cover the rows (FP64 162K rows: 3.3 us at 40 registers, 4.0 at 32; 304K rows, 2,000 threads:
+    // 4.4 and 4.2; FP32 511K rows, 1,680 threads: 3.9 and 3.5).  With more waves two rows per lane
+    // do better at 40 (878K two-entry rows 6.3, against 7.6 at 32), one row at 32 (1M rows 10.8,
+    // against 11.1 at 40 and 13.7 at 64)
+    const bool one_wave32 = threads > 1536 && threads <= 2048;
+    if (narrow) {
+        if (threads <= 1024) return go(two, two, regs64);
+        return one_wave32 ? go(two, two, regs32) : go(two, two, regs40);
+    }
+    if constexpr (f32) {
+        if (!two_rows) return longer ? go(one, u7, regs64) : go(one, u5, regs64);
+        if (longer) {  // 398K mixed 5.1 at 40 registers, 5.9 at 64; 942K 14.1 at 64 (U = 7: 14.4)
+            if (threads <= 1024) return go(two, u7, regs64);
+            return threads <= 1536 ? go(two, u7, regs40) : go(two, u6, regs64);
+        }
+        if (threads <= 1024) return go(two, u5, regs64);
+        return one_wave32 ? go(two, u5, regs32) : go(two, u5, regs40);
     } else {
-        if (A->n > kThinRows32) return go(integral_constant<int, 2>{}, integral_constant<int, 5>{});
-        if (longer) return go(integral_constant<int, 1>{}, integral_constant<int, 6>{});
-        return go(integral_constant<int, 1>{}, integral_constant<int, 5>{});
+        if (longer) return go(one, u6, regs64);
+        // rows whose gathers miss L1 (random cell order) are bound by the loads in flight: 1.3M
+        // rows 25.6 at 64 registers, 27.7 at 32
+        if (threads <= 1024 || (A->max_span > 65535 && A->n > 1000000))
+            return go(one, u5, regs64);
+        // y = alpha A x + beta y spills at 32 (1.3M rows 20.8 against 29.0)
+        return AXPBY || threads <= 1536 ? go(one, u5, regs40) : go(one, u5, regs32);
     }
 }
 
@@ -371,26 +376,18 @@ template <typename T, bool AXPBY = false>
 spmv_status_t launch_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha = T(1),
                           T beta = T(0), cudaStream_t st = nullptr) {
     if (A->n == 0) return SPMV_OK;
-    if (use_thin(A, sizeof(T) == 4, AXPBY))
-        return go_thin<T, AXPBY>(A, val, x, y, alpha, beta, st);
     if constexpr (sizeof(T) == 8) {
-        switch (A->S) {
-            case 32: return go_sell<T, 1, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
-            case 64: return go_sell<T, 2, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
-            case 128: return go_sell<T, 4, 32, 2, AXPBY>(A, val, x, y, alpha, beta, st);
-            case 256: return go_sell<T, 8, 32, 1, AXPBY>(A, val, x, y, alpha, beta, st);
-        }
-    } else {
-        switch (A->S) {
-            case 32: return go_sell<T, 4, 8, 4, AXPBY>(A, val, x, y, alpha, beta, st);
-            // five entries in flight per row: a whole row of the tetrahedral meshes in one
-            // round of loads (measured 41.0 -> 38.9 us at S = 64 on the 6M-row mesh)
-            case 64: return go_sell<T, 4, 16, 5, AXPBY>(A, val, x, y, alpha, beta, st);
-            case 128: return go_sell<T, 4, 32, 5, AXPBY>(A, val, x, y, alpha, beta, st);
-            case 256: return go_sell<T, 8, 32, 2, AXPBY>(A, val, x, y, alpha, beta, st);
+        if (!use_thin(A)) {
+            switch (A->S) {
+                case 32: return go_sell<T, 1, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
+                case 64: return go_sell<T, 2, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
+                case 128: return go_sell<T, 4, 32, 2, AXPBY>(A, val, x, y, alpha, beta, st);
+                case 256: return go_sell<T, 8, 32, 1, AXPBY>(A, val, x, y, alpha, beta, st);
+            }
+            return SPMV_ERR_INVALID_ARG;
         }
     }
-    return SPMV_ERR_INVALID_ARG;
+    return go_thin<T, AXPBY>(A, val, x, y, alpha, beta, st);
 }
 
 }  // namespace

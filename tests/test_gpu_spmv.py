@@ -559,15 +559,21 @@ def test_small_products_every_row_remainder(oracle, n, max_len, bits, S):
                                                              -0.25, y0))
 
 
-@pytest.mark.parametrize("rows", [64 * 1024, 64 * 1024 + 1, 256 * 1024, 256 * 1024 + 1, 512 * 1024,
-                                  512 * 1024 + 1, 1500000, 1500001, 2000000, 2000001])
-def test_product_kernels_agree_at_the_edges_of_their_ranges(rows):
-    """Products on both sides of each row count where another kernel is chosen, equal bit for bit
-    to the thread-per-row CSR kernel's (FP64) and to a mirrored matrix of another slice height."""
+@pytest.mark.parametrize("width,rows", [
+    (2, 1000), (2, 311000), (2, 311400), (2, 466000), (2, 467000), (2, 622000), (2, 623000),
+    (6, 1000), (6, 155000), (6, 156000), (6, 233000), (6, 234000), (6, 262144), (6, 262145),
+    (6, 311000), (6, 312000), (6, 622000), (6, 623000), (6, 1000000), (6, 1000001),
+    (6, 3500000), (6, 3500001), (9, 1000), (9, 194000), (9, 195000), (9, 311000), (9, 312000),
+    (9, 466000), (9, 467000), (9, 2000000), (9, 2000001)])
+def test_product_kernels_agree_at_the_edges_of_their_ranges(width, rows):
+    """Products on both sides of each row count where another kernel is chosen, for rows of up to
+    two, six and nine entries, equal bit for bit to the thread-per-row CSR kernel's (FP64) and to
+    mirrored matrices of other slice heights; with a span of over 65,535 columns the same."""
     i = np.arange(rows, dtype=np.int64)
-    offs = np.array([-777, -1, 0, 1, 777, 1201])
-    j = i[:, None] + offs[None, :]
-    keep = (j >= 0) & (j < rows) & ((np.arange(6)[None, :] < 5) | (i[:, None] % 3 == 0))
+    offs = np.array([0, 70001, -1, 1, -777, 777, 1201, -29, 29])[:width]
+    j = np.sort((i[:, None] + offs[None, :]) % rows if rows > 80000
+                else (i[:, None] + offs[None, :] % 512) % rows, axis=1)
+    keep = (np.diff(j, axis=1, prepend=-1) > 0) & ((np.arange(width) < 8) | (i[:, None] % 3 == 0))
     rp = np.zeros(rows + 1, np.int64)
     np.cumsum(keep.sum(1), out=rp[1:])
     ci = j[keep].astype(np.int32)
@@ -585,18 +591,22 @@ def test_product_kernels_agree_at_the_edges_of_their_ranges(rows):
         y32.append(z)
         w = torch.empty_like(x)
         A.apply_csr(x, w)
+        u, u32 = x.clone(), x.float()
+        A.apply_axpby(1.0, x, 1.0, u)
+        A.apply_axpby(1.0, x.float(), 1.0, u32)
         torch.cuda.synchronize()
         assert torch.equal(y, w)
+        assert torch.equal(u, y + x) and torch.equal(u32, z + x.float())
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
     assert torch.equal(y32[0], y32[1]) and torch.equal(y32[0], y32[2])
 
 
 @pytest.mark.parametrize("rows,per_row", [(33, 3), (5003, 4), (300000, 5), (1000003, 6),
-                                          (2000000, 5), (2000001, 5)])
+                                          (3500000, 5), (3500001, 5)])
 def test_products_that_wait_for_one_another(rows, per_row):
-    """Products in a row on one stream, each the next one's input (dependent launches up to 2M
-    rows), with a copy, another stream's product and other kernels between them; then the same
-    captured in a graph.  Equal bit for bit to the CSR kernel with a synchronisation after each."""
+    """Products in a row on one stream, each the next one's input (dependent launches, and plain
+    ones above 3.5M rows), with a copy, another stream's product and other kernels between them;
+    then the same captured in a graph.  Equal bit for bit to the CSR kernel with a synchronisation after each."""
     i = np.arange(rows, dtype=np.int64)
     j = (i[:, None] + np.array([0, 1, -1, 29, -29, 777])[None, :per_row]) % rows
     rp = np.arange(rows + 1, dtype=np.int64) * per_row
