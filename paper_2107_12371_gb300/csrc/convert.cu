@@ -52,7 +52,7 @@ __global__ void validate_csr(int32_t n, int32_t n_cols, int64_t nnz, const int32
 }
 
 // ---------------------------------------------------------------------------------------
-// Cuthill-McKee on the device.  A node's key is (degree, index); pos[v] = -1 until placed.
+// Cuthill-McKee on the device.  A node's key is (degree, index).
 // ---------------------------------------------------------------------------------------
 __global__ void degree_kernel(int32_t n, const int32_t *rp, const int32_t *ci, int32_t *deg) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -73,11 +73,29 @@ __device__ __forceinline__ int32_t ld_l2(const int32_t *p) {
     return v;
 }
 
+// *p = max(*p, x) if `on`: the value before, else x
+__device__ __forceinline__ int32_t max_if(bool on, int32_t *p, int32_t x) {
+    int32_t v = x;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t"
+                 "@q atom.global.max.s32 %0, [%1], %2;\n\t}"
+                 : "+r"(v) : "l"(p), "r"(x), "r"((int)on) : "memory");
+    return v;
+}
+// *p += 1 if `on`, in the shared memory of any CTA of the cluster: the value before, else 0
+__device__ __forceinline__ int32_t count_if(bool on, int *p) {
+    int32_t v = 0;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t"
+                 "@q atom.add.s32 %0, [%1], 1;\n\t}"
+                 : "+r"(v) : "l"(p), "r"((int)on) : "memory");
+    return v;
+}
+
 constexpr int kCmCluster = 16;
 constexpr int kCmThreads = 1024;  // at most; see cm_order_device
-constexpr int kCmPlaced = -2;   // stamp of a node that has its position
+constexpr int kCmPlaced = INT_MAX;  // stamp of a node that has its position
 constexpr int kCmBatch = 6;     // row entries in flight per thread
 constexpr int kCmComponents = 256;  // components that one launch orders
+constexpr int kCmQueue = 4096;  // frontier nodes that a CTA keeps in shared memory
 constexpr int kCmKids = 8;      // children of a node sorted in registers; more are selected one by one
 
 // Smallest key that each CTA of the cluster found, in every CTA; two sets in turn, so that one can
@@ -87,15 +105,24 @@ struct CmKeys {
     unsigned long long warp[kCmThreads / 32];
 };
 
+// A CTA's part of the frontier, one for the level that is read and one for the next, which the
+// other CTAs write too.
+struct CmFrontier {
+    int32_t node[2][kCmQueue];
+    // nodes that a BFS level has sent to this CTA: three words in turn, the next one cleared a level
+    // ahead, when every CTA has passed the barrier after the last one read it
+    int count[3];
+    int full[3];  // whether a CTA's part was full, likewise
+};
+
 // What the CTAs of the cluster keep in step (every thread of every CTA holds the same values).
 struct CmWalk {
     int32_t n;
     const int32_t *rp, *ci, *deg;
-    int32_t *pos, *claim, *stamp, *queue, *perm;
-    // nodes that a BFS level appends: three words in turn, the next one cleared a level ahead,
-    // when every CTA has passed the barrier after the last CTA read it
-    int32_t *grown;
+    int32_t *claim, *stamp, *queue, *perm;
+    int32_t *spilled;  // BFS nodes in `queue`, those that found their CTA's frontier full
     CmKeys *keys;
+    CmFrontier *front;
     cg::cluster_group cluster;
     int64_t gid, threads;  // threads are numbered across the CTAs: small levels use every SM
     int searches, levels;  // uses of the words above so far
@@ -110,18 +137,14 @@ struct CmWalk {
             if (v[j] == u) v[j] = -1;
     }
 
-    // smallest key over the nodes f(i), i in [0, count); f returns a node or -1
-    template <typename F>
-    __device__ __forceinline__ unsigned long long min_key(int64_t count, F &&f) {
+    __device__ __forceinline__ void take_min(unsigned long long &best, int32_t v) const {
+        const unsigned long long k = node_key(deg, v);
+        best = k < best ? k : best;
+    }
+
+    // smallest of the threads' keys
+    __device__ __forceinline__ unsigned long long min_key(unsigned long long best) {
         const int w = searches++ & 1, ranks = (int)cluster.num_blocks();
-        unsigned long long best = ~0ull;
-        for (int64_t i = gid; i < count; i += threads) {
-            const int32_t v = f(i);
-            if (v >= 0) {
-                const unsigned long long k = node_key(deg, v);
-                best = k < best ? k : best;
-            }
-        }
         auto warp_min = [&] {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -145,61 +168,100 @@ struct CmWalk {
     }
 
     // BFS levels from r over nodes without a position: the number of levels, and the node of
-    // the last one with the smallest key
+    // the last one with the smallest key.  Ids grow, and a stamp only grows, so that one atomicMax
+    // tells whether a node is new; it then goes to the CTA that its index hashes to.
     __device__ __forceinline__ void bfs(int32_t r, int32_t id, int32_t *ecc, int32_t *pick) {
-        if (gid == 0) {
-            stamp[r] = id;
-            queue[0] = r;
+        const int ranks = (int)cluster.num_blocks(), lane = threadIdx.x & 31;
+        const int shift = ranks == 16 ? 28 : 29;
+        int mine = 0;  // nodes of the level in this CTA's frontier
+        if (cluster.block_rank() == 0) {
+            mine = 1;
+            if (threadIdx.x == 0) {
+                stamp[r] = id;
+                front->node[levels & 1][0] = r;
+            }
         }
         cluster.sync();
-        int64_t ls = 0, le = 1;
+        int32_t ls = 0, le = 0;  // the level's nodes in `queue`
         int32_t depth = 0;
-        for (;;) {
-            const int w = levels++ % 3;
-            for (int64_t i = ls + gid; i < le; i += threads) {
-                const int32_t u = ld_l2(queue + i);
-                const int32_t b = rp[u + 1];
-                for (int32_t k = rp[u]; k < b; k += kCmBatch) {
-                    int32_t v[kCmBatch];
-                    bool fresh[kCmBatch];
-                    load_row(u, k, b, v);
+        auto owner = [&](int32_t v) {
+            return cluster.map_shared_rank(front, (uint32_t)v * 2654435761u >> shift);
+        };
+        auto visit = [&](int32_t u, int w) {
+            const int32_t b = rp[u + 1];
+            for (int32_t k = rp[u]; k < b; k += kCmBatch) {
+                int32_t v[kCmBatch], slot[kCmBatch];
+                load_row(u, k, b, v);
+                // (results are looked at after all of a kind have been requested: an atomic whose
+                // result decides a branch waits for it, 1,000 clocks each)
+                int32_t was[kCmBatch];
 #pragma unroll
-                    for (int j = 0; j < kCmBatch; ++j) {
-                        const int32_t st = v[j] >= 0 ? ld_l2(stamp + v[j]) : id;
-                        fresh[j] = st != id && st != kCmPlaced;
+                for (int j = 0; j < kCmBatch; ++j) was[j] = max_if(v[j] >= 0, stamp + v[j], id);
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j)
+                    if (was[j] >= id) v[j] = -1;
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j)
+                    slot[j] = count_if(v[j] >= 0, &owner(v[j])->count[w]);
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j) {
+                    if (v[j] < 0) continue;
+                    if (slot[j] < kCmQueue) {
+                        owner(v[j])->node[~levels & 1][slot[j]] = v[j];
+                    } else {
+                        queue[atomicAdd(spilled, 1)] = v[j];
+                        for (int r = 0; r < ranks; ++r)
+                            cluster.map_shared_rank(front, r)->full[w] = 1;
                     }
-                    int cnt = 0;
-#pragma unroll
-                    for (int j = 0; j < kCmBatch; ++j)
-                        if (fresh[j]) fresh[j] = atomicExch(&stamp[v[j]], id) != id;
-#pragma unroll
-                    for (int j = 0; j < kCmBatch; ++j) cnt += fresh[j];
-                    if (cnt == 0) continue;
-                    int64_t at = le + atomicAdd(&grown[w], cnt);
-#pragma unroll
-                    for (int j = 0; j < kCmBatch; ++j)
-                        if (fresh[j]) queue[at++] = v[j];
                 }
             }
-            if (gid == 0) grown[levels % 3] = 0;
+        };
+        int last = 0;  // the same of the level before
+        int32_t last_ls = 0;
+        for (bool first = true;; first = false) {
+            const int w = levels % 3;
+            // whether the level has any nodes is needed only once it has been visited
+            const int sent = first ? 1
+                             : lane < ranks
+                                 ? cluster.map_shared_rank(front, lane)->count[(levels + 2) % 3]
+                                 : 0;
+            const int share = mine + (le - ls + ranks - 1 - (int)cluster.block_rank()) / ranks;
+            for (int i = threadIdx.x; i < share; i += blockDim.x)
+                visit(i < mine ? front->node[levels & 1][i]
+                               : ld_l2(queue + ls + (i - mine) * ranks + cluster.block_rank()),
+                      w);
+            if (threadIdx.x == 0) front->count[(levels + 1) % 3] = front->full[(levels + 1) % 3] = 0;
             cluster.sync();
-            const int more = ld_l2(grown + w);
-            if (more == 0) break;
-            ++depth;
+            if (!__any_sync(0xffffffffu, sent > 0)) break;
+            last = mine;
+            last_ls = ls;
+            const int own = front->count[w];
+            mine = own < kCmQueue ? own : kCmQueue;
             ls = le;
-            le += more;
+            if (front->full[w]) {
+                const int all = lane < ranks ? cluster.map_shared_rank(front, lane)->count[w] : 0;
+                le += __reduce_add_sync(0xffffffffu, all > kCmQueue ? all - kCmQueue : 0);
+            }
+            ++depth;
+            ++levels;
         }
-        const int32_t *q = queue + ls;
-        const unsigned long long k = min_key(le - ls, [&](int64_t i) { return ld_l2(q + i); });
+        // the level after the last one was empty
+        unsigned long long best = ~0ull;
+        for (int i = threadIdx.x; i < last; i += blockDim.x)
+            take_min(best, front->node[~levels & 1][i]);
+        for (int64_t i = last_ls + gid; i < ls; i += threads) take_min(best, ld_l2(queue + i));
+        --depth;
+        ++levels;
+        if (gid == 0) *spilled = 0;
         *ecc = depth;
-        *pick = (int32_t)(k & 0xffffffffull);
+        *pick = (int32_t)(min_key(best) & 0xffffffffull);
     }
 };
 
-// Children of frontier position p (the unplaced neighbours of u = perm[p] that no earlier
-// position claimed): their number, and the first kCmKids keys, sorted.
-__device__ __forceinline__ int cm_kids(const CmWalk &w, int64_t p, int32_t u,
-                                       unsigned long long (&key)[kCmKids]) {
+// Children of frontier position p (the neighbours of its node u that no earlier position claimed):
+// their number, and the first kCmKids keys, sorted.
+__device__ __noinline__ int cm_kids(const CmWalk &w, int32_t p, int32_t u,
+                                    unsigned long long (&key)[kCmKids]) {
 #pragma unroll
     for (int j = 0; j < kCmKids; ++j) key[j] = ~0ull;
     int cnt = 0;
@@ -214,7 +276,7 @@ __device__ __forceinline__ int cm_kids(const CmWalk &w, int64_t p, int32_t u,
         }
 #pragma unroll
         for (int i = 0; i < kCmBatch; ++i) {
-            if (c[i] != (int32_t)p) continue;
+            if (c[i] != p) continue;
             // insertion into the sorted list (a full list keeps the smallest)
             unsigned long long x = (unsigned long long)(uint32_t)d[i] << 32 | (uint32_t)v[i];
 #pragma unroll
@@ -229,20 +291,44 @@ __device__ __forceinline__ int cm_kids(const CmWalk &w, int64_t p, int32_t u,
     return cnt;
 }
 
-__device__ __forceinline__ void cm_set(const CmWalk &w, int64_t at, int32_t v) {
-    w.perm[at] = v;
-    w.pos[v] = (int32_t)at;
-    w.stamp[v] = kCmPlaced;
-}
+// The next level of the order: its first position, how many nodes each CTA takes, and where they
+// are kept (in shared memory if every CTA's fit).
+struct CmNext {
+    int32_t first, run;
+    int buf;
+};
+// Sets positions from `at` on, a few of them: position at + i is node i of `slot`.
+struct CmSet {
+    const CmWalk &w;
+    const CmNext &next;
+    int32_t at;
+    int to, slot;
+    __device__ __forceinline__ CmSet(const CmWalk &w_, const CmNext &next_, int32_t at_)
+        : w(w_), next(next_), at(at_) {
+        to = (at - next.first) / next.run;
+        slot = at - next.first - to * next.run;
+    }
+    __device__ __forceinline__ void set(int i, int32_t v) const {
+        w.perm[at + i] = v;
+        w.stamp[v] = kCmPlaced;
+        if (next.run > kCmQueue) return;
+        int t = to, k = slot + i;
+        while (k >= next.run) {
+            k -= next.run;
+            ++t;
+        }
+        w.cluster.map_shared_rank(w.front, t)->node[next.buf][k] = v;
+    }
+};
 
 // Places the children of position p from position `at` on, in increasing (degree, index).
-__device__ __forceinline__ void cm_place_kids(const CmWalk &w, int64_t p, int32_t u, int cnt,
-                                              const unsigned long long (&key)[kCmKids],
-                                              int64_t at) {
+__device__ __forceinline__ void cm_place_kids(const CmWalk &w, const CmSet &set, int32_t p,
+                                              int32_t u, int cnt,
+                                              const unsigned long long (&key)[kCmKids]) {
     if (cnt <= kCmKids) {
 #pragma unroll
         for (int j = 0; j < kCmKids; ++j)
-            if (j < cnt) cm_set(w, at + j, (int32_t)(key[j] & 0xffffffffull));
+            if (j < cnt) set.set(j, (int32_t)(key[j] & 0xffffffffull));
         return;
     }
     // any number: repeated selection of the next larger key
@@ -251,11 +337,11 @@ __device__ __forceinline__ void cm_place_kids(const CmWalk &w, int64_t p, int32_
         unsigned long long best = ~0ull;
         for (int32_t k = w.rp[u]; k < w.rp[u + 1]; ++k) {
             const int32_t v = w.ci[k];
-            if (v == u || ld_l2(w.claim + v) != (int32_t)p) continue;
+            if (v == u || ld_l2(w.claim + v) != p) continue;
             const unsigned long long x = node_key(w.deg, v);
             if ((t == 0 || x > last) && x < best) best = x;
         }
-        cm_set(w, at + t, (int32_t)(best & 0xffffffffull));
+        set.set(t, (int32_t)(best & 0xffffffffull));
         last = best;
     }
 }
@@ -264,36 +350,43 @@ __device__ __forceinline__ void cm_place_kids(const CmWalk &w, int64_t p, int32_
 // launch is short whatever the graph), in one thread-block cluster: the levels of a mesh are
 // a few thousand nodes in some hundred steps, so what a level costs is its chain of dependent
 // loads and its barriers.  A cluster barrier is a hardware one, and nothing returns to the host
-// between levels.  Measured for a mesh of 796K cells (1,038 BFS levels of the start-node search,
-// 353 of the order): 42 -> 8.8 ms against a few kernels and a read-back per level; 48K cells 15.8
-// -> 2.8 ms, 6M about 115 -> 36 ms.  With the frontier spread over all CTAs a level of the
-// search takes 6 us and one of the order 8 us.
+// between levels.  The frontier lies in the CTAs' shared memory, spread over all of them, and is
+// written there by whichever CTA finds a node; a search's step is then row bounds, row, one
+// atomic per neighbour, a slot in the finder's choice of CTA and the barrier: 800 + 600 + 1,130 +
+// 700 + 1,700 of its 6,600 clocks (3.3 us; 6 with the frontier in global memory, a look at each
+// stamp before the atomic, and atomics that waited for one another).  A level of the order takes
+// 5.9 us.  Whole set-up of 796K cells (1,038 levels of the start-node search, 353 of the order)
+// 9.7 -> 6.4 ms, 48K 3.1 -> 2.2, 192K mixed 4.6 -> 3.7, 6M 40.6 -> 32.0.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
-cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, int32_t *pos,
-           int32_t *claim, int32_t *stamp, int32_t *queue, int32_t *perm, int peripheral,
-           int max_components, int64_t *placed_io, int32_t *bfs_id_io, int32_t *grown) {
+cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, int32_t *claim,
+           int32_t *stamp, int32_t *queue, int32_t *perm, int peripheral, int max_components,
+           int64_t *placed_io, int32_t *bfs_id_io, int32_t *spilled) {
     __shared__ CmKeys keys;
+    __shared__ CmFrontier front;
     __shared__ int totals[2][kCmCluster];
     __shared__ int warp_sums[THREADS / 32];
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (rank == 0 && threadIdx.x < 3) grown[threadIdx.x] = 0;
-    CmWalk w{n, rp, ci, deg, pos, claim, stamp, queue, perm, grown, &keys, cluster,
+    if (threadIdx.x < 3) front.count[threadIdx.x] = front.full[threadIdx.x] = 0;
+    CmWalk w{n, rp, ci, deg, claim, stamp, queue, perm, spilled, &keys, &front, cluster,
              (int64_t)threadIdx.x * ranks + rank, (int64_t)ranks * THREADS, 0, 0};
-    int64_t placed = *placed_io;
+    int32_t placed = (int32_t)*placed_io;
     int32_t bfs_id = *bfs_id_io;
+    const int log_ranks = ranks == 16 ? 4 : 3;
+    if (w.gid == 0) *spilled = 0;
     int turn = 0;
     cluster.sync();
     for (int comp = 0; comp < max_components && placed < n; ++comp) {
-        int32_t start = (int32_t)(w.min_key(n, [&](int64_t i) {
-                                      return ld_l2(pos + i) == -1 ? (int32_t)i : -1;
-                                  }) & 0xffffffffull);
+        // a node without a position is one that nothing has claimed
+        unsigned long long best = ~0ull;
+        for (int64_t i = w.gid; i < n; i += w.threads)
+            if (ld_l2(claim + i) == INT_MAX) w.take_min(best, (int32_t)i);
+        int32_t start = (int32_t)(w.min_key(best) & 0xffffffffull);
         if (peripheral) {
-            int32_t ecc, pick;
-            w.bfs(start, bfs_id++, &ecc, &pick);
-            for (int moves = 0; moves < 8; ++moves) {
+            int32_t ecc = -1, pick = start;
+            for (int searches = 0; searches <= 8; ++searches) {
                 int32_t ecc2, pick2;
                 w.bfs(pick, bfs_id++, &ecc2, &pick2);
                 if (ecc2 <= ecc) break;
@@ -302,40 +395,61 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
                 pick = pick2;
             }
         }
-        if (w.gid == 0) cm_set(w, placed, start);
+        if (w.gid == 0) {
+            claim[start] = -1;
+            CmSet(w, CmNext{placed, 1, 0}, placed).set(0, start);
+        }
         cluster.sync();
-        int64_t ls = placed, le = placed + 1;
+        int32_t ls = placed, le = placed + 1;
+        int buf = 0;
         while (le > ls) {
             // the CTAs take equal runs of the frontier, their threads `m` consecutive positions
             // each, so that the children's order is that of a scan over CTAs and threads
-            const int64_t run = (le - ls + ranks - 1) / ranks;
-            const int64_t m = (run + THREADS - 1) / THREADS;
-            const int64_t r1 = ls + (rank + 1) * run < le ? ls + (rank + 1) * run : le;
-            const int64_t p0 = ls + rank * run + threadIdx.x * m;
-            const int64_t p1 = p0 + m < r1 ? p0 + m : r1;
-            // every unplaced neighbour of a frontier node records the earliest position
-            for (int64_t p = p0; p < p1; ++p) {
-                const int32_t u = ld_l2(perm + p);
+            const int32_t run = ((le - ls - 1) >> log_ranks) + 1;
+            const int32_t m = (run + THREADS - 1) / THREADS;
+            // counted from ls (positions up to n + kCmCluster THREADS would overflow)
+            const int32_t size = le - ls, r1 = (rank + 1) * run < size ? (rank + 1) * run : size;
+            const int32_t q0 = rank * run + (int)threadIdx.x * m;
+            const int32_t p0 = ls + (q0 < r1 ? q0 : r1), p1 = ls + (q0 + m < r1 ? q0 + m : r1);
+            const int32_t r0 = ls + rank * run;
+            auto node = [&](int32_t p) {
+                return run <= kCmQueue ? front.node[buf][p - r0] : ld_l2(perm + p);
+            };
+            // every neighbour of a frontier node records the earliest position; one that has its
+            // own keeps the smaller claim of its parent
+            int32_t u = -1, v[kCmBatch], d[kCmBatch];
+            bool one = p1 - p0 == 1;  // one position, and a row that v holds
+            for (int32_t p = p0; p < p1; ++p) {
+                u = node(p);
                 const int32_t b = rp[u + 1];
                 for (int32_t k = rp[u]; k < b; k += kCmBatch) {
-                    int32_t v[kCmBatch];
                     w.load_row(u, k, b, v);
 #pragma unroll
                     for (int j = 0; j < kCmBatch; ++j)
-                        if (v[j] >= 0 && ld_l2(pos + v[j]) != -1) v[j] = -1;
-#pragma unroll
-                    for (int j = 0; j < kCmBatch; ++j)
-                        if (v[j] >= 0) atomicMin(&claim[v[j]], (int32_t)p);
+                        if (v[j] >= 0) atomicMin(&claim[v[j]], p);
+                    one = one && b - k <= kCmBatch;
                 }
+                one = one && rp[u] < b;
+            }
+            if (one) {
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j) d[j] = v[j] >= 0 ? deg[v[j]] : 0;
             }
             cluster.sync();
             // children per thread, their scan over the cluster
-            unsigned long long key[kCmKids];
-            int32_t u = -1;
             int mine = 0;
-            for (int64_t p = p0; p < p1; ++p) {
-                u = ld_l2(perm + p);
-                mine += cm_kids(w, p, u, key);
+            unsigned long long key[kCmKids];
+            if (one) {
+                int32_t c[kCmBatch];
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j) c[j] = v[j] >= 0 ? ld_l2(claim + v[j]) : -1;
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j) {
+                    if (c[j] != p0) v[j] = -1;
+                    else ++mine;
+                }
+            } else {
+                for (int32_t p = p0; p < p1; ++p) mine += cm_kids(w, p, node(p), key);
             }
             int incl = mine;
 #pragma unroll
@@ -356,23 +470,35 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
             if ((int)threadIdx.x < ranks)
                 *cluster.map_shared_rank(&totals[turn][rank], threadIdx.x) = all;
             cluster.sync();
-            int64_t at = le + before + incl - mine, total = 0;
+            int32_t at = le + before + incl - mine, total = 0;
             for (int r = 0; r < ranks; ++r) {
                 const int x = totals[turn][r];
                 if (r < rank) at += x;
                 total += x;
             }
-            if (m == 1) {
-                if (mine) cm_place_kids(w, p0, u, mine, key, at);
-            } else {
-                for (int64_t p = p0; p < p1; ++p) {
-                    u = ld_l2(perm + p);
-                    const int cnt = cm_kids(w, p, u, key);
-                    cm_place_kids(w, p, u, cnt, key, at);
+            const CmNext next{le, ((total - 1) >> log_ranks) + 1, buf ^ 1};
+            if (one && mine) {
+                const CmSet set(w, next, at);
+                // a child's place: how many siblings have a smaller key
+#pragma unroll
+                for (int j = 0; j < kCmBatch; ++j) {
+                    if (v[j] < 0) continue;
+                    int rank_of = 0;
+#pragma unroll
+                    for (int i = 0; i < kCmBatch; ++i)
+                        rank_of += v[i] >= 0 && (d[i] < d[j] || (d[i] == d[j] && v[i] < v[j]));
+                    set.set(rank_of, v[j]);
+                }
+            } else if (mine) {
+                for (int32_t p = p0; p < p1; ++p) {
+                    const int32_t x = node(p);
+                    const int cnt = p1 - p0 == 1 ? mine : cm_kids(w, p, x, key);
+                    if (cnt) cm_place_kids(w, CmSet(w, next, at), p, x, cnt, key);
                     at += cnt;
                 }
             }
             cluster.sync();
+            buf ^= 1;
             ls = le;
             le += total;
         }
@@ -398,25 +524,24 @@ __global__ void fill_i32(int32_t *p, int64_t n, int32_t v) {
 spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, bool reverse,
                               bool peripheral, int32_t *perm_out, cudaStream_t st) {
     if (n == 0) return SPMV_OK;
-    // six arrays of n words, then the progress words
+    // five arrays of n words, then the progress words
     int32_t *mem = nullptr;
     const size_t stride = ((size_t)n + 63) / 64 * 64;
-    GB_CUDA(gb_malloc_async((void **)&mem, sizeof(int32_t) * (6 * stride + 8), st));
-    int32_t *deg = mem, *pos = mem + stride, *claim = mem + 2 * stride, *stamp = mem + 3 * stride,
-            *queue = mem + 4 * stride, *cm = mem + 5 * stride;
-    int64_t *placed_d = (int64_t *)(mem + 6 * stride);
-    int32_t *bfs_id_d = mem + 6 * stride + 2, *grown_d = mem + 6 * stride + 3;
+    GB_CUDA(gb_malloc_async((void **)&mem, sizeof(int32_t) * (5 * stride + 8), st));
+    int32_t *deg = mem, *claim = mem + stride, *stamp = mem + 2 * stride,
+            *queue = mem + 3 * stride, *cm = mem + 4 * stride;
+    int64_t *placed_d = (int64_t *)(mem + 5 * stride);
+    int32_t *bfs_id_d = mem + 5 * stride + 2, *spilled_d = mem + 5 * stride + 3;
     spmv_status_t s = [&]() -> spmv_status_t {
         const unsigned nb = blocks_for(n);
         degree_kernel<<<nb, kT, 0, st>>>(n, rp, ci, deg);
-        fill_i32<<<nb, kT, 0, st>>>(pos, n, -1);
         fill_i32<<<nb, kT, 0, st>>>(claim, n, INT_MAX);
         fill_i32<<<nb, kT, 0, st>>>(stamp, n, -1);
         GB_LAUNCHED();
         GB_CUDA(cudaMemsetAsync(placed_d, 0, 4 * sizeof(int32_t), st));
         // 512 threads per CTA leave registers for a row's loads in flight; the frontiers of
         // larger graphs (about 10K nodes from 1.5M on) keep 1,024 busy.  Whole set-up, ms, 512 /
-        // 1,024: 48K cells 3.1 / 3.4, 796K 9.7 / 10.3, 3.1M 23.5 / 21.9, 6M 43.0 / 40.4.
+        // 1,024: 48K cells 2.2 / 3.1, 796K 6.6 / 8.5, 3.1M 18.5 / 17.8, 6M 34.4 / 33.7.
         const bool wide = n >= 1500000;
         auto *kern = wide ? cm_cluster<1024> : cm_cluster<512>;
         GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -438,9 +563,9 @@ spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, b
         }
         int64_t placed = 0;
         while (placed < n) {
-            GB_CUDA(cudaLaunchKernelEx(&cfg, kern, n, rp, ci, (const int32_t *)deg, pos,
+            GB_CUDA(cudaLaunchKernelEx(&cfg, kern, n, rp, ci, (const int32_t *)deg,
                                        claim, stamp, queue, cm, peripheral ? 1 : 0,
-                                       kCmComponents, placed_d, bfs_id_d, grown_d));
+                                       kCmComponents, placed_d, bfs_id_d, spilled_d));
             GB_CUDA(cudaMemcpyAsync(&placed, placed_d, sizeof(int64_t), cudaMemcpyDeviceToHost,
                                     st));
             GB_CUDA(cudaStreamSynchronize(st));

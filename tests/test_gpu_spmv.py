@@ -438,11 +438,21 @@ def ordering_graph(kind):
     if kind == "broad":          # levels wider than the cluster has threads
         n = 60000
         return graph_csr(n, [(k, (k - 1) // 300) for k in range(1, n)])
+    if kind == "flood":          # a level of 90,000 nodes: more than the shared frontiers hold
+        n = 150000
+        return graph_csr(n, [(k, (k - 1) // 300) for k in range(1, n)])
+    if kind == "one_way":        # no symmetric pattern: searches meet nodes that have their place
+        n = 4000
+        cols = [np.unique(np.append(rng.integers(0, n, k % 4), k)) for k in range(n)]
+        rp = np.zeros(n + 1, np.int32)
+        rp[1:] = np.cumsum([c.size for c in cols])
+        return rp, np.concatenate(cols).astype(np.int32), np.ones(rp[-1])
     n = 5000                     # random sparse graph, several components
     return graph_csr(n, rng.integers(0, n, (2 * n // 3, 2)))
 
 
-@pytest.mark.parametrize("kind", ["isolated", "paths", "star", "wheel", "broad", "random"])
+@pytest.mark.parametrize("kind", ["isolated", "paths", "star", "wheel", "broad", "flood",
+                                  "one_way", "random"])
 @pytest.mark.parametrize("peripheral", [0, 1])
 def test_gpu_cm_order_of_unusual_graphs(oracle, kind, peripheral):
     rp, ci, v = ordering_graph(kind)
