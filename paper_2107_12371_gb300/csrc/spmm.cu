@@ -17,6 +17,14 @@ inline unsigned grid_for(int64_t threads, int block) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
+// Threads of a CTA, but for spmm_sell_wide_gs.  A CTA ends with its longest rows, so small ones
+// give their place up sooner: k = 28 in FP64 on 312K mixed-mesh rows 193.8 us at 256, 182.8 at
+// 128, 180.2 at 64 (on 304K tetrahedra 135, 127 and 155).  All kernels are dependent launches:
+// those that hold a round of matrix entries before their first gather request it while the
+// kernel before still runs (us, before -> now, with 128 threads: f32 k = 5 on 312K mixed rows
+// 16.5 -> 13.4, 47K 7.2 -> 4.3; f64 k = 32 on 192K 72.5 -> 69.5).
+constexpr int kRowsBlock = 128;
+
 // SpMM: G lanes per row (G divides 32, so the RPW = 32 / G rows of a warp lie in one slice and
 // share its width), lane g owns columns g, g + G, ... (C of them).  The lanes of a row first
 // load G of its (value, column) pairs at once, one per lane; the pairs are then broadcast
@@ -34,6 +42,8 @@ spmm_sell(int32_t n, int32_t S, int32_t n_slices, int k, const int64_t *__restri
     const int sub = lane / G, g = lane % G;
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t row0 = gw * RPW;
+    dep_wait();
+    dep_allow();
     if (row0 >= rows_total) return;  // whole warp: rows_total is a multiple of RPW
     const int64_t row = row0 + sub;
     const int64_t slice = row0 / S;
@@ -144,6 +154,8 @@ spmm_sell_vec(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict_
     const int sub = lane / G, g = lane % G;
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t row0 = gw * RPW;
+    dep_wait();
+    dep_allow();
     if (row0 >= rows_total) return;  // whole warp: rows_total is a multiple of RPW
     const int64_t row = row0 + sub;
     const int64_t slice = row0 / S;
@@ -274,9 +286,10 @@ __device__ __forceinline__ void st_cols(T *p, const T (&v)[P]) {
 // are identical.  The product is bound by the latency of its gathers: several pieces per lane
 // put more rows into a warp and more bytes in flight, which is why C is three to five for
 // narrow pieces; two or three entries in flight leave more warps room than five (f32 k = 5 on
-// 312K mixed-mesh rows: 14.4 us with three, 16.1 with five).  Measured there against a power
-// of two of lanes per row with the pairs broadcast by shuffles (spmm_sell): f32 k = 5 30.9 ->
-// 14.4 us, 6 31.2 -> 13.8, 11 54.5 -> 28.9, 20 105 -> 36, 31 108 -> 67; f64 k = 5 51.7 -> 37.3.
+// 312K mixed-mesh rows: three 12 % faster), and fewer registers for more warps cost more than they
+// gain (42 instead of 64: 13.6 -> 21 us).  Measured there against a power of two of lanes per row
+// with the pairs broadcast by shuffles (spmm_sell): f32 k = 5 30.9 -> 13.4 us, 6 31.2 -> 12.3,
+// 20 105 -> 33, 31 108 -> 69; f64 k = 5 51.7 -> 35.6.
 constexpr int piece_unroll(int bytes, int elem) {
     return bytes <= (elem == 4 ? 24 : 16) ? 3 : 2;
 }
@@ -320,7 +333,7 @@ inline int piece_choice(int k, int P, int elem) {
 }
 
 template <typename T, int P, int C, typename ColT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ sp, ColT cols,
                 const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
     constexpr int U = piece_unroll(P * C * (int)sizeof(T), (int)sizeof(T));
@@ -328,7 +341,10 @@ spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ 
     const int lane = threadIdx.x & 31;
     const int sub = lane / G, g = lane - sub * G;
     const int64_t row = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * rpw + sub;
-    if (sub >= rpw || row >= n) return;
+    if (sub >= rpw || row >= n) {
+        dep_wait();
+        return;
+    }
     // (w is set under a test that always holds here: with its value plain, the compiler knows the
     // first entry of each round exists and branches around the others' loads instead of
     // predicating them, and they no longer overlap: f32 k = 31 56 against 39 us)
@@ -364,6 +380,10 @@ spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ 
                 cols.template load<1>(at + (int64_t)(t0 + u) * S, 0, pol, cb, c[u]);
             }
         }
+        if (t0 == 0) {
+            dep_wait();
+            dep_allow();
+        }
         T xv[U][C][P];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -382,6 +402,7 @@ spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ 
                 for (int e = 0; e < P; ++e) acc[j][e] = fma_t(a[u][0], xv[u][j][e], acc[j][e]);
         }
     }
+    if (w == 0) dep_wait();
     T *yr = Y + row * k + g * P;
 #pragma unroll
     for (int j = 0; j < C; ++j)
@@ -408,6 +429,8 @@ spmm_sell_wide(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict
     const int sub = lane / G, g = lane % G;
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t row0 = gw * RPW;
+    dep_wait();
+    dep_allow();
     if (row0 >= rows_total) return;  // whole warp: rows_total is a multiple of RPW
     const int64_t row = row0 + sub;
     const int64_t slice = row0 / S;
@@ -474,6 +497,8 @@ spmm_sell_wide_pipe(int32_t n, int32_t S, int32_t n_slices, const int64_t *__res
     const int sub = lane / G, g = lane % G;
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t row0 = gw * RPW;
+    dep_wait();
+    dep_allow();
     if (row0 >= rows_total) return;  // whole warp: rows_total is a multiple of RPW
     const int64_t row = row0 + sub;
     const int64_t slice = row0 / S;
@@ -622,6 +647,8 @@ spmm_sell_wide_gs(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restr
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t nblocks = (rows_total + RB - 1) / RB;
     const uint64_t pol = policy_evict_first();
+    dep_wait();
+    dep_allow();
     for (int64_t blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
         const int64_t nxt = blk + gridDim.x;
         if (warp == 0 && nxt < nblocks)
@@ -688,6 +715,8 @@ spmm_sell_unrolled(int32_t n, int32_t S, int32_t n_slices, const int64_t *__rest
     const int sub = lane / G, g = lane % G;
     const int64_t rows_total = (int64_t)n_slices * S;
     const int64_t row0 = gw * RPW;
+    dep_wait();  // here, not behind the row's entries: there it costs large products 2 %
+    dep_allow();
     if (row0 >= rows_total) return;  // whole warp: rows_total is a multiple of RPW
     const int64_t row = row0 + sub;
     const int64_t slice = row0 / S;
@@ -788,7 +817,6 @@ template <typename T>
 spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y,
                           cudaStream_t st) {
     if (A->n == 0) return SPMV_OK;
-    const int block = 256;
     const int64_t rows_total = (int64_t)A->n_slices * A->S;
     // 256-bit kernel when k is a power-of-two multiple of 32 bytes and X, Y allow it
     constexpr int WV = Wide<T>::n;
@@ -797,34 +825,26 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
         constexpr int G = decltype(gtag)::value;
         constexpr int gi = G == 1 ? 0 : (G == 2 ? 1 : (G == 4 ? 2 : 3));
         const int64_t warps = (rows_total + (32 / G) - 1) / (32 / G);
-        const unsigned grid = grid_for(warps * 32, block);
+        const unsigned grid = grid_for(warps * 32, kRowsBlock);
         const int sms = device_facts().sm_count;
         const int form = spmm_form_of(A, sizeof(T) == 4, gi);
         auto go = [&](auto cols) -> spmv_status_t {
             using ColT = decltype(cols);
+            auto rows = [&](auto *kern) {
+                return launch_dependent(kern, grid, kRowsBlock, st, A->n, A->S, A->n_slices,
+                                        A->slice_ptr.p, cols, val, X, Y);
+            };
+            auto strided = [&](auto *kern, int per_sm) {  // rows per step fixed at 256 threads
+                return launch_dependent(kern, sms * per_sm, 256, st, A->n, A->S, A->n_slices,
+                                        A->slice_ptr.p, cols, val, X, Y);
+            };
             switch (form) {
-                case SPMV_SPMM_WIDE_PIPE:
-                    spmm_sell_wide_pipe<T, G, ColT><<<grid, block, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, X, Y);
-                    break;
-                case SPMV_SPMM_WIDE_GS4:
-                    spmm_sell_wide_gs<T, G, 4, ColT><<<sms * 4, block, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, X, Y);
-                    break;
-                case SPMV_SPMM_WIDE_GS6:
-                    spmm_sell_wide_gs<T, G, 6, ColT><<<sms * 6, block, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, X, Y);
-                    break;
-                case SPMV_SPMM_UNROLLED:
-                    spmm_sell_unrolled<T, G, 6, 10, ColT><<<grid, block, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, X, Y);
-                    break;
-                default:
-                    spmm_sell_wide<T, G, ColT><<<grid, block, 0, st>>>(
-                        A->n, A->S, A->n_slices, A->slice_ptr.p, cols, val, X, Y);
+                case SPMV_SPMM_WIDE_PIPE: return rows(spmm_sell_wide_pipe<T, G, ColT>);
+                case SPMV_SPMM_WIDE_GS4: return strided(spmm_sell_wide_gs<T, G, 4, ColT>, 4);
+                case SPMV_SPMM_WIDE_GS6: return strided(spmm_sell_wide_gs<T, G, 6, ColT>, 6);
+                case SPMV_SPMM_UNROLLED: return rows(spmm_sell_unrolled<T, G, 6, 10, ColT>);
+                default: return rows(spmm_sell_wide<T, G, ColT>);
             }
-            GB_LAUNCHED();
-            return SPMV_OK;
         };
         if (A->index_bits == 16) return go(Cols16{A->sell_col16.p, A->col_start.p});
         return go(Cols32{A->sell_col.p});
@@ -843,16 +863,13 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
     auto vec = [&](auto gtag) -> spmv_status_t {
         constexpr int G = decltype(gtag)::value;
         const int64_t warps = (rows_total + (32 / G) - 1) / (32 / G);
-        const unsigned grid = grid_for(warps * 32, block);
+        const unsigned grid = grid_for(warps * 32, kRowsBlock);
         if (A->index_bits == 16)
-            spmm_sell_vec<T, VW, G, Cols16><<<grid, block, 0, st>>>(
-                A->n, A->S, A->n_slices, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p},
-                val, X, Y);
-        else
-            spmm_sell_vec<T, VW, G, Cols32><<<grid, block, 0, st>>>(
-                A->n, A->S, A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
-        GB_LAUNCHED();
-        return SPMV_OK;
+            return launch_dependent(spmm_sell_vec<T, VW, G, Cols16>, grid, kRowsBlock, st, A->n,
+                                    A->S, A->n_slices, A->slice_ptr.p,
+                                    Cols16{A->sell_col16.p, A->col_start.p}, val, X, Y);
+        return launch_dependent(spmm_sell_vec<T, VW, G, Cols32>, grid, kRowsBlock, st, A->n, A->S,
+                                A->n_slices, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
     };
     using std::integral_constant;
     if constexpr (sizeof(T) == 4) {
@@ -871,17 +888,14 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
             constexpr int C = decltype(ctag)::value;
             const int G = (pieces + C - 1) / C;
             const int64_t warps = ((int64_t)A->n + 32 / G - 1) / (32 / G);
-            const unsigned grid = grid_for(warps * 32, block);
-            if (A->index_bits == 16)
-                spmm_sell_piece<T, P, C, Cols16><<<grid, block, 0, st>>>(
-                    A->n, A->S, k, G, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p}, val,
-                    X, Y);
-            else
-                spmm_sell_piece<T, P, C, Cols32><<<grid, block, 0, st>>>(
-                    A->n, A->S, k, G, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
+            const unsigned grid = grid_for(warps * 32, kRowsBlock);
             done = true;
-            GB_LAUNCHED();
-            return SPMV_OK;
+            if (A->index_bits == 16)
+                return launch_dependent(spmm_sell_piece<T, P, C, Cols16>, grid, kRowsBlock, st,
+                                        A->n, A->S, k, G, A->slice_ptr.p,
+                                        Cols16{A->sell_col16.p, A->col_start.p}, val, X, Y);
+            return launch_dependent(spmm_sell_piece<T, P, C, Cols32>, grid, kRowsBlock, st, A->n,
+                                    A->S, k, G, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
         };
         switch (piece_choice(k, P, (int)sizeof(T))) {
             case 1: return go(integral_constant<int, 1>{});
@@ -907,16 +921,13 @@ spmv_status_t launch_spmm(spmv_matrix_t A, int k, const T *val, const T *X, T *Y
         constexpr int G = decltype(gtag)::value;
         constexpr int C = decltype(ctag)::value;
         const int64_t warps = (rows_total + (32 / G) - 1) / (32 / G);
-        const unsigned grid = grid_for(warps * 32, block);
+        const unsigned grid = grid_for(warps * 32, kRowsBlock);
         if (A->index_bits == 16)
-            spmm_sell<T, G, C, Cols16><<<grid, block, 0, st>>>(
-                A->n, A->S, A->n_slices, k, A->slice_ptr.p, Cols16{A->sell_col16.p, A->col_start.p},
-                val, X, Y);
-        else
-            spmm_sell<T, G, C, Cols32><<<grid, block, 0, st>>>(
-                A->n, A->S, A->n_slices, k, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
-        GB_LAUNCHED();
-        return SPMV_OK;
+            return launch_dependent(spmm_sell<T, G, C, Cols16>, grid, kRowsBlock, st, A->n, A->S,
+                                    A->n_slices, k, A->slice_ptr.p,
+                                    Cols16{A->sell_col16.p, A->col_start.p}, val, X, Y);
+        return launch_dependent(spmm_sell<T, G, C, Cols32>, grid, kRowsBlock, st, A->n, A->S,
+                                A->n_slices, k, A->slice_ptr.p, Cols32{A->sell_col.p}, val, X, Y);
     };
     using I1 = std::integral_constant<int, 1>;
     if (k == 1) return go(I1{}, I1{});

@@ -614,9 +614,9 @@ def test_product_kernels_agree_at_the_edges_of_their_ranges(width, rows):
 @pytest.mark.parametrize("rows,per_row", [(33, 3), (5003, 4), (300000, 5), (1000003, 6),
                                           (3500000, 5), (3500001, 5)])
 def test_products_that_wait_for_one_another(rows, per_row):
-    """Products in a row on one stream, each the next one's input (dependent launches, and plain
-    ones above 3.5M rows), with a copy, another stream's product and other kernels between them;
-    then the same captured in a graph.  Equal bit for bit to the CSR kernel with a synchronisation after each."""
+    """Products in a row on one stream, each the next one's input (dependent launches), with a
+    copy, another stream's product and other kernels between them; then the same captured in a
+    graph.  Equal bit for bit to the CSR kernel with a synchronisation after each."""
     i = np.arange(rows, dtype=np.int64)
     j = (i[:, None] + np.array([0, 1, -1, 29, -29, 777])[None, :per_row]) % rows
     rp = np.arange(rows + 1, dtype=np.int64) * per_row
@@ -653,6 +653,30 @@ def test_products_that_wait_for_one_another(rows, per_row):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("dtype,k,form", [
+    (torch.float64, 1, 0), (torch.float64, 5, 0), (torch.float64, 7, 0), (torch.float32, 4, 0),
+    (torch.float32, 5, 0)] + [(torch.float32, 16, form) for form in range(6)])
+def test_spmm_products_that_wait_for_one_another(dtype, k, form):
+    """Multi-vector products in a row on one stream, each the next one's input, one for every
+    kernel: equal bit for bit to the same with a synchronisation after each."""
+    n = 20011
+    i = np.arange(n, dtype=np.int64)
+    j = np.sort((i[:, None] + np.array([0, 1, -1, 29, -777])[None, :]) % n, 1)
+    v = np.random.default_rng(1).uniform(-0.3, 0.3, 5 * n)
+    A = capi.Matrix(n, np.arange(n + 1, dtype=np.int32) * 5, j.astype(np.int32).ravel(), v,
+                    precision=capi.SPMV_PREC_DUAL, spmm_form=form)
+    x = dev(np.random.default_rng(2).uniform(-1, 1, (n, k))).to(dtype)
+    out = []
+    for sync in (torch.cuda.synchronize, lambda: None):
+        b = [x.clone(), torch.empty_like(x), torch.empty_like(x)]
+        sync()
+        for step in range(12):
+            A.apply_multi(b[step % 3], b[(step + 1) % 3])
+            sync()
+        out.append(b[0])
+    assert torch.equal(out[0], out[1])
 
 
 @pytest.mark.parametrize("bits", [16, 32])
