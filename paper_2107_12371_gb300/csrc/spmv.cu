@@ -93,6 +93,8 @@ __global__ void __launch_bounds__(1024)
 spmv_sell(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
           const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
           T beta) {
+    dep_wait();
+    dep_allow();
     spmv_sell_body<T, R, L, U, ColT, AXPBY>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
                                             n_slices, sp, cols, val, x, y, alpha, beta);
 }
@@ -105,6 +107,8 @@ __global__ void __launch_bounds__(1024, 2)
 spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
               const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
               T beta) {
+    dep_wait();
+    dep_allow();
     spmv_sell_body<T, R, L, U, ColT, AXPBY>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n,
                                             n_slices, sp, cols, val, x, y, alpha, beta);
 }
@@ -112,8 +116,10 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
 // FP64 with one or two rows per lane: a grid of at most kGsCtasPerSm 256-thread CTAs per SM
 // strides over the slice-lanes, each thread keeping U = 5 entries of its rows in flight (a
 // whole row of the tetrahedral meshes) at 64 registers.  Measured on the 6M-row mesh (S = 64):
-// 66.0 us, against 69.6 us for one slice-lane per thread at 32 registers and 2,048 threads per
-// SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.
+// 66.3 us, against 69.6 us for one slice-lane per thread at 32 registers and 2,048 threads per
+// SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.  A
+// dependent launch, as are the other two: 68.1 -> 66.3 us in a stream of products with the wait
+// first thing in the kernel; behind the first requests for entries it cost 69.6.
 constexpr int kGsBlock = 256;
 constexpr int kGsCtasPerSm = 4;
 template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
@@ -121,6 +127,8 @@ __global__ void __launch_bounds__(kGsBlock, kGsCtasPerSm)
 spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
              const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
              T beta) {
+    dep_wait();
+    dep_allow();
     const int64_t items = (int64_t)n_slices * L;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gt < items; gt += stride)
@@ -265,25 +273,22 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
                 const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
                 const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
                 const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
-                spmv_sell_gs<T, R, L, 5, ColT, AXPBY><<<g, kGsBlock, 0, st>>>(
-                    A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
-            } else {
-                spmv_sell_occ<T, R, L, U, ColT, AXPBY><<<grid, block, 0, st>>>(
-                    A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
+                return launch_dependent(spmv_sell_gs<T, R, L, 5, ColT, AXPBY>, g, kGsBlock, st,
+                                        A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha,
+                                        beta);
             }
-        } else {
-            spmv_sell<T, R, L, U, ColT, AXPBY><<<grid, block, 0, st>>>(
-                A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
+            return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
+                                    A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
         }
-        GB_LAUNCHED();
-        return SPMV_OK;
+        return launch_dependent(spmv_sell<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
+                                A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
     };
     if (A->index_bits == 16) return go(Cols16{A->sell_col16.p, A->col_start.p});
     return go(Cols32{A->sell_col.p});
 }
 
 // FP64 products that spmv_sell_thin takes (us, spmv_sell_gs or _occ / thin).  Rows of up to six
-// entries in Cuthill-McKee order: 304K 4.5 / 4.2, 796K 10.5 / 8.7, 3.1M 35.1 / 29.9, 6M 68.1 /
+// entries in Cuthill-McKee order: 304K 4.5 / 4.2, 796K 10.5 / 8.7, 3.1M 33.4 / 29.9, 6M 66.3 /
 // 71.1; of two entries (a gradient's faces): 600K 5.3 / 4.5, 2.6M 22.6 / 17.2.  Longer rows: 647K
 // 20.8 / 17.1, 1.8M 44.6 / 43.5, 3M 70.8 / 69.9 but with alpha and beta 82.6 / 84.5.
 bool use_thin(const spmv_matrix_t A) {
