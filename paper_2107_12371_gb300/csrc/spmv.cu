@@ -23,6 +23,16 @@
 namespace gb {
 namespace {
 
+// Hint: bring bytes (a multiple of 16) from p (16-byte aligned) on into L2.
+__device__ __forceinline__ void prefetch_l2_bulk(const void *p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+}
+// 8 bytes from global to shared memory, not waited for.
+__device__ __forceinline__ void copy_async8(volatile void *to, const void *from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared((const void *)to)), "l"(from));
+}
+
 // y = A x, or with AXPBY y = alpha (A x) + beta y evaluated as fma(alpha, t, beta y) (y is not
 // read when beta == 0), t being the row sum in column order.
 // gt: the slice-lane this thread computes (slice gt / L, lane gt % L).  The entries of a row
@@ -119,10 +129,12 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
 // 66.3 us, against 69.6 us for one slice-lane per thread at 32 registers and 2,048 threads per
 // SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.  A
 // dependent launch, as are the other two: 68.1 -> 66.3 us in a stream of products with the wait
-// first thing in the kernel; behind the first requests for entries it cost 69.6.
+// first thing in the kernel; behind the first requests for entries it cost 69.6.  AHEAD (a matrix of
+// more than twice the L2): 66.3 -> 63.2 us, 88 % of what HBM gives a copy; where the product before
+// leaves a good part of the matrix in L2 it costs more than it saves (3.7M rows 39.7 -> 41.3).
 constexpr int kGsBlock = 256;
 constexpr int kGsCtasPerSm = 4;
-template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
+template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool AHEAD>
 __global__ void __launch_bounds__(kGsBlock, kGsCtasPerSm)
 spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
              const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
@@ -131,8 +143,30 @@ spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT c
     dep_allow();
     const int64_t items = (int64_t)n_slices * L;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gt < items; gt += stride)
+    // AHEAD: thread 0 brings the entries of the CTA's next step into L2 in two bulk requests.  Their
+    // bounds come a step earlier into shared memory, so that no register holds them.
+    __shared__ volatile int64_t bound[2];
+    bool first = true;
+    for (int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gt < items; gt += stride) {
+        if (AHEAD && threadIdx.x == 0) {
+            if (!first) {
+                asm volatile("cp.async.wait_all;");
+                const int64_t e0 = bound[0], count = bound[1] - e0;
+                if (gt + stride < items && count > 0 && count <= 65536) {
+                    prefetch_l2_bulk(val + e0, (uint32_t)count * (uint32_t)sizeof(T));
+                    prefetch_l2_bulk(cols.col + e0, (uint32_t)count * (uint32_t)sizeof(cols.col[0]));
+                }
+            }
+            first = false;
+            const int64_t s0 = (gt + 2 * stride) / L;
+            if (s0 < n_slices) {
+                const int64_t s1 = s0 + kGsBlock / L < n_slices ? s0 + kGsBlock / L : n_slices;
+                copy_async8(&bound[0], sp + s0);
+                copy_async8(&bound[1], sp + s1);
+            }
+        }
         spmv_sell_body<T, R, L, U, ColT, AXPBY>(gt, n, n_slices, sp, cols, val, x, y, alpha, beta);
+    }
 }
 
 // One or two rows per lane, S / R lanes per slice (a slice may span several warps), U entries in
@@ -273,9 +307,12 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
                 const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
                 const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
                 const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
-                return launch_dependent(spmv_sell_gs<T, R, L, 5, ColT, AXPBY>, g, kGsBlock, st,
-                                        A->n, A->n_slices, A->slice_ptr.p, c, val, x, y, alpha,
-                                        beta);
+                const double bytes = (double)A->sell_entries * (sizeof(T) + A->index_bits / 8);
+                auto *kern = bytes > 2.0 * device_facts().l2_bytes
+                                 ? spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>
+                                 : spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false>;
+                return launch_dependent(kern, g, kGsBlock, st, A->n, A->n_slices, A->slice_ptr.p, c,
+                                        val, x, y, alpha, beta);
             }
             return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
                                     A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);

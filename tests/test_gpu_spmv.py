@@ -573,7 +573,7 @@ def test_small_products_every_row_remainder(oracle, n, max_len, bits, S):
     (2, 1000), (2, 311000), (2, 311400), (2, 466000), (2, 467000), (2, 622000), (2, 623000),
     (6, 1000), (6, 155000), (6, 156000), (6, 233000), (6, 234000), (6, 262144), (6, 262145),
     (6, 311000), (6, 312000), (6, 622000), (6, 623000), (6, 1000000), (6, 1000001),
-    (6, 3500000), (6, 3500001), (9, 1000), (9, 194000), (9, 195000), (9, 311000), (9, 312000),
+    (6, 3500000), (6, 3500001), (6, 4000001), (9, 1000), (9, 194000), (9, 195000), (9, 311000), (9, 312000),
     (9, 466000), (9, 467000), (9, 2000000), (9, 2000001)])
 def test_product_kernels_agree_at_the_edges_of_their_ranges(width, rows):
     """Products on both sides of each row count where another kernel is chosen, for rows of up to
