@@ -2,8 +2,8 @@
 // solves built on the sliced-ELLPACK product.  Neither solver is in the paper; the paper puts
 // the SpMV at the heart of the linear solver of an incompressible-flow time step (Sec. 2).
 //
-// One CG iteration is three kernels, each a grid-stride sweep over a fixed grid (the product
-// over a grid of its own, see cg_pq_grid):
+// One CG iteration is three kernels of one CTA per SM, each CTA with an equal contiguous chunk (the
+// product over a grid of its own, see cg_pq_grid):
 //   cg_spmv_pq   q = A p, partial p.q
 //   cg_update_xr alpha = rho / (p.q); x += alpha p, r -= alpha q, partial r.(D^-1 r), r.r
 //   cg_update_p  beta, rho, convergence; p = D^-1 r + beta p
@@ -11,11 +11,15 @@
 // kernel adds all of them in one fixed order (reduce_parts), so results do not depend on CTA
 // scheduling.  Measured against a last-CTA reduction at the end of every kernel (atomic ticket,
 // four 256-thread CTAs per SM, plain launches), per FP64 iteration of a CUDA-graph batch: 10K
-// rows 16.9 -> 7.7 us, 48K 17.3 -> 8.5, 304K 24.1 -> 15.5, 1M 44.6 -> 36.6, 6M 175.0 -> 167.0;
-// FP32 6M 76.2 -> 71.8, 1M 28.9 -> 18.7.  Each kernel is a programmatic dependent of the one before: its CTAs start as
-// the previous kernel's leave, request what no kernel of the solve writes (matrix, D^-1) and
-// then wait.  A "done" flag turns the remaining kernels of a CUDA-graph batch into no-ops, so
-// the host only checks convergence once per batch of iterations.
+// rows 16.9 -> 7.4 us, 48K 17.3 -> 8.2, 304K 24.1 -> 14.9, 1M 44.6 -> 35.0, 6M 175.0 -> 164.5;
+// FP32 6M 76.2 -> 71.1, 1M 28.9 -> 17.6.  What is left is the FP64 pipe (13 operations per row) and
+// HBM for large systems, and for small ones three chains of dependent loads, sums and a division.
+// Each kernel is a programmatic dependent of the one before: its CTAs start as the previous
+// kernel's leave, request what no kernel of the solve writes (matrix, D^-1) and then wait.  A
+// "done" flag turns the remaining kernels of a CUDA-graph batch into no-ops, so the host only
+// checks convergence once per batch of iterations.  Forming p = D^-1 r + beta p while gathering,
+// in two kernels, is bit-identical and no faster: FP64 48K 8.2 / 8.4 us, 304K 14.9 / 16.4, FP32
+// 48K 9.5 / 8.3 with its share of the solve, 105K 9.4 / 10.7.
 #include <algorithm>
 #include <atomic>
 #include <chrono>

@@ -18,8 +18,8 @@
 // the row's own update.
 //
 // Measured per iteration against three atomic-counter barriers per iteration on 256-thread CTAs
-// (us, whole solve over its iterations): FP64 10K rows 20.4 -> 10.8, 304K 28.5 -> 19.2, 1M 56.3
-// -> 41.6, 6M 188 -> 163; FP32 inner iterations 304K 21.8 -> 15.1, 6M 82.3 -> 72.0.
+// (us, whole solve over its iterations): FP64 10K rows 20.4 -> 9.5, 304K 28.5 -> 18.7, 1M 56.3
+// -> 40.1, 6M 188 -> 164; FP32 inner iterations 304K 21.8 -> 12.5, 6M 82.3 -> 70.2.
 //
 // Every wait is bounded: after 2 s without progress the waiting CTA records done = 4 (timeout)
 // and leaves; the others then leave by their own limits, so a fault can never leave the GPU
@@ -93,7 +93,8 @@ struct PersSmem {
 // Sums over CTAs [0, ctas) of their first TT threads' v[k]: use(k, sum) runs in one thread of
 // each CTA per quantity, and the other threads see what it wrote after the call.  Every CTA of
 // the grid waits.  PUBLISH: the CTAs' earlier writes are visible to all after the exchange.
-// meanwhile runs in every thread while the sums travel.  Returns false on a wait that ran out or CTA 0's vote to stop.
+// meanwhile runs in every thread while the sums travel.  Returns false on a wait that ran out or
+// CTA 0's vote to stop.
 template <int NV, bool PUBLISH, typename T, typename F, typename M>
 __device__ __forceinline__ bool exchange(const T (&v)[NV], int TT, int ctas,
                                          ulonglong2 *slots, unsigned long long iter, int my_vote,
