@@ -307,10 +307,14 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
                 const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
                 const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
                 const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
-                const double bytes = (double)A->sell_entries * (sizeof(T) + A->index_bits / 8);
-                auto *kern = bytes > 2.0 * device_facts().l2_bytes
-                                 ? spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>
-                                 : spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false>;
+                // (not where x is gathered from all over: the entries then drive x out of L2, 6M rows
+                // in random order 111 -> 130 us)
+                const double l2 = device_facts().l2_bytes;
+                const bool ahead =
+                    (double)A->sell_entries * (sizeof(T) + A->index_bits / 8) > 2.0 * l2 &&
+                    (double)A->max_span * sizeof(T) < l2 / 16;
+                auto *kern = ahead ? spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>
+                                   : spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false>;
                 return launch_dependent(kern, g, kGsBlock, st, A->n, A->n_slices, A->slice_ptr.p, c,
                                         val, x, y, alpha, beta);
             }
