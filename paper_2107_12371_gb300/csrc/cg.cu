@@ -159,8 +159,13 @@ cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, bool keep, const int64_t 
 // alpha = rho / (p.q) from the product's partials; x += alpha p; r -= alpha q; the CTA's partial
 // r.(D^-1 r) and r.r.  ONE: the grid has a thread for every vector, whose loads then travel with
 // those of the partials (one round trip); otherwise the sweep's own loads overlap each other.
-template <typename T, bool ONE>
-__global__ void __launch_bounds__(kIterThreads)
+// CTAS: at 2, with 32 registers and one vector in flight per thread, an SM has room for a sweep of
+// another stream.  That is for solves that run beside others: 16 requests of 200K to 2M rows in
+// the solve server 257 -> 233 ms.  A solve by itself wants the SM full: with room for two, dependent
+// launches put two of a sweep's CTAs on one SM and none on another (3M rows 89 -> 128 us per
+// iteration).  The sums are the same.
+template <typename T, bool ONE, int CTAS>
+__global__ void __launch_bounds__(kIterThreads, CTAS)
 cg_update_xr(int32_t n, int64_t chunk, bool keep, T *x, T *r, const T *p, const T *q,
              const T *dinv, const double *pq_part, int pq_count, double *part, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
@@ -198,15 +203,15 @@ cg_update_xr(int32_t n, int64_t chunk, bool keep, T *x, T *r, const T *p, const 
     const T alpha = step.coef;
     T vz = T(0), vr = T(0);
     if (ONE && mine) v.update(alpha, x, r, k0 * V, pol, vz, vr);
-    else sweep_update_xr<T>(n, k0, end, blockDim.x, pol, alpha, x, r, p, q, dinv, vz, vr);
+    else sweep_update_xr<T, CTAS == 1 ? 4 : 1>(n, k0, end, blockDim.x, pol, alpha, x, r, p, q, dinv, vz, vr);
     const T t[2] = {vz, vr};
     store_parts<2>(t, part);
 }
 
 // beta, rho and the convergence test from the x/r update's partials; p = D^-1 r + beta p.  ONE as
 // in cg_update_xr.
-template <typename T, bool ONE>
-__global__ void __launch_bounds__(kIterThreads)
+template <typename T, bool ONE, int CTAS>
+__global__ void __launch_bounds__(kIterThreads, CTAS)
 cg_update_p(int32_t n, int64_t chunk, bool keep, const T *r, const T *dinv, T *p,
             const double *part, int count, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
@@ -260,7 +265,7 @@ cg_update_p(int32_t n, int64_t chunk, bool keep, const T *r, const T *dinv, T *p
     if (step.done) return;
     const T beta = step.coef;
     if (ONE && mine) v.update(beta, p, k0 * V);
-    else sweep_update_p<T>(n, k0, end, blockDim.x, pol, beta, r, dinv, p);
+    else sweep_update_p<T, CTAS == 1 ? 4 : 1>(n, k0, end, blockDim.x, pol, beta, r, dinv, p);
 }
 
 // refinement: right-hand side of the inner solve r32 = fp32(r64 / ||r64||), start of the
@@ -433,44 +438,54 @@ static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q,
 }
 template <typename T>
 static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const T *p, const T *q,
-                                const T *dinv, CgScalars *sc, cudaStream_t st) {
+                                const T *dinv, CgScalars *sc, bool beside, cudaStream_t st) {
     constexpr int V = Vec16<T>::n;
     const IterGrid g = cg_sweep_grid(A, V);
-    return launch_dependent(g.single() ? cg_update_xr<T, true> : cg_update_xr<T, false>, g.ctas,
+    auto *kern = g.single() ? cg_update_xr<T, true, 1>
+                 : beside   ? cg_update_xr<T, false, 2>
+                            : cg_update_xr<T, false, 1>;
+    return launch_dependent(kern, g.ctas,
                             g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, x, r, p, q,
                             dinv, A->cg.part.p, pq_count, A->cg.part.p + A->cg.pq_len, sc);
 }
 template <typename T>
 static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p, CgScalars *sc,
-                               cudaStream_t st) {
+                               bool beside, cudaStream_t st) {
     constexpr int V = Vec16<T>::n;
     const IterGrid g = cg_sweep_grid(A, V);
-    return launch_dependent(g.single() ? cg_update_p<T, true> : cg_update_p<T, false>, g.ctas,
+    auto *kern = g.single() ? cg_update_p<T, true, 1>
+                 : beside   ? cg_update_p<T, false, 2>
+                            : cg_update_p<T, false, 1>;
+    return launch_dependent(kern, g.ctas,
                             g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, r, dinv, p,
                             A->cg.part.p + A->cg.pq_len, g.ctas, sc);
 }
 template <typename T>
 static spmv_status_t enqueue_iterations(spmv_matrix_t A, int iters, const T *val, T *x, T *r, T *p,
-                                        T *q, const T *dinv, CgScalars *sc, cudaStream_t st) {
+                                        T *q, const T *dinv, CgScalars *sc, bool beside,
+                                        cudaStream_t st) {
     for (int it = 0; it < iters; ++it) {
         int pq_count = 0;
         GB_TRY(enqueue_pq<T>(A, val, p, q, sc, st, &pq_count));
-        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, st));
-        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, st));
+        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, beside, st));
+        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, beside, st));
     }
     return SPMV_OK;
 }
 
-// enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each)
-static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st) {
+// enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each);
+// beside: other solves are expected to run at the same time (see cg_update_xr)
+static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st,
+                                  bool beside = false) {
     CgWork &w = A->cg;
     return enqueue_iterations<double>(A, iters, A->sell_val.p, w.x.p, w.r.p, w.p.p, w.q.p,
-                                      w.dinv.p, outer_scalars(A), st);
+                                      w.dinv.p, outer_scalars(A), beside, st);
 }
-static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st) {
+static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st,
+                                  bool beside = false) {
     CgWork &w = A->cg;
     return enqueue_iterations<float>(A, iters, A->sell_val32.p, w.d32.p, w.r32.p, w.p32.p, w.q32.p,
-                                     w.dinv32.p, inner_scalars(A), st);
+                                     w.dinv32.p, inner_scalars(A), beside, st);
 }
 
 __global__ void fill_value(int32_t n, double *v, double value) {
@@ -673,7 +688,7 @@ static spmv_status_t solve64(spmv_matrix_t A, const double *b, const cg_options_
             if (ctl.graphs) GB_TRY(get_graph(A, false, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg64(A, batch, st));
+                else GB_TRY(enqueue_cg64(A, batch, st, true));
                 GB_TRY(read_scalars(A, st, &h, nullptr));
                 if (h.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -766,7 +781,7 @@ static spmv_status_t solve_mixed(spmv_matrix_t A, const double *b, const cg_opti
             if (ctl.graphs) GB_TRY(get_graph(A, true, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg32(A, batch, st));
+                else GB_TRY(enqueue_cg32(A, batch, st, true));
                 GB_TRY(read_scalars(A, st, nullptr, &hi));
                 if (hi.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -871,8 +886,8 @@ spmv_status_t cg_timing(spmv_matrix_t A, int iters, double *out, cudaStream_t st
                 s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, st, &pq_count);
             else if (k == 1)
                 s = enqueue_xr<double>(A, pq_count, w.x.p, w.r.p, w.p.p, w.q.p, w.dinv.p, sc,
-                                       st);
-            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, st);
+                                       false, st);
+            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, false, st);
             if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e[1], st));
             if (s == SPMV_OK) s = elapsed(&ms);
             sum[k] += ms;

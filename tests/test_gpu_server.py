@@ -275,3 +275,28 @@ def test_priority_streams_leave_results_unchanged(oracle):
         assert r0["status"] == capi.SPMV_OK and relres(oracle, m, x0, b) <= 1e-8
         for out in outs[1:]:
             assert np.array_equal(out[i][0], x0)
+
+
+@pytest.mark.parametrize("mixed,edge", [(0, 38), (1, 48)])
+def test_large_requests_equal_a_solve_of_their_own(mixed, edge):
+    """Systems with several vectors per thread (329K rows FP64, 664K FP32), whose sweeps leave room
+    for other solves in the server: bit for bit what cg_solve returns."""
+    m, rng = meshgen.kuhn_tet_matrix_fast(edge, seed=3, dirichlet=True)
+    b = meshgen.uniform_vectors(rng, m.n)
+    A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values,
+                    precision=capi.SPMV_PREC_DUAL if mixed else capi.SPMV_PREC_FP64)
+    x = torch.zeros(m.n, dtype=torch.float64, device="cuda")
+    A.solve(torch.from_numpy(b).cuda(), x, rtol=1e-8, mixed=mixed)
+    srv = capi.spmv_server_create(8 << 30, 2)
+    try:
+        opt = capi.cg_default_options(rtol=1e-8, mixed=mixed)
+        tickets = [capi.spmv_server_submit(srv, m.n, m.row_ptr, m.col_idx, m.values, b, opt)
+                   for _ in range(2)]
+        for t in tickets:
+            got, r = np.empty(m.n), None
+            while r is None:
+                r = capi.spmv_server_poll(srv, t, got)
+            assert r["status"] == capi.SPMV_OK
+            assert np.array_equal(got, x.cpu().numpy())
+    finally:
+        capi.spmv_server_destroy(srv)
