@@ -846,6 +846,9 @@ spmv_status_t build_sell(spmv_matrix_t A, int S, cudaStream_t st) {
         GB_LAUNCHED();
         A->index_bits = 16;
     }
+    // a product is a dependent launch that reads matrix entries before its dep_wait: its kernel
+    // may start while a kernel that has not been waited for here still writes them
+    GB_CUDA(cudaStreamSynchronize(st));
     return SPMV_OK;
 }
 

@@ -173,3 +173,23 @@ def test_every_multi_cg_gather_width_matches_oracle(oracle, gather, k):
     A.solve_multi(Bd, X2, rtol=1e-10, persistent=1)
     torch.cuda.synchronize()
     assert torch.equal(X2, Xd)
+
+
+@pytest.mark.parametrize("size", [6, 26, 80])
+@pytest.mark.parametrize("precision", [capi.SPMV_PREC_FP64, capi.SPMV_PREC_FP32])
+def test_tuned_handles_with_16_bit_columns_keep_the_bits(size, precision):
+    """The tuner launches products right after the kernels that write a slice height's arrays
+    (16-bit columns last): 1K, 105K and 3.1M rows, equal to an untuned handle's product."""
+    m, x = workloads.kuhn(size, seed=size, dirichlet=True)
+    dt = np.float64 if precision == capi.SPMV_PREC_FP64 else np.float32
+    xd = dev(x.astype(dt))
+    out = []
+    for tuned in (0, 1):
+        A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values, reorder=capi.SPMV_REORDER_RCM,
+                        precision=precision, index_bits=16, autotune=tuned)
+        assert A.info()["index_bits"] == 16
+        y = torch.full_like(xd, float("nan"))
+        (A.apply if dt == np.float64 else A.apply_f32)(xd, y)
+        out.append(y)
+        A.close()
+    assert torch.equal(out[0], out[1])
