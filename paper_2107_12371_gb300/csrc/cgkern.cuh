@@ -304,7 +304,7 @@ __device__ __forceinline__ double reduce_parts(const double *part, int count) {
     double a[kPartLoads];
 #pragma unroll
     for (int j = 0; j < kPartLoads; ++j)
-        a[j] = lane + 32 * j < count ? __ldcg(part + lane + 32 * j) : 0.0;
+        a[j] = lane + 32 * j < count ? ld_l2(part + lane + 32 * j) : 0.0;
     return sum_parts(a);
 }
 
@@ -329,7 +329,7 @@ __device__ bool grid_sum_last(double (&v)[NV], double *part, unsigned *ticket, d
     for (int k = 0; k < NV; ++k) {
         s[k] = 0.0;
         for (int i = threadIdx.x; i < (int)gridDim.x; i += kCgBlock)
-            s[k] += __ldcg(part + k * gridDim.x + i);
+            s[k] += ld_l2(part + k * gridDim.x + i);
     }
     block_sum<NV>(s);
     if (threadIdx.x == 0) {

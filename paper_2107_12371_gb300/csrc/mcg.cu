@@ -83,25 +83,6 @@ struct Piece {
     static constexpr int n = BYTES / (int)sizeof(T);
 };
 
-// read-only (.nc) gather: for arrays no thread writes while the kernel runs
-template <int BYTES, typename T>
-__device__ __forceinline__ void ld_piece_nc(const T *p, T (&v)[Piece<T, BYTES>::n]) {
-    if constexpr (BYTES == 32 && sizeof(T) == 8) {
-        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-            : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
-    } else if constexpr (BYTES == 32) {
-        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
-              "=f"(v[6]), "=f"(v[7])
-            : "l"(p));
-    } else if constexpr (sizeof(T) == 8) {
-        asm("ld.global.nc.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p));
-    } else {
-        asm("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];"
-            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
-    }
-}
-
 // coherent gather (weak ld.global, L1 allocating): for the persistent kernel, where other CTAs
 // rewrite the array between grid barriers
 template <int BYTES, typename T>
@@ -125,7 +106,7 @@ __device__ __forceinline__ void ld_piece_co(const T *p, T (&v)[Piece<T, BYTES>::
 template <int BYTES, bool COH, typename T>
 __device__ __forceinline__ void ld_piece(const T *p, T (&v)[Piece<T, BYTES>::n]) {
     if constexpr (COH) ld_piece_co<BYTES>(p, v);
-    else ld_piece_nc<BYTES>(p, v);
+    else ld_x(p, v);
 }
 
 template <int BYTES, typename T>
@@ -257,7 +238,7 @@ __device__ __forceinline__ void last_cols(const double *part, int count, double 
     for (int qc = warp; qc < NQ * KP; qc += kMcgWarps) {
         const double *pp = part + (int64_t)qc * count;
         double s = 0.0;
-        for (int i = lane; i < count; i += 32) s += __ldcg(pp + i);
+        for (int i = lane; i < count; i += 32) s += ld_l2(pp + i);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) tot[qc / KP][qc % KP] = s;
@@ -928,7 +909,7 @@ mcg_persistent(IterGrid pq, IterGrid sw, int32_t n, int32_t S, int32_t n_slices,
             timed_out = true;
             break;
         }
-        if (__ldcg(vote) != 0.0) {
+        if (ld_l2(vote) != 0.0) {
             timed_out = true;
             break;
         }

@@ -160,14 +160,53 @@ struct Cols16 {
     __device__ __forceinline__ int32_t base(int64_t slice) const { return col_start[slice]; }
 };
 
-// ---- gathers of the multiplying vector (read-only path, L1 allocating) ----------------
-// Only for vectors that no thread writes while the kernel runs.
-__device__ __forceinline__ double ld_x(const double *p) { return __ldg(p); }
-__device__ __forceinline__ float ld_x(const float *p) { return __ldg(p); }
+// ---- reads of vectors ------------------------------------------------------------------
+// Vectors that an earlier kernel of the stream may still be writing when a dependent launch
+// begins (see dep_wait) are read with ordinary loads, never through the read-only .nc path, whose
+// data must not change while the kernel runs.  The loads are volatile, so the compiler keeps them
+// behind the wait, also where their addresses are known before it; they leave it free to move
+// other memory accesses.
+__device__ __forceinline__ double ld_x(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_x(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void ld_x(const double *p, double (&v)[1]) { v[0] = ld_x(p); }
+__device__ __forceinline__ void ld_x(const float *p, float (&v)[1]) { v[0] = ld_x(p); }
+__device__ __forceinline__ void ld_x(const double *p, double (&v)[2]) {
+    asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p));
+}
+__device__ __forceinline__ void ld_x(const float *p, float (&v)[2]) {
+    asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "l"(p));
+}
+__device__ __forceinline__ void ld_x(const float *p, float (&v)[4]) {
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
+}
+__device__ __forceinline__ void ld_x(const double *p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+__device__ __forceinline__ void ld_x(const float *p, float (&v)[8]) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                   "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+// One that other CTAs write while the kernel runs, between barriers or before a wait, from L2.
+__device__ __forceinline__ double ld_l2(const double *p) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
 
-// Coherent gathers (weak ld.global, L1 allocating) for vectors that other CTAs rewrite during
-// the same kernel, between grid barriers whose fences order the writes before these loads
-// (the read-only .nc path above would be allowed to return stale data there).
+// Gathers (weak ld.global, L1 allocating) for vectors that other CTAs rewrite during the same
+// kernel, between grid barriers whose fences order the writes before these loads.
 __device__ __forceinline__ double ld_x_coherent(const double *p) {
     double v;
     asm volatile("ld.global.ca.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
@@ -211,7 +250,9 @@ __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fma
 
 // Programmatic dependent launch (a kernel launched by launch_dependent).  dep_wait: returns once
 // the kernels this one depends on have finished and their writes are visible; before it, only
-// data that no kernel still running may write is read (a handle's matrix, a solve's D^-1).
+// data that no kernel still running may write is read (a handle's matrix, a solve's D^-1: both are
+// synchronised with when they are made).  Vectors are read behind it with ld_x or through pointers
+// without __restrict__, since a restricted one lets the compiler move its loads across the wait.
 // dep_allow: lets the next kernel's CTAs start as SM slots become free; they stop at their own
 // dep_wait.  Called after dep_wait, so that no more than two kernels of a stream are in flight.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -35,7 +35,7 @@ constexpr int kRowsBlock = 128;
 template <typename T, int G, int C, typename ColT>
 __global__ void __launch_bounds__(256)
 spmm_sell(int32_t n, int32_t S, int32_t n_slices, int k, const int64_t *__restrict__ sp,
-          ColT cols, const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
+          ColT cols, const T *__restrict__ val, const T *X, T *Y) {
     constexpr int RPW = 32 / G;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -117,24 +117,12 @@ template <typename T, int VW>
 struct VecOf;
 template <>
 struct VecOf<double, 2> {
-    static __device__ __forceinline__ void load(const double *p, double (&v)[2]) {
-        const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
-        v[0] = t.x;
-        v[1] = t.y;
-    }
     static __device__ __forceinline__ void store(double *p, const double (&v)[2]) {
         *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
     }
 };
 template <>
 struct VecOf<float, 4> {
-    static __device__ __forceinline__ void load(const float *p, float (&v)[4]) {
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = t.x;
-        v[1] = t.y;
-        v[2] = t.z;
-        v[3] = t.w;
-    }
     static __device__ __forceinline__ void store(float *p, const float (&v)[4]) {
         *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
     }
@@ -143,7 +131,7 @@ struct VecOf<float, 4> {
 template <typename T, int VW, int G, typename ColT>
 __global__ void __launch_bounds__(256)
 spmm_sell_vec(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
-              const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
+              const T *__restrict__ val, const T *X, T *Y) {
     constexpr int K = VW * G;
     constexpr int RPW = 32 / G;
     constexpr int PE = 16;                      // pairs preloaded per round
@@ -199,7 +187,7 @@ spmm_sell_vec(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict_
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (c[u] >= 0) VecOf<T, VW>::load(X + (int64_t)c[u] * K + g * VW, xv[u]);
+                if (c[u] >= 0) ld_x(X + (int64_t)c[u] * K + g * VW, xv[u]);
                 else {
 #pragma unroll
                     for (int j = 0; j < VW; ++j) xv[u][j] = T(0);
@@ -215,18 +203,12 @@ spmm_sell_vec(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict_
     if (row < n) VecOf<T, VW>::store(Y + row * K + g * VW, acc);
 }
 
-// 32-byte gathers and stores of X / Y rows (256-bit accesses, sm_100 and later).
+// Columns of a 32-byte piece of a row, gathered and stored by one 256-bit access.
 template <typename T>
 struct Wide;
 template <>
 struct Wide<float> {
     static constexpr int n = 8;
-    static __device__ __forceinline__ void load(const float *p, float (&v)[8]) {
-        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
-              "=f"(v[7])
-            : "l"(p));
-    }
     static __device__ __forceinline__ void store(float *p, const float (&v)[8]) {
         asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]),
                      "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
@@ -236,11 +218,6 @@ struct Wide<float> {
 template <>
 struct Wide<double> {
     static constexpr int n = 4;
-    static __device__ __forceinline__ void load(const double *p, double (&v)[4]) {
-        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-            : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
-            : "l"(p));
-    }
     static __device__ __forceinline__ void store(double *p, const double (&v)[4]) {
         asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(v[0]), "d"(v[1]),
                      "d"(v[2]), "d"(v[3])
@@ -248,24 +225,7 @@ struct Wide<double> {
     }
 };
 
-// Loads and stores of P consecutive elements (4 to 32 bytes) of a row of X or Y.
-template <typename T, int P>
-__device__ __forceinline__ void ld_cols(const T *p, T (&v)[P]) {
-    if constexpr (P == 1) {
-        v[0] = __ldg(p);
-    } else if constexpr (P == 2 && sizeof(T) == 8) {
-        const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
-        v[0] = t.x, v[1] = t.y;
-    } else if constexpr (P == 2) {
-        const float2 t = __ldg(reinterpret_cast<const float2 *>(p));
-        v[0] = t.x, v[1] = t.y;
-    } else if constexpr (P == 4 && sizeof(T) == 4) {
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-    } else {
-        Wide<T>::load(p, v);
-    }
-}
+// Stores of P consecutive elements (4 to 32 bytes) of a row of Y.
 template <typename T, int P>
 __device__ __forceinline__ void st_cols(T *p, const T (&v)[P]) {
     if constexpr (P == 1) *p = v[0];
@@ -335,7 +295,7 @@ inline int piece_choice(int k, int P, int elem) {
 template <typename T, int P, int C, typename ColT>
 __global__ void __launch_bounds__(256, 1)
 spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ sp, ColT cols,
-                const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
+                const T *__restrict__ val, const T *X, T *Y) {
     constexpr int U = piece_unroll(P * C * (int)sizeof(T), (int)sizeof(T));
     const int rpw = 32 / G;
     const int lane = threadIdx.x & 31;
@@ -391,7 +351,7 @@ spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ 
             const T *xr = xg + (int64_t)c[u][0] * k;
 #pragma unroll
             for (int j = 0; j < C; ++j)
-                if (has[j]) ld_cols<T, P>(xr + j * G * P, xv[u][j]);
+                if (has[j]) ld_x(xr + j * G * P, xv[u][j]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -420,7 +380,7 @@ spmm_sell_piece(int32_t n, int32_t S, int k, int G, const int64_t *__restrict__ 
 template <typename T, int G, typename ColT>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4)
 spmm_sell_wide(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict__ sp,
-               ColT cols, const T *__restrict__ val, const T *__restrict__ X, T *__restrict__ Y) {
+               ColT cols, const T *__restrict__ val, const T *X, T *Y) {
     constexpr int VW = Wide<T>::n;
     constexpr int K = VW * G;
     constexpr int RPW = 32 / G;
@@ -456,7 +416,7 @@ spmm_sell_wide(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict
         T xv[2][VW];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            if (c[u][0] >= 0) Wide<T>::load(xg + (int64_t)c[u][0] * K, xv[u]);
+            if (c[u][0] >= 0) ld_x(xg + (int64_t)c[u][0] * K, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u)
@@ -472,7 +432,7 @@ spmm_sell_wide(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict
         cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c);
         if (c[0] >= 0) {
             T xv[VW];
-            Wide<T>::load(xg + (int64_t)c[0] * K, xv);
+            ld_x(xg + (int64_t)c[0] * K, xv);
 #pragma unroll
             for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[0], xv[j], acc[j]);
         }
@@ -487,8 +447,7 @@ spmm_sell_wide(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict
 template <typename T, int G, typename ColT>
 __global__ void __launch_bounds__(256, 4)
 spmm_sell_wide_pipe(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict__ sp,
-                    ColT cols, const T *__restrict__ val, const T *__restrict__ X,
-                    T *__restrict__ Y) {
+                    ColT cols, const T *__restrict__ val, const T *X, T *Y) {
     constexpr int VW = Wide<T>::n;
     constexpr int K = VW * G;
     constexpr int RPW = 32 / G;
@@ -540,7 +499,7 @@ spmm_sell_wide_pipe(int32_t n, int32_t S, int32_t n_slices, const int64_t *__res
         T xv[2][VW];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
-            if (c[u] >= 0) Wide<T>::load(xg + (int64_t)c[u] * K, xv[u]);
+            if (c[u] >= 0) ld_x(xg + (int64_t)c[u] * K, xv[u]);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
             if (c[u] >= 0) {
@@ -562,7 +521,7 @@ template <typename T, int G, typename ColT>
 __device__ __forceinline__ void wide_warp_rows(int64_t row0, int32_t n, int32_t S,
                                                const int64_t *__restrict__ sp, ColT cols,
                                                const T *__restrict__ val,
-                                               const T *__restrict__ X, T *__restrict__ Y,
+                                               const T *X, T *Y,
                                                uint64_t pol) {
     constexpr int VW = Wide<T>::n;
     constexpr int K = VW * G;
@@ -591,7 +550,7 @@ __device__ __forceinline__ void wide_warp_rows(int64_t row0, int32_t n, int32_t 
         T xv[2][VW];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            if (c[u][0] >= 0) Wide<T>::load(xg + (int64_t)c[u][0] * K, xv[u]);
+            if (c[u][0] >= 0) ld_x(xg + (int64_t)c[u][0] * K, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u)
@@ -607,7 +566,7 @@ __device__ __forceinline__ void wide_warp_rows(int64_t row0, int32_t n, int32_t 
         cols.template load<1>(cat + (int64_t)t * S, slice, pol, cbase, c);
         if (c[0] >= 0) {
             T xv[VW];
-            Wide<T>::load(xg + (int64_t)c[0] * K, xv);
+            ld_x(xg + (int64_t)c[0] * K, xv);
 #pragma unroll
             for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[0], xv[j], acc[j]);
         }
@@ -639,8 +598,7 @@ __device__ __forceinline__ void prefetch_rows_l2(int64_t rlo, int64_t rhi, int32
 template <typename T, int G, int MINB, typename ColT>
 __global__ void __launch_bounds__(256, MINB)
 spmm_sell_wide_gs(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict__ sp,
-                  ColT cols, const T *__restrict__ val, const T *__restrict__ X,
-                  T *__restrict__ Y) {
+                  ColT cols, const T *__restrict__ val, const T *X, T *Y) {
     constexpr int RPW = 32 / G;
     constexpr int64_t RB = 8 * RPW;
     const int warp = threadIdx.x >> 5;
@@ -686,7 +644,7 @@ __device__ __forceinline__ void wide_row_w(int64_t at, int32_t S, ColT cols, int
         T xv[2][VW];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
-            if (t + u < W && c[t + u] >= 0) Wide<T>::load(xg + (int64_t)c[t + u] * K, xv[u]);
+            if (t + u < W && c[t + u] >= 0) ld_x(xg + (int64_t)c[t + u] * K, xv[u]);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
             if (t + u < W && c[t + u] >= 0) {
@@ -705,8 +663,7 @@ __device__ __forceinline__ void wide_row_w(int64_t at, int32_t S, ColT cols, int
 template <typename T, int G, int MINB, int WMAX, typename ColT>
 __global__ void __launch_bounds__(256, MINB)
 spmm_sell_unrolled(int32_t n, int32_t S, int32_t n_slices, const int64_t *__restrict__ sp,
-                   ColT cols, const T *__restrict__ val, const T *__restrict__ X,
-                   T *__restrict__ Y) {
+                   ColT cols, const T *__restrict__ val, const T *X, T *Y) {
     constexpr int VW = Wide<T>::n;
     constexpr int K = VW * G;
     constexpr int RPW = 32 / G;
@@ -774,7 +731,7 @@ spmm_sell_unrolled(int32_t n, int32_t S, int32_t n_slices, const int64_t *__rest
                 T xv[2][VW];
 #pragma unroll
                 for (int u = 0; u < 2; ++u)
-                    if (c[u][0] >= 0) Wide<T>::load(xg + (int64_t)c[u][0] * K, xv[u]);
+                    if (c[u][0] >= 0) ld_x(xg + (int64_t)c[u][0] * K, xv[u]);
 #pragma unroll
                 for (int u = 0; u < 2; ++u)
                     if (c[u][0] >= 0) {
@@ -789,7 +746,7 @@ spmm_sell_unrolled(int32_t n, int32_t S, int32_t n_slices, const int64_t *__rest
                 cols.template load<1>(at + (int64_t)t * S, 0, pol, cb, c);
                 if (c[0] >= 0) {
                     T xv[VW];
-                    Wide<T>::load(xg + (int64_t)c[0] * K, xv);
+                    ld_x(xg + (int64_t)c[0] * K, xv);
 #pragma unroll
                     for (int j = 0; j < VW; ++j) acc[j] = fma_t(a[0], xv[j], acc[j]);
                 }

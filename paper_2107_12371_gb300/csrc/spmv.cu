@@ -42,7 +42,7 @@ template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_slices,
                                                const int64_t *__restrict__ sp, ColT cols,
                                                const T *__restrict__ val,
-                                               const T *__restrict__ x, T *__restrict__ y,
+                                               const T *x, T *y,
                                                T alpha, T beta) {
     // L lanes per slice, R rows per lane: S = L R rows per slice
     constexpr int S = L * R;
@@ -101,7 +101,7 @@ __device__ __forceinline__ void spmv_sell_body(int64_t gt, int32_t n, int32_t n_
 template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __global__ void __launch_bounds__(1024)
 spmv_sell(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
-          const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
+          const T *__restrict__ val, const T *x, T *y, T alpha,
           T beta) {
     dep_wait();
     dep_allow();
@@ -115,7 +115,7 @@ spmv_sell(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols
 template <typename T, int R, int L, int U, typename ColT, bool AXPBY>
 __global__ void __launch_bounds__(1024, 2)
 spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
-              const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
+              const T *__restrict__ val, const T *x, T *y, T alpha,
               T beta) {
     dep_wait();
     dep_allow();
@@ -137,7 +137,7 @@ constexpr int kGsCtasPerSm = 4;
 template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool AHEAD>
 __global__ void __launch_bounds__(kGsBlock, kGsCtasPerSm)
 spmv_sell_gs(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
-             const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
+             const T *__restrict__ val, const T *x, T *y, T alpha,
              T beta) {
     dep_wait();
     dep_allow();
@@ -183,7 +183,7 @@ constexpr int kThinBlock = 128;
 template <typename T, int R, int L, int U, int CTAS, typename ColT, bool AXPBY>
 __global__ void __launch_bounds__(kThinBlock, CTAS)
 spmv_sell_thin(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT cols,
-               const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y, T alpha,
+               const T *__restrict__ val, const T *x, T *y, T alpha,
                T beta, bool add) {
     constexpr int S = L * R;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
