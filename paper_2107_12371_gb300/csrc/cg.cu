@@ -108,13 +108,16 @@ cg_residual(int32_t n, int32_t n_slices, const int64_t *sp, ColT col, const T *v
 // q = A p and the CTA's partial p.q.  Grid cg_pq_grid (see cgkern.cuh).  UU: entries in flight
 // per lane (pq_unroll, or 2 for matrices whose widest slice needs fewer load rounds that way;
 // the per-row order, hence the result, is the same).  The first round of matrix entries is
-// requested before the previous kernel (which finishes p) has ended.
-template <typename T, int R, int L, typename ColT, int UU>
-__global__ void __launch_bounds__(kCgBlock * pq_min_ctas((int)sizeof(T) * R))
-cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, bool keep, const int64_t *sp, ColT col,
-           const T *val, const T *p, T *q, double *part, CgScalars *sc) {
+// requested before the previous kernel (which finishes p) has ended.  Q: CTAs that share one of
+// the grid (1, or kSplit; see IterForm).
+template <typename T, int R, int L, typename ColT, int UU, int Q>
+__global__ void __launch_bounds__(kCgBlock * pq_min_ctas((int)sizeof(T) * R) / Q, Q)
+cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, int threads, bool keep, const int64_t *sp,
+           ColT col, const T *val, const T *p, T *q, double *part, SplitSums *split,
+           CgScalars *sc) {
     const uint64_t pol = policy_stream(keep);
-    const int64_t g0 = iter_begin(chunk), end = iter_end(chunk, (int64_t)n_slices * L);
+    const IterSlot<Q> slot(threads);
+    const int64_t g0 = slot.begin(chunk), end = slot.end(chunk, (int64_t)n_slices * L);
     // lanes of 64 bytes per entry have no registers for a round held across the wait
     constexpr bool kEarly = sizeof(T) * R <= 32;
     SliceLane s{};
@@ -135,7 +138,7 @@ cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, bool keep, const int64_t 
     }
     if (done) return;
     T vt = T(0);
-    for (int64_t g = g0; g < end; g += blockDim.x) {
+    for (int64_t g = g0; g < end; g += Q == 1 ? (int)blockDim.x : threads) {
         T acc[R];
         if constexpr (kEarly) {
             if (g != g0) {
@@ -153,23 +156,22 @@ cg_spmv_pq(int32_t n, int32_t n_slices, int64_t chunk, bool keep, const int64_t 
             if (row0 + i < n) vt = fma_t(p[row0 + i], acc[i], vt);
     }
     const T v[1] = {vt};
-    store_parts<1>(v, part);
+    store_parts<Q, 1>(slot, threads, v, split, part);
 }
 
 // alpha = rho / (p.q) from the product's partials; x += alpha p; r -= alpha q; the CTA's partial
 // r.(D^-1 r) and r.r.  ONE: the grid has a thread for every vector, whose loads then travel with
 // those of the partials (one round trip); otherwise the sweep's own loads overlap each other.
-// CTAS: at 2, with 32 registers and one vector in flight per thread, an SM has room for a sweep of
-// another stream.  That is for solves that run beside others: 16 requests of 200K to 2M rows in
-// the solve server 257 -> 233 ms.  A solve by itself wants the SM full: with room for two, dependent
-// launches put two of a sweep's CTAs on one SM and none on another (3M rows 89 -> 128 us per
-// iteration).  The sums are the same.
-template <typename T, bool ONE, int CTAS>
-__global__ void __launch_bounds__(kIterThreads, CTAS)
-cg_update_xr(int32_t n, int64_t chunk, bool keep, T *x, T *r, const T *p, const T *q,
-             const T *dinv, const double *pq_part, int pq_count, double *part, CgScalars *sc) {
+// Q: CTAs that share one of the grid (1, or kSplit with 32 registers and one vector in flight per
+// thread; see IterForm).
+template <typename T, bool ONE, int Q>
+__global__ void __launch_bounds__(kIterThreads / Q, Q == 1 ? 1 : 2 * Q)
+cg_update_xr(int32_t n, int64_t chunk, int threads, bool keep, T *x, T *r, const T *p, const T *q,
+             const T *dinv, const double *pq_part, int pq_count, double *part,
+             SplitSums *split, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
-    const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
+    const IterSlot<Q> slot(threads);
+    const int64_t k0 = slot.begin(chunk), end = slot.end(chunk, ((int64_t)n + V - 1) / V);
     const bool mine = k0 < end && k0 < n / V;
     XrVec<T> v;
     if (mine) {
@@ -203,19 +205,22 @@ cg_update_xr(int32_t n, int64_t chunk, bool keep, T *x, T *r, const T *p, const 
     const T alpha = step.coef;
     T vz = T(0), vr = T(0);
     if (ONE && mine) v.update(alpha, x, r, k0 * V, pol, vz, vr);
-    else sweep_update_xr<T, CTAS == 1 ? 4 : 1>(n, k0, end, blockDim.x, pol, alpha, x, r, p, q, dinv, vz, vr);
+    else
+        sweep_update_xr<T, Q == 1 ? 4 : 1>(n, k0, end, Q == 1 ? (int)blockDim.x : threads, pol,
+                                           alpha, x, r, p, q, dinv, vz, vr);
     const T t[2] = {vz, vr};
-    store_parts<2>(t, part);
+    store_parts<Q, 2>(slot, threads, t, split, part);
 }
 
 // beta, rho and the convergence test from the x/r update's partials; p = D^-1 r + beta p.  ONE as
 // in cg_update_xr.
-template <typename T, bool ONE, int CTAS>
-__global__ void __launch_bounds__(kIterThreads, CTAS)
-cg_update_p(int32_t n, int64_t chunk, bool keep, const T *r, const T *dinv, T *p,
+template <typename T, bool ONE, int Q>
+__global__ void __launch_bounds__(kIterThreads / Q, Q == 1 ? 1 : 2 * Q)
+cg_update_p(int32_t n, int64_t chunk, int threads, bool keep, const T *r, const T *dinv, T *p,
             const double *part, int count, CgScalars *sc) {
     constexpr int V = Vec16<T>::n;
-    const int64_t k0 = iter_begin(chunk), end = iter_end(chunk, ((int64_t)n + V - 1) / V);
+    const IterSlot<Q> slot(threads);
+    const int64_t k0 = slot.begin(chunk), end = slot.end(chunk, ((int64_t)n + V - 1) / V);
     const bool mine = k0 < end && k0 < n / V;
     const uint64_t pol = policy_stream(keep);
     PVec<T> v;
@@ -265,7 +270,9 @@ cg_update_p(int32_t n, int64_t chunk, bool keep, const T *r, const T *dinv, T *p
     if (step.done) return;
     const T beta = step.coef;
     if (ONE && mine) v.update(beta, p, k0 * V);
-    else sweep_update_p<T, CTAS == 1 ? 4 : 1>(n, k0, end, blockDim.x, pol, beta, r, dinv, p);
+    else
+        sweep_update_p<T, Q == 1 ? 4 : 1>(n, k0, end, Q == 1 ? (int)blockDim.x : threads, pol,
+                                          beta, r, dinv, p);
 }
 
 // refinement: right-hand side of the inner solve r32 = fp32(r64 / ||r64||), start of the
@@ -418,74 +425,112 @@ static spmv_status_t with_cols(spmv_matrix_t A, F &&f) {
     return f(Cols32{A->sell_col.p});
 }
 
+// How the kernels of an iteration are run: by themselves (a CTA per SM), or beside other solves.
+// There a CTA that fills an SM waits for one to be empty and then keeps the other streams' kernels
+// out, so those of more than kSplitThreads threads are run by four smaller ones each, the sweeps
+// at 32 registers, and nothing is kept in an L2 that several solves share.  Each thread of the grid
+// does what it does otherwise and the sums are formed from the same warps' (store_parts), so the
+// bits are the same.  Measured, whole kernels / four 256-thread CTAs per SM with last-CTA
+// reductions and FP64 shuffle trees / this form: saturated stream of 700 requests (1e4 to 2e6
+// cells), eight slots, 143 / 152 / 159 solves/s; 16 requests of 200K to 2M cells 304 / 297 / 279 ms,
+// 100K to 600K 92 / 92 / 81 ms.  Halves instead of quarters 125-134 solves/s, sweeps at 64
+// registers 131, L2 hints as for a single solve 2-4 % less; splitting smaller CTAs too costs the
+// small requests 8 %.
+// kYield: a solve whose stream has priority over the others'.  A dependent CTA that waits holds its
+// place, and with priority it takes that from kernels that have work: the large kernels are launched
+// plainly (p99 of the stream at 75/s with the requests of 256 MB and more prioritised 187 -> 141 ms;
+// at equal priority dependent launches have the better p99, 145 against 152).
+enum class IterForm { kAlone, kBeside, kYield };
+constexpr int kSplit = 4, kSplitThreads = 512;
+
+struct IterLaunch {
+    IterGrid g;
+    IterKeep keep;
+    bool split, dependent;
+    IterLaunch(const spmv_matrix_t A, IterForm form, const IterGrid &grid, int elem_bytes)
+        : g(grid), keep(cg_keep(A, elem_bytes)) {
+        split = form != IterForm::kAlone && g.threads > kSplitThreads;
+        dependent = form != IterForm::kYield || g.single();
+        if (form != IterForm::kAlone) keep = {false, false};
+    }
+    unsigned ctas() const { return (unsigned)(split ? g.ctas * kSplit : g.ctas); }
+    unsigned threads() const {
+        return (unsigned)(split ? (g.threads + 32 * kSplit - 1) / (32 * kSplit) * 32 : g.threads);
+    }
+};
+
 // the product, the x/r sweep and the p sweep of an iteration (pq_count: CTAs of the product)
 template <typename T>
 static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q, CgScalars *sc,
-                                cudaStream_t st, int *pq_count) {
+                                IterForm form, cudaStream_t st, int *pq_count) {
     return with_cols(A, [&](auto cols) -> spmv_status_t {
         using ColT = decltype(cols);
         return with_shape<T>(A->S, [&](auto rt, auto lt) -> spmv_status_t {
             constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
             constexpr int UU = pq_unroll((int)sizeof(T) * R);
-            const IterGrid g = cg_pq_grid(A, L, (int)sizeof(T) * R);
-            *pq_count = g.ctas;
-            return launch_dependent(cg_pq_deep(A, UU) ? cg_spmv_pq<T, R, L, ColT, UU>
-                                                      : cg_spmv_pq<T, R, L, ColT, 2>,
-                                    g.ctas, g.threads, st, A->n, A->n_slices, g.chunk,
-                                    cg_keep(A, sizeof(T)).matrix, A->slice_ptr.p, cols, val, p, q, A->cg.part.p, sc);
+            const IterLaunch l(A, form, cg_pq_grid(A, L, (int)sizeof(T) * R), sizeof(T));
+            *pq_count = l.g.ctas;
+            auto go = [&](auto *kern) {
+                return launch_ordered(l.dependent, kern, l.ctas(), l.threads(), st, A->n,
+                                      A->n_slices, l.g.chunk, l.g.threads, l.keep.matrix,
+                                      A->slice_ptr.p, cols, val, p, q, A->cg.part.p,
+                                      A->cg.split.p, sc);
+            };
+            if (cg_pq_deep(A, UU))
+                return go(l.split ? cg_spmv_pq<T, R, L, ColT, UU, kSplit>
+                                  : cg_spmv_pq<T, R, L, ColT, UU, 1>);
+            return go(l.split ? cg_spmv_pq<T, R, L, ColT, 2, kSplit>
+                              : cg_spmv_pq<T, R, L, ColT, 2, 1>);
         });
     });
 }
 template <typename T>
 static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const T *p, const T *q,
-                                const T *dinv, CgScalars *sc, bool beside, cudaStream_t st) {
-    constexpr int V = Vec16<T>::n;
-    const IterGrid g = cg_sweep_grid(A, V);
-    auto *kern = g.single() ? cg_update_xr<T, true, 1>
-                 : beside   ? cg_update_xr<T, false, 2>
-                            : cg_update_xr<T, false, 1>;
-    return launch_dependent(kern, g.ctas,
-                            g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, x, r, p, q,
-                            dinv, A->cg.part.p, pq_count, A->cg.part.p + A->cg.pq_len, sc);
+                                const T *dinv, CgScalars *sc, IterForm form, cudaStream_t st) {
+    const IterLaunch l(A, form, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
+    auto *kern = l.split        ? cg_update_xr<T, false, kSplit>
+                 : l.g.single() ? cg_update_xr<T, true, 1>
+                                : cg_update_xr<T, false, 1>;
+    return launch_ordered(l.dependent, kern, l.ctas(), l.threads(), st, A->n, l.g.chunk,
+                          l.g.threads, l.keep.vectors, x, r, p, q, dinv, A->cg.part.p, pq_count,
+                          A->cg.part.p + A->cg.pq_len, A->cg.split.p, sc);
 }
 template <typename T>
 static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p, CgScalars *sc,
-                               bool beside, cudaStream_t st) {
-    constexpr int V = Vec16<T>::n;
-    const IterGrid g = cg_sweep_grid(A, V);
-    auto *kern = g.single() ? cg_update_p<T, true, 1>
-                 : beside   ? cg_update_p<T, false, 2>
-                            : cg_update_p<T, false, 1>;
-    return launch_dependent(kern, g.ctas,
-                            g.threads, st, A->n, g.chunk, cg_keep(A, sizeof(T)).vectors, r, dinv, p,
-                            A->cg.part.p + A->cg.pq_len, g.ctas, sc);
+                               IterForm form, cudaStream_t st) {
+    const IterLaunch l(A, form, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
+    auto *kern = l.split        ? cg_update_p<T, false, kSplit>
+                 : l.g.single() ? cg_update_p<T, true, 1>
+                                : cg_update_p<T, false, 1>;
+    return launch_ordered(l.dependent, kern, l.ctas(), l.threads(), st, A->n, l.g.chunk,
+                          l.g.threads, l.keep.vectors, r, dinv, p, A->cg.part.p + A->cg.pq_len,
+                          l.g.ctas, sc);
 }
 template <typename T>
 static spmv_status_t enqueue_iterations(spmv_matrix_t A, int iters, const T *val, T *x, T *r, T *p,
-                                        T *q, const T *dinv, CgScalars *sc, bool beside,
+                                        T *q, const T *dinv, CgScalars *sc, IterForm form,
                                         cudaStream_t st) {
     for (int it = 0; it < iters; ++it) {
         int pq_count = 0;
-        GB_TRY(enqueue_pq<T>(A, val, p, q, sc, st, &pq_count));
-        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, beside, st));
-        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, beside, st));
+        GB_TRY(enqueue_pq<T>(A, val, p, q, sc, form, st, &pq_count));
+        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, form, st));
+        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, form, st));
     }
     return SPMV_OK;
 }
 
-// enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each);
-// beside: other solves are expected to run at the same time (see cg_update_xr)
+// enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each)
 static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st,
-                                  bool beside = false) {
+                                  IterForm form = IterForm::kAlone) {
     CgWork &w = A->cg;
     return enqueue_iterations<double>(A, iters, A->sell_val.p, w.x.p, w.r.p, w.p.p, w.q.p,
-                                      w.dinv.p, outer_scalars(A), beside, st);
+                                      w.dinv.p, outer_scalars(A), form, st);
 }
 static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st,
-                                  bool beside = false) {
+                                  IterForm form = IterForm::kAlone) {
     CgWork &w = A->cg;
     return enqueue_iterations<float>(A, iters, A->sell_val32.p, w.d32.p, w.r32.p, w.p32.p, w.q32.p,
-                                     w.dinv32.p, inner_scalars(A), beside, st);
+                                     w.dinv32.p, inner_scalars(A), form, st);
 }
 
 __global__ void fill_value(int32_t n, double *v, double value) {
@@ -529,7 +574,8 @@ static spmv_status_t tune_cg_product(spmv_matrix_t A, cudaStream_t st) {
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e0, st));
                 int count = 0;
                 if (s == SPMV_OK)
-                    s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, st, &count);
+                    s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, IterForm::kAlone, st,
+                                           &count);
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e1, st));
                 if (s == SPMV_OK) s = cuda_status(cudaEventSynchronize(e1));
                 if (s == SPMV_OK && i >= 0) s = cuda_status(cudaEventElapsedTime(&t[i], e0, e1));
@@ -650,6 +696,13 @@ static bool cancelled(const std::atomic<int> *cancel) {
     return cancel && cancel->load(std::memory_order_relaxed) != 0;
 }
 
+// The form of the next batch of directly launched iterations.
+static IterForm iter_form(const spmv_matrix_t A, const SolveControl &ctl) {
+    if (!A->cg.split.p || ctl.running->load(std::memory_order_relaxed) < 2)
+        return IterForm::kAlone;
+    return ctl.high_priority ? IterForm::kYield : IterForm::kBeside;
+}
+
 // read both scalar blocks to the host
 static spmv_status_t read_scalars(spmv_matrix_t A, cudaStream_t st, CgScalars *outer,
                                   CgScalars *inner) {
@@ -688,7 +741,7 @@ static spmv_status_t solve64(spmv_matrix_t A, const double *b, const cg_options_
             if (ctl.graphs) GB_TRY(get_graph(A, false, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg64(A, batch, st, true));
+                else GB_TRY(enqueue_cg64(A, batch, st, iter_form(A, ctl)));
                 GB_TRY(read_scalars(A, st, &h, nullptr));
                 if (h.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -781,7 +834,7 @@ static spmv_status_t solve_mixed(spmv_matrix_t A, const double *b, const cg_opti
             if (ctl.graphs) GB_TRY(get_graph(A, true, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg32(A, batch, st, true));
+                else GB_TRY(enqueue_cg32(A, batch, st, iter_form(A, ctl)));
                 GB_TRY(read_scalars(A, st, nullptr, &hi));
                 if (hi.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -827,7 +880,7 @@ void release_cg(spmv_matrix_t A) {
     CgWork &w = A->cg;
     w.x.release(t); w.r.release(t); w.p.release(t); w.q.release(t); w.dinv.release(t);
     w.r32.release(t); w.p32.release(t); w.q32.release(t); w.d32.release(t); w.dinv32.release(t);
-    w.part.release(t); w.scal.release(t); w.slots.release(t); w.zp.release(t);
+    w.part.release(t); w.scal.release(t); w.split.release(t); w.slots.release(t); w.zp.release(t);
     w.zp32.release(t); w.flags.release(t);
     if (w.graph64) cudaGraphExecDestroy(w.graph64);
     if (w.graph32) cudaGraphExecDestroy(w.graph32);
@@ -883,11 +936,12 @@ spmv_status_t cg_timing(spmv_matrix_t A, int iters, double *out, cudaStream_t st
             s = cuda_status(cudaEventRecord(e[0], st));
             if (s != SPMV_OK) break;
             if (k == 0)
-                s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, st, &pq_count);
+                s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, IterForm::kAlone, st,
+                                       &pq_count);
             else if (k == 1)
                 s = enqueue_xr<double>(A, pq_count, w.x.p, w.r.p, w.p.p, w.q.p, w.dinv.p, sc,
-                                       false, st);
-            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, false, st);
+                                       IterForm::kAlone, st);
+            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, IterForm::kAlone, st);
             if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e[1], st));
             if (s == SPMV_OK) s = elapsed(&ms);
             sum[k] += ms;
@@ -969,6 +1023,11 @@ spmv_status_t gb::cg_solve_ex(spmv_matrix_t A, const double *b, double *x,
     NvtxRange nvtx(o.mixed ? "cg_solve/mixed" : "cg_solve/fp64");
     const auto t0 = Clock::now();
     spmv_status_t s = ensure_cg_work(A, o.mixed != 0, st);
+    if (s == SPMV_OK && ctl.running && !A->cg.split.p) {
+        s = A->cg.split.alloc(1, &A->bytes);
+        if (s == SPMV_OK)
+            s = cuda_status(cudaMemsetAsync(A->cg.split.p, 0, sizeof(SplitSums), st));
+    }
     if (s != SPMV_OK) return (res->status = s);
     if (A->opt.autotune && !A->pq_tuned) {
         s = tune_cg_product(A, st);

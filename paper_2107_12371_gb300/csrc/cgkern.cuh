@@ -52,6 +52,23 @@ __device__ __forceinline__ int64_t iter_end(int64_t chunk, int64_t items) {
     const int64_t e = ((int64_t)blockIdx.x + 1) * chunk;
     return e < items ? e : items;
 }
+// The calling thread's place in an IterGrid each of whose CTAs is run by Q smaller ones (a
+// solve beside others, see IterForm); Q = 1: the grid as it is.
+template <int Q>
+struct IterSlot {
+    int cta, id;   // CTA of the grid, thread of it
+    bool in;       // whether the grid has that thread
+    __device__ __forceinline__ explicit IterSlot(int threads) {
+        cta = (int)blockIdx.x / Q;
+        id = (int)(blockIdx.x % Q * blockDim.x + threadIdx.x);
+        in = Q == 1 || id < threads;
+    }
+    __device__ __forceinline__ int64_t begin(int64_t chunk) const { return cta * chunk + id; }
+    __device__ __forceinline__ int64_t end(int64_t chunk, int64_t items) const {
+        const int64_t e = (cta + 1) * chunk;
+        return !in ? 0 : e < items ? e : items;
+    }
+};
 // What an iteration leaves in L2 for the next one.  The matrix is streamed evict-first unless it
 // and the vectors fit (three quarters of) the L2 together; the vectors that a FP32 sweep is the
 // last to touch are, unless the five vectors take no more than half of it.  Per FP32 iteration,
@@ -260,13 +277,49 @@ __device__ __forceinline__ double sum_parts(const double (&a)[kPartLoads]) {
     return fx_value(fx_warp<kPartLoads>(a));
 }
 
-// The CTA's sums of v to part[k * ctas + cta].
-template <int NV, typename T>
-__device__ __forceinline__ void store_parts(const T (&v)[NV], double *part) {
-    __shared__ FoldSmem<NV> sm;
-    const double s = fold_block<NV>(v, blockDim.x, sm);
+// Where the CTAs that share one of an IterGrid leave their warps' sums.
+struct SplitSums {
+    int4 fx[32 * kPartLoads][2][kIterThreads / 32];
+    unsigned arrived[32 * kPartLoads];
+};
+
+// The sums of v over a CTA of the grid, to part[k * ctas + cta].  Of Q CTAs that share it the last
+// one to arrive adds what all their warps left, in the order and with the bits of a single one.
+template <int Q, int NV, typename T>
+__device__ __forceinline__ void store_parts(const IterSlot<Q> &slot, int threads, const T (&v)[NV],
+                                            SplitSums *split, double *part) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp < NV && lane == 0) part[warp * gridDim.x + blockIdx.x] = s;
+    if constexpr (Q == 1) {
+        __shared__ FoldSmem<NV> sm;
+        const double s = fold_block<NV>(v, blockDim.x, sm);
+        if (warp < NV && lane == 0) part[warp * gridDim.x + blockIdx.x] = s;
+    } else {
+        __shared__ bool last;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const T one[1] = {v[k]};
+            const Fx f = fx_warp<1>(one);
+            if (lane == 0 && slot.in)
+                split->fx[slot.cta][k][slot.id >> 5] = make_int4(f.l0, f.l1, f.l2, f.e);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(&split->arrived[slot.cta], 1u) == Q - 1;
+            if (last) split->arrived[slot.cta] = 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (last && warp < NV) {
+            Fx f = {0, 0, 0, 0};
+            if (32 * lane < threads) {
+                const int4 q = ld_l2(&split->fx[slot.cta][warp][lane]);
+                f = {q.x, q.y, q.z, q.w};
+            }
+            const double s = fx_value(fx_combine(f));
+            if (lane == 0) part[warp * (gridDim.x / Q) + slot.cta] = s;
+        }
+    }
 }
 
 // The scalars of an iteration from its sums, computed by one thread of each CTA and shared: an

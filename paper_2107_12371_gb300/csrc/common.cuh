@@ -54,10 +54,10 @@ inline spmv_status_t cuda_status(cudaError_t e) {
 #define GB_LAUNCHED() GB_CUDA(cudaGetLastError())
 
 // Launches a kernel that begins with dep_wait so that it may start while the kernel before it on
-// the stream still runs (also as an edge of a captured graph).
+// the stream still runs (also as an edge of a captured graph); plainly if not `dependent`.
 template <typename... K, typename... A>
-spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t st,
-                               A... args) {
+spmv_status_t launch_ordered(bool dependent, void (*kern)(K...), unsigned grid, unsigned block,
+                             cudaStream_t st, A... args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -66,8 +66,13 @@ spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block
     cfg.blockDim = dim3(block);
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
     return cuda_status(cudaLaunchKernelEx(&cfg, kern, K(args)...));
+}
+template <typename... K, typename... A>
+spmv_status_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t st,
+                               A... args) {
+    return launch_ordered(true, kern, grid, block, st, args...);
 }
 
 // Stream on which handle buffers are allocated and freed (stream-ordered allocator), set for
@@ -140,12 +145,15 @@ struct CgScalars {
     long long budget_ns;            // persistent kernel: wall-clock budget (0 = none)
 };
 
+struct SplitSums;  // cgkern.cuh
+
 // Work vectors of a CG solve (allocated on first use, kept with the handle).
 struct CgWork {
     DevBuf<double> x, r, p, q, dinv;
     DevBuf<float> r32, p32, q32, d32, dinv32;
     DevBuf<double> part;        // per-CTA partial sums
     DevBuf<double> scal;        // two CgScalars blocks (outer / inner)
+    DevBuf<SplitSums> split;    // solves beside others (see cg.cu)
     DevBuf<double> zp;          // persistent kernel, resident form: (D^-1 r, p) of every row
     DevBuf<float> zp32;
     DevBuf<ulonglong2> slots;   // persistent kernel: what each CTA posts to the others
@@ -281,6 +289,10 @@ struct SolveControl {
     // same kernels launched directly (for one-off handles: capturing, instantiating and
     // destroying a graph per handle was measured to stall concurrent solves)
     bool graphs = true;
+    // direct launches: solves in progress, this one among them, looked at once per batch.  While
+    // there are several, the iteration runs in the form that leaves them room (same bits)
+    const std::atomic<int> *running = nullptr;
+    bool high_priority = false;  // the stream's priority is above the others'
 };
 spmv_status_t cg_solve_ex(spmv_matrix_t A, const double *b, double *x, const cg_options_t *opt,
                           cg_result_t *result, cudaStream_t st, const SolveControl &ctl);

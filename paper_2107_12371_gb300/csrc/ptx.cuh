@@ -205,6 +205,13 @@ __device__ __forceinline__ double ld_l2(const double *p) {
     return v;
 }
 
+__device__ __forceinline__ int4 ld_l2(const int4 *p) {
+    int4 v;
+    asm volatile("ld.global.cg.v4.s32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 // Gathers (weak ld.global, L1 allocating) for vectors that other CTAs rewrite during the same
 // kernel, between grid barriers whose fences order the writes before these loads.
 __device__ __forceinline__ double ld_x_coherent(const double *p) {

@@ -79,7 +79,7 @@ struct spmv_server_s {
     std::deque<gb::Request *> queue;
     std::unordered_map<uint64_t, gb::Request *> all;
     size_t bytes_in_use = 0, peak = 0;
-    int active = 0;
+    std::atomic<int> active{0};  // changed under mu; solves in progress look at it
     uint64_t next_ticket = 1, submitted = 0, completed = 0, rejected = 0, cancelled = 0;
     std::vector<double> latencies;
     double setup_s = 0, solve_s = 0, teardown_s = 0;
@@ -107,7 +107,7 @@ std::deque<Request *>::iterator admissible(spmv_server_t S) {
     return S->queue.end();
 }
 
-void run_request(Request *r, cudaStream_t st) {
+void run_request(spmv_server_t S, Request *r, cudaStream_t st, bool high_priority) {
     AllocStream scope(st);
     NvtxRange nvtx("server/request");
     auto t0 = Clock::now();
@@ -139,6 +139,8 @@ void run_request(Request *r, cudaStream_t st) {
         SolveControl ctl;
         ctl.cancel = &r->cancel;
         ctl.graphs = false;  // a request's handle solves once: launch its kernels directly
+        ctl.running = &S->active;
+        ctl.high_priority = high_priority;
         s = cg_solve_ex(A, d_b, d_x, &co, &r->result, st, ctl);
         r->solve_s = since(t0);
         t0 = Clock::now();
@@ -191,8 +193,9 @@ void worker(spmv_server_t S) {
         }
         r->t_start = Clock::now();
         const size_t pb = S->priority_bytes.load(std::memory_order_relaxed);
-        cudaStream_t use = (pb > 0 && r->est_bytes >= pb && st_hi) ? st_hi : st;
-        if (use) run_request(r, use);
+        const bool high = pb > 0 && r->est_bytes >= pb && st_hi;
+        cudaStream_t use = high ? st_hi : st;
+        if (use) run_request(S, r, use, high);
         else r->status = SPMV_ERR_CUDA;
         r->t_done = Clock::now();
         {

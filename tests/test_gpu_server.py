@@ -300,3 +300,33 @@ def test_large_requests_equal_a_solve_of_their_own(mixed, edge):
             assert np.array_equal(got, x.cpu().numpy())
     finally:
         capi.spmv_server_destroy(srv)
+
+
+@pytest.mark.parametrize("threshold", [0, 1])
+@pytest.mark.parametrize("mixed,edge", [(0, 29), (0, 30), (0, 37), (0, 45), (1, 37), (1, 40), (1, 50)])
+def test_solves_beside_others_equal_a_solve_of_their_own(mixed, edge, threshold):
+    """Kernels that four CTAs run in the place of one while other solves are in progress, at the
+    default priority and (threshold 1) as prioritised requests: grids just below and above the
+    size from which that is done, a vector or several per thread, FP64 and FP32.  Three requests
+    at once, a small one keeping the server busy beside the last: the bits of cg_solve."""
+    m, rng = meshgen.kuhn_tet_matrix_fast(edge, seed=4, dirichlet=True)
+    b = meshgen.uniform_vectors(rng, m.n)
+    A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values,
+                    precision=capi.SPMV_PREC_DUAL if mixed else capi.SPMV_PREC_FP64)
+    x = torch.zeros(m.n, dtype=torch.float64, device="cuda")
+    want = A.solve(torch.from_numpy(b).cuda(), x, rtol=1e-8, mixed=mixed)
+    (ms, bs), = requests([2e4], seed0=7)
+    srv = capi.spmv_server_create(8 << 30, 4)
+    try:
+        capi.spmv_server_set_priority_bytes(srv, threshold)
+        endless = capi.cg_default_options(rtol=0.0, max_iter=10 ** 7)
+        busy = capi.spmv_server_submit(srv, ms.n, ms.row_ptr, ms.col_idx, ms.values, bs, endless)
+        opt = capi.cg_default_options(rtol=1e-8, mixed=mixed)
+        tickets = [capi.spmv_server_submit(srv, m.n, m.row_ptr, m.col_idx, m.values, b, opt)
+                   for _ in range(3)]
+        for got, r in wait_all(srv, tickets, [m] * 3):
+            assert r["status"] == capi.SPMV_OK and r["iterations"] == want["iterations"]
+            assert np.array_equal(got, x.cpu().numpy())
+        capi.spmv_server_cancel(srv, busy)
+    finally:
+        capi.spmv_server_destroy(srv)
