@@ -320,9 +320,10 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
             }
             return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
                                     A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
+        } else {
+            return launch_dependent(spmv_sell<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
+                                    A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
         }
-        return launch_dependent(spmv_sell<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
-                                A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
     };
     if (A->index_bits == 16) return go(Cols16{A->sell_col16.p, A->col_start.p});
     return go(Cols32{A->sell_col.p});
