@@ -1,13 +1,13 @@
-// autotune.cu -- picks the slice height S, the CTA size and the product variant of a handle by
-// timing every candidate on the matrix itself with x = 1 (CUDA events, median of 5 launches
-// after 2 warm-up launches, L2 overwritten before each timed launch).  Each slice height needs
-// its own sliced-ELLPACK arrays, so the arrays are rebuilt per candidate and finally for the
-// winner.  Candidates: S in {32, 64, 128, 256}
-// (S = 512 of the FPGA design is a pipelining depth, Sec. 6.1, and has no GPU meaning),
-// CTA sizes {128, 256, 512}, the matrix staged by bulk copies, the shared-memory window
-// variant, and the naive CSR kernel (FP64 handles).
+// autotune.cu -- picks the slice height S and the form, CTA size and variant of a handle's product
+// by timing every candidate on the matrix itself with x = 1 (CUDA events; launches in a row, and
+// single ones with the L2 overwritten before each).  Each slice height needs its own
+// sliced-ELLPACK arrays, so the arrays are rebuilt per candidate and finally for the winner.
+// Candidates: S in {32, 64, 128, 256} (S = 512 of the FPGA design is a pipelining depth, Sec. 6.1,
+// and has no GPU meaning), the two forms of the sliced product (spmv.cu), CTA sizes {128, 256, 512}
+// where the form's kernel leaves the size open, the matrix staged by bulk copies, the shared-memory
+// window variant, and the naive CSR kernel (FP64 handles).  A handle of both precisions is tuned by
+// its FP64 product, and the form of its FP32 product at the height that gives.
 #include <algorithm>
-#include <vector>
 
 #include "common.cuh"
 
@@ -23,28 +23,36 @@ __global__ void fill_ones(size_t n, double *x64, float *x32) {
     }
 }
 
-// median of 5 launches after 2 warm-up launches, each timed launch after writing a buffer of
-// twice the L2 size, so that the matrix and x come from DRAM as in steady use
-spmv_status_t time_launch(spmv_matrix_t A, const void *x, void *y, void *flush, size_t fb,
+// Time of a product as programs call it: one launch with nothing in the caches (mean of the eight
+// fastest of ten, each after writing a buffer of twice the L2 size) plus one of ten in a row.  Forms
+// differ in both: FP64, 1.3M rows, strided 20.9 and 16.8 us, thin 21.9 and 13.9.  (Events resolve 2
+// us: candidates that close are told apart by the mean only.)
+spmv_status_t time_launch(spmv_matrix_t A, bool f32, const void *x, void *y, void *flush, size_t fb,
                           cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, float *ms_out) {
     auto launch = [&]() -> spmv_status_t {
-        if (A->has64()) return launch_spmv64(A, (const double *)x, (double *)y, st);
-        return launch_spmv32(A, (const float *)x, (float *)y, st);
+        if (f32) return launch_spmv32(A, (const float *)x, (float *)y, st);
+        return launch_spmv64(A, (const double *)x, (double *)y, st);
     };
+    constexpr int kTimed = 10, kKept = 8;
+    float t[kTimed], row = 0.f;
     for (int i = 0; i < 2; ++i) GB_TRY(launch());
-    std::vector<float> t;
-    for (int i = 0; i < 5; ++i) {
+    GB_CUDA(cudaEventRecord(e0, st));
+    for (int i = 0; i < kTimed; ++i) GB_TRY(launch());
+    GB_CUDA(cudaEventRecord(e1, st));
+    GB_CUDA(cudaEventSynchronize(e1));
+    GB_CUDA(cudaEventElapsedTime(&row, e0, e1));
+    for (int i = 0; i < kTimed; ++i) {
         GB_CUDA(cudaMemsetAsync(flush, i + 1, fb, st));
         GB_CUDA(cudaEventRecord(e0, st));
         GB_TRY(launch());
         GB_CUDA(cudaEventRecord(e1, st));
         GB_CUDA(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        GB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        t.push_back(ms);
+        GB_CUDA(cudaEventElapsedTime(&t[i], e0, e1));
     }
-    std::sort(t.begin(), t.end());
-    *ms_out = t[t.size() / 2];
+    std::sort(t, t + kTimed);
+    float sum = 0.f;
+    for (int i = 0; i < kKept; ++i) sum += t[i];
+    *ms_out = sum / kKept + row / kTimed;
     return SPMV_OK;
 }
 
@@ -53,7 +61,8 @@ spmv_status_t time_launch(spmv_matrix_t A, const void *x, void *y, void *flush, 
 spmv_status_t autotune_matrix(spmv_matrix_t A, cudaStream_t st) {
     if (A->n == 0) return SPMV_OK;
     NvtxRange nvtx("spmv_create/autotune");
-    const size_t eb = A->has64() ? sizeof(double) : sizeof(float);
+    const bool f32 = !A->has64();
+    const size_t eb = f32 ? sizeof(float) : sizeof(double);
     void *x = nullptr, *y = nullptr;
     const size_t nx = (size_t)(A->n_cols > 0 ? A->n_cols : 1);
     GB_CUDA(gb_malloc_async(&x, eb * nx, st));
@@ -74,30 +83,39 @@ spmv_status_t autotune_matrix(spmv_matrix_t A, cudaStream_t st) {
     const int blocks[] = {128, 256, 512};
     float best = 1e30f;
     int best_S = A->S, best_block = A->block, best_variant = SPMV_VARIANT_SELL;
+    int best_form = kFormBySize;
     const int user_variant = A->opt.variant;
     for (int S : heights) {
         if (s != SPMV_OK) break;
         s = build_sell(A, S, st);
         if (s != SPMV_OK) break;
-        for (int b : blocks) {
-            A->block = b;
-            A->variant = SPMV_VARIANT_SELL;
-            float ms;
-            s = time_launch(A, x, y, flush, fb, st, e0, e1, &ms);
-            if (s != SPMV_OK) break;
-            if (ms < best) {
-                best = ms;
-                best_S = S;
-                best_block = b;
-                best_variant = SPMV_VARIANT_SELL;
+        A->variant = SPMV_VARIANT_SELL;
+        for (int form : {kFormThin, kFormStrided}) {
+            A->spmv_form[f32] = form;
+            int timed = 0;  // (a kernel with a size of its own is one candidate)
+            for (int b : blocks) {
+                A->block = b;
+                if (product_block(A) == timed) continue;
+                timed = product_block(A);
+                float ms;
+                s = time_launch(A, f32, x, y, flush, fb, st, e0, e1, &ms);
+                if (s != SPMV_OK) break;
+                if (ms < best) {
+                    best = ms;
+                    best_S = S;
+                    best_block = b;
+                    best_form = form;
+                    best_variant = SPMV_VARIANT_SELL;
+                }
             }
+            if (s != SPMV_OK) break;
         }
         if (s != SPMV_OK) break;
         if (user_variant == SPMV_VARIANT_AUTO || user_variant == SPMV_VARIANT_SELL_BULK) {
             // matrix staged through shared memory by bulk copies (one CTA per SM)
             A->variant = SPMV_VARIANT_SELL_BULK;
             float ms;
-            s = time_launch(A, x, y, flush, fb, st, e0, e1, &ms);
+            s = time_launch(A, f32, x, y, flush, fb, st, e0, e1, &ms);
             if (s != SPMV_OK) break;
             if (ms < best) {
                 best = ms;
@@ -109,7 +127,7 @@ spmv_status_t autotune_matrix(spmv_matrix_t A, cudaStream_t st) {
             // shared-memory window of x (one 1024-thread CTA per SM)
             A->variant = SPMV_VARIANT_SELL_WINDOW;
             float ms;
-            s = time_launch(A, x, y, flush, fb, st, e0, e1, &ms);
+            s = time_launch(A, f32, x, y, flush, fb, st, e0, e1, &ms);
             if (s != SPMV_OK) break;
             if (ms < best) {
                 best = ms;
@@ -121,7 +139,7 @@ spmv_status_t autotune_matrix(spmv_matrix_t A, cudaStream_t st) {
     if (s == SPMV_OK && A->has64() && user_variant == SPMV_VARIANT_AUTO) {
         A->variant = SPMV_VARIANT_CSR;
         float ms;
-        s = time_launch(A, x, y, flush, fb, st, e0, e1, &ms);
+        s = time_launch(A, f32, x, y, flush, fb, st, e0, e1, &ms);
         if (s == SPMV_OK && ms < best) {
             best = ms;
             best_variant = SPMV_VARIANT_CSR;
@@ -129,6 +147,26 @@ spmv_status_t autotune_matrix(spmv_matrix_t A, cudaStream_t st) {
     }
     if (s == SPMV_OK && best_S != A->S) s = build_sell(A, best_S, st);
     A->block = best_block;
+    A->spmv_form[f32] = best_form;
+    if (s == SPMV_OK && A->has64() && A->has32()) {  // the other precision's form
+        A->variant = SPMV_VARIANT_SELL;
+        fill_ones<<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, st>>>(
+            nx, nullptr, (float *)x);
+        s = cuda_status(cudaGetLastError());
+        float fastest = 1e30f;
+        int pick = kFormBySize;
+        for (int form : {kFormThin, kFormStrided}) {
+            if (s != SPMV_OK) break;
+            float ms;
+            A->spmv_form[1] = form;
+            s = time_launch(A, true, x, y, flush, fb, st, e0, e1, &ms);
+            if (s == SPMV_OK && ms < fastest) {
+                fastest = ms;
+                pick = form;
+            }
+        }
+        A->spmv_form[1] = pick;
+    }
     if (user_variant == SPMV_VARIANT_AUTO) A->variant = best_variant;
     else A->variant = user_variant;
     A->window_words = A->variant == SPMV_VARIANT_SELL_WINDOW

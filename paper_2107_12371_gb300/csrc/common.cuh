@@ -170,6 +170,8 @@ struct CgWork {
 
 struct McgWork;  // multi-right-hand-side CG work (mcg.cu)
 
+enum { kFormBySize, kFormThin, kFormStrided };  // spmv.cu
+
 }  // namespace gb
 
 struct spmv_matrix_s {
@@ -213,6 +215,8 @@ struct spmv_matrix_s {
     int pq_ctas = 0;             // CG product grid: CTAs per SM (0: pq_min_ctas)
     int pq_unroll = 0;           // CG product entries in flight (0: by load rounds)
     bool pq_tuned = false;       // pq_ctas / pq_unroll chosen by the tuner
+    // form of the single-vector product per precision (0 FP64, 1 FP32) chosen by the tuner
+    int spmv_form[2] = {};       // kFormBySize, kFormThin, kFormStrided
     // SpMM form per precision (0 FP64, 1 FP32) and lanes per row (1, 2, 4, 8) chosen by the
     // tuner on the first multi-vector product of that shape (SPMV_SPMM_AUTO: not tuned)
     int spmm_tuned[2][4] = {};
@@ -255,6 +259,8 @@ spmv_status_t launch_axpby64(spmv_matrix_t A, double alpha, const double *x, dou
 spmv_status_t launch_axpby32(spmv_matrix_t A, float alpha, const float *x, float beta, float *y,
                              cudaStream_t st);
 spmv_status_t launch_spmv32(spmv_matrix_t A, const float *x, float *y, cudaStream_t st);
+bool product_is_thin(const spmv_matrix_t A, bool f32);
+int product_block(const spmv_matrix_t A);
 spmv_status_t launch_spmv_csr64(spmv_matrix_t A, const double *x, double *y, cudaStream_t st);
 spmv_status_t launch_spmm64(spmv_matrix_t A, int k, const double *X, double *Y, cudaStream_t st);
 spmv_status_t launch_spmm32(spmv_matrix_t A, int k, const float *X, float *Y, cudaStream_t st);

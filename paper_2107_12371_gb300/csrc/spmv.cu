@@ -9,11 +9,11 @@
 //   in ascending column order with fused multiply-add from +0.0; padding entries (column -1)
 //   are skipped.  Column indices come as int32 or (when every slice spans fewer than 65,535
 //   columns) as 16-bit offsets from the slice's col_start (Sec. 5.1), 10 instead of 12 bytes
-//   per FP64 non-zero.  All FP32 products, and the FP64 ones up to a few million rows (use_thin).
-// spmv_sell_occ / spmv_sell_gs: FP64 products of larger matrices at one or two rows per lane, one
-//   slice-lane per thread at 32 registers, or a grid of four CTAs per SM striding over the
-//   slice-lanes with five entries of each row in flight; the one whose widest slice needs fewer
-//   dependent load rounds is launched.  spmv_sell: the same at four or eight rows per lane.
+//   per FP64 non-zero.  Matrices up to a few million rows (use_thin).
+// spmv_sell_gs / spmv_sell_occ: larger matrices, one or two rows per lane in FP64 and four in FP32;
+//   a grid of four CTAs per SM striding over the slice-lanes with five entries of each row in
+//   flight, or (FP64) one slice-lane per thread at 32 registers; the one whose widest slice needs
+//   fewer dependent load rounds is launched.  spmv_sell: FP64 at four or eight rows per lane.
 // spmv_csr: the naive baseline of Sec. 4.3, thread per CSR row.
 #include <type_traits>
 
@@ -123,7 +123,7 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
                                             n_slices, sp, cols, val, x, y, alpha, beta);
 }
 
-// FP64 with one or two rows per lane: a grid of at most kGsCtasPerSm 256-thread CTAs per SM
+// One or two rows per lane (FP32 four): a grid of at most kGsCtasPerSm 256-thread CTAs per SM
 // strides over the slice-lanes, each thread keeping U = 5 entries of its rows in flight (a
 // whole row of the tetrahedral meshes) at 64 registers.  Measured on the 6M-row mesh (S = 64):
 // 66.3 us, against 69.6 us for one slice-lane per thread at 32 registers and 2,048 threads per
@@ -293,30 +293,43 @@ inline unsigned grid_for(int64_t threads, int block) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// The FP64 products of larger matrices; (R, L) per slice height: lanes read 8 R bytes of values per
-// entry (16 B at S = 64, 32 B at S = 128).
+// A matrix of which a product leaves nothing in L2 for the next one.
+template <typename T>
+bool beyond_l2(const spmv_matrix_t A) {
+    return (double)A->sell_entries * (sizeof(T) + A->index_bits / 8) >
+           2.0 * device_facts().l2_bytes;
+}
+
+// Whether the strided form of FP64 rows at one or two per lane is spmv_sell_gs (else _occ).
+bool strided_rows(const spmv_matrix_t A) {
+    return load_rounds(A->max_width, 5) < load_rounds(A->max_width, 4);
+}
+
+// The products of larger matrices; (R, L) per slice height: lanes read 8 R bytes of values per
+// entry in FP64 (16 B at S = 64, 32 B at S = 128), 16 in FP32.
 template <typename T, int R, int L, int U, bool AXPBY>
 spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, T beta,
                       cudaStream_t st) {
     const int block = A->block;
     const unsigned grid = grid_for((int64_t)A->n_slices * L, block);
+    auto strided = [&](auto c, auto aheadt) -> spmv_status_t {
+        const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
+        const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
+        return launch_dependent(spmv_sell_gs<T, R, L, 5, decltype(c), AXPBY, decltype(aheadt)::value>,
+                                (int64_t)want < cap ? want : (unsigned)cap, kGsBlock, st, A->n,
+                                A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
+    };
     auto go = [&](auto c) -> spmv_status_t {
         using ColT = decltype(c);
-        if constexpr (R <= 2) {
-            if (load_rounds(A->max_width, 5) < load_rounds(A->max_width, 4)) {
-                const int64_t cap = (int64_t)device_facts().sm_count * kGsCtasPerSm;
-                const unsigned want = grid_for((int64_t)A->n_slices * L, kGsBlock);
-                const unsigned g = (int64_t)want < cap ? want : (unsigned)cap;
+        if constexpr (sizeof(T) == 4) {  // (ahead, 10.4M rows: 61.7 us cold and 61.3 in a row, without 60.9 and 62.0)
+            return strided(c, std::false_type{});
+        } else if constexpr (R <= 2) {
+            if (strided_rows(A)) {
                 // (not where x is gathered from all over: the entries then drive x out of L2, 6M rows
                 // in random order 111 -> 130 us)
-                const double l2 = device_facts().l2_bytes;
-                const bool ahead =
-                    (double)A->sell_entries * (sizeof(T) + A->index_bits / 8) > 2.0 * l2 &&
-                    (double)A->max_span * sizeof(T) < l2 / 16;
-                auto *kern = ahead ? spmv_sell_gs<T, R, L, 5, ColT, AXPBY, true>
-                                   : spmv_sell_gs<T, R, L, 5, ColT, AXPBY, false>;
-                return launch_dependent(kern, g, kGsBlock, st, A->n, A->n_slices, A->slice_ptr.p, c,
-                                        val, x, y, alpha, beta);
+                const bool ahead = beyond_l2<T>(A) && (double)A->max_span * sizeof(T) <
+                                                          device_facts().l2_bytes / 16.0;
+                return ahead ? strided(c, std::true_type{}) : strided(c, std::false_type{});
             }
             return launch_dependent(spmv_sell_occ<T, R, L, U, ColT, AXPBY>, grid, block, st, A->n,
                                     A->n_slices, A->slice_ptr.p, c, val, x, y, alpha, beta);
@@ -329,12 +342,21 @@ spmv_status_t go_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha, 
     return go(Cols32{A->sell_col.p});
 }
 
-// FP64 products that spmv_sell_thin takes (us, spmv_sell_gs or _occ / thin).  Rows of up to six
-// entries in Cuthill-McKee order: 304K 4.5 / 4.2, 796K 10.5 / 8.7, 3.1M 33.4 / 29.9, 6M 66.3 /
-// 71.1; of two entries (a gradient's faces): 600K 5.3 / 4.5, 2.6M 22.6 / 17.2.  Longer rows: 647K
-// 20.8 / 17.1, 1.8M 44.6 / 43.5, 3M 70.8 / 69.9 but with alpha and beta 82.6 / 84.5.
+// Products that spmv_sell_thin takes, unless the tuner has picked a form for the handle.  Products
+// in a row (us, spmv_sell_gs or _occ / thin): FP64 rows of up to six entries in Cuthill-McKee
+// order 304K 4.5 / 4.2, 796K 10.5 / 8.7, 3.1M 33.4 / 29.9, 6M 66.3 / 71.1; of two entries (a
+// gradient's faces) 600K 5.3 / 4.5, 2.6M 22.6 / 17.2; longer rows 647K 20.8 / 17.1, 1.8M 44.6 /
+// 43.5, 3M 70.8 / 69.9 but with alpha and beta 82.6 / 84.5.  FP32: 3.1M 17.7 / 17.0, 6M 33.5 /
+// 32.4, and beyond the L2, 10.4M, 62.0 / 64.7; longer rows 1.8M 27.6 / 23.8.  With nothing in the
+// caches the line lies lower, since thin's CTAs come and go with their chains of loads (FP64 1.3M
+// 21.9 / 21.9, 3.1M 37.9 / 39.9, FP32 6M 38.7 / 40.7): that is the tuner's to find.
+template <typename T>
 bool use_thin(const spmv_matrix_t A) {
-    return A->n <= (A->max_width > 2 && A->mean_width > 6.f ? 2000000 : 3500000);
+    constexpr bool f32 = sizeof(T) == 4;
+    if (A->spmv_form[f32]) return A->spmv_form[f32] == kFormThin;
+    const bool longer = A->max_width > 2 && A->mean_width > 6.f;
+    if (f32) return longer || A->max_width <= 2 || !beyond_l2<T>(A);
+    return A->n <= (longer ? 2000000 : 3500000);
 }
 
 // Rows per lane, entries in flight and registers of spmv_sell_thin, by the threads that an SM
@@ -423,21 +445,38 @@ template <typename T, bool AXPBY = false>
 spmv_status_t launch_sell(spmv_matrix_t A, const T *val, const T *x, T *y, T alpha = T(1),
                           T beta = T(0), cudaStream_t st = nullptr) {
     if (A->n == 0) return SPMV_OK;
+    if (use_thin<T>(A)) return go_thin<T, AXPBY>(A, val, x, y, alpha, beta, st);
     if constexpr (sizeof(T) == 8) {
-        if (!use_thin(A)) {
-            switch (A->S) {
-                case 32: return go_sell<T, 1, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
-                case 64: return go_sell<T, 2, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
-                case 128: return go_sell<T, 4, 32, 2, AXPBY>(A, val, x, y, alpha, beta, st);
-                case 256: return go_sell<T, 8, 32, 1, AXPBY>(A, val, x, y, alpha, beta, st);
-            }
-            return SPMV_ERR_INVALID_ARG;
+        switch (A->S) {
+            case 32: return go_sell<T, 1, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 64: return go_sell<T, 2, 32, 4, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 128: return go_sell<T, 4, 32, 2, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 256: return go_sell<T, 8, 32, 1, AXPBY>(A, val, x, y, alpha, beta, st);
+        }
+    } else {
+        switch (A->S) {
+            case 32: return go_sell<T, 4, 8, 5, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 64: return go_sell<T, 4, 16, 5, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 128: return go_sell<T, 4, 32, 5, AXPBY>(A, val, x, y, alpha, beta, st);
+            case 256: return go_sell<T, 4, 64, 5, AXPBY>(A, val, x, y, alpha, beta, st);
         }
     }
-    return go_thin<T, AXPBY>(A, val, x, y, alpha, beta, st);
+    return SPMV_ERR_INVALID_ARG;
 }
 
 }  // namespace
+
+bool product_is_thin(const spmv_matrix_t A, bool f32) {
+    return f32 ? use_thin<float>(A) : use_thin<double>(A);
+}
+
+// CTA size of the product (the handle's first precision); A->block where the kernel leaves it open.
+int product_block(const spmv_matrix_t A) {
+    const bool f32 = !A->has64();
+    if (A->variant != SPMV_VARIANT_SELL) return A->block;
+    if (product_is_thin(A, f32)) return A->block < kThinBlock ? A->block : kThinBlock;
+    return f32 || (A->S <= 64 && strided_rows(A)) ? kGsBlock : A->block;
+}
 
 spmv_status_t launch_spmv64(spmv_matrix_t A, const double *x, double *y, cudaStream_t st) {
     if (A->variant == SPMV_VARIANT_CSR) return launch_spmv_csr64(A, x, y, st);

@@ -919,3 +919,39 @@ def test_c2_full_size_parity(oracle, reorder, bits, variant):
     ref32 = oracle.spmv_f32(ro, co, np.asarray(vo).astype(np.float32), x32, use_fma=True)
     assert np.array_equal(y32, ref32)
     assert capi.spmv_device_status(A.handle) == capi.SPMV_OK
+
+
+@pytest.mark.parametrize("S", [32, 64, 128, 256])
+def test_fp32_products_beyond_the_l2(oracle, S):
+    """FP32 matrices of more than twice the L2 take the strided kernel at four rows per lane: rows of
+    0 to 6 entries (slices of width 6: a round of five and one more), a ragged last slice; plain and
+    with alpha and beta, bit for bit."""
+    n, offsets = 6000017, np.array([-977, -31, -1, 0, 2, 40])
+    rng = np.random.default_rng(S)
+    j = np.arange(n, dtype=np.int64)[:, None] + offsets
+    has = (rng.random((n, 6)) < 0.6) & (j >= 0) & (j < n)
+    rp = np.zeros(n + 1, np.int64)
+    rp[1:] = np.cumsum(has.sum(1))
+    ci = j[has].astype(np.int32)
+    v = rng.uniform(-1, 1, ci.size)
+    x = rng.uniform(-1, 1, n).astype(np.float32)
+    y0 = rng.uniform(-1, 1, n).astype(np.float32)
+    A = capi.Matrix(n, rp, ci, v, precision=capi.SPMV_PREC_FP32, slice_height=S, index_bits=32)
+    l2 = torch.cuda.get_device_properties(0).L2_cache_size
+    assert 8 * A.info()["sell_entries"] > 2 * l2
+    t = oracle.spmm(rp, ci, v.astype(np.float32), x[:, None], use_fma=True)[:, 0]
+    xd, y = dev(x), torch.full((n,), float("nan"), device="cuda")
+    A.apply_f32(xd, y)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), t)
+    y = torch.full((n,), float("nan"), device="cuda")
+    A.apply_axpby(0.75, xd, 0.0, y)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), np.float32(0.75) * t)
+    y = dev(y0)
+    A.apply_axpby(0.75, xd, 0.5, y)
+    torch.cuda.synchronize()
+    # fma(0.75, t, 0.5 y) rounds once; here the sum is rounded to FP64 and then to FP32
+    want = (0.75 * t.astype(np.float64) + 0.5 * y0.astype(np.float64)).astype(np.float32)
+    assert np.all(np.abs(y.cpu().numpy() - want) <= np.spacing(np.abs(want)))
+    A.close()
