@@ -71,15 +71,16 @@ typedef enum {
 
 typedef struct {
     int slice_height;    /* S, rows per slice: 32, 64, 128 or 256 (0 = default 64)            */
-    int block;           /* threads per CTA for the SpMV kernels that take one slice-lane per
-                          * thread: 64..1024, multiple of 32 (0 = 256; at most 128 are used for
-                          * matrices that do not fill the GPU).  The FP64 kernel that
-                          * strides over the slice-lanes with five entries in flight (chosen when
-                          * the widest slice needs fewer load rounds that way) uses 256. */
+    int block;           /* threads per CTA: 64..1024, multiple of 32 (0 = 256), for the FP64
+                          * kernels of matrices past some two million rows that take one
+                          * slice-lane per thread.  The kernel of smaller matrices uses at most
+                          * 128 of them; the one that strides over the slice-lanes with five
+                          * entries in flight (FP64 when the widest slice needs fewer load rounds
+                          * that way, FP32 past twice the L2, or the tuner's choice) uses 256. */
     int variant;         /* SPMV_VARIANT_*                                                   */
     int reorder;         /* SPMV_REORDER_*                                                   */
     int precision;       /* SPMV_PREC_*                                                      */
-    int autotune;        /* 1: time the candidate (S, block, variant) on this matrix and keep the fastest */
+    int autotune;        /* 1: time the candidates (S, form, block, variant) on this matrix, keep the fastest */
     int peripheral;      /* 1: George-Liu pseudo-peripheral start node for (R)CM             */
     int window_words;    /* SELL_WINDOW capacity in x entries per CTA (0 = largest that fits) */
     int index_bits;      /* 0 = 16 when every slice spans < 65,535 columns, else 32;

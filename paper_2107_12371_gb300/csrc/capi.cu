@@ -250,7 +250,7 @@ spmv_status_t spmv_get_info(spmv_matrix_t A, spmv_info_t *info) {
     info->n_cols = A->n_cols;
     info->nnz = A->nnz;
     info->slice_height = A->S;
-    info->block = A->block;
+    info->block = product_block(A);
     info->variant = A->variant;
     info->precision = A->opt.precision;
     info->reorder = A->opt.reorder;

@@ -193,3 +193,23 @@ def test_tuned_handles_with_16_bit_columns_keep_the_bits(size, precision):
         out.append(y)
         A.close()
     assert torch.equal(out[0], out[1])
+
+
+def test_reported_block_is_the_kernels():
+    """spmv_get_info's CTA size is that of the product's kernel, not the option it ignores: a small
+    matrix (at most 128 threads), FP64 past 3.5M rows of five entries (256, strided) and of four
+    (the option: four entries in flight are one round, five four)."""
+    m, _ = workloads.kuhn(8, seed=1)
+    for opt, used in ((0, 128), (64, 64), (96, 96), (512, 128)):
+        for precision in (capi.SPMV_PREC_FP64, capi.SPMV_PREC_FP32):
+            A = capi.Matrix(m.n, m.row_ptr, m.col_idx, m.values, block=opt, precision=precision)
+            assert A.info()["block"] == used
+            A.close()
+    n = 3500100
+    for w, used in ((5, 256), (4, 512)):
+        rp = np.arange(n + 1, dtype=np.int32) * w
+        ci = (np.arange(n, dtype=np.int32)[:, None] // w * w)[:, :1] + np.arange(w, dtype=np.int32)
+        A = capi.Matrix(n, rp, np.minimum(ci, n - w + np.arange(w, dtype=np.int32)).ravel(),
+                        np.ones(n * w), block=512)
+        assert A.info()["block"] == used
+        A.close()
