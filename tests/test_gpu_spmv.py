@@ -955,3 +955,21 @@ def test_fp32_products_beyond_the_l2(oracle, S):
     want = (0.75 * t.astype(np.float64) + 0.5 * y0.astype(np.float64)).astype(np.float32)
     assert np.all(np.abs(y.cpu().numpy() - want) <= np.spacing(np.abs(want)))
     A.close()
+
+
+@pytest.mark.parametrize("peripheral", [0, 1])
+def test_gpu_cm_order_of_nodes_with_many_children(oracle, peripheral):
+    """Hubs of 8 to 18 leaves, some of 40 and 300, in a chain and of unlike degrees: more children
+    than are sorted in registers, by insertion and by heap."""
+    rng = np.random.default_rng(3)
+    size = np.array([8, 9, 10, 15, 16, 17, 18, 40, 300])[np.arange(300) % 9]
+    hub = np.concatenate([[0], np.cumsum(size)])
+    n = hub[-1] + 1
+    leaf = np.arange(hub[-1])
+    edges = np.concatenate([np.stack([np.repeat(hub[:-1], size), leaf], 1),
+                            np.stack([hub[:-1], hub[1:]], 1), rng.integers(0, n, (n // 8, 2))])
+    p = rng.permutation(n)
+    rp, ci, v = graph_csr(n, p[edges])
+    A = capi.Matrix(n, rp, ci, v, reorder=capi.SPMV_REORDER_CM, peripheral=peripheral)
+    ref = oracle.cm_order(rp, ci, reverse=False, peripheral=bool(peripheral))
+    assert np.array_equal(A.permutation(), ref)
