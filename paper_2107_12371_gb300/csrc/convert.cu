@@ -97,6 +97,21 @@ constexpr int kCmBatch = 6;     // row entries in flight per thread
 constexpr int kCmComponents = 256;  // components that one launch orders
 constexpr int kCmQueue = 4096;  // frontier nodes that a CTA keeps in shared memory
 constexpr int kCmKids = 8;      // children of a node sorted in registers; more are sorted in memory
+// Row entries per level, on average from the first one on, from which a component's levels go to
+// the whole GPU.  A level costs a handful of launches and a read-back there (some 60 us), while the
+// cluster's 16 SMs take some 0.2 ns per entry and level.  Whole set-up of connected random graphs, in
+// ms, all levels launched from the host / all in the cluster / as here: 1M nodes of 7 entries 5.3 /
+// 7.2 / 4.3, 4M 13.9 / 25.7 / 10.3, 300K of 43 14.6 / 21.1 / 8.7, 1M of 23 13.0 / 33.9 / 10.3.
+constexpr int64_t kCmWide = 400000;
+
+// How far an order has got.  A launch of cm_cluster ends early when it meets a component with wide
+// levels: `wide` says whether while looking for its start node (from `start`) or between levels of
+// its order, and then [ls, le) are the last level's positions.
+enum { kCmNarrow, kCmWideSearch, kCmWideOrder };
+struct CmProgress {
+    int64_t placed, ls, le;
+    int32_t bfs_id, spilled, wide, start;
+};
 
 // Smallest key that each CTA of the cluster found, in every CTA; two sets in turn, so that one can
 // be written while another CTA still reads the last one.
@@ -121,6 +136,7 @@ struct CmWalk {
     const int32_t *rp, *ci, *deg;
     int32_t *claim, *stamp, *queue, *perm;
     int32_t *spilled;  // BFS nodes in `queue`, those that found their CTA's frontier full
+    int row;           // mean row entries
     CmKeys *keys;
     CmFrontier *front;
     cg::cluster_group cluster;
@@ -167,10 +183,15 @@ struct CmWalk {
         return best;
     }
 
+    // Whether `levels` levels of `nodes` nodes together are too wide for the cluster.
+    __device__ __forceinline__ bool wide(int64_t nodes, int64_t levels_) const {
+        return nodes * row > kCmWide * levels_;
+    }
+
     // BFS levels from r over nodes without a position: the number of levels, and the node of
-    // the last one with the smallest key.  Ids grow, and a stamp only grows, so that one atomicMax
+    // the last one with the smallest key; false if they are too wide.  Ids grow, and a stamp only grows, so that one atomicMax
     // tells whether a node is new; it then goes to the CTA that its index hashes to.
-    __device__ __forceinline__ void bfs(int32_t r, int32_t id, int32_t *ecc, int32_t *pick) {
+    __device__ __forceinline__ bool bfs(int32_t r, int32_t id, int32_t *ecc, int32_t *pick) {
         const int ranks = (int)cluster.num_blocks(), lane = threadIdx.x & 31;
         const int shift = ranks == 16 ? 28 : 29;
         int mine = 0;  // nodes of the level in this CTA's frontier
@@ -218,10 +239,11 @@ struct CmWalk {
         };
         int last = 0;  // the same of the level before
         int32_t last_ls = 0;
+        int64_t seen = 0;  // nodes of the levels so far
         for (bool first = true;; first = false) {
             const int w = levels % 3;
-            // whether the level has any nodes is needed only once it has been visited
-            const int sent = first ? 1
+            // how many nodes the level has is needed only once it has been visited
+            const int sent = first ? lane == 0
                              : lane < ranks
                                  ? cluster.map_shared_rank(front, lane)->count[(levels + 2) % 3]
                                  : 0;
@@ -232,7 +254,10 @@ struct CmWalk {
                       w);
             if (threadIdx.x == 0) front->count[(levels + 1) % 3] = front->full[(levels + 1) % 3] = 0;
             cluster.sync();
-            if (!__any_sync(0xffffffffu, sent > 0)) break;
+            const int size = __reduce_add_sync(0xffffffffu, sent);
+            if (size == 0) break;
+            seen += size;
+            int64_t known = seen;
             last = mine;
             last_ls = ls;
             const int own = front->count[w];
@@ -241,9 +266,11 @@ struct CmWalk {
             if (front->full[w]) {
                 const int all = lane < ranks ? cluster.map_shared_rank(front, lane)->count[w] : 0;
                 le += __reduce_add_sync(0xffffffffu, all > kCmQueue ? all - kCmQueue : 0);
+                known += __reduce_add_sync(0xffffffffu, all);
             }
             ++depth;
             ++levels;
+            if (wide(known, depth)) return false;
         }
         // the level after the last one was empty
         unsigned long long best = ~0ull;
@@ -255,6 +282,7 @@ struct CmWalk {
         if (gid == 0) *spilled = 0;
         *ecc = depth;
         *pick = (int32_t)(min_key(best) & 0xffffffffull);
+        return true;
     }
 };
 
@@ -392,7 +420,7 @@ __device__ __forceinline__ void cm_place_kids(const CmWalk &w, const CmSet &set,
     for (int t = 0; t < cnt; ++t) set.set(t, w.perm[set.at + t]);
 }
 
-// Cuthill-McKee from position *placed_io on, up to max_components further components (so that a
+// Cuthill-McKee from position io->placed on, up to max_components further components (so that a
 // launch is short whatever the graph), in one thread-block cluster: the levels of a mesh are
 // a few thousand nodes in some hundred steps, so what a level costs is its chain of dependent
 // loads and its barriers.  A cluster barrier is a hardware one, and nothing returns to the host
@@ -407,7 +435,7 @@ template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
 cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, int32_t *claim,
            int32_t *stamp, int32_t *queue, int32_t *perm, int peripheral, int max_components,
-           int64_t *placed_io, int32_t *bfs_id_io, int32_t *spilled) {
+           CmProgress *io) {
     __shared__ CmKeys keys;
     __shared__ CmFrontier front;
     __shared__ int totals[2][kCmCluster];
@@ -416,39 +444,48 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
     const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < 3) front.count[threadIdx.x] = front.full[threadIdx.x] = 0;
-    CmWalk w{n, rp, ci, deg, claim, stamp, queue, perm, spilled, &keys, &front, cluster,
+    CmWalk w{n, rp, ci, deg, claim, stamp, queue, perm, &io->spilled, rp[n] / n + 1, &keys, &front,
+             cluster,
              (int64_t)threadIdx.x * ranks + rank, (int64_t)ranks * THREADS, 0, 0};
-    int32_t placed = (int32_t)*placed_io;
-    int32_t bfs_id = *bfs_id_io;
+    int32_t placed = (int32_t)io->placed;
+    int32_t bfs_id = io->bfs_id;
     const int log_ranks = ranks == 16 ? 4 : 3;
-    if (w.gid == 0) *spilled = 0;
-    int turn = 0;
+    int turn = 0, wide = kCmNarrow;
+    int32_t start = 0, ls = 0, le = 0;
     cluster.sync();
+    if (w.gid == 0) io->spilled = 0;
     for (int comp = 0; comp < max_components && placed < n; ++comp) {
         // a node without a position is one that nothing has claimed
         unsigned long long best = ~0ull;
         for (int64_t i = w.gid; i < n; i += w.threads)
             if (ld_l2(claim + i) == INT_MAX) w.take_min(best, (int32_t)i);
-        int32_t start = (int32_t)(w.min_key(best) & 0xffffffffull);
+        start = (int32_t)(w.min_key(best) & 0xffffffffull);
         if (peripheral) {
+            const int32_t first = start;
             int32_t ecc = -1, pick = start;
             for (int searches = 0; searches <= 8; ++searches) {
                 int32_t ecc2, pick2;
-                w.bfs(pick, bfs_id++, &ecc2, &pick2);
+                if (!w.bfs(pick, bfs_id++, &ecc2, &pick2)) {
+                    wide = kCmWideSearch;
+                    start = first;
+                    break;
+                }
                 if (ecc2 <= ecc) break;
                 start = pick;
                 ecc = ecc2;
                 pick = pick2;
             }
+            if (wide) break;
         }
         if (w.gid == 0) {
             claim[start] = -1;
             CmSet(w, CmNext{placed, 1, 0}, placed).set(0, start);
         }
         cluster.sync();
-        int32_t ls = placed, le = placed + 1;
+        ls = placed;
+        le = placed + 1;
         int buf = 0;
-        while (le > ls) {
+        for (int64_t level = 1; le > ls; ++level) {
             // the CTAs take equal runs of the frontier, their threads `m` consecutive positions
             // each, so that the children's order is that of a scan over CTAs and threads
             const int32_t run = ((le - ls - 1) >> log_ranks) + 1;
@@ -547,14 +584,88 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
             buf ^= 1;
             ls = le;
             le += total;
+            if (total && w.wide(le - placed, level + 1)) {
+                wide = kCmWideOrder;
+                break;
+            }
         }
         placed = le;
+        if (wide) break;
     }
     if (w.gid == 0) {
-        *placed_io = placed;
-        *bfs_id_io = bfs_id;
+        io->placed = placed;
+        io->bfs_id = bfs_id;
+        io->wide = wide;
+        io->start = start;
+        io->ls = ls;
+        io->le = le;
     }
     cluster.sync();  // no CTA leaves while another may use its shared memory
+}
+
+// ---- levels too wide for the cluster, a thread per node of the level; the same arrays ----------
+__global__ void wide_seed(int32_t r, int32_t id, int32_t *stamp, int32_t *queue, int32_t *tail) {
+    stamp[r] = id;
+    queue[0] = r;
+    *tail = 1;
+}
+
+// queue[ls, le): a BFS level; its unvisited neighbours without a position are appended
+__global__ void wide_expand(const int32_t *rp, const int32_t *ci, int32_t id, int32_t *stamp,
+                            int32_t *queue, int32_t ls, int32_t le, int32_t *tail) {
+    const int64_t i = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= le) return;
+    const int32_t u = queue[i];
+    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
+        const int32_t v = ci[k];
+        if (v != u && stamp[v] < id && atomicMax(&stamp[v], id) < id) queue[atomicAdd(tail, 1)] = v;
+    }
+}
+
+__global__ void wide_min_key(const int32_t *queue, int32_t ls, int32_t le, const int32_t *deg,
+                             unsigned long long *out) {
+    const int64_t i = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < le) atomicMin(out, node_key(deg, queue[i]));
+}
+
+__global__ void wide_start(int32_t v, int32_t at, int32_t *claim, int32_t *stamp, int32_t *perm) {
+    claim[v] = -1;
+    stamp[v] = kCmPlaced;
+    perm[at] = v;
+}
+
+__global__ void wide_claim(const int32_t *rp, const int32_t *ci, const int32_t *perm,
+                           int32_t *claim, int32_t ls, int32_t le) {
+    const int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= le) return;
+    const int32_t u = perm[p];
+    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) {
+        const int32_t v = ci[k];
+        if (v != u && claim[v] > (int32_t)p) atomicMin(&claim[v], (int32_t)p);
+    }
+}
+
+__global__ void wide_count(const int32_t *rp, const int32_t *ci, const int32_t *perm,
+                           const int32_t *claim, int32_t ls, int32_t le, int64_t *counts) {
+    const int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= le) return;
+    const int32_t u = perm[p];
+    int64_t c = 0;
+    for (int32_t k = rp[u]; k < rp[u + 1]; ++k) c += ci[k] != u && claim[ci[k]] == (int32_t)p;
+    counts[p - ls] = c;
+}
+
+__global__ void wide_place(const int32_t *rp, const int32_t *ci, const int32_t *deg,
+                           const int32_t *claim, int32_t *stamp, int32_t *perm, int32_t ls,
+                           int32_t le, const int64_t *offsets) {
+    const int64_t p = ls + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= le) return;
+    const int64_t first = offsets[p - ls];
+    const int cnt = (int)(offsets[p - ls + 1] - first);
+    if (!cnt) return;
+    int32_t *out = perm + le + first;
+    cm_sort_kids(rp, ci, deg, claim, (int32_t)p, perm[p], out);
+    for (int t = 0; t < cnt; ++t) stamp[out[t]] = kCmPlaced;
 }
 
 __global__ void reverse_kernel(int32_t n, const int32_t *src, int32_t *dst) {
@@ -567,29 +678,117 @@ __global__ void fill_i32(int32_t *p, int64_t n, int32_t v) {
     if (i < n) p[i] = v;
 }
 
+// The arrays of an order: five of n words, then the progress.
+struct CmArrays {
+    int32_t n;
+    const int32_t *rp, *ci;
+    int32_t *deg, *claim, *stamp, *queue, *perm;
+    CmProgress *progress;
+};
+
+// Component whose levels are too wide for cm_cluster, from where that left off (*g): its start node
+// if need be, then its levels to the end.
+spmv_status_t cm_wide_component(const CmArrays &a, bool peripheral, CmProgress *g,
+                                cudaStream_t st) {
+    struct Words {
+        unsigned long long key;
+        int32_t tail;
+    } h, *d = nullptr;
+    int64_t *counts = nullptr;
+    auto read = [&]() -> spmv_status_t {
+        GB_CUDA(cudaMemcpyAsync(&h, d, sizeof(Words), cudaMemcpyDeviceToHost, st));
+        GB_CUDA(cudaStreamSynchronize(st));
+        return SPMV_OK;
+    };
+    // levels from r: their number less one, and the node of the last one with the smallest key
+    auto bfs = [&](int32_t r, int32_t *ecc, int32_t *pick) -> spmv_status_t {
+        const int32_t id = g->bfs_id++;
+        wide_seed<<<1, 1, 0, st>>>(r, id, a.stamp, a.queue, &d->tail);
+        int32_t ls = 0, le = 1, last = 0;
+        *ecc = -1;
+        while (le > ls) {
+            wide_expand<<<blocks_for(le - ls), kT, 0, st>>>(a.rp, a.ci, id, a.stamp, a.queue, ls,
+                                                            le, &d->tail);
+            GB_LAUNCHED();
+            GB_TRY(read());
+            last = ls;
+            ls = le;
+            le = h.tail;
+            ++*ecc;
+        }
+        GB_CUDA(cudaMemsetAsync(&d->key, 0xff, sizeof(d->key), st));
+        wide_min_key<<<blocks_for(ls - last), kT, 0, st>>>(a.queue, last, ls, a.deg, &d->key);
+        GB_LAUNCHED();
+        GB_TRY(read());
+        *pick = (int32_t)(h.key & 0xffffffffull);
+        return SPMV_OK;
+    };
+    spmv_status_t s = [&]() -> spmv_status_t {
+        GB_CUDA(gb_malloc_async((void **)&d, sizeof(Words), st));
+        GB_CUDA(gb_malloc_async((void **)&counts, sizeof(int64_t) * ((size_t)a.n + 1), st));
+        if (g->wide == kCmWideSearch) {
+            int32_t start = g->start;
+            if (peripheral) {
+                int32_t ecc = -1, pick = start;
+                for (int searches = 0; searches <= 8; ++searches) {
+                    int32_t ecc2, pick2;
+                    GB_TRY(bfs(pick, &ecc2, &pick2));
+                    if (ecc2 <= ecc) break;
+                    start = pick;
+                    ecc = ecc2;
+                    pick = pick2;
+                }
+            }
+            wide_start<<<1, 1, 0, st>>>(start, (int32_t)g->placed, a.claim, a.stamp, a.perm);
+            GB_LAUNCHED();
+            g->ls = g->placed;
+            g->le = g->placed + 1;
+        }
+        int32_t ls = (int32_t)g->ls, le = (int32_t)g->le;
+        while (le > ls) {
+            const unsigned nb = blocks_for(le - ls);
+            wide_claim<<<nb, kT, 0, st>>>(a.rp, a.ci, a.perm, a.claim, ls, le);
+            wide_count<<<nb, kT, 0, st>>>(a.rp, a.ci, a.perm, a.claim, ls, le, counts);
+            GB_LAUNCHED();
+            GB_TRY(exclusive_scan_i64(counts, le - ls, st));
+            wide_place<<<nb, kT, 0, st>>>(a.rp, a.ci, a.deg, a.claim, a.stamp, a.perm, ls, le,
+                                          counts);
+            GB_LAUNCHED();
+            int64_t total = 0;
+            GB_CUDA(cudaMemcpyAsync(&total, counts + (le - ls), sizeof(int64_t),
+                                    cudaMemcpyDeviceToHost, st));
+            GB_CUDA(cudaStreamSynchronize(st));
+            ls = le;
+            le += (int32_t)total;
+        }
+        g->placed = le;
+        return SPMV_OK;
+    }();
+    if (d) cudaFreeAsync(d, st);
+    if (counts) cudaFreeAsync(counts, st);
+    return s;
+}
+
 spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, bool reverse,
                               bool peripheral, int32_t *perm_out, cudaStream_t st) {
     if (n == 0) return SPMV_OK;
-    // five arrays of n words, then the progress words
     int32_t *mem = nullptr;
     const size_t stride = ((size_t)n + 63) / 64 * 64;
-    GB_CUDA(gb_malloc_async((void **)&mem, sizeof(int32_t) * (5 * stride + 8), st));
-    int32_t *deg = mem, *claim = mem + stride, *stamp = mem + 2 * stride,
-            *queue = mem + 3 * stride, *cm = mem + 4 * stride;
-    int64_t *placed_d = (int64_t *)(mem + 5 * stride);
-    int32_t *bfs_id_d = mem + 5 * stride + 2, *spilled_d = mem + 5 * stride + 3;
+    GB_CUDA(gb_malloc_async((void **)&mem, sizeof(int32_t) * 5 * stride + sizeof(CmProgress), st));
+    const CmArrays a{n,          rp, ci, mem, mem + stride, mem + 2 * stride, mem + 3 * stride,
+                     mem + 4 * stride, (CmProgress *)(mem + 5 * stride)};
     spmv_status_t s = [&]() -> spmv_status_t {
         const unsigned nb = blocks_for(n);
-        degree_kernel<<<nb, kT, 0, st>>>(n, rp, ci, deg);
-        fill_i32<<<nb, kT, 0, st>>>(claim, n, INT_MAX);
-        fill_i32<<<nb, kT, 0, st>>>(stamp, n, -1);
+        degree_kernel<<<nb, kT, 0, st>>>(n, rp, ci, a.deg);
+        fill_i32<<<nb, kT, 0, st>>>(a.claim, n, INT_MAX);
+        fill_i32<<<nb, kT, 0, st>>>(a.stamp, n, -1);
         GB_LAUNCHED();
-        GB_CUDA(cudaMemsetAsync(placed_d, 0, 4 * sizeof(int32_t), st));
+        GB_CUDA(cudaMemsetAsync(a.progress, 0, sizeof(CmProgress), st));
         // 512 threads per CTA leave registers for a row's loads in flight; the frontiers of
         // larger graphs (about 10K nodes from 1.5M on) keep 1,024 busy.  Whole set-up, ms, 512 /
         // 1,024: 48K cells 2.2 / 3.1, 796K 6.6 / 8.5, 3.1M 18.5 / 17.8, 6M 34.4 / 33.7.
-        const bool wide = n >= 1500000;
-        auto *kern = wide ? cm_cluster<1024> : cm_cluster<512>;
+        const bool large = n >= 1500000;
+        auto *kern = large ? cm_cluster<1024> : cm_cluster<512>;
         GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -597,7 +796,7 @@ spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, b
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(kCmCluster);
-        cfg.blockDim = dim3(wide ? 1024 : 512);
+        cfg.blockDim = dim3(large ? 1024 : 512);
         cfg.stream = st;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
@@ -607,20 +806,23 @@ spmv_status_t cm_order_device(int32_t n, const int32_t *rp, const int32_t *ci, b
             attr[0].val.clusterDim.x = 8;  // the portable size
             cfg.gridDim = dim3(8);
         }
-        int64_t placed = 0;
-        while (placed < n) {
-            GB_CUDA(cudaLaunchKernelEx(&cfg, kern, n, rp, ci, (const int32_t *)deg,
-                                       claim, stamp, queue, cm, peripheral ? 1 : 0,
-                                       kCmComponents, placed_d, bfs_id_d, spilled_d));
-            GB_CUDA(cudaMemcpyAsync(&placed, placed_d, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                                    st));
+        CmProgress g{};
+        while (g.placed < n) {
+            GB_CUDA(cudaLaunchKernelEx(&cfg, kern, n, rp, ci, (const int32_t *)a.deg, a.claim,
+                                       a.stamp, a.queue, a.perm, peripheral ? 1 : 0, kCmComponents,
+                                       a.progress));
+            GB_CUDA(cudaMemcpyAsync(&g, a.progress, sizeof(g), cudaMemcpyDeviceToHost, st));
             GB_CUDA(cudaStreamSynchronize(st));
+            if (g.wide) {
+                GB_TRY(cm_wide_component(a, peripheral, &g, st));
+                GB_CUDA(cudaMemcpyAsync(a.progress, &g, sizeof(g), cudaMemcpyHostToDevice, st));
+            }
         }
         if (reverse)
-            reverse_kernel<<<nb, kT, 0, st>>>(n, cm, perm_out);
+            reverse_kernel<<<nb, kT, 0, st>>>(n, a.perm, perm_out);
         else
-            GB_CUDA(cudaMemcpyAsync(perm_out, cm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice,
-                                    st));
+            GB_CUDA(cudaMemcpyAsync(perm_out, a.perm, sizeof(int32_t) * n,
+                                    cudaMemcpyDeviceToDevice, st));
         GB_LAUNCHED();
         return SPMV_OK;
     }();

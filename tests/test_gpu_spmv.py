@@ -973,3 +973,47 @@ def test_gpu_cm_order_of_nodes_with_many_children(oracle, peripheral):
     A = capi.Matrix(n, rp, ci, v, reorder=capi.SPMV_REORDER_CM, peripheral=peripheral)
     ref = oracle.cm_order(rp, ci, reverse=False, peripheral=bool(peripheral))
     assert np.array_equal(A.permutation(), ref)
+
+
+def wide_graph(kind):
+    """Patterns whose levels go to the whole GPU: (row_ptr, columns)."""
+    rng = np.random.default_rng(11)
+    if kind == "one_way":        # no symmetric pattern
+        n = 50000
+        i, j = np.repeat(np.arange(n), 40), rng.integers(0, n, 40 * n)
+    elif kind == "hubs":         # nodes of 9 to 17, 40 and 300 children, in wide levels
+        n = 300000
+        size = np.array([9, 10, 11, 12, 13, 14, 15, 16, 17, 40, 300])[np.arange(5000) % 11]
+        hub = np.concatenate([[0], np.cumsum(size)])[:-1]
+        leaf = np.arange(size.sum())
+        owner = np.repeat(hub, size)
+        # the hubs hang on one root, and a few thousand random links tie the leaves
+        i = np.concatenate([owner, np.zeros(hub.size, int), rng.integers(0, n, 2 * n)])
+        j = np.concatenate([leaf, hub, rng.integers(0, n, 2 * n)])
+    else:                        # two dense components among small ones and single nodes
+        n, parts = 105000, [(0, 60000, 30), (60300, 40000, 40)]
+        i = np.concatenate([rng.integers(0, m, m * d) + a for a, m, d in parts])
+        j = np.concatenate([rng.integers(0, m, m * d) + a for a, m, d in parts])
+        path = np.arange(100300, 104000)
+        path = path[path % 37 != 0]
+        i, j = np.concatenate([i, path]), np.concatenate([j, path + 1])
+    key = np.concatenate([i * n + j, np.arange(n) * (n + 1)])
+    if kind != "one_way":
+        key = np.concatenate([key, j * n + i])
+    key = np.unique(key)
+    rp = np.zeros(n + 1, np.int64)
+    rp[1:] = np.cumsum(np.bincount(key // n, minlength=n))
+    return rp.astype(np.int32), (key % n).astype(np.int32)
+
+
+@pytest.mark.parametrize("kind", ["components", "one_way", "hubs"])
+@pytest.mark.parametrize("peripheral", [0, 1])
+def test_gpu_cm_order_of_graphs_with_wide_levels(oracle, kind, peripheral):
+    """Left by the cluster while it looks for a start node (peripheral) or between two levels of the
+    order (not), finished by the whole GPU, and taken up again for the next component."""
+    rp, ci = wide_graph(kind)
+    n = rp.size - 1
+    A = capi.Matrix(n, rp, ci, np.ones(ci.size), reorder=capi.SPMV_REORDER_CM,
+                    peripheral=peripheral)
+    ref = oracle.cm_order(rp, ci, reverse=False, peripheral=bool(peripheral))
+    assert np.array_equal(A.permutation(), ref)
