@@ -684,7 +684,7 @@ def test_spmm_products_that_wait_for_one_another(dtype, k, form):
                                63, 64])
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_spmm_any_column_count(oracle, dtype, k, bits):
-    """Products whose rows are gathered in pieces of 4 to 32 bytes, one to three per lane: ragged
+    """Products whose rows are gathered in pieces of 4 to 32 bytes, one to five per lane: ragged
     rows (0 to 17 entries, so every remainder of the load rounds), a row count that is no
     multiple of a warp's rows or of a slice, warps whose rows lie in two slices; bit-exact."""
     n = 1237
@@ -1017,3 +1017,31 @@ def test_gpu_cm_order_of_graphs_with_wide_levels(oracle, kind, peripheral):
                     peripheral=peripheral)
     ref = oracle.cm_order(rp, ci, reverse=False, peripheral=bool(peripheral))
     assert np.array_equal(A.permutation(), ref)
+
+
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("which", ["X", "Y", "both"])
+@pytest.mark.parametrize("k", [2, 6, 12, 20, 24, 40, 48, 56, 64])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_spmm_pieces_of_16_byte_aligned_blocks(oracle, dtype, k, which, bits):
+    """Rows that are a multiple of 16 or 32 bytes with X, Y or both 16 bytes past a 32-byte boundary
+    are gathered and stored in 16-byte pieces: bit-exact, and nothing beside Y is written."""
+    n = 1237
+    m = ragged_matrix(n, seed=k, max_len=17)
+    X = np.random.default_rng(k).uniform(-1, 1, (n, k)).astype(dtype)
+    A = capi.Matrix(n, m.row_ptr, m.col_idx, m.values, precision=capi.SPMV_PREC_DUAL,
+                    index_bits=bits, slice_height=32)
+    off, size = 16 // X.itemsize, n * k
+    dt = torch.float64 if dtype == np.float64 else torch.float32
+    xb = torch.full((size + 2 * off,), float("nan"), dtype=dt, device="cuda")
+    yb = torch.full((size + 2 * off,), float("nan"), dtype=dt, device="cuda")
+    xo, yo = (0 if which == "Y" else off), (0 if which == "X" else off)
+    Xd, Y = xb[xo:xo + size].view(n, k), yb[yo:yo + size].view(n, k)
+    assert (Xd.data_ptr() % 32 == 16) == (which != "Y")
+    assert (Y.data_ptr() % 32 == 16) == (which != "X")
+    Xd.copy_(dev(X))
+    A.apply_multi(Xd, Y)
+    torch.cuda.synchronize()
+    ref = oracle.spmm(m.row_ptr, m.col_idx, m.values.astype(dtype), X, use_fma=True)
+    assert np.array_equal(Y.cpu().numpy(), ref)
+    assert torch.isnan(yb[:yo]).all() and torch.isnan(yb[yo + size:]).all()
