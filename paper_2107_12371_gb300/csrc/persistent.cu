@@ -180,8 +180,8 @@ __device__ __forceinline__ void st_pair(float *p, float z, float v) {
 
 // RES: the resident form.  Otherwise vectors and matrix are streamed from L2 / HBM; `own` there
 // says that each thread's product rows are its sweep rows (q needs no publishing).
-template <typename T, int R, int L, typename ColT, int UU, bool RES, bool PAIRS, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1)
+template <typename T, int R, int L, typename ColT, int UU, bool RES, bool PAIRS, int THREADS, int CTAS = 1>
+__global__ void __launch_bounds__(THREADS, CTAS)
 cg_persistent(PersArgs<T> a, ColT col) {
     __shared__ PersSmem<T> sm;
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -475,9 +475,17 @@ static spmv_status_t run_persistent(spmv_matrix_t A, PersArgs<T> a, const cg_opt
                 const size_t room = device_facts().max_smem_optin - sizeof(PersSmem<T>) - 1024;
                 if (a.same && a.pq.single() && need <= room) {
                     const bool pairs = threads <= 512;
-                    kern = pairs ? (const void *)cg_persistent<T, R, L, ColT, 5, true, true, 512>
-                                 : (const void *)cg_persistent<T, R, L, ColT, 5, true, false,
-                                                               1024>;
+                    // CTAs of up to 128 threads take the registers of five entries in flight
+                    // (up to 128 a thread); larger ones three at 64 registers, so that the SMs hold the
+                    // kernels of several streams: solves/s of 1 / 4 / 16 host threads, five and
+                    // three: 48K rows 435 / 835 / 894 and 431 / 1,273 / 1,480, 118K rows 261 / 303
+                    // / 300 and 270 / 467 / 464 (256-thread CTAs that streamed the matrix: 243 /
+                    // 850 / 1,099 and 185 / 322 / 430)
+                    kern = pairs && threads <= 128
+                               ? (const void *)cg_persistent<T, R, L, ColT, 5, true, true, 512>
+                           : pairs
+                               ? (const void *)cg_persistent<T, R, L, ColT, 3, true, true, 512, 2>
+                               : (const void *)cg_persistent<T, R, L, ColT, 5, true, false, 1024>;
                     if (pairs) {
                         DevBuf<T> &zp = pair_buffer(w, T{});
                         if (!zp.p) GB_TRY(zp.alloc(2 * (size_t)A->n, &A->bytes));

@@ -154,6 +154,24 @@ def test_iteration_grids_at_their_edges(oracle, rows_per_sm, extra, width, mixed
     assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b)
 
 
+@pytest.mark.parametrize("mixed", [0, 1])
+@pytest.mark.parametrize("extra", [0, 1])
+@pytest.mark.parametrize("width", [1, 3, 5, 7, 25])
+def test_resident_solves_on_both_sides_of_128_threads(width, extra, mixed):
+    """Up to 128 threads per CTA the resident form gathers five entries of a row at once, above
+    three (rows of one entry to several rounds of either, with and without a remainder): the
+    persistent solve equals the graph path bit for bit."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = (512 if mixed else 256) * sms + extra
+    rp, ci, v = banded(n, width)
+    b = np.random.default_rng(n + width).uniform(-1, 1, n)
+    A = capi.Matrix(n, rp, ci, v, precision=capi.SPMV_PREC_DUAL)
+    x1, r1 = solve(A, b, rtol=1e-10, mixed=mixed)
+    x2, r2 = solve(A, b, rtol=1e-10, mixed=mixed, persistent=1)
+    assert r1["status"] == r2["status"] == capi.SPMV_OK, (r1, r2)
+    assert r1["iterations"] == r2["iterations"] and np.array_equal(x1, x2)
+
+
 def test_concurrent_persistent_solves_of_different_sizes(oracle):
     """Host threads that launch the persistent kernel for handles of different sizes (so with
     different amounts of shared memory) on streams of their own do not disturb each other."""
