@@ -23,8 +23,10 @@ int cg_grid(int32_t n);
 // entries in flight (a whole row of the tetrahedral meshes) at 1,024 threads per SM and 64
 // registers -- measured on the 6M-row mesh against two entries at 1,536 threads (40
 // registers): FP64 CG 185 -> 176 us per iteration, the FP32 refinement solve 4.7 % faster;
-// wider lanes keep two entries, and so do matrices whose widest slice needs fewer load
-// rounds that way (load_rounds).
+// wider lanes keep two entries, and so do matrices whose widest slice has no fewer load_rounds in
+// fives than in twos.  (That count charges a round's missing entries, which are masked here but
+// still take the FP64 pipe: us per FP64 iteration of 3M rows, two / five in flight, rows of 3
+// entries 82 / 88, 4 85 / 90, 8 107 / 113, 9 117 / 115, 5 95 / 88.)
 constexpr int kIterThreads = 1024;
 constexpr int pq_min_ctas(int value_bytes) { return value_bytes >= 64 ? 3 : 4; }
 constexpr int pq_unroll(int value_bytes) { return value_bytes <= 16 ? 5 : 2; }
@@ -327,7 +329,7 @@ __device__ __forceinline__ void store_parts(const IterSlot<Q> &slot, int threads
 // SM's 2-per-clock pipe in 3 us.
 template <typename T>
 struct StepScalars {
-    double rho, rr;
+    double rr;
     T coef;    // alpha, or beta
     int done;  // 0, or the reason to stop after this step (CgScalars::done)
 };
@@ -341,7 +343,6 @@ __device__ __forceinline__ void step_alpha(double rho, double pq, StepScalars<T>
 // beta = r.z / rho, from the sums r.z and r.r
 template <typename T>
 __device__ __forceinline__ void step_beta(double rho, double rz, StepScalars<T> &s) {
-    s.rho = rz;
     s.coef = (T)(rz / rho);
 }
 __device__ __forceinline__ int step_done(double rr, double limit, int iters, int max_iter) {

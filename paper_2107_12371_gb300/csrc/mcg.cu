@@ -191,7 +191,7 @@ __device__ __forceinline__ void cta_cols_fx(const E (&v)[NQ][V], ColsSmem<E, CG,
     for (int qc = warp; qc < NQ * KP; qc += (int)blockDim.x >> 5) {
         const int q = qc / KP, c = qc % KP;
         const E *src = sm.v[q * V + c % V] + (c / V) * ColsSmem<E, CG, V, NQ>::kPitch;
-        // at most 512 / 32 values per lane, eight at a time
+        // at most 1,024 / 32 values per lane, eight at a time
         constexpr int M = 8;
         double s = 0.0;
         for (int i0 = 0; i0 < per; i0 += 32 * M) {

@@ -11,9 +11,8 @@
 // library is loaded if CUDA_MODULE_LOADING=EAGER; from then on the device holds it until the
 // process exits.  Systems up to kNoallocMaxRows rows fit.
 //
-// The iteration is the one of cg_solve (Jacobi-preconditioned CG, last-CTA reductions in a
-// fixed order, true-residual check with at most two restarts), with a thread-per-row CSR
-// product instead of the sliced-ELLPACK one.
+// The recurrence is cg_solve's (Jacobi-preconditioned CG, true-residual check with at most two
+// restarts), on a thread-per-row CSR product, with last-CTA reductions in a fixed order.
 #include <cuda.h>
 
 #include <chrono>

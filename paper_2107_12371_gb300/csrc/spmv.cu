@@ -130,8 +130,9 @@ spmv_sell_occ(int32_t n, int32_t n_slices, const int64_t *__restrict__ sp, ColT 
 // SM (four entries in flight), 77.1 us with four entries and 68.3 us with two at six CTAs.  A
 // dependent launch, as are the other two: 68.1 -> 66.3 us in a stream of products with the wait
 // first thing in the kernel; behind the first requests for entries it cost 69.6.  AHEAD (a matrix of
-// more than twice the L2): 66.3 -> 63.2 us, 88 % of what HBM gives a copy; where the product before
-// leaves a good part of the matrix in L2 it costs more than it saves (3.7M rows 39.7 -> 41.3).
+// more than twice the L2): 66.3 -> 62.9 us, the 396 MB that the product cannot do without at 93 % of
+// the copy rate; where the product before leaves a good part of the matrix in L2 it costs more than
+// it saves (3.7M rows 39.7 -> 41.3).
 constexpr int kGsBlock = 256;
 constexpr int kGsCtasPerSm = 4;
 template <typename T, int R, int L, int U, typename ColT, bool AXPBY, bool AHEAD>
