@@ -335,8 +335,8 @@ IterGrid cg_iter_grid(int64_t items, int max_threads) {
     return g;
 }
 
-IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes) {
-    const double l2 = device_facts().l2_bytes;
+IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes, int solves) {
+    const double l2 = (double)device_facts().l2_bytes / solves;
     const double vectors = 5.0 * elem_bytes * A->n;
     const double matrix = (double)A->sell_entries * (elem_bytes + A->index_bits / 8);
     return {matrix + vectors <= 0.75 * l2, vectors <= 0.5 * l2};
@@ -428,7 +428,7 @@ static spmv_status_t with_cols(spmv_matrix_t A, F &&f) {
 // How the kernels of an iteration are run: by themselves (a CTA per SM), or beside other solves.
 // There a CTA that fills an SM waits for one to be empty and then keeps the other streams' kernels
 // out, so those of more than kSplitThreads threads are run by four smaller ones each, the sweeps
-// at 32 registers, and nothing is kept in an L2 that several solves share.  Each thread of the grid
+// at 32 registers, and the L2 hints go by an equal share of it.  Each thread of the grid
 // does what it does otherwise and the sums are formed from the same warps' (store_parts), so the
 // bits are the same.  Measured, whole kernels / four 256-thread CTAs per SM with last-CTA
 // reductions and FP64 shuffle trees / this form: saturated stream of 700 requests (1e4 to 2e6
@@ -441,17 +441,20 @@ static spmv_status_t with_cols(spmv_matrix_t A, F &&f) {
 // plainly (p99 of the stream at 75/s with the requests of 256 MB and more prioritised 187 -> 141 ms;
 // at equal priority dependent launches have the better p99, 145 against 152).
 enum class IterForm { kAlone, kBeside, kYield };
+struct IterMode {
+    IterForm form = IterForm::kAlone;
+    int solves = 1;  // in progress, this one among them
+};
 constexpr int kSplit = 4, kSplitThreads = 512;
 
 struct IterLaunch {
     IterGrid g;
     IterKeep keep;
     bool split, dependent;
-    IterLaunch(const spmv_matrix_t A, IterForm form, const IterGrid &grid, int elem_bytes)
-        : g(grid), keep(cg_keep(A, elem_bytes)) {
-        split = form != IterForm::kAlone && g.threads > kSplitThreads;
-        dependent = form != IterForm::kYield || g.single();
-        if (form != IterForm::kAlone) keep = {false, false};
+    IterLaunch(const spmv_matrix_t A, IterMode mode, const IterGrid &grid, int elem_bytes)
+        : g(grid), keep(cg_keep(A, elem_bytes, mode.solves)) {
+        split = mode.form != IterForm::kAlone && g.threads > kSplitThreads && A->cg.split.p;
+        dependent = mode.form != IterForm::kYield || g.single();
     }
     unsigned ctas() const { return (unsigned)(split ? g.ctas * kSplit : g.ctas); }
     unsigned threads() const {
@@ -462,13 +465,13 @@ struct IterLaunch {
 // the product, the x/r sweep and the p sweep of an iteration (pq_count: CTAs of the product)
 template <typename T>
 static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q, CgScalars *sc,
-                                IterForm form, cudaStream_t st, int *pq_count) {
+                                IterMode mode, cudaStream_t st, int *pq_count) {
     return with_cols(A, [&](auto cols) -> spmv_status_t {
         using ColT = decltype(cols);
         return with_shape<T>(A->S, [&](auto rt, auto lt) -> spmv_status_t {
             constexpr int R = decltype(rt)::value, L = decltype(lt)::value;
             constexpr int UU = pq_unroll((int)sizeof(T) * R);
-            const IterLaunch l(A, form, cg_pq_grid(A, L, (int)sizeof(T) * R), sizeof(T));
+            const IterLaunch l(A, mode, cg_pq_grid(A, L, (int)sizeof(T) * R), sizeof(T));
             *pq_count = l.g.ctas;
             auto go = [&](auto *kern) {
                 return launch_ordered(l.dependent, kern, l.ctas(), l.threads(), st, A->n,
@@ -486,8 +489,8 @@ static spmv_status_t enqueue_pq(spmv_matrix_t A, const T *val, const T *p, T *q,
 }
 template <typename T>
 static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const T *p, const T *q,
-                                const T *dinv, CgScalars *sc, IterForm form, cudaStream_t st) {
-    const IterLaunch l(A, form, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
+                                const T *dinv, CgScalars *sc, IterMode mode, cudaStream_t st) {
+    const IterLaunch l(A, mode, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
     auto *kern = l.split        ? cg_update_xr<T, false, kSplit>
                  : l.g.single() ? cg_update_xr<T, true, 1>
                                 : cg_update_xr<T, false, 1>;
@@ -497,8 +500,8 @@ static spmv_status_t enqueue_xr(spmv_matrix_t A, int pq_count, T *x, T *r, const
 }
 template <typename T>
 static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p, CgScalars *sc,
-                               IterForm form, cudaStream_t st) {
-    const IterLaunch l(A, form, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
+                               IterMode mode, cudaStream_t st) {
+    const IterLaunch l(A, mode, cg_sweep_grid(A, Vec16<T>::n), sizeof(T));
     auto *kern = l.split        ? cg_update_p<T, false, kSplit>
                  : l.g.single() ? cg_update_p<T, true, 1>
                                 : cg_update_p<T, false, 1>;
@@ -508,29 +511,29 @@ static spmv_status_t enqueue_p(spmv_matrix_t A, const T *r, const T *dinv, T *p,
 }
 template <typename T>
 static spmv_status_t enqueue_iterations(spmv_matrix_t A, int iters, const T *val, T *x, T *r, T *p,
-                                        T *q, const T *dinv, CgScalars *sc, IterForm form,
+                                        T *q, const T *dinv, CgScalars *sc, IterMode mode,
                                         cudaStream_t st) {
     for (int it = 0; it < iters; ++it) {
         int pq_count = 0;
-        GB_TRY(enqueue_pq<T>(A, val, p, q, sc, form, st, &pq_count));
-        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, form, st));
-        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, form, st));
+        GB_TRY(enqueue_pq<T>(A, val, p, q, sc, mode, st, &pq_count));
+        GB_TRY(enqueue_xr<T>(A, pq_count, x, r, p, q, dinv, sc, mode, st));
+        GB_TRY(enqueue_p<T>(A, r, dinv, p, sc, mode, st));
     }
     return SPMV_OK;
 }
 
 // enqueue `iters` FP64 iterations, or FP32 ones of a refinement's inner solve (3 kernels each)
 static spmv_status_t enqueue_cg64(spmv_matrix_t A, int iters, cudaStream_t st,
-                                  IterForm form = IterForm::kAlone) {
+                                  IterMode mode = {}) {
     CgWork &w = A->cg;
     return enqueue_iterations<double>(A, iters, A->sell_val.p, w.x.p, w.r.p, w.p.p, w.q.p,
-                                      w.dinv.p, outer_scalars(A), form, st);
+                                      w.dinv.p, outer_scalars(A), mode, st);
 }
 static spmv_status_t enqueue_cg32(spmv_matrix_t A, int iters, cudaStream_t st,
-                                  IterForm form = IterForm::kAlone) {
+                                  IterMode mode = {}) {
     CgWork &w = A->cg;
     return enqueue_iterations<float>(A, iters, A->sell_val32.p, w.d32.p, w.r32.p, w.p32.p, w.q32.p,
-                                     w.dinv32.p, inner_scalars(A), form, st);
+                                     w.dinv32.p, inner_scalars(A), mode, st);
 }
 
 __global__ void fill_value(int32_t n, double *v, double value) {
@@ -574,8 +577,7 @@ static spmv_status_t tune_cg_product(spmv_matrix_t A, cudaStream_t st) {
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e0, st));
                 int count = 0;
                 if (s == SPMV_OK)
-                    s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, IterForm::kAlone, st,
-                                           &count);
+                    s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, {}, st, &count);
                 if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e1, st));
                 if (s == SPMV_OK) s = cuda_status(cudaEventSynchronize(e1));
                 if (s == SPMV_OK && i >= 0) s = cuda_status(cudaEventElapsedTime(&t[i], e0, e1));
@@ -696,11 +698,11 @@ static bool cancelled(const std::atomic<int> *cancel) {
     return cancel && cancel->load(std::memory_order_relaxed) != 0;
 }
 
-// The form of the next batch of directly launched iterations.
-static IterForm iter_form(const spmv_matrix_t A, const SolveControl &ctl) {
-    if (!A->cg.split.p || ctl.running->load(std::memory_order_relaxed) < 2)
-        return IterForm::kAlone;
-    return ctl.high_priority ? IterForm::kYield : IterForm::kBeside;
+// How the next batch of directly launched iterations runs.
+static IterMode iter_mode(const SolveControl &ctl) {
+    const int solves = ctl.running ? ctl.running->load(std::memory_order_relaxed) : 1;
+    if (solves < 2) return {};
+    return {ctl.high_priority ? IterForm::kYield : IterForm::kBeside, solves};
 }
 
 // read both scalar blocks to the host
@@ -741,7 +743,7 @@ static spmv_status_t solve64(spmv_matrix_t A, const double *b, const cg_options_
             if (ctl.graphs) GB_TRY(get_graph(A, false, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg64(A, batch, st, iter_form(A, ctl)));
+                else GB_TRY(enqueue_cg64(A, batch, st, iter_mode(ctl)));
                 GB_TRY(read_scalars(A, st, &h, nullptr));
                 if (h.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -834,7 +836,7 @@ static spmv_status_t solve_mixed(spmv_matrix_t A, const double *b, const cg_opti
             if (ctl.graphs) GB_TRY(get_graph(A, true, batch, &g));
             for (;;) {
                 if (g) GB_CUDA(cudaGraphLaunch(g, st));
-                else GB_TRY(enqueue_cg32(A, batch, st, iter_form(A, ctl)));
+                else GB_TRY(enqueue_cg32(A, batch, st, iter_mode(ctl)));
                 GB_TRY(read_scalars(A, st, nullptr, &hi));
                 if (hi.done || cancelled(cancel)) break;
                 if (o.timeout_s > 0 && seconds_since(t0) > o.timeout_s) break;
@@ -936,12 +938,11 @@ spmv_status_t cg_timing(spmv_matrix_t A, int iters, double *out, cudaStream_t st
             s = cuda_status(cudaEventRecord(e[0], st));
             if (s != SPMV_OK) break;
             if (k == 0)
-                s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, IterForm::kAlone, st,
-                                       &pq_count);
+                s = enqueue_pq<double>(A, A->sell_val.p, w.p.p, w.q.p, sc, {}, st, &pq_count);
             else if (k == 1)
                 s = enqueue_xr<double>(A, pq_count, w.x.p, w.r.p, w.p.p, w.q.p, w.dinv.p, sc,
-                                       IterForm::kAlone, st);
-            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, IterForm::kAlone, st);
+                                       {}, st);
+            else s = enqueue_p<double>(A, w.r.p, w.dinv.p, w.p.p, sc, {}, st);
             if (s == SPMV_OK) s = cuda_status(cudaEventRecord(e[1], st));
             if (s == SPMV_OK) s = elapsed(&ms);
             sum[k] += ms;
@@ -1023,7 +1024,9 @@ spmv_status_t gb::cg_solve_ex(spmv_matrix_t A, const double *b, double *x,
     NvtxRange nvtx(o.mixed ? "cg_solve/mixed" : "cg_solve/fp64");
     const auto t0 = Clock::now();
     spmv_status_t s = ensure_cg_work(A, o.mixed != 0, st);
-    if (s == SPMV_OK && ctl.running && !A->cg.split.p) {
+    // (a grid of a row per thread has at least the threads of any other)
+    if (s == SPMV_OK && ctl.running && !A->cg.split.p &&
+        cg_iter_grid((int64_t)A->n_slices * A->S, kIterThreads).threads > kSplitThreads) {
         s = A->cg.split.alloc(1, &A->bytes);
         if (s == SPMV_OK)
             s = cuda_status(cudaMemsetAsync(A->cg.split.p, 0, sizeof(SplitSums), st));

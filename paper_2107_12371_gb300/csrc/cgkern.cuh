@@ -79,7 +79,7 @@ struct IterSlot {
 struct IterKeep {
     bool matrix, vectors;
 };
-IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes);
+IterKeep cg_keep(const spmv_matrix_t A, int elem_bytes, int solves = 1);  // that share the L2
 
 IterGrid cg_iter_grid(int64_t items, int max_threads);
 IterGrid cg_pq_grid(const spmv_matrix_t A, int L, int value_bytes);
