@@ -136,7 +136,7 @@ struct CmWalk {
     const int32_t *rp, *ci, *deg;
     int32_t *claim, *stamp, *queue, *perm;
     int32_t *spilled;  // BFS nodes in `queue`, those that found their CTA's frontier full
-    int row;           // mean row entries
+    int row, limit;    // mean row entries; nodes of a level of kCmWide of them
     CmKeys *keys;
     CmFrontier *front;
     cg::cluster_group cluster;
@@ -183,9 +183,10 @@ struct CmWalk {
         return best;
     }
 
-    // Whether `levels` levels of `nodes` nodes together are too wide for the cluster.
-    __device__ __forceinline__ bool wide(int64_t nodes, int64_t levels_) const {
-        return nodes * row > kCmWide * levels_;
+    // Whether `levels_` levels of `nodes` nodes together, `last` of them in the last, are too wide for
+    // the cluster (the average passes kCmWide at a level that does).
+    __device__ __forceinline__ bool wide(int32_t last, int64_t nodes, int32_t levels_) const {
+        return last > limit && nodes * row > kCmWide * levels_;
     }
 
     // BFS levels from r over nodes without a position: the number of levels, and the node of
@@ -239,7 +240,8 @@ struct CmWalk {
         };
         int last = 0;  // the same of the level before
         int32_t last_ls = 0;
-        int64_t seen = 0;  // nodes of the levels so far
+        int size = 0;      // nodes of the last level, and of all so far
+        int64_t seen = 0;
         for (bool first = true;; first = false) {
             const int w = levels % 3;
             // how many nodes the level has is needed only once it has been visited
@@ -254,10 +256,11 @@ struct CmWalk {
                       w);
             if (threadIdx.x == 0) front->count[(levels + 1) % 3] = front->full[(levels + 1) % 3] = 0;
             cluster.sync();
-            const int size = __reduce_add_sync(0xffffffffu, sent);
-            if (size == 0) break;
+            if (!__any_sync(0xffffffffu, sent > 0)) break;
+            // (the level's size is looked at a level later, so that nothing waits for it)
+            if (wide(size, seen, depth)) return false;
+            size = __reduce_add_sync(0xffffffffu, sent);
             seen += size;
-            int64_t known = seen;
             last = mine;
             last_ls = ls;
             const int own = front->count[w];
@@ -266,11 +269,11 @@ struct CmWalk {
             if (front->full[w]) {
                 const int all = lane < ranks ? cluster.map_shared_rank(front, lane)->count[w] : 0;
                 le += __reduce_add_sync(0xffffffffu, all > kCmQueue ? all - kCmQueue : 0);
-                known += __reduce_add_sync(0xffffffffu, all);
+                const int next = __reduce_add_sync(0xffffffffu, all);
+                if (wide(next, seen + next, depth + 1)) return false;
             }
             ++depth;
             ++levels;
-            if (wide(known, depth)) return false;
         }
         // the level after the last one was empty
         unsigned long long best = ~0ull;
@@ -444,7 +447,8 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
     const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < 3) front.count[threadIdx.x] = front.full[threadIdx.x] = 0;
-    CmWalk w{n, rp, ci, deg, claim, stamp, queue, perm, &io->spilled, rp[n] / n + 1, &keys, &front,
+    CmWalk w{n, rp, ci, deg, claim, stamp, queue, perm, &io->spilled, rp[n] / n + 1,
+             (int)(kCmWide / (rp[n] / n + 1)), &keys, &front,
              cluster,
              (int64_t)threadIdx.x * ranks + rank, (int64_t)ranks * THREADS, 0, 0};
     int32_t placed = (int32_t)io->placed;
@@ -485,7 +489,7 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
         ls = placed;
         le = placed + 1;
         int buf = 0;
-        for (int64_t level = 1; le > ls; ++level) {
+        for (int32_t level = 1; le > ls; ++level) {
             // the CTAs take equal runs of the frontier, their threads `m` consecutive positions
             // each, so that the children's order is that of a scan over CTAs and threads
             const int32_t run = ((le - ls - 1) >> log_ranks) + 1;
@@ -584,7 +588,7 @@ cm_cluster(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *deg, 
             buf ^= 1;
             ls = le;
             le += total;
-            if (total && w.wide(le - placed, level + 1)) {
+            if (w.wide(total, le - placed, level + 1)) {
                 wide = kCmWideOrder;
                 break;
             }
